@@ -353,7 +353,16 @@ void launch_syrk_fp64(Ctx *ctx, const double *A, int64_t m, int64_t n, int64_t l
 size_t syrk_fp64_scratch_bytes(int64_t m, int64_t n, int num_sms);
 void launch_syrk_fp64_ws(cudaStream_t s, int num_sms, const double *A, int64_t m, int64_t n,
                          int64_t lda, const double *w, double beta, double *C, int64_t ldc,
-                         double *work, int bm = 0);
+                         double *work, int bm = 0, void *rns_ws = nullptr);
+// The same product by residue numbers on the tensor cores (syrk_rns.cu), the
+// faster form from syrk_rns_pays on; ws as syrk_rns_workspace_bytes.  The
+// returned device flag is nonzero afterwards when the operands were outside
+// its range and C is untouched.
+bool syrk_rns_pays(int64_t m, int64_t n);
+size_t syrk_rns_workspace_bytes(int64_t m, int64_t n, int num_sms);
+inline const int *syrk_rns_err(const void *ws) { return static_cast<const int *>(ws) + 1; }   // nonzero: a wait expired
+const int *launch_syrk_rns(cudaStream_t s, int num_sms, const double *A, int64_t m, int64_t n, int64_t lda,
+                           const double *w, double beta, double *C, int64_t ldc, void *ws);
 
 // Tensor-core SYRK (syrk_tc.cu)
 struct TcPlan {

@@ -110,7 +110,8 @@ struct Problem {
     DBuf bgrad, bgrad_t, bcg, bcg_t, bch, bch_t, bgl, bATy, bJdh, bHss, bHdd;
     DBuf bsig_x, bq, bsig_d, bw, bbt_g, bu, bATu, brhs, bAdx;
     // reduced matrix and factors
-    DBuf bS, bL, bDd, bDoff, bperm, bkind, binertia, bldlt_ws, berr, bsyrk_ws, btune;
+    DBuf bS, bL, bDd, bDoff, bperm, bkind, binertia, bldlt_ws, berr, bsyrk_ws, brns_ws, btune;
+    bool rns_oom = false;   // the residue workspace did not fit once: the DFMA product from then on
     // tensor-core condensation and refinement
     DBuf bAfT, bvf, btc_ws, btc_err, bref_b, bref_u, bref_r, bref_d, btmp_nd2, bsolve_ws, bsolve_err, bAu_run;
     DBuf bcpre, bcw, bwf, bATv, bAsd;   // the refinement's fused residual pass
@@ -704,13 +705,31 @@ static int tuned_syrk_tile(Problem *P) {
     int v = 0;
     if (tune_get(TUNE_SYRK_TILE, D.m_E, D.n_d, &v)) return v;
     double *C = P->btune.get<double>(P->ctx, (size_t)std::max<int64_t>(D.n_d * D.n_d, 1));
-    v = tune_pick(P, {64, 80}, [&](int bm) {
+    v = tune_pick(P, D.n_d <= 64 ? std::vector<int>{32, 64} : std::vector<int>{64, 80}, [&](int bm) {
         launch_syrk_fp64_ws(P->ctx->stream, P->ctx->num_sms, P->Mv.A, D.m_E, D.n_d, D.lda, P->bw.as<double>(),
                             0.0, C, D.n_d, P->bsyrk_ws.as<double>(), bm);
     });
     P->btune.reset();
     tune_put(TUNE_SYRK_TILE, D.m_E, D.n_d, v);
     return v;
+}
+
+// Workspace of the residue form of the FP64 product, allocated at its first
+// use (a mixed-precision problem needs it only when a step falls back to the
+// FP64 product); null where that form does not pay or does not fit.
+static void *rns_workspace(Problem *P) {
+    const Dims &D = P->D;
+    if (P->rns_oom || !syrk_rns_pays(D.m_E, D.n_d)) return nullptr;
+    if (!P->brns_ws.ptr) {
+        try {
+            P->brns_ws.get<char>(P->ctx, syrk_rns_workspace_bytes(D.m_E, D.n_d, P->ctx->num_sms));
+        } catch (const Error &e) {
+            if (e.status != MDSIP_ERR_OOM) throw;
+            P->rns_oom = true;
+            return nullptr;
+        }
+    }
+    return P->brns_ws.ptr;
 }
 
 // Run the factorization phase `enqueue` on the problem's stream: eagerly on
@@ -815,6 +834,7 @@ static Inertia factor_attempt(Problem *P, double dw, double dc, bool force_fp64 
     const bool p2 = P->path == MDSIP_PATH_P2;
     double *sig_x = P->bsig_x.as<double>(), *q = P->bq.as<double>(), *sig_d = P->bsig_d.as<double>(),
            *w = P->bw.as<double>(), *S = P->bS.as<double>();
+    const int *rns_err = nullptr;
     MDSIP_CUDA(cudaEventRecord(P->ev[0], st));
     P->V.newton_diag(P->I, P->bHss.as<double>(), dw, dc, p2, sig_x, q, sig_d, w, sc + SC_DIAG);
     if (p2) {
@@ -831,10 +851,12 @@ static Inertia factor_attempt(Problem *P, double dw, double dc, bool force_fp64 
             launch_syrk_tc(st, P->ctx->num_sms, (int)P->opt.precision, P->bAfT.as<float>(), D.m_E, D.n_d, w,
                            1.0, S, P->N, P->btc_ws.ptr, P->btc_err.as<int>());
         } else {
-            const int bm = tuned_syrk_tile(P);
+            void *rns = rns_workspace(P);
+            const int bm = rns ? 0 : tuned_syrk_tile(P);
             MDSIP_CUDA(cudaEventRecord(P->ev[8], st));   // the tile choice's trial runs are not the product
             launch_syrk_fp64_ws(st, P->ctx->num_sms, P->Mv.A, D.m_E, D.n_d, D.lda, w, 1.0, S, P->N,
-                                P->bsyrk_ws.as<double>(), bm);
+                                P->bsyrk_ws.as<double>(), bm, rns);
+            rns_err = rns ? syrk_rns_err(rns) : nullptr;
         }
         MDSIP_CUDA(cudaEventRecord(P->ev[9], st));
     } else {
@@ -863,9 +885,10 @@ static Inertia factor_attempt(Problem *P, double dw, double dc, bool force_fp64 
     MDSIP_CUDA(cudaMemcpyAsync(P->hint + 4, P->berr.ptr, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     const bool tc = p2 && P->opt.precision != MDSIP_PREC_FP64 && !force_fp64;
     if (tc) MDSIP_CUDA(cudaMemcpyAsync(P->hint + 5, P->btc_err.ptr, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+    if (rns_err) MDSIP_CUDA(cudaMemcpyAsync(P->hint + 5, rns_err, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
     P->sync_scalars();
     MDSIP_REQUIRE(P->hint[4] == 0, MDSIP_ERR_DEVICE, "LDL^T: a bounded device wait expired");
-    MDSIP_REQUIRE(!tc || P->hint[5] == 0, MDSIP_ERR_DEVICE, "tensor-core product: a bounded device wait expired");
+    MDSIP_REQUIRE((!tc && !rns_err) || P->hint[5] == 0, MDSIP_ERR_DEVICE, "tensor-core product: a bounded device wait expired");
     float a = 0, b = 0, c = 0;
     cudaEventElapsedTime(&a, P->ev[0], P->ev[1]);
     cudaEventElapsedTime(&b, P->ev[1], P->ev[2]);

@@ -4,11 +4,15 @@
 //     C[p][q] = beta C[p][q] + sum_i A[i][p] A[i][q] / w_i        (p >= q)
 //
 // A is m x n row-major (the dense Jacobian block J_{x_d} g), C column-major.
-// GB300 FP64 runs on the SIMT DFMA pipe only (about 2 DFMA per clock per SM),
-// so the kernel is arranged to keep that pipe saturated with useful FMAs:
-// 64x64 or 80x80 output tiles of the lower triangle (whichever executes the
-// fewest FMAs on the ragged edge and the diagonal tiles), 4x4 or 5x5
-// accumulators per thread, 16-row K slabs staged in shared memory with
+// Two forms.  Where the product is large the residue form of syrk_rns.cu runs
+// on the tensor cores (syrk_rns_pays); the kernel here takes the small ones,
+// and the operands outside that form's range (the launch is gated on its
+// device flag).  FP64 on the SIMT DFMA pipe runs at about 2 DFMA per clock
+// per SM, so this kernel is arranged to keep that pipe saturated with useful
+// FMAs: 64x64 or 80x80 output tiles of the lower triangle (whichever executes
+// the fewest FMAs on the ragged edge and the diagonal tiles; 32x32 up to order
+// 64, whose few tiles would leave SMs idle), 4x4, 5x5 or 2x2 accumulators per
+// thread, 16-row K slabs staged in shared memory with
 // 16-byte loads and register prefetch, the reciprocals 1/w computed once per
 // call, diagonal tiles skipping the accumulators that hold only entries above
 // the diagonal, and split-K chosen so that the (tile, split) work items fill
@@ -35,6 +39,7 @@ struct SyrkArgs {
     double *C;         // final output (nsplit == 1)
     int64_t ldc;
     double *work;      // nsplit x n x n partials (nsplit > 1)
+    const int *gate;   // null, or a device flag: zero = the product is already formed
 };
 
 __device__ __forceinline__ void tile_of(int t, int &tp, int &tq) {
@@ -55,6 +60,7 @@ __global__ void __launch_bounds__(SYRK_THREADS, 2) k_syrk_fp64(SyrkArgs a) {
     constexpr int LPT = (VTOT + SYRK_THREADS - 1) / SYRK_THREADS;
     __shared__ __align__(16) double As[KB][BM];  // p side, scaled by 1/w
     __shared__ __align__(16) double Bs[KB][BM];  // q side
+    if (a.gate && *a.gate == 0) return;
     int tp, tq;
     tile_of(blockIdx.x, tp, tq);
     const int64_t p0 = (int64_t)tp * BM, q0 = (int64_t)tq * BM;
@@ -174,7 +180,8 @@ __global__ void k_recip(int64_t m, const double *__restrict__ w, double *__restr
 }
 
 __global__ void k_syrk_reduce(int64_t n, int nsplit, const double *__restrict__ work, double beta,
-                              double *__restrict__ C, int64_t ldc) {
+                              double *__restrict__ C, int64_t ldc, const int *__restrict__ gate) {
+    if (gate && *gate == 0) return;
     for (int64_t q = blockIdx.x; q < n; q += gridDim.x) {
         for (int64_t p = q + threadIdx.x; p < n; p += blockDim.x) {
             double s = 0.0;
@@ -192,13 +199,13 @@ struct Plan {
 };
 
 // Tile edge with the least executed work (ragged edge + diagonal tiles), or
-// bm_force (64 or 80) when given, then the split count whose (tile, split)
+// bm_force (32, 64 or 80) when given, then the split count whose (tile, split)
 // items fill whole waves of 2 CTAs per SM.
 Plan plan_for(int64_t m, int64_t n, int num_sms, int bm_force = 0) {
-    Plan best{64, 0, 1};
+    Plan best{bm_force ? bm_force : 64, 0, 1};
     double best_work = 0;
-    for (int bm : {64, 80}) {
-        if (bm_force && bm != bm_force) continue;
+    for (int bm : {32, 64, 80}) {
+        if (bm_force ? bm != bm_force : (bm == 32) != (n <= 64)) continue;
         const int64_t nt = (n + bm - 1) / bm;
         const int64_t T = nt * (nt + 1) / 2;
         const double work = (double)T * bm * bm;
@@ -210,8 +217,10 @@ Plan plan_for(int64_t m, int64_t n, int num_sms, int bm_force = 0) {
     const int64_t slots = (int64_t)num_sms * 2;
     const size_t cap = (size_t)1 << 30;  // split partials at most 1 GiB
     double best_eff = 0.0;
-    for (int s = 1; s <= 32; ++s) {
-        if (s > 1 && (m / s < 512 || (size_t)s * n * n * sizeof(double) > cap)) break;
+    // at least one slab per split: an order below one tile (n_d = 32, m = 1000)
+    // has one tile; one CTA alone took 719 us, 62 splits of a 32 x 32 tile take 23
+    for (int s = 1; s <= 64; ++s) {
+        if (s > 1 && (m / s < KB || (size_t)s * n * n * sizeof(double) > cap)) break;
         const double waves = (double)(best.tiles * s) / (double)slots;
         const double eff = waves / std::ceil(waves);
         if (eff > best_eff + 0.005) {
@@ -225,10 +234,10 @@ Plan plan_for(int64_t m, int64_t n, int num_sms, int bm_force = 0) {
 
 }  // namespace
 
-// enough for either tile edge
+// enough for any tile edge
 size_t syrk_fp64_scratch_bytes(int64_t m, int64_t n, int num_sms) {
     size_t part = 0;
-    for (int bm : {64, 80}) {
+    for (int bm : {32, 64, 80}) {
         const Plan pl = plan_for(m, n, num_sms, bm);
         if (pl.nsplit > 1) part = std::max(part, (size_t)pl.nsplit * (size_t)n * (size_t)n * sizeof(double));
     }
@@ -238,9 +247,10 @@ size_t syrk_fp64_scratch_bytes(int64_t m, int64_t n, int num_sms) {
 // work: syrk_fp64_scratch_bytes(m, n, num_sms) bytes (split partials, then 1/w)
 void launch_syrk_fp64_ws(cudaStream_t st, int num_sms, const double *A, int64_t m, int64_t n,
                          int64_t lda, const double *w, double beta, double *C, int64_t ldc,
-                         double *work, int bm) {
+                         double *work, int bm, void *rns_ws) {
     if (n <= 0) return;
-    const Plan pl = plan_for(m, n, num_sms, bm == 64 || bm == 80 ? bm : 0);
+    const int *gate = rns_ws ? launch_syrk_rns(st, num_sms, A, m, n, lda, w, beta, C, ldc, rns_ws) : nullptr;
+    const Plan pl = plan_for(m, n, num_sms, bm == 32 || bm == 64 || bm == 80 ? bm : 0);
     SyrkArgs a{};
     a.A = A;
     a.m = m;
@@ -251,7 +261,9 @@ void launch_syrk_fp64_ws(cudaStream_t st, int num_sms, const double *A, int64_t 
     a.ldc = ldc;
     a.nsplit = m > 0 ? pl.nsplit : 1;
     a.kchunk = ((std::max<int64_t>(m, 1) + a.nsplit - 1) / a.nsplit + KB - 1) / KB * KB;
+    a.nsplit = std::max(1, (int)((m + a.kchunk - 1) / a.kchunk));   // no empty split
     a.work = work;
+    a.gate = gate;
     double *rw = work + (pl.nsplit > 1 ? (size_t)pl.nsplit * n * n : 0);
     a.rw = rw;
     if (m > 0) {
@@ -260,21 +272,36 @@ void launch_syrk_fp64_ws(cudaStream_t st, int num_sms, const double *A, int64_t 
     }
     MDSIP_REQUIRE(pl.tiles < (1LL << 31), MDSIP_ERR_INVALID_ARG, "syrk: n too large");
     const dim3 grid((unsigned)pl.tiles, (unsigned)a.nsplit);
-    if (pl.bm == 80)
+    if (pl.bm == 32)
+        k_syrk_fp64<32><<<grid, SYRK_THREADS, 0, st>>>(a);
+    else if (pl.bm == 80)
         k_syrk_fp64<80><<<grid, SYRK_THREADS, 0, st>>>(a);
     else
         k_syrk_fp64<64><<<grid, SYRK_THREADS, 0, st>>>(a);
     MDSIP_LAUNCHED();
     if (a.nsplit > 1) {
         k_syrk_reduce<<<(unsigned)std::min<int64_t>(n, 4096), 256, 0, st>>>(n, a.nsplit, work, beta, C,
-                                                                            ldc);
+                                                                            ldc, gate);
         MDSIP_LAUNCHED();
     }
 }
 
 void launch_syrk_fp64(Ctx *ctx, const double *A, int64_t m, int64_t n, int64_t lda, const double *w,
                       double beta, double *C, int64_t ldc) {
-    const size_t ws = syrk_fp64_scratch_bytes(m, n, ctx->num_sms);
+    const size_t ws = (syrk_fp64_scratch_bytes(m, n, ctx->num_sms) + 1023) / 1024 * 1024;
+    if (syrk_rns_pays(m, n)) {
+        char *base = nullptr;
+        try {
+            base = static_cast<char *>(ctx->scratch_at_least(ws + syrk_rns_workspace_bytes(m, n, ctx->num_sms)));
+        } catch (const Error &e) {   // not enough memory for the residues: the DFMA kernel needs less
+            if (e.status != MDSIP_ERR_OOM) throw;
+        }
+        if (base) {
+            launch_syrk_fp64_ws(ctx->stream, ctx->num_sms, A, m, n, lda, w, beta, C, ldc,
+                                reinterpret_cast<double *>(base), 0, base + ws);
+            return;
+        }
+    }
     double *work = static_cast<double *>(ctx->scratch_at_least(ws));
     launch_syrk_fp64_ws(ctx->stream, ctx->num_sms, A, m, n, lda, w, beta, C, ldc, work);
 }
