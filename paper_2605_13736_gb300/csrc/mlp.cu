@@ -8,8 +8,10 @@
 // standardised units, L = sum (yn - (y* - out_mean) / out_std)^2 / (B O), with
 // Adam.  Every contraction (three forward, five backward) runs on the BF16
 // tcgen05 GEMM with FP32 accumulation; parameters, moments and gradients are
-// FP32; the bias, ReLU, loss and transposes are fused into the kernels that
-// produce the BF16 operands of the next contraction.
+// FP32; the bias and ReLU are fused into the kernels that produce the BF16
+// operands of the next contraction, the output layer's bias, scaling, loss and
+// Adam step into its contractions.  No operand is stored twice: where a
+// contraction needs the other orientation the tensor core reads it MN-major.
 //
 // BF16 operand points (each value rounded to nearest even once): the
 // standardised input, W1, W2, W3, h1, h2, the output gradient dL/dyn, and the
@@ -20,142 +22,89 @@
 #include <algorithm>
 
 #include "internal.cuh"
+#include "mlp.cuh"
 
 namespace mdsip {
-
-size_t gemm_bf16_ws_bytes(int64_t M, int64_t N, int64_t K, int num_sms);
-void launch_gemm_bf16(cudaStream_t s, int num_sms, const __nv_bfloat16 *A, int64_t lda, const __nv_bfloat16 *B,
-                      int64_t ldb, int64_t M, int64_t N, int64_t K, float *C, int64_t ldc, void *ws, int *err_dev);
 
 namespace {
 
 using bf16 = __nv_bfloat16;
 
-constexpr int TT = 32;  // transpose tile edge
-
 int64_t r8(int64_t v) { return (std::max<int64_t>(v, 1) + 7) / 8 * 8; }
 
-// Xb[b][i] = bf16((X[row(b)][i] - mean_i) / std_i), XbT[i][b] = Xb[b][i]
+// Xb[b][i] = bf16((X[row(b)][i] - mean_i) / std_i)
 __global__ void k_gather_x(int64_t B, int64_t I, const double *__restrict__ X, int64_t ldx,
                            const int32_t *__restrict__ idx, const float *__restrict__ mean,
-                           const float *__restrict__ sd, bf16 *__restrict__ Xb, int64_t ldI, bf16 *__restrict__ XbT,
-                           int64_t ldB) {
-    __shared__ bf16 t[TT][TT + 2];
-    const int64_t i0 = (int64_t)blockIdx.x * TT, b0 = (int64_t)blockIdx.y * TT;
-    for (int r = threadIdx.y; r < TT; r += blockDim.y) {
-        const int64_t b = b0 + r, i = i0 + threadIdx.x;
-        bf16 v = __float2bfloat16_rn(0.0f);
-        if (b < B && i < I) {
-            const int64_t row = idx ? (int64_t)idx[b] : b;
-            v = __float2bfloat16_rn((float)((X[row * ldx + i] - (double)mean[i]) / (double)sd[i]));
-            Xb[b * ldI + i] = v;
-        }
-        t[r][threadIdx.x] = v;
-    }
-    __syncthreads();
-    if (!XbT) return;
-    for (int r = threadIdx.y; r < TT; r += blockDim.y) {
-        const int64_t i = i0 + r, b = b0 + threadIdx.x;
-        if (i < I && b < B) XbT[i * ldB + b] = t[threadIdx.x][r];
+                           const float *__restrict__ sd, bf16 *__restrict__ Xb, int64_t ldI) {
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < B * I; e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t b = e / I, i = e - b * I;
+        const int64_t row = idx ? (int64_t)idx[b] : b;
+        Xb[b * ldI + i] = __float2bfloat16_rn((float)((X[row * ldx + i] - (double)mean[i]) / (double)sd[i]));
     }
 }
 
-// Hh[b][j] = bf16(relu(Z[b][j] + bias[j])), HT[j][b] = Hh[b][j]
+// Hh[b][j] = bf16(relu(Z[b][j] + bias[j]))
 __global__ void k_bias_relu(int64_t B, int64_t Hn, const float *__restrict__ Z, int64_t ldz,
-                            const float *__restrict__ bias, bf16 *__restrict__ Hh, int64_t ldh, bf16 *__restrict__ HT,
-                            int64_t ldB) {
-    __shared__ bf16 t[TT][TT + 2];
-    const int64_t j0 = (int64_t)blockIdx.x * TT, b0 = (int64_t)blockIdx.y * TT;
-    for (int r = threadIdx.y; r < TT; r += blockDim.y) {
-        const int64_t b = b0 + r, j = j0 + threadIdx.x;
-        bf16 v = __float2bfloat16_rn(0.0f);
-        if (b < B && j < Hn) {
-            v = __float2bfloat16_rn(fmaxf(Z[b * ldz + j] + bias[j], 0.0f));
-            Hh[b * ldh + j] = v;
-        }
-        t[r][threadIdx.x] = v;
-    }
-    __syncthreads();
-    for (int r = threadIdx.y; r < TT; r += blockDim.y) {
-        const int64_t j = j0 + r, b = b0 + threadIdx.x;
-        if (j < Hn && b < B) HT[j * ldB + b] = t[threadIdx.x][r];
+                            const float *__restrict__ bias, bf16 *__restrict__ Hh, int64_t ldh) {
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < B * Hn; e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t b = e / Hn, j = e - b * Hn;
+        Hh[b * ldh + j] = __float2bfloat16_rn(fmaxf(Z[b * ldz + j] + bias[j], 0.0f));
     }
 }
 
-// Output layer and loss: yn = Z + b3, target tn = (Y[row(b)][o] - mean_o) /
-// std_o, dY = bf16(scale (yn - tn)) in both orientations; per-block partial of
-// sum (yn - tn)^2 in FP64.
-__global__ void k_out_loss(int64_t B, int64_t O, const float *__restrict__ Z, int64_t ldz,
-                           const float *__restrict__ b3, const double *__restrict__ Y, int64_t ldy,
-                           const int32_t *__restrict__ idx, const float *__restrict__ mean,
-                           const float *__restrict__ sd, float scale, bf16 *__restrict__ dY, int64_t ldO,
-                           bf16 *__restrict__ dYT, int64_t ldB, double *__restrict__ part) {
-    __shared__ bf16 t[TT][TT + 2];
-    __shared__ double red[TT * 8];
-    const int64_t o0 = (int64_t)blockIdx.x * TT, b0 = (int64_t)blockIdx.y * TT;
-    double acc = 0.0;
-    for (int r = threadIdx.y; r < TT; r += blockDim.y) {
-        const int64_t b = b0 + r, o = o0 + threadIdx.x;
-        bf16 g = __float2bfloat16_rn(0.0f);
-        if (b < B && o < O) {
-            const int64_t row = idx ? (int64_t)idx[b] : b;
-            const float yn = Z[b * ldz + o] + b3[o];
-            const float tn = (float)((Y[row * ldy + o] - (double)mean[o]) / (double)sd[o]);
-            const float d = yn - tn;
-            acc += (double)d * (double)d;
-            g = __float2bfloat16_rn(scale * d);
-            dY[b * ldO + o] = g;
-        }
-        t[r][threadIdx.x] = g;
-    }
-    const int tid = threadIdx.y * TT + threadIdx.x;
-    red[tid] = acc;
+// Sum of the 32 row groups of a block's columns (groups halved pairwise) by
+// the threads with threadIdx.y == 0.
+__device__ __forceinline__ float group_sum(float s, float (&red)[32][33]) {
+    red[threadIdx.y][threadIdx.x] = s;
     __syncthreads();
-    for (int w = TT * 8 / 2; w > 0; w >>= 1) {
-        if (tid < w) red[tid] += red[tid + w];
+    for (int w = 16; w > 0; w >>= 1) {
+        if ((int)threadIdx.y < w) red[threadIdx.y][threadIdx.x] += red[threadIdx.y + w][threadIdx.x];
         __syncthreads();
     }
-    if (tid == 0) part[(int64_t)blockIdx.y * gridDim.x + blockIdx.x] = red[0];
-    for (int r = threadIdx.y; r < TT; r += blockDim.y) {
-        const int64_t o = o0 + r, b = b0 + threadIdx.x;
-        if (o < O && b < B) dYT[o * ldB + b] = t[threadIdx.x][r];
-    }
+    return red[0][threadIdx.x];
 }
 
-// dZ = bf16(dH * [Hact > 0]) in both orientations (dZ optional)
-__global__ void k_relu_back(int64_t B, int64_t Hn, const float *__restrict__ dH, int64_t ldd,
-                            const bf16 *__restrict__ Hact, int64_t ldh, bf16 *__restrict__ dZ,
-                            bf16 *__restrict__ dZT, int64_t ldB) {
-    __shared__ bf16 t[TT][TT + 2];
-    const int64_t j0 = (int64_t)blockIdx.x * TT, b0 = (int64_t)blockIdx.y * TT;
-    for (int r = threadIdx.y; r < TT; r += blockDim.y) {
-        const int64_t b = b0 + r, j = j0 + threadIdx.x;
-        bf16 v = __float2bfloat16_rn(0.0f);
-        if (b < B && j < Hn) {
+// dZ = bf16(dH * [Hact > 0]) and its column sums (the bias gradient): 32
+// columns x 32 row groups per block, fixed order
+__global__ void __launch_bounds__(1024) k_relu_back(int64_t B, int64_t Hn, const float *__restrict__ dH, int64_t ldd,
+                                                    const bf16 *__restrict__ Hact, int64_t ldh, bf16 *__restrict__ dZ,
+                                                    float *__restrict__ db) {
+    __shared__ float red[32][33];
+    const int64_t j = (int64_t)blockIdx.x * 32 + threadIdx.x;
+    float s = 0.0f;
+    if (j < Hn) {
+#pragma unroll 4
+        for (int64_t b = threadIdx.y; b < B; b += 32) {
             const float h = __bfloat162float(Hact[b * ldh + j]);
-            v = __float2bfloat16_rn(h > 0.0f ? dH[b * ldd + j] : 0.0f);
-            if (dZ) dZ[b * ldh + j] = v;
+            const bf16 v = __float2bfloat16_rn(h > 0.0f ? dH[b * ldd + j] : 0.0f);
+            dZ[b * ldh + j] = v;
+            s += __bfloat162float(v);
         }
-        t[r][threadIdx.x] = v;
     }
-    __syncthreads();
-    for (int r = threadIdx.y; r < TT; r += blockDim.y) {
-        const int64_t j = j0 + r, b = b0 + threadIdx.x;
-        if (j < Hn && b < B) dZT[j * ldB + b] = t[threadIdx.x][r];
-    }
+    s = group_sum(s, red);
+    if (threadIdx.y == 0 && j < Hn) db[j] = s;
 }
 
-// out[r] = sum_{c < cols} T[r][c]  (one warp per row, fixed order)
-__global__ void k_rowsum_bf16(int64_t rows, int64_t cols, const bf16 *__restrict__ T, int64_t ld,
-                              float *__restrict__ out) {
-    const int lane = threadIdx.x & 31;
-    const int64_t wpb = blockDim.x / 32;
-    for (int64_t r = (int64_t)blockIdx.x * wpb + threadIdx.x / 32; r < rows; r += (int64_t)gridDim.x * wpb) {
-        float s = 0.0f;
-        for (int64_t c = lane; c < cols; c += 32) s += __bfloat162float(T[r * ld + c]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) out[r] = s;
+// out[j] = sum_b T[b][j] in the same order, two columns per thread (ld even);
+// HBM / L2-bound, one read of T
+__global__ void __launch_bounds__(1024) k_colsum_bf16(int64_t B, int64_t cols, const bf16 *__restrict__ T, int64_t ld,
+                                                      float *__restrict__ out) {
+    __shared__ float red[2][32][33];
+    const int64_t j = (int64_t)blockIdx.x * 64 + 2 * threadIdx.x;
+    float s0 = 0.0f, s1 = 0.0f;
+    if (j < cols) {
+#pragma unroll 8
+        for (int64_t b = threadIdx.y; b < B; b += 32) {
+            const float2 v = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(T + b * ld + j));
+            s0 += v.x;
+            s1 += v.y;
+        }
+    }
+    s0 = group_sum(s0, red[0]);
+    s1 = group_sum(s1, red[1]);
+    if (threadIdx.y == 0 && j < cols) {
+        out[j] = s0;
+        if (j + 1 < cols) out[j + 1] = s1;
     }
 }
 
@@ -173,49 +122,24 @@ __global__ void k_sum_partials(int64_t n, const double *__restrict__ part, doubl
     if (threadIdx.x == 0) *out = red[0];
 }
 
-// Adam (bias-corrected first and second moments)
 __global__ void k_adam(int64_t n, float *__restrict__ w, const float *__restrict__ g, float *__restrict__ m,
-                       float *__restrict__ v, float lr, float b1, float b2, float eps, float bc1, float bc2) {
+                       float *__restrict__ v, AdamStep st) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.0f - b1) * gi;
-        const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
+        float wi = w[i], mi = m[i], vi = v[i];
+        adam_update(st, g[i], wi, mi, vi);
         m[i] = mi;
         v[i] = vi;
-        w[i] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+        w[i] = wi;
     }
 }
 
-// dst[r][c] = bf16(src[r][c]) and/or dstT[c][r] = bf16(src[r][c])
+// dst[r][c] = bf16(src[r][c])
 __global__ void k_cast_bf16(int64_t rows, int64_t cols, const float *__restrict__ src, int64_t lds,
-                            bf16 *__restrict__ dst, int64_t ldd, bf16 *__restrict__ dstT, int64_t ldt) {
-    __shared__ bf16 t[TT][TT + 2];
-    const int64_t c0 = (int64_t)blockIdx.x * TT, r0 = (int64_t)blockIdx.y * TT;
-    for (int rr = threadIdx.y; rr < TT; rr += blockDim.y) {
-        const int64_t r = r0 + rr, c = c0 + threadIdx.x;
-        bf16 v = __float2bfloat16_rn(0.0f);
-        if (r < rows && c < cols) {
-            v = __float2bfloat16_rn(src[r * lds + c]);
-            if (dst) dst[r * ldd + c] = v;
-        }
-        t[rr][threadIdx.x] = v;
-    }
-    if (!dstT) return;
-    __syncthreads();
-    for (int rr = threadIdx.y; rr < TT; rr += blockDim.y) {
-        const int64_t c = c0 + rr, r = r0 + threadIdx.x;
-        if (c < cols && r < rows) dstT[c * ldt + r] = t[threadIdx.x][rr];
-    }
-}
-
-// y[b][o] = (Z[b][o] + b3[o]) * std_o + mean_o
-__global__ void k_out_denorm(int64_t B, int64_t O, const float *__restrict__ Z, int64_t ldz,
-                             const float *__restrict__ b3, const float *__restrict__ mean,
-                             const float *__restrict__ sd, float *__restrict__ Yo, int64_t ldy) {
-    const int64_t total = B * O;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t b = e / O, o = e % O;
-        Yo[b * ldy + o] = (Z[b * ldz + o] + b3[o]) * sd[o] + mean[o];
+                            bf16 *__restrict__ dst, int64_t ldd) {
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < rows * cols;
+         e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t r = e / cols, c = e - r * cols;
+        dst[r * ldd + c] = __float2bfloat16_rn(src[r * lds + c]);
     }
 }
 
@@ -247,8 +171,6 @@ int grid_for(int64_t n, int num_sms) {
     return (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)num_sms * 16, ceil_div(n, 256)));
 }
 
-dim3 tgrid(int64_t cols, int64_t rows) { return dim3((unsigned)ceil_div(cols, TT), (unsigned)ceil_div(rows, TT)); }
-
 }  // namespace
 
 struct Mlp {
@@ -259,110 +181,159 @@ struct Mlp {
     double beta1 = 0.9, beta2 = 0.999, eps = 1e-8;
     int64_t t = 0;  // Adam steps taken
     DBuf params, grads, m1, m2;
-    DBuf W1b, W2b, W2bT, W3b, W3bT;
+    DBuf W1b, W2b, W3b;
     DBuf in_mean, in_std, out_mean, out_std;
     DBuf err, loss;
     // activations, sized for `cap` rows
-    int64_t cap = 0, ldB = 8;
-    DBuf Xb, XbT, H1, H1T, H2, H2T, dY, dYT, dZ2, dZ2T, dZ1T, Zbuf, lpart, gws;
+    int64_t cap = 0, tcap = 0;   // rows of the forward and of the training buffers
+    DBuf Xb, H1, H2, Zbuf, gws, dY, dZ2, dZ1, lpart, tws;
     size_t gws_bytes = 0;
 
     float *P() const { return params.as<float>(); }
     float *G() const { return grads.as<float>(); }
 
-    void ensure(int64_t B) {
-        if (B <= cap) return;
-        cap = std::max<int64_t>(B, 64);
-        ldB = r8(cap);
-        Xb.get<bf16>(ctx, cap * ldI);
-        XbT.get<bf16>(ctx, I * ldB);
-        H1.get<bf16>(ctx, cap * ldH);
-        H1T.get<bf16>(ctx, H * ldB);
-        H2.get<bf16>(ctx, cap * ldH);
-        H2T.get<bf16>(ctx, H * ldB);
-        dY.get<bf16>(ctx, cap * ldO);
-        dYT.get<bf16>(ctx, O * ldB);
-        dZ2.get<bf16>(ctx, cap * ldH);
-        dZ2T.get<bf16>(ctx, H * ldB);
-        dZ1T.get<bf16>(ctx, H * ldB);
-        Zbuf.get<float>(ctx, cap * std::max(ldO, ldH));
-        lpart.get<double>(ctx, ceil_div(O, TT) * ceil_div(cap, TT));
+    // buffers for batches of B rows: the forward pass's, and with `train` the
+    // backward pass's (a prediction needs no batch x outputs gradient)
+    void ensure(int64_t B, bool train) {
         const int sms = ctx->num_sms;
-        gws_bytes = std::max({gemm_bf16_ws_bytes(cap, H, I, sms), gemm_bf16_ws_bytes(cap, H, H, sms),
-                              gemm_bf16_ws_bytes(cap, O, H, sms), gemm_bf16_ws_bytes(O, H, cap, sms),
-                              gemm_bf16_ws_bytes(cap, H, O, sms), gemm_bf16_ws_bytes(H, H, cap, sms),
-                              gemm_bf16_ws_bytes(H, I, cap, sms), (size_t)16});
-        gws.get<uint8_t>(ctx, gws_bytes);
+        if (B > cap) {
+            const int64_t c = std::max<int64_t>(B, 64);
+            Xb.get<bf16>(ctx, c * ldI);
+            H1.get<bf16>(ctx, c * ldH);
+            H2.get<bf16>(ctx, c * ldH);
+            Zbuf.get<float>(ctx, c * ldH);
+            gws.get<uint8_t>(ctx, std::max({split_ws(c, H, I, false, false), split_ws(c, H, H, false, false), (size_t)16}));
+            cap = c;
+        }
+        if (train && B > tcap) {
+            const int64_t c = std::max<int64_t>(B, 64);
+            dY.get<bf16>(ctx, c * ldO);
+            dZ2.get<bf16>(ctx, c * ldH);
+            dZ1.get<bf16>(ctx, c * ldH);
+            lpart.get<double>(ctx, (int64_t)8 * sms);
+            tws.get<uint8_t>(ctx, std::max({split_ws(c, H, O, false, true),
+                                            split_ws(H, H, c, true, true), split_ws(c, H, H, false, true),
+                                            split_ws(H, I, c, true, true), (size_t)16}));
+            tcap = c;
+        }
+    }
+
+    // largest split workspace over batches of up to B rows (the plan's split
+    // count is not monotone in the batch): dimensions M, N, K with the batch as
+    // M (or as K, for the weight gradients)
+    size_t split_ws(int64_t M, int64_t N, int64_t K, bool amn, bool bmn) const {
+        const bool batch_k = amn;   // weight gradients contract over the batch
+        const int64_t c = batch_k ? K : M;
+        size_t best = 0;
+        for (int64_t b = 1; b <= c; b = b < c && b + 64 > c ? c : b + 64)
+            best = std::max(best, gemm_bf16_ws_bytes(batch_k ? M : std::min(c, (b + 127) / 128 * 128), N,
+                                                     batch_k ? b : K, ctx->num_sms, amn, bmn));
+        return std::max(best, gemm_bf16_ws_bytes(M, N, K, ctx->num_sms, amn, bmn));
     }
 
     void gemm(const bf16 *A, int64_t lda, const bf16 *Bm, int64_t ldb, int64_t M, int64_t N, int64_t K, float *C,
-              int64_t ldc) {
-        launch_gemm_bf16(ctx->stream, ctx->num_sms, A, lda, Bm, ldb, M, N, K, C, ldc, gws.ptr, err.as<int>());
+              int64_t ldc, void *ws, bool amn = false, bool bmn = false) {
+        launch_gemm_bf16(ctx->stream, ctx->num_sms, A, lda, Bm, ldb, M, N, K, C, ldc, ws, err.as<int>(), amn, bmn);
     }
 
-    // BF16 copies of the weights (W2 and W3 also transposed)
-    void cast_weights() {
+    // BF16 copies of the hidden layers' weights, and of W3 (the training step's
+    // fused update writes that one itself)
+    void cast_hidden() {
         cudaStream_t s = ctx->stream;
-        const dim3 blk(TT, 8);
-        k_cast_bf16<<<tgrid(I, H), blk, 0, s>>>(H, I, P() + off_W1, I, W1b.as<bf16>(), ldI, nullptr, 0);
+        k_cast_bf16<<<grid_for(H * I, ctx->num_sms), 256, 0, s>>>(H, I, P() + off_W1, I, W1b.as<bf16>(), ldI);
         MDSIP_LAUNCHED();
-        k_cast_bf16<<<tgrid(H, H), blk, 0, s>>>(H, H, P() + off_W2, H, W2b.as<bf16>(), ldH, W2bT.as<bf16>(), ldH);
+        k_cast_bf16<<<grid_for(H * H, ctx->num_sms), 256, 0, s>>>(H, H, P() + off_W2, H, W2b.as<bf16>(), ldH);
         MDSIP_LAUNCHED();
-        k_cast_bf16<<<tgrid(H, O), blk, 0, s>>>(O, H, P() + off_W3, H, W3b.as<bf16>(), ldH, W3bT.as<bf16>(), ldO);
+    }
+    void cast_weights() {
+        cast_hidden();
+        k_cast_bf16<<<grid_for(O * H, ctx->num_sms), 256, 0, ctx->stream>>>(O, H, P() + off_W3, H, W3b.as<bf16>(), ldH);
         MDSIP_LAUNCHED();
     }
 
-    // forward through h2 (kept for the backward pass); Zbuf ends with the
-    // output-layer pre-bias values (B x O, row stride ldO)
+    // forward through h2 (kept for the backward pass)
     void forward(const double *X, int64_t ldx, const int32_t *idx, int64_t B) {
         cudaStream_t s = ctx->stream;
-        const dim3 blk(TT, 8);
         float *Z = Zbuf.as<float>();
-        k_gather_x<<<tgrid(I, B), blk, 0, s>>>(B, I, X, ldx, idx, in_mean.as<float>(), in_std.as<float>(),
-                                               Xb.as<bf16>(), ldI, XbT.as<bf16>(), ldB);
+        k_gather_x<<<grid_for(B * I, ctx->num_sms), 256, 0, s>>>(B, I, X, ldx, idx, in_mean.as<float>(),
+                                                                 in_std.as<float>(), Xb.as<bf16>(), ldI);
         MDSIP_LAUNCHED();
-        gemm(Xb.as<bf16>(), ldI, W1b.as<bf16>(), ldI, B, H, I, Z, ldH);
-        k_bias_relu<<<tgrid(H, B), blk, 0, s>>>(B, H, Z, ldH, P() + off_b1, H1.as<bf16>(), ldH, H1T.as<bf16>(), ldB);
+        gemm(Xb.as<bf16>(), ldI, W1b.as<bf16>(), ldI, B, H, I, Z, ldH, gws.ptr);
+        k_bias_relu<<<grid_for(B * H, ctx->num_sms), 256, 0, s>>>(B, H, Z, ldH, P() + off_b1, H1.as<bf16>(), ldH);
         MDSIP_LAUNCHED();
-        gemm(H1.as<bf16>(), ldH, W2b.as<bf16>(), ldH, B, H, H, Z, ldH);
-        k_bias_relu<<<tgrid(H, B), blk, 0, s>>>(B, H, Z, ldH, P() + off_b2, H2.as<bf16>(), ldH, H2T.as<bf16>(), ldB);
+        gemm(H1.as<bf16>(), ldH, W2b.as<bf16>(), ldH, B, H, H, Z, ldH, gws.ptr);
+        k_bias_relu<<<grid_for(B * H, ctx->num_sms), 256, 0, s>>>(B, H, Z, ldH, P() + off_b2, H2.as<bf16>(), ldH);
         MDSIP_LAUNCHED();
-        gemm(H2.as<bf16>(), ldH, W3b.as<bf16>(), ldH, B, O, H, Z, ldO);
     }
 
-    // loss (device scalar) and gradients into G()
-    void backward(const double *Y, int64_t ldy, const int32_t *idx, int64_t B) {
+    OutLayer out_layer() const {
+        OutLayer o{};
+        o.b3 = params.as<float>() + off_b3;
+        o.mean = out_mean.as<float>();
+        o.sd = out_std.as<float>();
+        return o;
+    }
+
+    // loss (device scalar) and gradients into G(); without w3_grad the output
+    // layer's weight gradient is left to the fused update
+    void backward(const double *Y, int64_t ldy, const int32_t *idx, int64_t B, bool w3_grad) {
         cudaStream_t s = ctx->stream;
-        const dim3 blk(TT, 8);
         float *Z = Zbuf.as<float>();
         float *G_ = G();
-        const float scale = (float)(2.0 / ((double)B * (double)O));
-        const dim3 lg = tgrid(O, B);
-        k_out_loss<<<lg, blk, 0, s>>>(B, O, Z, ldO, P() + off_b3, Y, ldy, idx, out_mean.as<float>(),
-                                      out_std.as<float>(), scale, dY.as<bf16>(), ldO, dYT.as<bf16>(), ldB,
-                                      lpart.as<double>());
+        OutLayer o = out_layer();
+        o.Y = Y;
+        o.ldy = ldy;
+        o.idx = idx;
+        o.scale = (float)(2.0 / ((double)B * (double)O));
+        o.dY = dY.as<bf16>();
+        o.ldo = ldO;
+        o.part = lpart.as<double>();
+        // yn = W3 h2 + b3, loss partials, dL/dyn and db3
+        const int np = launch_out_layer(s, ctx->num_sms, H2.as<bf16>(), ldH, W3b.as<bf16>(), ldH, B, O, H, o, nullptr,
+                                        0, err.as<int>());
+        k_sum_partials<<<1, 256, 0, s>>>(np, lpart.as<double>(), loss.as<double>());
         MDSIP_LAUNCHED();
-        k_sum_partials<<<1, 256, 0, s>>>((int64_t)lg.x * lg.y, lpart.as<double>(), loss.as<double>());
+        k_colsum_bf16<<<ceil_div(O, 64), dim3(32, 32), 0, s>>>(B, O, dY.as<bf16>(), ldO, G_ + off_b3);
         MDSIP_LAUNCHED();
-        // output layer: dW3 = dY^T h2, db3 = column sums of dY
-        gemm(dYT.as<bf16>(), ldB, H2T.as<bf16>(), ldB, O, H, B, G_ + off_W3, H);
-        k_rowsum_bf16<<<grid_for(O * 32, ctx->num_sms), 256, 0, s>>>(O, B, dYT.as<bf16>(), ldB, G_ + off_b3);
-        MDSIP_LAUNCHED();
+        // output layer: dW3 = dY^T h2
+        if (w3_grad)
+            launch_gemm_w3_grad(s, ctx->num_sms, H2.as<bf16>(), ldH, dY.as<bf16>(), ldO, B, O, H, G_ + off_W3,
+                                err.as<int>());
         // second hidden layer: dh2 = dY W3, dz2 = dh2 [h2 > 0]
-        gemm(dY.as<bf16>(), ldO, W3bT.as<bf16>(), ldO, B, H, O, Z, ldH);
-        k_relu_back<<<tgrid(H, B), blk, 0, s>>>(B, H, Z, ldH, H2.as<bf16>(), ldH, dZ2.as<bf16>(), dZ2T.as<bf16>(),
-                                               ldB);
+        const int hb = ceil_div(H, 32);
+        gemm(dY.as<bf16>(), ldO, W3b.as<bf16>(), ldH, B, H, O, Z, ldH, tws.ptr, false, true);
+        k_relu_back<<<hb, dim3(32, 32), 0, s>>>(B, H, Z, ldH, H2.as<bf16>(), ldH, dZ2.as<bf16>(), G_ + off_b2);
         MDSIP_LAUNCHED();
-        gemm(dZ2T.as<bf16>(), ldB, H1T.as<bf16>(), ldB, H, H, B, G_ + off_W2, H);
-        k_rowsum_bf16<<<grid_for(H * 32, ctx->num_sms), 256, 0, s>>>(H, B, dZ2T.as<bf16>(), ldB, G_ + off_b2);
-        MDSIP_LAUNCHED();
+        gemm(dZ2.as<bf16>(), ldH, H1.as<bf16>(), ldH, H, H, B, G_ + off_W2, H, tws.ptr, true, true);
         // first hidden layer: dh1 = dz2 W2, dz1 = dh1 [h1 > 0]
-        gemm(dZ2.as<bf16>(), ldH, W2bT.as<bf16>(), ldH, B, H, H, Z, ldH);
-        k_relu_back<<<tgrid(H, B), blk, 0, s>>>(B, H, Z, ldH, H1.as<bf16>(), ldH, nullptr, dZ1T.as<bf16>(), ldB);
+        gemm(dZ2.as<bf16>(), ldH, W2b.as<bf16>(), ldH, B, H, H, Z, ldH, tws.ptr, false, true);
+        k_relu_back<<<hb, dim3(32, 32), 0, s>>>(B, H, Z, ldH, H1.as<bf16>(), ldH, dZ1.as<bf16>(), G_ + off_b1);
         MDSIP_LAUNCHED();
-        gemm(dZ1T.as<bf16>(), ldB, XbT.as<bf16>(), ldB, H, I, B, G_ + off_W1, I);
-        k_rowsum_bf16<<<grid_for(H * 32, ctx->num_sms), 256, 0, s>>>(H, B, dZ1T.as<bf16>(), ldB, G_ + off_b1);
-        MDSIP_LAUNCHED();
+        gemm(dZ1.as<bf16>(), ldH, Xb.as<bf16>(), ldI, H, I, B, G_ + off_W1, I, tws.ptr, true, true);
+    }
+
+    // the fused update moves rows of W3 by TMA: whole 16-byte units
+    bool fused_w3() const { return H % 4 == 0; }
+
+    // one Adam step on the gradients of the last backward pass: W3 from its
+    // fused gradient where that applies, the rest from G()
+    void adam(const AdamStep &st, int64_t B) {
+        cudaStream_t s = ctx->stream;
+        auto range = [&](int64_t a, int64_t b) {
+            k_adam<<<grid_for(b - a, ctx->num_sms), 256, 0, s>>>(b - a, P() + a, G() + a, m1.as<float>() + a,
+                                                                 m2.as<float>() + a, st);
+            MDSIP_LAUNCHED();
+        };
+        if (!fused_w3()) {
+            range(0, n_params);
+            cast_weights();
+            return;
+        }
+        launch_gemm_w3_adam(s, ctx->num_sms, H2.as<bf16>(), ldH, dY.as<bf16>(), ldO, B, O, H, P() + off_W3,
+                            m1.as<float>() + off_W3, m2.as<float>() + off_W3, W3b.as<bf16>(), ldH, st, err.as<int>());
+        range(0, off_W3);
+        range(off_b3, n_params);
+        cast_hidden();
     }
 
     void check_err() {
@@ -439,9 +410,7 @@ mdsip_status mdsip_mlp_create(mdsip_ctx *hctx, int64_t n_in, int64_t n_hidden, i
             }
             m->W1b.get<__nv_bfloat16>(ctx, n_hidden * m->ldI);
             m->W2b.get<__nv_bfloat16>(ctx, n_hidden * m->ldH);
-            m->W2bT.get<__nv_bfloat16>(ctx, n_hidden * m->ldH);
             m->W3b.get<__nv_bfloat16>(ctx, n_out * m->ldH);
-            m->W3bT.get<__nv_bfloat16>(ctx, n_hidden * m->ldO);
             m->in_mean.get<float>(ctx, n_in);
             m->in_std.get<float>(ctx, n_in);
             m->out_mean.get<float>(ctx, n_out);
@@ -595,23 +564,22 @@ mdsip_status mdsip_mlp_forward(mdsip_mlp *hm, const double *X, int64_t ldx, int6
         if (batch == 0) return;
         MDSIP_REQUIRE(X && Y, MDSIP_ERR_INVALID_ARG, "mlp: null data pointer");
         DeviceGuard g(m->ctx->device);
-        m->ensure(batch);
+        m->ensure(batch, false);
         m->forward(X, ldx, nullptr, batch);
-        mdsip::k_out_denorm<<<mdsip::grid_for(batch * m->O, m->ctx->num_sms), 256, 0, m->ctx->stream>>>(
-            batch, m->O, m->Zbuf.as<float>(), m->ldO, m->P() + m->off_b3, m->out_mean.as<float>(),
-            m->out_std.as<float>(), Y, ldy);
-        MDSIP_LAUNCHED();
+        mdsip::launch_out_layer(m->ctx->stream, m->ctx->num_sms, m->H2.as<__nv_bfloat16>(), m->ldH,
+                                m->W3b.as<__nv_bfloat16>(), m->ldH, batch, m->O, m->H, m->out_layer(), Y, ldy,
+                                m->err.as<int>());
         m->check_err();
     });
 }
 
 static void run_gradient(Mlp *m, const double *X, int64_t ldx, const double *Y, int64_t ldy, const int32_t *idx,
-                         int64_t batch) {
+                         int64_t batch, bool w3_grad) {
     MDSIP_REQUIRE(X && Y && batch > 0 && ldx >= m->I && ldy >= m->O, MDSIP_ERR_INVALID_ARG,
                   "mlp: bad training arguments");
-    m->ensure(batch);
+    m->ensure(batch, true);
     m->forward(X, ldx, idx, batch);
-    m->backward(Y, ldy, idx, batch);
+    m->backward(Y, ldy, idx, batch, w3_grad);
 }
 
 mdsip_status mdsip_mlp_gradient(mdsip_mlp *hm, const double *X, int64_t ldx, const double *Y, int64_t ldy,
@@ -620,7 +588,7 @@ mdsip_status mdsip_mlp_gradient(mdsip_mlp *hm, const double *X, int64_t ldx, con
     Mlp *m = M_(hm);
     return guarded(m->ctx, [&] {
         DeviceGuard g(m->ctx->device);
-        run_gradient(m, X, ldx, Y, ldy, idx, batch);
+        run_gradient(m, X, ldx, Y, ldy, idx, batch, true);
         m->check_err();
         if (grad) copy_out(grad, m->grads.ptr, m->n_params * sizeof(float), MDSIP_MEM_DEVICE, m->ctx->stream);
         if (loss) copy_out(loss, m->loss.ptr, sizeof(double), MDSIP_MEM_HOST, m->ctx->stream);
@@ -635,18 +603,15 @@ mdsip_status mdsip_mlp_train_step(mdsip_mlp *hm, const double *X, int64_t ldx, c
     return guarded(m->ctx, [&] {
         MDSIP_REQUIRE(lr >= 0.0, MDSIP_ERR_INVALID_ARG, "mlp: negative learning rate");
         DeviceGuard g(m->ctx->device);
-        run_gradient(m, X, ldx, Y, ldy, idx, batch);
+        run_gradient(m, X, ldx, Y, ldy, idx, batch, !m->fused_w3());
         m->t += 1;
         // the moments decay with the FP32 rates the kernel uses, so the bias
         // corrections 1 - beta^t take those same rates (Kingma-Ba Algorithm 1);
         // with the FP64 rates 1 - 0.999 and 1 - fl32(0.999) differ by 1.3e-5
         const float b1f = (float)m->beta1, b2f = (float)m->beta2;
         const double bc1 = 1.0 - std::pow((double)b1f, (double)m->t), bc2 = 1.0 - std::pow((double)b2f, (double)m->t);
-        mdsip::k_adam<<<mdsip::grid_for(m->n_params, m->ctx->num_sms), 256, 0, m->ctx->stream>>>(
-            m->n_params, m->P(), m->G(), m->m1.as<float>(), m->m2.as<float>(), (float)lr, b1f, b2f,
-            (float)m->eps, (float)bc1, (float)bc2);
-        MDSIP_LAUNCHED();
-        m->cast_weights();
+        m->adam(mdsip::AdamStep{(float)lr, b1f, b2f, (float)m->eps, (float)bc1, (float)bc2, 1.0f / (float)bc1,
+                               1.0f / (float)bc2}, batch);
         if (loss) {
             m->check_err();
             copy_out(loss, m->loss.ptr, sizeof(double), MDSIP_MEM_HOST, m->ctx->stream);

@@ -87,7 +87,7 @@ constexpr int T_M = 128, T_N = 256;    // output tile: 128 rows p, 256 columns q
 constexpr int SLAB = 64;               // rows of A (K) per pipeline stage
 constexpr int STAGES = 4;
 constexpr int FOLD = 4;                // stages per exact accumulation (256 rows)
-constexpr int BOX_BYTES = 64 * SLAB * 2;           // one 64-column x 64-row TMA box
+constexpr int BOX_BYTES = (int)tc::kMnBoxBytes;    // one 64-column x 64-row TMA box
 constexpr int STAGE_BYTES = (T_M + T_N) / 64 * BOX_BYTES;   // 48 KiB
 constexpr int MMA_THREADS = 384;       // warp 0 loads, warp 1 issues, warps 4-11 fold
 constexpr size_t kMmaSmem = 1024 + (size_t)STAGES * STAGE_BYTES + 256;
@@ -259,38 +259,6 @@ __global__ void __launch_bounds__(256) k_rns_residues(const double *__restrict__
     }
 }
 
-// Shared-memory descriptor of an operand stored with its M/N index contiguous
-// (MN-major), 128-byte swizzle: 64-element x 8-row atoms of 1024 bytes, atoms
-// 1024 bytes apart along K, 64-element groups BOX_BYTES apart along M/N.
-__device__ __forceinline__ uint64_t sw128_mnmajor_desc(uint32_t saddr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
-    d |= (uint64_t)(BOX_BYTES >> 4) << 16;
-    d |= (uint64_t)(1024 >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)2 << 61;
-    return d;
-}
-
-constexpr uint32_t mn_idesc(int N) {   // BF16 x BF16 -> FP32, both operands MN-major
-    return tc::instr_desc(false, T_M, N) | (1u << 15) | (1u << 16);
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-          "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
 // packed FP32 pairs
 __device__ __forceinline__ uint64_t pk(float a, float b) {
     uint64_t r;
@@ -417,12 +385,12 @@ __global__ void __launch_bounds__(MMA_THREADS, 1) k_rns_mma(const __grid_constan
                     const uint32_t ab = tc::smem_u32(smem + (size_t)st * STAGE_BYTES), bb = ab + 2 * BOX_BYTES;
 #pragma unroll
                     for (int k = 0; k < SLAB / 16; ++k) {
-                        const uint64_t da = sw128_mnmajor_desc(ab + 2048 * k), db = sw128_mnmajor_desc(bb + 2048 * k);
+                        const uint64_t da = tc::sw128_mnmajor_desc(ab + 2048 * k), db = tc::sw128_mnmajor_desc(bb + 2048 * k);
                         const uint32_t on = (ks > f0 || k > 0) ? 1u : 0u;
                         if (half)
-                            tc::mma<false, mn_idesc(128)>(acc, da, db, on);
+                            tc::mma<false, tc::instr_desc(false, T_M, 128, true, true)>(acc, da, db, on);
                         else
-                            tc::mma<false, mn_idesc(256)>(acc, da, db, on);
+                            tc::mma<false, tc::instr_desc(false, T_M, 256, true, true)>(acc, da, db, on);
                     }
                     tc::commit(&empty[st]);
                 }
@@ -459,7 +427,7 @@ __global__ void __launch_bounds__(MMA_THREADS, 1) k_rns_mma(const __grid_constan
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {
                         uint32_t r[16];
-                        tmem_ld16(base + 16 * c, r);
+                        tc::tmem_ld16(base + 16 * c, r);
 #pragma unroll
                         for (int j = 0; j < 8; ++j) {
                             const uint64_t x = pk(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
@@ -470,7 +438,7 @@ __global__ void __launch_bounds__(MMA_THREADS, 1) k_rns_mma(const __grid_constan
                 }
                 tc::fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&tempty[buf]);
+                if (lane == 0) tc::mbar_arrive(&tempty[buf]);
             }
             if (ok && !skip) {
                 int16_t *out = a.W + ((size_t)w * T_N + 128 * hc) * T_M + 32 * quad + lane;

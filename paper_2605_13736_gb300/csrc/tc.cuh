@@ -53,6 +53,18 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, u
         : "memory");
 }
 
+// shared -> global; the caller commits and waits the bulk group
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, const void *src, int x, int y) {
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
+                     reinterpret_cast<uint64_t>(map)),
+                 "r"(smem_u32(src)), "r"(x), "r"(y)
+                 : "memory");
+}
+__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+__device__ __forceinline__ void bulk_wait() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
+__device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
@@ -83,12 +95,33 @@ __device__ __forceinline__ uint64_t sw128_kmajor_desc(uint32_t saddr) {
     return d;
 }
 
+// The same for an operand stored with its M/N index contiguous (MN-major), as
+// 64-element x 64-row boxes of 8192 bytes (one TMA box each): 64-element x
+// 8-row atoms of 1024 bytes, the atoms 1024 bytes apart along K and the
+// 64-element groups one box apart along M/N.  A K step of 16 advances the
+// start address by 2048 bytes.
+constexpr uint32_t kMnBoxBytes = 64 * 64 * 2;
+__device__ __forceinline__ uint64_t sw128_mnmajor_desc(uint32_t saddr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)(kMnBoxBytes >> 4) << 16;
+    d |= (uint64_t)(1024 >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)2 << 61;
+    return d;
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
 // Instruction descriptor: FP32 accumulator, A and B of one type (BF16 or
-// TF32), both K-major, tile M x N.
-__host__ __device__ constexpr uint32_t instr_desc(bool tf32, int M, int N) {
+// TF32), each K-major or MN-major, tile M x N.
+__host__ __device__ constexpr uint32_t instr_desc(bool tf32, int M, int N, bool a_mn = false, bool b_mn = false) {
     return (1u << 4)                        // D = F32
            | ((tf32 ? 2u : 1u) << 7)        // A = TF32 / BF16
            | ((tf32 ? 2u : 1u) << 10)       // B = TF32 / BF16
+           | ((a_mn ? 1u : 0u) << 15) | ((b_mn ? 1u : 0u) << 16)
            | ((uint32_t)(N >> 3) << 17)     // N / 8
            | ((uint32_t)(M >> 4) << 24);    // M / 16
 }
@@ -123,11 +156,23 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
+          "=r"(r[15])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
 // Host: 2-D tiled tensor map (inner extent `inner` elements of `esz` bytes,
 // `outer` rows `ld` elements apart; box `box_inner` x `box_outer`; 128-byte
-// swizzle; out-of-range elements read as zero).  Throws on failure.
+// swizzle, or rows of the box packed without one; out-of-range elements read
+// as zero and are not written).  Throws on failure.
 void encode_2d(CUtensorMap *map, const void *base, bool f32, uint64_t inner, uint64_t outer, uint64_t ld,
-               uint32_t box_inner, uint32_t box_outer);
+               uint32_t box_inner, uint32_t box_outer, bool swizzle = true);
 
 }  // namespace tc
 }  // namespace mdsip
