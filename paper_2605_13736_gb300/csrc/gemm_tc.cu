@@ -854,10 +854,10 @@ void launch_gemm_w3_adam(cudaStream_t s, int num_sms, const __nv_bfloat16 *H2, i
     CUtensorMap hmap, ymap, wmap, mmap, vmap, bmap;
     tc::encode_2d(&hmap, H2, false, (uint64_t)H, (uint64_t)batch, (uint64_t)ldh, 64, G_SLAB);
     tc::encode_2d(&ymap, dY, false, (uint64_t)O, (uint64_t)batch, (uint64_t)ldo, 64, G_SLAB);
-    tc::encode_2d(&wmap, w, true, (uint64_t)H, (uint64_t)O, (uint64_t)H, 128, D_ROWS, false);
-    tc::encode_2d(&mmap, m, true, (uint64_t)H, (uint64_t)O, (uint64_t)H, 128, D_ROWS, false);
-    tc::encode_2d(&vmap, v, true, (uint64_t)H, (uint64_t)O, (uint64_t)H, 128, D_ROWS, false);
-    tc::encode_2d(&bmap, wb, false, (uint64_t)H, (uint64_t)O, (uint64_t)ldb, 128, D_ROWS, false);
+    tc::encode_2d(&wmap, w, true, (uint64_t)H, (uint64_t)O, (uint64_t)H, 128, D_ROWS, 0);
+    tc::encode_2d(&mmap, m, true, (uint64_t)H, (uint64_t)O, (uint64_t)H, 128, D_ROWS, 0);
+    tc::encode_2d(&vmap, v, true, (uint64_t)H, (uint64_t)O, (uint64_t)H, 128, D_ROWS, 0);
+    tc::encode_2d(&bmap, wb, false, (uint64_t)H, (uint64_t)O, (uint64_t)ldb, 128, D_ROWS, 0);
     GemmAdamArgs a = w3_args(batch, O, H, err_dev);
     a.s = st;
     static PerDeviceOnce once;

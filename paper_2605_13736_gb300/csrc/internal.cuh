@@ -393,12 +393,12 @@ void launch_ldlt(cudaStream_t s, int num_sms, int64_t N, const double *S, int64_
 size_t ldlt_blocked_scratch_bytes(int64_t N);
 bool ldlt_blocked_available(int64_t N);
 // Speculation mode of the blocked factorization: 0 every panel pivots; 1 (auto)
-// no-interchange panels, the persistent kernel from order kPersistentMinOrder
-// on or where the pivoting panel does not fit; 2 the persistent kernel at any
-// order.  The persistent kernel reads back where it stopped (synchronises the
+// no-interchange panels, the persistent kernel with FP64 updates, and with FP32
+// updates from order kPersistentMinOrder on or where the pivoting panel does
+// not fit; 2 the persistent kernel at any order.  The persistent kernel reads back where it stopped (synchronises the
 // stream).
 constexpr int64_t kPersistentMinOrder = 2048;
-bool ldlt_persistent_path(int64_t N, int spec);
+bool ldlt_persistent_path(int64_t N, int spec, bool fp32_update);
 std::vector<int> ldlt_blocked_widths(int64_t N, bool f32);
 void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, const double *maxabs_dev,
                          double zero_tol, LdltOut out, void *scratch, bool fp32_update, int nb = 0,

@@ -37,6 +37,7 @@
 #include <vector>
 
 #include "internal.cuh"
+#include "ldlt_panel.cuh"
 #include "tc.cuh"
 
 namespace cg = cooperative_groups;
@@ -55,17 +56,6 @@ constexpr int kUT = 64;   // trailing-update tile edge
 // memory) before touching data, then lets its own successor launch.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
-struct PanelState {
-    int k;       // first column of the next panel
-    int kb;      // columns factored by the last panel
-    int npos, nneg, nzero;
-    int spec;    // 1: the last panel was taken by the verified no-interchange path
-    int nacc, nrej;   // panels that path accepted / handed to the pivoting panel
-    unsigned done;    // k_bk_spec CTAs done with the current panel (reset by the last)
-    int nfail;        // columns of the pending panel whose row test k_bk_spec_rows evaluates
-    unsigned done2;   // k_bk_spec_rows CTAs done (reset by the last)
-};
 
 struct Cand {                  // one CTA's candidate of a cluster-wide arg-max
     unsigned long long bits;   // |v| bit pattern
@@ -86,10 +76,6 @@ struct PanelArgs {
     const double *maxabs;
     double zero_tol;
 };
-
-__device__ __forceinline__ unsigned long long absbits64(double v) {
-    return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL;
-}
 
 __device__ __forceinline__ void cand_combine(unsigned long long &b, int &i, unsigned long long b2, int i2) {
     if (b2 > b || (b2 == b && i2 < i)) {
@@ -137,22 +123,6 @@ __device__ void block_cand_to(unsigned long long b, int idx, const double *diag,
             out->abits = absbits64(alpha * __longlong_as_double((long long)b));
         }
     }
-}
-
-// 1/d by Newton-Raphson iteration x <- x (2 - d x) (two steps, as fused
-// multiply-adds) from the single-precision reciprocal of d: each step squares
-// the relative error, 2^-23 -> 2^-46 -> below the double rounding.  Takes six
-// FP64 instructions; d outside the normal float range goes through the
-// division operator.
-__device__ __forceinline__ double rcp_newton(double d) {
-    if (d == 0.0) return 0.0;
-    const float df = (float)d;
-    if (!(fabsf(df) >= 1.17549435e-38f && fabsf(df) <= 3.0e38f)) return 1.0 / d;
-    double x = (double)__frcp_rn(df);
-    double e = fma(-d, x, 1.0);
-    x = fma(x, e, x);
-    e = fma(-d, x, 1.0);
-    return fma(x, e, x);
 }
 
 // Cluster-wide arg-max of the candidates cand[slot] of all C CTAs (C <= 32),
@@ -1014,107 +984,10 @@ __global__ void __launch_bounds__(kSpecThreads) k_bk_spec_rows(SpecArgs a) {
     }
 }
 
-// ---------------------------------------------------------------------------
-// Persistent speculative factorization (one cooperative launch for all panels),
-// FP64 form (the FP32-update form is k_bk_persist32 below).
-//
-// The same no-interchange speculation as k_bk_spec, organised so that a kept
-// panel costs no launch: one grid of co-resident CTAs walks the panels of 64
-// columns, with a grid barrier after the panel (all column maxima known) and
-// one after its trailing update.  Per panel:
-//   A1 every CTA factors the 64 x 64 diagonal block in shared memory without
-//      interchanges, in four sub-panels of 16 columns: warp 0 factors the
-//      16 x 16 diagonal sub-block with register shuffles, one thread per row
-//      solves the rows below it, and a rank-16 update brings the rest of the
-//      block up to date (three block barriers per sub-panel instead of one
-//      per column);
-//   A2 each CTA takes a slice of the rows below the block, one thread per
-//      row: 64-row chunks in shared memory, solved against the block's
-//      factor in the same 16-column steps; the FP64 values w = A - sum L W,
-//      L = w / d and the column maxima of |w| (exact FP64 bit patterns,
-//      atomicMax) follow;
-//   B  after the grid barrier every CTA applies the rule's column test to the
-//      64 columns with the same data: the panel is kept when every column
-//      keeps its diagonal pivot (|a_jj| >= alpha colmax_j, or a zero column)
-//      and no pivot is within zero_tol max|S| of zero;
-//   C  the trailing update of a kept panel, tiles of the lower triangle over
-//      all CTAs; grid barrier.
-// The first panel that fails the column test (the rule would look at a row
-// or interchange) ends the kernel with st->k at its first column; the host
-// then runs the pivoting panels from there.  All arithmetic is FP64.
-// ---------------------------------------------------------------------------
+// (The FP64 form of the persistent no-interchange factorization is in
+// ldlt_persist64.cu.)
 constexpr int kPThreads = 256;
 constexpr int kPP = 65;      // shared-memory row pitch of the diagonal block
-
-struct PanelBar {
-    unsigned count;   // grid-barrier arrivals of the current launch
-    unsigned pad0;
-    int err, pad;
-};
-
-struct PersistArgs {
-    int N;
-    double *A;                      // lower triangle, column-major, ld N (trailing part updated in place)
-    double *L, *Dd, *Doff;
-    int32_t *kind;
-    double *Wg;                     // FP64 W of the current panel (T = double), ld N
-    float *Lf, *Wf;                 // FP32 L and W of the current panel (T = float), ld N
-    unsigned long long *cmax;       // [2][64]: per-column maxima of |w| (bit patterns), by panel parity
-    PanelState *st;
-    PanelBar *bar;
-    const double *maxabs;
-    double zero_tol;
-    long long wait_ns;              // bound of each grid-barrier wait
-    float *Af;                      // FP32 copy of the lower triangle, ld N (FP32-update kernel)
-    float *Lf2, *Wf2;               // FP32-update kernel: the odd panels' L and W columns (ld N)
-    unsigned *colcnt;               // FP32-update kernel: per 64-column block, trailing tiles updated
-};
-
-__device__ __forceinline__ long long global_ns() {
-    long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-// Grid-wide barrier of a cooperative launch (all CTAs co-resident).  The
-// arrival counter only grows within a launch (k_bk_init clears it): the
-// barrier numbered `epoch` (counted by each CTA's thread 0) completes when
-// the counter reaches epoch x gridDim.x, so arriving is one release-add with
-// no reply to wait for and nobody resets anything.  Every wait is bounded: a
-// CTA that waits longer than wait_ns sets the error word and returns false,
-// and so does every CTA that sees the word set.
-__device__ bool panel_barrier(PanelBar *b, unsigned &epoch, long long wait_ns) {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        const unsigned target = ++epoch * gridDim.x;
-        __threadfence();
-        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&b->count) : "memory");
-        const long long t0 = global_ns();
-        for (unsigned it = 0;; ++it) {
-            unsigned v;
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&b->count) : "memory");
-            if ((int)(v - target) >= 0) break;
-            if ((it & 63) == 63) {
-                if (*(volatile int *)&b->err) {
-                    ok = 0;
-                    break;
-                }
-                if (global_ns() - t0 > wait_ns) {
-                    atomicExch(&b->err, 1);
-                    ok = 0;
-                    break;
-                }
-            }
-        }
-        __threadfence();
-        if (*(volatile int *)&b->err) ok = 0;
-        s_ok = ok;
-    }
-    __syncthreads();
-    return s_ok != 0;
-}
 
 // Wait (thread 0, then the whole CTA) until *cnt reaches target; bounded like
 // panel_barrier and sharing its error word.
@@ -1146,19 +1019,9 @@ __device__ bool wait_count(const unsigned *cnt, unsigned target, PanelBar *b, lo
     return s_ok != 0;
 }
 
-template <typename T>
-__device__ __forceinline__ T chain_rcp(T d) {
-    if constexpr (sizeof(T) == sizeof(float)) return d != 0.0f ? __frcp_rn(d) : 0.0f;
-    else return d != 0.0 ? 1.0 / d : 0.0;
-}
-
-// w in FP64 from a chain value v: for FP32 chains the part of A that the FP32
-// copy dropped is added back (v started as float(A))
-template <typename T>
-__device__ __forceinline__ double chain_w64(T v, double a) {
-    if constexpr (sizeof(T) == sizeof(float)) return (double)v + (a - (double)(float)a);
-    else return v;
-}
+// w in FP64 from an FP32 chain value v: the part of A that the FP32 copy
+// dropped is added back (v started as float(A))
+__device__ __forceinline__ double chain_w64(float v, double a) { return (double)v + (a - (double)(float)a); }
 
 // The rule's column test for the panel at k (all threads of every CTA take
 // the same decision from the FP64 pivots s_d and the maxima gathered in
@@ -1197,221 +1060,14 @@ __device__ bool persist_keep(const PersistArgs &a, int k, int nb, int buf, int c
     return true;
 }
 
-__global__ void __launch_bounds__(kPThreads, 1) k_bk_persist(PersistArgs a) {
-    using T = double;
-    extern __shared__ __align__(16) unsigned char psm[];
-    T *V = reinterpret_cast<T *>(psm);      // [64][kPP]: the diagonal block; W values once factored
-                                            // (then [64][kPP]: a chunk of the rows below it)
-    __shared__ double s_d[64], s_rd[64];    // FP64 pivots and their reciprocals
-    __shared__ T s_rc[64];                  // the chain's reciprocals
-    __shared__ unsigned long long s_cmax[64];
-    const int N = a.N, G = (int)gridDim.x, g = (int)blockIdx.x, tid = threadIdx.x;
-    const int lane = tid & 31;
-    const double ztol = a.zero_tol * __ldg(a.maxabs);
-    unsigned epoch = 0;   // grid barriers passed (thread 0)
-    int p = 0;
-    for (int k = a.st->k; k < N; k += 64, ++p) {
-        const int nb = min(64, N - k);
-        const int buf = p & 1;
-        // ---------------- A1: the diagonal block
-        for (int e = tid; e < 64 * 64; e += kPThreads) {
-            const int c = e >> 6, r = e & 63;
-            T v = (T)0;
-            if (r < nb && c <= r) v = (T)a.A[(int64_t)(k + r) + (int64_t)(k + c) * N];
-            V[r * kPP + c] = v;
-        }
-        if (tid < 64) {
-            s_cmax[tid] = 0ULL;
-            s_rc[tid] = (T)0;      // columns beyond a narrow last panel stay zero
-        }
-        __syncthreads();
-        for (int c0 = 0; c0 < nb; c0 += 16) {
-            const int cw = min(16, nb - c0);
-            if (tid < 32) {   // warp 0: the 16 x 16 sub-block, lane = row c0 + lane
-                T v[16];
-#pragma unroll
-                for (int j = 0; j < 16; ++j) v[j] = (lane < cw && j <= lane) ? V[(c0 + lane) * kPP + c0 + j] : (T)0;
-                // (lanes that take no part get a zero multiplier: a conditional
-                // update kept v in local memory; the entries above a lane's
-                // diagonal that the zero-free form touches are never read)
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const T dj = __shfl_sync(0xffffffffu, v[j], j);
-                    const T rj = j < cw ? chain_rcp(dj) : (T)0;
-                    const T l = (lane > j && lane < cw) ? v[j] * rj : (T)0;
-#pragma unroll
-                    for (int t = 0; t < 16; ++t)
-                        if (t > j) v[t] = fma(-l, __shfl_sync(0xffffffffu, v[j], t), v[t]);
-                    if (lane == j && j < cw) s_rc[c0 + j] = rj;
-                }
-#pragma unroll
-                for (int j = 0; j < 16; ++j)
-                    if (lane < cw && j <= lane) V[(c0 + lane) * kPP + c0 + j] = v[j];
-            }
-            __syncthreads();
-            // rows of the block below the sub-block
-            for (int r = c0 + 16 + tid; r < nb; r += kPThreads) {
-                T v[16];
-#pragma unroll
-                for (int j = 0; j < 16; ++j) v[j] = j < cw ? V[r * kPP + c0 + j] : (T)0;
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const T l = j < cw ? v[j] * s_rc[c0 + j] : (T)0;
-#pragma unroll
-                    for (int t = j + 1; t < 16; ++t)
-                        if (t < cw) v[t] = fma(-l, V[(c0 + t) * kPP + c0 + j], v[t]);
-                }
-#pragma unroll
-                for (int j = 0; j < 16; ++j)
-                    if (j < cw) V[r * kPP + c0 + j] = v[j];
-            }
-            __syncthreads();
-            // rank-16 update of the rest of the block (lower triangle)
-            const int m0 = c0 + 16, mw = nb - m0;
-            if (mw > 0) {
-                const int npairs = mw * (mw + 1) / 2;
-                for (int e = tid; e < npairs; e += kPThreads) {
-                    int rr = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
-                    while ((rr + 1) * (rr + 2) / 2 <= e) ++rr;
-                    while (rr * (rr + 1) / 2 > e) --rr;
-                    const int r = m0 + rr, c = m0 + (e - rr * (rr + 1) / 2);
-                    T acc = V[r * kPP + c];
-#pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        if (j < cw) acc = fma(-(V[r * kPP + c0 + j] * s_rc[c0 + j]), V[c * kPP + c0 + j], acc);
-                    V[r * kPP + c] = acc;
-                }
-            }
-            __syncthreads();
-        }
-        // FP64 pivots
-        if (tid < 64) {
-            double d = 0.0, rd = 0.0;
-            if (tid < nb) {
-                d = chain_w64<T>(V[tid * kPP + tid], a.A[(int64_t)(k + tid) * (N + 1)]);
-                rd = rcp_newton(d);
-            }
-            s_d[tid] = d;
-            s_rd[tid] = rd;
-        }
-        __syncthreads();
-        const int wid = tid >> 5;
-        constexpr int kWarps = kPThreads / 32;
-        // the block's L and D and the column maxima of its rows: column c by
-        // CTA c mod G, one warp per column, lanes over rows (warp maxima)
-        for (int c = g + G * wid; c < nb; c += G * kWarps) {
-            unsigned long long bm = 0ULL;
-            for (int r = c + lane; r < nb; r += 32) {
-                const int64_t o = (int64_t)(k + r) + (int64_t)(k + c) * N;
-                if (r == c) {
-                    a.L[o] = 1.0;
-                    a.Dd[k + c] = s_d[c];
-                } else {
-                    const T w = V[r * kPP + c];
-                    a.L[o] = w * s_rd[c];
-                    const unsigned long long bw = absbits64((double)w);
-                    bm = bw > bm ? bw : bm;
-                }
-            }
-            const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(bm >> 32));
-            const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(bm >> 32) == hi ? (unsigned)bm : 0u);
-            if (lane == 0 && (hi | lo)) atomicMax(&s_cmax[c], ((unsigned long long)hi << 32) | lo);
-        }
-        // ---------------- A2: this CTA's rows below the block, 64 at a time
-        // in shared memory, solved against the block's factor in the same
-        // 16-column steps (row solves, then a rank-16 update of the rest)
-        T *U = V + 64 * kPP;                  // [64][kPP]: a chunk of rows
-        const int brow = N - k - nb;
-        const int R = (brow + G - 1) / G;
-        const int r_begin = k + nb + g * R, r_end = min(N, r_begin + R);
-        for (int cb = r_begin; cb < r_end; cb += 64) {
-            const int nr = min(64, r_end - cb);
-            __syncthreads();                   // the previous chunk is written out
-            for (int e = tid; e < 64 * 64; e += kPThreads) {
-                const int c = e >> 6, r = e & 63;
-                U[r * kPP + c] = (r < nr && c < nb) ? (T)a.A[(int64_t)(cb + r) + (int64_t)(k + c) * N] : (T)0;
-            }
-            __syncthreads();
-            for (int c0 = 0; c0 < nb; c0 += 16) {
-                const int cw = min(16, nb - c0);
-                for (int r = tid; r < nr; r += kPThreads) {
-                    T v[16];
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) v[j] = j < cw ? U[r * kPP + c0 + j] : (T)0;
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const T l = j < cw ? v[j] * s_rc[c0 + j] : (T)0;
-#pragma unroll
-                        for (int t = j + 1; t < 16; ++t)
-                            if (t < cw) v[t] = fma(-l, V[(c0 + t) * kPP + c0 + j], v[t]);
-                    }
-#pragma unroll
-                    for (int j = 0; j < 16; ++j)
-                        if (j < cw) U[r * kPP + c0 + j] = v[j];
-                }
-                __syncthreads();
-                const int m0 = c0 + 16, mw = nb - m0;
-                if (mw > 0) {
-                    for (int e = tid; e < nr * mw; e += kPThreads) {
-                        const int r = e / mw, c = m0 + (e - (e / mw) * mw);
-                        T acc = U[r * kPP + c];
-#pragma unroll
-                        for (int j = 0; j < 16; ++j)
-                            if (j < cw) acc = fma(-(U[r * kPP + c0 + j] * s_rc[c0 + j]), V[c * kPP + c0 + j], acc);
-                        U[r * kPP + c] = acc;
-                    }
-                }
-                __syncthreads();
-            }
-            // outputs and column maxima: one warp per column, lanes over rows
-            for (int c = wid; c < nb; c += kWarps) {
-                unsigned long long bm = 0ULL;
-                for (int r = lane; r < nr; r += 32) {
-                    const int i = cb + r;
-                    const int64_t o = (int64_t)i + (int64_t)(k + c) * N;
-                    const double w = U[r * kPP + c];
-                    a.L[o] = w * s_rd[c];
-                    a.Wg[(int64_t)i + (int64_t)c * N] = w;
-                    const unsigned long long bw = absbits64(w);
-                    bm = bw > bm ? bw : bm;
-                }
-                const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(bm >> 32));
-                const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(bm >> 32) == hi ? (unsigned)bm : 0u);
-                if (lane == 0 && (hi | lo)) atomicMax(&s_cmax[c], ((unsigned long long)hi << 32) | lo);
-            }
-        }
-        __syncthreads();
-        if (tid < 64 && s_cmax[tid]) atomicMax(&a.cmax[buf * 64 + tid], s_cmax[tid]);
-        if (!panel_barrier(a.bar, epoch, a.wait_ns)) return;
-        // ---------------- B: the rule's column test, the same in every CTA
-        if (!persist_keep(a, k, nb, buf, buf ^ 1, ztol, s_d)) {
-            if (g == 0 && tid == 0) {   // the panel loop takes over at column k
-                a.st->k = k;
-                a.st->kb = 0;
-                a.st->spec = 0;
-            }
-            return;
-        }
-        if (k + nb >= N) break;
-        // ---------------- C: trailing update
-        {
-            const int base = k + nb;
-            const int nt = (N - base + kUT - 1) / kUT;
-            const int tiles = nt * (nt + 1) / 2;
-            for (int t = g; t < tiles; t += G) {
-                trailing_tile<T>(t, N, nb, k, 65, a.A, a.L, a.Wg, a.Lf, a.Wf, psm);
-                __syncthreads();
-            }
-        }
-        __threadfence();
-        if (!panel_barrier(a.bar, epoch, a.wait_ns)) return;
-    }
-}
-
 // ---------------------------------------------------------------------------
 // Persistent no-interchange factorization, FP32-update form (the refined
-// mixed-precision path).  The same panel sequence, column test and hand-over
-// as k_bk_persist, with the arithmetic of the loop in FP32 only:
+// mixed-precision path): one cooperative launch walks panels of 64 columns; a
+// panel is kept when the rule's column test on the computed columns keeps every
+// diagonal pivot and no pivot is within zero_tol max|S| of zero, and the first
+// one that is not ends the kernel with st->k at its first column (the host
+// then runs the pivoting panels from there).  The arithmetic of the loop is
+// FP32:
 //   - the prologue copies the lower triangle of S into Af (FP32, ld N); the
 //     trailing updates run on Af in place, and the FP64 matrix keeps S;
 //   - each 64-column panel is factored in Q-column sub-panels (Q = 16).  A
@@ -1898,7 +1554,7 @@ __global__ void __launch_bounds__(kPThreads, 1) k_bk_persist32(PersistArgs a) {
                 // its rows: column c by CTA c mod G, one warp per column
                 if (tid < 64) {
                     double d = 0.0;
-                    if (tid < nb) d = chain_w64<float>(Rb[tid * kPP + tid], adiag);
+                    if (tid < nb) d = chain_w64(Rb[tid * kPP + tid], adiag);
                     s_d[tid] = d;
                 }
                 __syncthreads();
@@ -2153,7 +1809,7 @@ void launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned block, size_t sm
 // (2 x 64), the pending row tests (64) and their partial row maxima
 // ((ceil(N / 32) + 2) x 64)
 struct BlockedScratch {
-    size_t wg, st, lf, wf, cmax, fail, rowpart, af, lf2, wf2, colcnt, total;
+    size_t wg, st, lf, wf, cmax, fail, rowpart, af, lf2, wf2, colcnt, p64, total;
 };
 
 BlockedScratch blocked_scratch(int64_t N) {
@@ -2171,7 +1827,8 @@ BlockedScratch blocked_scratch(int64_t N) {
     l.lf2 = l.af + up(n * n * sizeof(float));   // the FP32 copy of the persistent FP32-update kernel
     l.wf2 = l.lf2 + up(n * 64 * sizeof(float));
     l.colcnt = l.wf2 + up(n * 64 * sizeof(float));
-    l.total = l.colcnt + up(((n + 63) / 64 + 1) * sizeof(unsigned));
+    l.p64 = l.colcnt + up(((n + 63) / 64 + 1) * sizeof(unsigned));
+    l.total = l.p64 + up(persist64_scratch_bytes(N));   // residues of the FP64 persistent kernel
     return l;
 }
 
@@ -2180,34 +1837,18 @@ BlockedScratch blocked_scratch(int64_t N) {
 // the grid barrier of the persistent kernel shares the panel state's slot
 PanelBar *grid_bar(char *w, const BlockedScratch &lay) { return reinterpret_cast<PanelBar *>(w + lay.st + 128); }
 
-// dynamic shared memory of k_bk_persist<T>: the diagonal block, or the staged
-// rows of a trailing-update tile
-template <typename T>
-size_t persist_smem() {
-    if constexpr (sizeof(T) == sizeof(float))   // k_bk_persist32: staged rows, or a trailing tile's panel rows
-        return std::max({(size_t)kRowsBuf * kPP * sizeof(float), 2 * (size_t)64 * kUT * sizeof(float), kTcSmem});
-    return std::max(2 * (size_t)64 * kPP * sizeof(T), 2 * (size_t)65 * kUT * sizeof(T));
+// dynamic shared memory of k_bk_persist32: staged rows, or a trailing tile's panel rows
+constexpr size_t persist32_smem() {
+    return std::max({(size_t)kRowsBuf * kPP * sizeof(float), 2 * (size_t)64 * kUT * sizeof(float), kTcSmem});
 }
 
-template <typename T>
-const void *persist_kernel() {
-    if constexpr (sizeof(T) == sizeof(float)) return (const void *)k_bk_persist32<kPersistQ>;
-    else return (const void *)k_bk_persist;
-}
-
-// Run k_bk_persist from column 0; returns the column where it stopped (N: all
-// panels kept).  One cooperative launch; reads two words back (synchronises
-// the stream).
-template <typename T>
-int run_persistent(cudaStream_t s, int num_sms, int N, const PersistArgs &pa, PanelState *st, PanelBar *bar) {
+void launch_persist32(cudaStream_t s, int num_sms, int N, const PersistArgs &pa) {
+    const void *kern = (const void *)k_bk_persist32<kPersistQ>;
     static PerDeviceOnce once;
-    MDSIP_CUDA(once.run([] {
-        return cudaFuncSetAttribute(persist_kernel<T>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)persist_smem<T>());
-    }));
+    MDSIP_CUDA(once.run(
+        [&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)persist32_smem()); }));
     int per_sm = 0;
-    MDSIP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persist_kernel<T>(), kPThreads,
-                                                             persist_smem<T>()));
+    MDSIP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPThreads, persist32_smem()));
     MDSIP_REQUIRE(per_sm >= 1, MDSIP_ERR_CUDA, "ldlt: persistent factorization does not fit an SM");
     // about three trailing tiles per CTA after the first panel, at most one CTA per SM
     const int64_t nt = std::max<int64_t>(1, (N - 64 + kUT - 1) / kUT);
@@ -2215,9 +1856,13 @@ int run_persistent(cudaStream_t s, int num_sms, int N, const PersistArgs &pa, Pa
     const int G = (int)std::min<int64_t>(want, (int64_t)num_sms);
     PersistArgs args = pa;
     void *kargs[] = {&args};
-    MDSIP_CUDA(cudaLaunchCooperativeKernel(persist_kernel<T>(), dim3(G), dim3(kPThreads), kargs,
-                                           persist_smem<T>(), s));
+    MDSIP_CUDA(cudaLaunchCooperativeKernel(kern, dim3(G), dim3(kPThreads), kargs, persist32_smem(), s));
     count_launch();
+}
+
+// Where the persistent kernel stopped (N: all panels kept); reads two words
+// back (synchronises the stream).
+int persist_stopped_at(cudaStream_t s, const PanelState *st, const PanelBar *bar) {
     thread_local int *h = nullptr;
     if (!h) MDSIP_CUDA(cudaMallocHost(&h, 4 * sizeof(int)));
     MDSIP_CUDA(cudaMemcpyAsync(h, &st->k, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -2240,17 +1885,17 @@ std::vector<int> ldlt_blocked_widths(int64_t N, bool f32) {
 bool ldlt_blocked_available(int64_t N) { return blocked_config(N, true).C > 0 && blocked_config(N, false).C > 0; }
 
 // The persistent no-interchange factorization runs first (and the host reads
-// back where it stopped) in mode 2, and in mode 1 from kPersistentMinOrder on
-// (measured on the convex Newton-step shape, persistent against per-panel
-// launches: N = 2050 FP32 updates 1.65 / 1.73 ms, FP64 8.3 / 11.1 ms; N = 4050
-// 4.8 / 6.0 and 31 / 36 ms; N = 8003 27.5 / 42.9 and 179 / 194 ms) and
-// wherever the pivoting panel does not fit shared memory: it needs no
-// pivoting panel unless a panel fails the column test.  Below that order --
-// the many small instances of a batch among them -- the per-panel launches
-// (captured in a graph from their second use) stay.
-bool ldlt_persistent_path(int64_t N, int spec) {
+// back where it stopped) in mode 2, in mode 1 at every order with FP64 updates
+// and from kPersistentMinOrder on with FP32 updates, and wherever the pivoting
+// panel does not fit shared memory: it needs no pivoting panel unless a panel
+// fails the column test, and a first panel that fails costs one short launch.
+// FP64, convex Newton-step shape, persistent / per-panel launches: N = 33
+// 0.10 / 0.14 ms, 351 0.46 / 1.47, 1036 1.31 / 4.46, 2050 2.83 / 11.1.
+// FP32 updates (the many small instances of a batch among them, whose
+// per-panel launches replay as one graph): N = 2050 0.82 / 1.73 ms.
+bool ldlt_persistent_path(int64_t N, int spec, bool fp32_update) {
     if (spec == 0 || N <= 0 || N > (int64_t)0x7fffffff / 2) return false;
-    return spec == 2 || N >= kPersistentMinOrder || !ldlt_blocked_available(N);
+    return spec == 2 || !fp32_update || N >= kPersistentMinOrder || !ldlt_blocked_available(N);
 }
 
 // S (lower, ld N) is overwritten.  scratch: ldlt_blocked_scratch_bytes(N),
@@ -2264,7 +1909,7 @@ void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, cons
     }
     BlockedConfig cfg = blocked_config(N, fp32_update, nb);
     if (cfg.C == 0) cfg = blocked_config(N, fp32_update);
-    const bool persist = ldlt_persistent_path(N, spec);
+    const bool persist = ldlt_persistent_path(N, spec, fp32_update);
     MDSIP_REQUIRE(cfg.C > 0 || persist, MDSIP_ERR_INVALID_ARG, "ldlt: N too large for the blocked factorization");
     char *w = static_cast<char *>(scratch);
     MDSIP_REQUIRE((reinterpret_cast<uintptr_t>(w) & 255) == 0, MDSIP_ERR_INVALID_ARG, "ldlt: misaligned scratch");
@@ -2285,7 +1930,6 @@ void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, cons
         pa.Dd = out.Dd;
         pa.Doff = out.Doff;
         pa.kind = out.kind;
-        pa.Wg = Wg;
         pa.Lf = reinterpret_cast<float *>(w + lay.lf);
         pa.Wf = reinterpret_cast<float *>(w + lay.wf);
         pa.cmax = reinterpret_cast<unsigned long long *>(w + lay.cmax);
@@ -2298,8 +1942,9 @@ void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, cons
         pa.Wf2 = reinterpret_cast<float *>(w + lay.wf2);
         pa.colcnt = reinterpret_cast<unsigned *>(w + lay.colcnt);
         pa.wait_ns = 20LL * 1000 * 1000 * 1000;   // 20 s: far above the longest phase (FP64 update at N ~ 44000)
-        k0 = fp32_update ? run_persistent<float>(s, num_sms, (int)N, pa, st, bar)
-                         : run_persistent<double>(s, num_sms, (int)N, pa, st, bar);
+        if (fp32_update) launch_persist32(s, num_sms, (int)N, pa);
+        else launch_persist64(s, num_sms, N, pa, w + lay.p64);
+        k0 = persist_stopped_at(s, st, bar);
         MDSIP_REQUIRE(k0 >= N || cfg.C > 0, MDSIP_ERR_INVALID_ARG,
                       "ldlt: a panel needs interchanges and N is too large for the pivoting panel");
         // the panel loop's no-interchange kernels expect their column maxima and

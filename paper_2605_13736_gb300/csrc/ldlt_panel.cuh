@@ -1,0 +1,131 @@
+// Declarations shared by the blocked LDL^T (ldlt_blocked.cu) and its
+// persistent FP64 kernel (ldlt_persist64.cu).
+#pragma once
+
+#include "internal.cuh"
+
+namespace mdsip {
+
+struct PanelState {
+    int k;       // first column of the next panel
+    int kb;      // columns factored by the last panel
+    int npos, nneg, nzero;
+    int spec;    // 1: the last panel was taken by the verified no-interchange path
+    int nacc, nrej;   // panels that path accepted / handed to the pivoting panel
+    unsigned done;    // k_bk_spec CTAs done with the current panel (reset by the last)
+    int nfail;        // columns of the pending panel whose row test k_bk_spec_rows evaluates
+    unsigned done2;   // k_bk_spec_rows CTAs done (reset by the last)
+};
+
+struct PanelBar {
+    unsigned count;   // grid-barrier arrivals of the current launch
+    unsigned pad0;
+    int err, pad;
+};
+
+struct PersistArgs {
+    int N;
+    double *A;                      // lower triangle, column-major, ld N (trailing part updated in place)
+    double *L, *Dd, *Doff;
+    int32_t *kind;
+    float *Lf, *Wf;                 // FP32-update kernel: L and W of the current panel, ld N
+    unsigned long long *cmax;       // [2][64]: per-column maxima of |w| (bit patterns), by panel parity
+    PanelState *st;
+    PanelBar *bar;
+    const double *maxabs;
+    double zero_tol;
+    long long wait_ns;              // bound of each grid-barrier wait
+    float *Af;                      // FP32 copy of the lower triangle, ld N (FP32-update kernel)
+    float *Lf2, *Wf2;               // FP32-update kernel: the odd panels' L and W columns (ld N)
+    unsigned *colcnt;               // FP32-update kernel: per 64-column block, trailing tiles updated
+};
+
+namespace {
+
+__device__ __forceinline__ unsigned long long absbits64(double v) {
+    return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL;
+}
+
+// 1/d by Newton-Raphson iteration x <- x (2 - d x) (0 for d = 0): the first
+// step in FP32 and integers on the mantissa m of d -- hardware reciprocal q of
+// m's upper 24 bits, the residual 1 - m q with all of m, x = q + q (e + e^2) in
+// units of 2^-53, good to about 2^-46 -- and the last in FP64.  Two FP64
+// instructions, where the FP32 conversions and two FP64 steps were six: on
+// GB300 each occupies a warp's FP64 pipe for 64 cycles and every pivot waits
+// for this value.  d near the ends of the range goes through the division
+// operator.
+__device__ __forceinline__ double rcp_newton(double d) {
+    const int hi = __double2hiint(d);
+    const unsigned lo = (unsigned)__double2loint(d);
+    const int ef = (hi >> 20) & 0x7ff;
+    if (ef < 100 || ef > 1946) return d == 0.0 ? 0.0 : 1.0 / d;
+    const float mh = __uint_as_float(0x3f800000u | (((unsigned)hi & 0xfffffu) << 3) | (lo >> 29));
+    const float ml = (float)(lo & 0x1fffffffu) * 0x1p-52f;
+    float q;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(mh));
+    const float e = fmaf(-ml, q, fmaf(-mh, q, 1.0f));
+    const float qe = q * e;
+    const int c = __float2int_rn(fmaf(qe, e, qe) * 0x1p52f);       // |q e| < 2^-21
+    const unsigned qb = __float_as_uint(q);                        // 1/2 <= q <= 1
+    const long long X = ((long long)((qb & 0x7fffffu) | 0x800000u) << (29 + (int)(qb >> 23) - 126)) + 2LL * c;
+    const double x = __longlong_as_double((1021LL << 52) + X);     // 2^52 <= X <= 2^53 (as 1022 << 52 plus X - 2^52)
+    const double m = __hiloint2double((hi & 0xfffff) | 0x3ff00000, (int)lo);
+    const double y = fma(x, fma(-m, x, 1.0), x);                   // 1 / m
+    return __hiloint2double((__double2hiint(y) - ((ef - 1023) << 20)) | (hi & (int)0x80000000), __double2loint(y));
+}
+
+__device__ __forceinline__ long long global_ns() {
+    long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
+// Grid-wide barrier of a cooperative launch (all CTAs co-resident).  The
+// arrival counter only grows within a launch (k_bk_init clears it): the
+// barrier numbered `epoch` (counted by each CTA's thread 0) completes when
+// the counter reaches epoch x gridDim.x, so arriving is one release-add with
+// no reply to wait for and nobody resets anything.  Every wait is bounded: a
+// CTA that waits longer than wait_ns sets the error word and returns false,
+// and so does every CTA that sees the word set.
+__device__ bool panel_barrier(PanelBar *b, unsigned &epoch, long long wait_ns) {
+    __shared__ int s_ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int ok = 1;
+        const unsigned target = ++epoch * gridDim.x;
+        __threadfence();
+        asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&b->count) : "memory");
+        const long long t0 = global_ns();
+        for (unsigned it = 0;; ++it) {
+            unsigned v;
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&b->count) : "memory");
+            if ((int)(v - target) >= 0) break;
+            if ((it & 63) == 63) {
+                if (*(volatile int *)&b->err) {
+                    ok = 0;
+                    break;
+                }
+                if (global_ns() - t0 > wait_ns) {
+                    atomicExch(&b->err, 1);
+                    ok = 0;
+                    break;
+                }
+            }
+        }
+        __threadfence();
+        if (*(volatile int *)&b->err) ok = 0;
+        s_ok = ok;
+    }
+    __syncthreads();
+    return s_ok != 0;
+}
+
+}  // namespace
+
+// ldlt_persist64.cu: the persistent no-interchange factorization, FP64.  One
+// cooperative launch from column pa.st->k on; it stops (st->k) at the first
+// panel the rule's column test rejects.  scratch: persist64_scratch_bytes(N).
+size_t persist64_scratch_bytes(int64_t N);
+void launch_persist64(cudaStream_t s, int num_sms, int64_t N, const PersistArgs &pa, void *scratch);
+
+}  // namespace mdsip

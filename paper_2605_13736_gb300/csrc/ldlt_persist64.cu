@@ -1,0 +1,545 @@
+// Persistent no-interchange LDL^T, FP64 (Section 2.3; the form that runs first
+// on the FP64 path): one cooperative launch walks panels of 32 columns; a panel
+// is kept when the Bunch-Kaufman rule's column test, evaluated on the computed
+// columns, keeps every diagonal pivot, and the first one that is not ends the
+// kernel with st->k at its first column (the pivoting panels take over).
+//
+// GB300 issues an FP64 instruction of a warp in 64 cycles per sub-partition
+// (76 with all four busy), whatever its lanes do, and one chain of dependent
+// FP64 instructions runs at that same rate.  So the kernel counts FP64 warp
+// instructions: element-wise parallel steps spread over the four
+// sub-partitions, and the N^3 / 6 multiply-adds of the trailing updates taken
+// off that pipe altogether.  Per panel:
+//   A  every CTA factors the 32 x 32 diagonal block and its own rows below it
+//      in shared memory, in two 16-column sub-panels: the 16 x 16 sub-block one
+//      lower-triangle element per thread (one multiply, one FMA and a
+//      reciprocal per column and warp), the rows four threads each, then a
+//      rank-16 update of the rest; L, D, the column maxima;
+//   R  the rows' W scaled by |d|^-1/2 and rounded once to 54-bit integers per
+//      row, as residues modulo 13 coprime moduli in BF16 (rns.cuh);
+//   B  grid barrier, the column test, the same decision in every CTA;
+//   C  the trailing update A -= W D^-1 W^T of a kept panel as 13 exact
+//      tensor-core contractions per 128 x 32 tile (bulk copies, tcgen05 into TMEM, the
+//      Chinese remainder in 128-bit integers on 16 warps, one rounding to FP64, one FP64
+//      subtraction per entry): sum_j sign(d_j) X_ij X_cj <= 32 2^108 in exact
+//      integers, an error below that of a 32-term FP64 dot product; grid barrier.
+// Against the 64-column form with DFMA trailing tiles (its first panel's tiles
+// alone took 215 us): N = 2050 7.90 -> 2.83 ms, 4050 30.6 -> 8.9 ms.  Of the 45
+// us a panel takes at N = 2050 the pivot chain is 10 (32 columns of three
+// dependent FP64 instructions, a reciprocal's FP32 part and a barrier), the
+// rows and the rank-16 update 8, the tiles 16, grid barriers with the skew
+// between CTAs 5.
+#include <cuda_bf16.h>
+
+#include <algorithm>
+
+#include "internal.cuh"
+#include "ldlt_panel.cuh"
+#include "rns.cuh"
+#include "tc.cuh"
+
+namespace mdsip {
+
+namespace {
+
+using bf16 = __nv_bfloat16;
+
+constexpr int RL = 13;                  // moduli: log2 of their product 116.3
+constexpr int QB = 54;                  // 2 QB + 5 + 2 <= 116
+constexpr int QN = 32;                  // panel width
+constexpr int Q_THREADS = 576;          // warps 0-7 factor; 0-15 update, 16 loads, 17 issues
+constexpr int Q_COMP = 256;             // threads of the factorization
+constexpr int Q_EPI = 16;               // warps of the trailing update
+constexpr int Q_OWN = 96;               // rows below the block staged at a time
+constexpr int VP = 33, LP = 17;         // shared-memory row pitches (doubles)
+constexpr int QA_BYTES = 128 * 64, QB_BYTES = 32 * 64;   // residues of 128 rows / 32 rows, 32 BF16 each
+constexpr int Q_STAGE = QA_BYTES + QB_BYTES;             // one modulus; a tile's 13 are loaded together
+constexpr size_t kQSmem = 1024 + (size_t)RL * Q_STAGE + (size_t)(QN + Q_OWN) * (VP + LP) * sizeof(double);
+
+__constant__ rns::Tab<RL> c_tab13 = rns::make_tab<RL>();
+
+struct P64Args {
+    PersistArgs p;
+    // [modulus][row][32]: X, and sign(d) X (M/p)^-1, modulo p, each 8 rows laid out as
+    // the tensor core's 64-byte-swizzled shared-memory atom (16-byte unit c of row r
+    // at unit c ^ (r / 2) mod 4), so that a tile's operand is one contiguous copy
+    bf16 *RA, *RB;
+    int *rowE;           // row exponents
+    int npad;
+};
+
+__device__ __forceinline__ void bar_comp() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+__device__ __forceinline__ void bar_chain() { asm volatile("bar.sync 2, 128;" ::: "memory"); }
+
+// The 16 x 16 diagonal sub-block at c0 (threads 0 .. 127): thread = one element
+// (ei, ej) of the lower triangle, ej >= 1.  Column j goes through `col` (two
+// buffers, one barrier per column); v_it -= (w_i w_t) / d.
+__device__ void q_chain(double *V, double *col, double *s_rc, int c0, int cw, int ei, int ej) {
+    const int tid = threadIdx.x;
+    double v = ei < cw && ej > 0 ? V[(c0 + ei) * VP + c0 + ej] : 0.0;
+    for (int j = 0; j < cw; ++j) {
+        double *cb = col + (j & 1) * 16;
+        if (j == 0) {
+            if (tid < 16) cb[tid] = V[(c0 + tid) * VP + c0];
+        } else if (ej == j) {
+            cb[ei] = v;
+            V[(c0 + ei) * VP + c0 + j] = v;
+        }
+        bar_chain();
+        const double d = cb[j];
+        const double u = ej > j ? cb[ei] * cb[ej] : 0.0;
+        const double r = rcp_newton(d);
+        if (tid == 0) s_rc[c0 + j] = r;
+        if (ej > j) v = fma(-u, r, v);
+    }
+}
+
+// Rows below the sub-block at c0 (block rows c0 + 16 .. nb - 1 when blk, then
+// the nr staged own rows): four threads per row, columns strided by four.
+__device__ void q_rows(double *V, double *Ls, const double *s_rc, int c0, int nb, bool blk, int nr) {
+    const int nblk = blk ? max(0, nb - c0 - 16) : 0;
+    const int total = nblk + nr;
+    const int lane = threadIdx.x & 31, q = lane & 3;
+    for (int x0 = 0; x0 < total; x0 += Q_COMP / 4) {
+        const int x = x0 + (threadIdx.x >> 2);
+        const bool live = x < total;
+        if (!__any_sync(0xffffffffu, live)) break;   // warp-uniform: no row in this warp
+        const int row = live ? (x < nblk ? c0 + 16 + x : QN + x - nblk) : 0;
+        double v[4];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) v[s] = live ? V[row * VP + c0 + q + 4 * s] : 0.0;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            const double w = __shfl_sync(0xffffffffu, v[j >> 2], (lane & ~3) | (j & 3));
+            const double l = w * s_rc[c0 + j];
+            if (live && (j & 3) == q) Ls[row * LP + j] = l;
+            if (j < 15) {
+#pragma unroll
+                for (int s = j >> 2; s < 4; ++s) {
+                    if ((j & 3) == 3 && s == (j >> 2)) continue;   // no column of this slot beyond j
+                    const int t = q + 4 * s;
+                    const double w2 = t > j ? V[(c0 + t) * VP + c0 + j] : 0.0;
+                    v[s] = fma(-l, w2, v[s]);
+                }
+            }
+        }
+        if (live) {
+#pragma unroll
+            for (int s = 0; s < 4; ++s) V[row * VP + c0 + q + 4 * s] = v[s];
+        }
+    }
+}
+
+// Rank-16 update of columns 16 .. 31 with the first sub-panel, two columns per
+// thread: block rows 16 .. nb - 1 (lower triangle, when blk), own rows.
+__device__ void q_rank16(double *V, const double *Ls, int nb, bool blk, int nr) {
+    const int nblk = blk ? nb - 16 : 0;
+    for (int e = threadIdx.x; e < (nblk + nr) * 8; e += Q_COMP) {
+        const int x = e >> 3, c = 16 + 2 * (e & 7);
+        const int row = x < nblk ? 16 + x : QN + x - nblk;
+        if (x < nblk && c > row) continue;
+        double a0 = V[row * VP + c], a1 = V[row * VP + c + 1];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            const double l = Ls[row * LP + j];
+            a0 = fma(-l, V[c * VP + j], a0);
+            a1 = fma(-l, V[(c + 1) * VP + j], a1);
+        }
+        V[row * VP + c] = a0;
+        V[row * VP + c + 1] = a1;
+    }
+}
+
+// column maximum of |w| over a warp's rows into s_cmax (bit patterns)
+__device__ __forceinline__ void q_colmax(unsigned long long bm, unsigned long long *dst, int lane) {
+    const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(bm >> 32));
+    const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(bm >> 32) == hi ? (unsigned)bm : 0u);
+    if (lane == 0 && (hi | lo)) atomicMax(dst, ((unsigned long long)hi << 32) | lo);
+}
+
+__global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
+    const PersistArgs &a = q.p;
+    extern __shared__ uint8_t psm_raw[];
+    uint8_t *ring = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(psm_raw) + 1023) & ~uintptr_t(1023));
+    double *V = reinterpret_cast<double *>(ring + RL * Q_STAGE);   // [32 + Q_OWN][VP]: block rows, own rows
+    double *Ls = V + (QN + Q_OWN) * VP;                                  // [32 + Q_OWN][LP]: L of the first sub-panel
+    __shared__ double s_d[QN], s_rc[QN], s_col[32];
+    __shared__ unsigned long long s_cmax[QN], s_sm[QN];
+    __shared__ int s_se[QN];
+    __shared__ uint4 s_km[16];   // -(bias + k M) modulo 2^128, k = -8 .. 7 at k + 8
+    __shared__ __align__(8) uint64_t full, tfull, tempty;   // operands loaded, products done, accumulators read
+    __shared__ uint32_t s_tmem;
+    const int N = a.N, G = (int)gridDim.x, g = (int)blockIdx.x, tid = threadIdx.x;
+    const int lane = tid & 31, wid = tid >> 5;
+    const double maxabs = __ldg(a.maxabs), ztol = a.zero_tol * maxabs;
+    // entries near the subnormal range would lose bits in the integer form: the
+    // pivoting panels take such a matrix (st->k stays where it is)
+    if (!(maxabs > 0x1p-900)) return;
+    if (tid == 0) {
+        tc::mbar_init(&full, 1);
+        tc::mbar_init(&tfull, 1);
+        tc::mbar_init(&tempty, Q_EPI);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (tid < 16) {
+        unsigned __int128 M = 0, B = 0;
+        for (int m = 3; m >= 0; --m) {
+            M = (M << 32) | c_tab13.mod32[m];
+            B = (B << 32) | c_tab13.bias32[m];
+        }
+        const unsigned __int128 v = (unsigned __int128)0 - B - M * (unsigned __int128)(__int128)(tid - 8);
+        s_km[tid] = make_uint4((unsigned)v, (unsigned)(v >> 32), (unsigned)(v >> 64), (unsigned)(v >> 96));
+    }
+    if (wid == 0) tc::tmem_alloc(&s_tmem, 512);
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    const uint32_t tmem = s_tmem;
+    int tl = 0;   // tiles this warp's role has gone through
+    auto release = [&]() {
+        if (wid == Q_EPI && tl > 0) tc::mbar_wait(&full, (tl - 1) & 1);   // no copy is in flight when the CTA leaves
+        tc::fence_before();
+        __syncthreads();
+        if (wid == 0) tc::tmem_dealloc(tmem, 512);
+    };
+    // this thread's element of a 16 x 16 lower triangle without its first column
+    int ei = 0, ej = 0;
+    if (tid < 120) {
+        int e = tid;
+        for (ej = 1; e >= 16 - ej; ++ej) e -= 16 - ej;
+        ei = ej + e;
+    }
+
+    unsigned epoch = 0;   // grid barriers passed (thread 0)
+    int p = 0;
+    for (int k = a.st->k; k < N; k += QN, ++p) {
+        const int nb = min(QN, N - k);
+        const int buf = p & 1;
+        // own rows: multiples of 8 per CTA
+        const int brow = N - k - nb;
+        const int R = ((brow + G - 1) / G + 7) / 8 * 8;
+        const int r_begin = k + nb + g * R, r_end = min(N, r_begin + R);
+        if (wid < 8) {
+            for (int cb = r_begin, first = 1; first || cb < r_end; cb += Q_OWN, first = 0) {
+                const int nr = max(0, min(Q_OWN, r_end - cb));
+                // ---- stage the block (first time) and the own rows
+                if (first) {
+                    for (int e = tid; e < QN * QN; e += Q_COMP) {
+                        const int c = e >> 5, r = e & 31;
+                        V[r * VP + c] = (r < nb && c <= r) ? __ldcg(a.A + (int64_t)(k + r) + (int64_t)(k + c) * N) : 0.0;
+                    }
+                    if (tid < QN) {
+                        s_cmax[tid] = 0ULL;
+                        s_rc[tid] = 0.0;    // columns beyond a narrow last panel stay zero
+                    }
+                }
+#pragma unroll
+                for (int c = wid; c < QN; c += 8)
+                    for (int r = lane; r < nr; r += 32)
+                        V[(QN + r) * VP + c] = c < nb ? __ldcg(a.A + (int64_t)(cb + r) + (int64_t)(k + c) * N) : 0.0;
+                bar_comp();
+                // ---- factor and solve
+                for (int c0 = 0; c0 < nb; c0 += 16) {
+                    if (first) {
+                        if (tid < 128) q_chain(V, s_col, s_rc, c0, min(16, nb - c0), ei, ej);
+                        bar_comp();
+                    }
+                    q_rows(V, Ls, s_rc, c0, nb, first, nr);
+                    bar_comp();
+                    if (c0 == 0 && nb > 16) {
+                        q_rank16(V, Ls, nb, first, nr);
+                        bar_comp();
+                    }
+                }
+                if (first) {
+                    if (wid == 0) {   // pivots and their scaling |d|^-1/2
+                        const double d = lane < nb ? V[lane * VP + lane] : 0.0;
+                        s_d[lane] = d;
+                        unsigned long long m = 0ULL;
+                        int e = 0;
+                        const double ad = fabs(d);
+                        if (ad > 0x1p-1000 && isfinite(ad)) rns::rsqrt64(ad, m, e);   // else the panel is rejected
+                        s_sm[lane] = m;
+                        s_se[lane] = e;
+                    } else {
+                        // the block's L and D and the column maxima of its rows: column c by
+                        // CTA c mod G, one warp per column, lanes over rows
+                        for (int c = g + G * (wid - 1); c < nb; c += G * 7) {
+                            const int r = lane;
+                            unsigned long long bm = 0ULL;
+                            if (r >= c && r < nb) {
+                                const int64_t o = (int64_t)(k + r) + (int64_t)(k + c) * N;
+                                const double w = V[r * VP + c];
+                                if (r == c) {
+                                    a.L[o] = 1.0;
+                                    a.Dd[k + c] = w;
+                                } else {
+                                    a.L[o] = w * s_rc[c];
+                                    bm = absbits64(w);
+                                }
+                            }
+                            q_colmax(bm, &s_cmax[c], lane);
+                        }
+                    }
+                    bar_comp();
+                }
+                // ---- own rows: L, column maxima (a warp per column)
+                for (int c = wid; c < nb; c += 8) {
+                    unsigned long long bm = 0ULL;
+                    for (int r = lane; r < nr; r += 32) {
+                        const double w = V[(QN + r) * VP + c];
+                        a.L[(int64_t)(cb + r) + (int64_t)(k + c) * N] = w * s_rc[c];
+                        const unsigned long long bw = absbits64(w);
+                        bm = bw > bm ? bw : bm;
+                    }
+                    q_colmax(bm, &s_cmax[c], lane);
+                }
+                // ---- own rows: residues (a warp per row, lane = panel column)
+                for (int r = wid; r < nr; r += 8) {
+                    const double w = lane < nb ? V[(QN + r) * VP + lane] : 0.0;
+                    const unsigned long long sm = s_sm[lane];
+                    const int se = s_se[lane];
+                    const int ef = (int)((__double_as_longlong(w) >> 52) & 0x7ff);
+                    const int E = __reduce_max_sync(0xffffffffu, ef != 0 ? ef - 1023 + se : -100000) + 2;
+                    const rns::Limbs x = rns::limbs(rns::scaled_int(w, sm, se, E, QB));
+                    const uint32_t sa = w < 0.0 ? 0x8000u : 0u, sb = sa ^ (s_d[lane] < 0.0 ? 0x8000u : 0u);
+                    const int64_t row = cb + r;
+                    if (lane == 0) q.rowE[row] = E;
+                    const int64_t at = row * QN + ((((lane >> 3) ^ (int)(row >> 1)) & 3) << 3) + (lane & 7);
+                    uint16_t *ra = reinterpret_cast<uint16_t *>(q.RA) + at;
+                    uint16_t *rb = reinterpret_cast<uint16_t *>(q.RB) + at;
+                    const int64_t ls = (int64_t)q.npad * QN;
+#pragma unroll
+                    for (int l = 0; l < RL; ++l) {
+                        const float v = rns::residue(c_tab13, l, x);
+                        const float vi = rns::mod(v * c_tab13.inv[l], c_tab13.p[l], c_tab13.pinv[l]);
+                        // the BF16 of an integer of magnitude <= 256: the upper half of its FP32
+                        ra[l * ls] = (uint16_t)((__float_as_uint(v) >> 16) ^ sa);
+                        rb[l * ls] = (uint16_t)((__float_as_uint(vi) >> 16) ^ sb);
+                    }
+                }
+                bar_comp();
+            }
+            if (tid < nb && s_cmax[tid]) atomicMax(&a.cmax[buf * 64 + tid], s_cmax[tid]);
+            asm volatile("fence.proxy.async;" ::: "memory");   // the residues are read by bulk copies
+        }
+        if (!panel_barrier(a.bar, epoch, a.wait_ns)) break;
+        // ---------------- the rule's column test, the same in every CTA
+        {
+            const double alpha = 0.6403882032022076;   // (1 + sqrt 17) / 8
+            int keep = 1;
+            if (tid < nb) {
+                const double d = s_d[tid];
+                const double colmax = __longlong_as_double((long long)__ldcg(&a.cmax[buf * 64 + tid]));
+                if (absbits64(d) < absbits64(alpha * colmax) || d == 0.0 || fabs(d) <= ztol || !isfinite(d) ||
+                    !isfinite(colmax))
+                    keep = 0;
+            }
+            if (!__syncthreads_and(keep)) {
+                if (g == 0 && tid == 0) {   // the panel loop takes over at column k
+                    a.st->k = k;
+                    a.st->kb = 0;
+                    a.st->spec = 0;
+                }
+                break;
+            }
+            if (g == 0) {
+                int pos = 0;
+                if (tid < nb) {
+                    a.kind[k + tid] = 1;
+                    a.Doff[k + tid] = 0.0;
+                    pos = s_d[tid] > 0.0 ? 1 : 0;
+                }
+                if (tid < QN) a.cmax[(buf ^ 1) * 64 + tid] = 0ULL;   // the next panel's maxima start at zero
+                const int np = __syncthreads_count(pos);
+                if (tid == 0) {
+                    a.st->npos += np;
+                    a.st->nneg += nb - np;
+                    a.st->k = k + nb;
+                    a.st->kb = nb;
+                    // counted in panels of 64 columns, as the panel loop's
+                    if (k + nb >= N || (k + nb) % 64 == 0) a.st->nacc += 1;
+                }
+            }
+        }
+        if (k + nb >= N) break;
+        // ---------------- trailing update: 128 x 32 tiles of the lower triangle
+        const int base = k + nb, nbr = (N - base + 127) / 128;
+        const int tiles = 2 * nbr * (nbr + 1);
+        bool ok = true;
+        auto tile_at = [&](int t, int &i0, int &c0) {   // false: beyond the last column
+            int tr = (int)((sqrtf(2.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+            while (2 * (tr + 1) * (tr + 2) <= t) ++tr;
+            while (2 * tr * (tr + 1) > t) --tr;
+            i0 = base + 128 * tr;
+            c0 = base + 32 * (t - 2 * tr * (tr + 1));
+            return c0 < N;
+        };
+        if (wid == Q_EPI) {   // loads: lane l takes modulus l (one thread issuing all 26 copies took 750 cycles each)
+            asm volatile("fence.proxy.async;" ::: "memory");
+            for (int t = g; t < tiles && ok; t += G) {
+                int i0, c0;
+                if (!tile_at(t, i0, c0)) continue;
+                if (tl > 0 && !tc::mbar_wait(&tfull, (tl - 1) & 1)) {   // the previous tile's operands are read
+                    ok = false;
+                    break;
+                }
+                ++tl;
+                if (lane == 0) tc::mbar_expect_tx(&full, RL * Q_STAGE);
+                __syncwarp();
+                if (lane < RL) {
+                    uint8_t *d = ring + lane * Q_STAGE;
+                    tc::bulk_load(d, q.RA + ((int64_t)lane * q.npad + i0) * QN, QA_BYTES, &full);
+                    tc::bulk_load(d + QA_BYTES, q.RB + ((int64_t)lane * q.npad + c0) * QN, QB_BYTES, &full);
+                }
+                __syncwarp();
+            }
+        } else if (wid == Q_EPI + 1 && lane == 0) {
+            for (int t = g; t < tiles && ok; t += G) {
+                int i0, c0;
+                if (!tile_at(t, i0, c0)) continue;
+                if (!tc::mbar_wait(&tempty, (tl & 1) ^ 1) || !tc::mbar_wait(&full, tl & 1)) {
+                    ok = false;
+                    break;
+                }
+                ++tl;
+                tc::fence_after();
+                const uint32_t ab0 = tc::smem_u32(ring);
+#pragma unroll
+                for (int l = 0; l < RL; ++l) {
+                    const uint32_t ab = ab0 + l * Q_STAGE, bb = ab + QA_BYTES;
+#pragma unroll
+                    for (int s = 0; s < 2; ++s)
+                        tc::mma<false, tc::instr_desc(false, 128, 32)>(tmem + 32 * l, tc::sw64_kmajor_desc(ab + 32 * s),
+                                                                       tc::sw64_kmajor_desc(bb + 32 * s), s ? 1u : 0u);
+                }
+                tc::commit(&tfull);
+            }
+        } else if (wid < Q_EPI) {
+            const int quad = wid & 3, quarter = wid >> 2;
+            for (int t = g; t < tiles && ok; t += G) {
+                int i0, c0;
+                if (!tile_at(t, i0, c0)) continue;
+                const int i = i0 + 32 * quad + lane, cb = c0 + 8 * quarter;
+                const int Ei = i < N ? __ldcg(q.rowE + i) : 0;
+                const int Ecl = lane < 8 && cb + lane < N ? __ldcg(q.rowE + cb + lane) : 0;
+                // two entries of A in use, the next two in flight
+                double old[2], nxt[2];
+                auto fetch = [&](double (&d)[2], int c) {
+#pragma unroll
+                    for (int j = 0; j < 2; ++j)
+                        d[j] = i < N && c + j <= i ? __ldcg(a.A + i + (int64_t)(c + j) * N) : 0.0;
+                };
+                fetch(nxt, cb);
+                if (!tc::mbar_wait(&tfull, tl & 1)) {
+                    ok = false;
+                    break;
+                }
+                ++tl;
+                tc::fence_after();
+                // parts of the tile above the diagonal or beyond N: nothing to do (warp-uniform)
+                const int nbatch = i0 + 32 * quad < N && cb <= i0 + 32 * quad + 31 ? 4 : 0;
+#pragma unroll 1
+                for (int b = 0; b < nbatch; ++b) {
+                    const int c = cb + 2 * b;
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) old[j] = nxt[j];
+                    if (b < 3) fetch(nxt, c + 2);
+                    uint32_t r[RL][2];
+                    __syncwarp();
+#pragma unroll
+                    for (int l = 0; l < RL; ++l)
+                        tc::tmem_ld2_async(tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(32 * l + 8 * quarter + 2 * b), r[l]);
+                    tc::tmem_wait_ld();
+#pragma unroll
+                    for (int l = 0; l < RL; ++l)   // the values exist only after the wait
+                        asm volatile("" : "+r"(r[l][0]), "+r"(r[l][1]));
+                    unsigned long long acc[2][4] = {};   // per entry, 32-bit limbs
+                    uint64_t yp = 0;                     // the pair's first residues
+#pragma unroll
+                    for (int l = 0; l < RL; ++l) {
+                        const float pf = c_tab13.p[l], pi = c_tab13.pinv[l];
+                        const uint64_t x = rns::pk(__uint_as_float(r[l][0]), __uint_as_float(r[l][1]));
+                        const uint64_t qq = rns::add2(rns::fma2(x, rns::pk(pi, pi), rns::pk(rns::kMagic, rns::kMagic)),
+                                                      rns::pk(-rns::kMagic, -rns::kMagic));
+                        const uint64_t y = rns::fma2(rns::pk(-pf, -pf), qq, x);   // x mod p
+                        if (l % 2 == 0 && l + 1 < RL) {
+                            yp = y;
+                            continue;
+                        }
+                        // z = y_p q + y_q p (exact); z + 2^19 is the low 23 bits of z + 2^23 + 2^19
+                        const uint64_t zb = rns::pk(8912896.0f, 8912896.0f);
+                        const float pp = c_tab13.p[l > 0 ? l - 1 : 0];
+                        const uint64_t z =
+                            l % 2 ? rns::add2(rns::fma2(yp, rns::pk(pf, pf), rns::mul2(y, rns::pk(pp, pp))), zb) : rns::add2(y, zb);
+                        const float2 zf = rns::upk(z);
+                        const uint32_t u0 = __float_as_uint(zf.x) & 0x7fffffu, u1 = __float_as_uint(zf.y) & 0x7fffffu;
+#pragma unroll
+                        for (int m = 0; m < 4; ++m) {
+                            acc[0][m] += (unsigned long long)u0 * c_tab13.mpair32[l / 2][m];
+                            acc[1][m] += (unsigned long long)u1 * c_tab13.mpair32[l / 2][m];
+                        }
+                    }
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        // T = sum z M/(p q) + bias; X = T - bias - k M with k = rint((T - bias) / M)
+                        unsigned __int128 T = ((unsigned __int128)acc[j][3] << 96) + ((unsigned __int128)acc[j][2] << 64) +
+                                              ((unsigned __int128)acc[j][1] << 32) + acc[j][0];
+                        const float f = fmaf((float)(uint32_t)(T >> 96), c_tab13.top, -c_tab13.btop) + rns::kMagic;
+                        const uint4 km = s_km[(__float_as_uint(f) + 8u) & 15u];   // kMagic's low bits are zero
+                        T += ((unsigned __int128)(((unsigned long long)km.w << 32) | km.z) << 64) |
+                             (((unsigned long long)km.y << 32) | km.x);
+                        const int Ec = __shfl_sync(0xffffffffu, Ecl, 2 * b + j);
+                        if (i < N && c + j <= i)
+                            a.A[i + (int64_t)(c + j) * N] = old[j] - rns::to_double(T, Ei + Ec - 2 * QB);
+                    }
+                }
+                tc::fence_before();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&tempty);
+            }
+        }
+        if (!ok) atomicExch(&a.bar->err, 1);
+        __threadfence();
+        if (!panel_barrier(a.bar, epoch, a.wait_ns)) break;
+    }
+    release();
+}
+
+int64_t q_npad(int64_t N) { return (N + 127) / 128 * 128 + 128; }
+size_t al256(size_t b) { return (b + 255) / 256 * 256; }
+
+}  // namespace
+
+size_t persist64_scratch_bytes(int64_t N) {
+    const size_t np = (size_t)q_npad(std::max<int64_t>(N, 1));
+    return 2 * al256(RL * np * QN * sizeof(bf16)) + al256(np * sizeof(int));
+}
+
+void launch_persist64(cudaStream_t s, int num_sms, int64_t N, const PersistArgs &pa, void *scratch) {
+    P64Args q{};
+    q.p = pa;
+    q.npad = (int)q_npad(N);
+    const size_t rb = al256((size_t)RL * q.npad * QN * sizeof(bf16));
+    char *w = static_cast<char *>(scratch);
+    q.RA = reinterpret_cast<bf16 *>(w);
+    q.RB = reinterpret_cast<bf16 *>(w + rb);
+    q.rowE = reinterpret_cast<int *>(w + 2 * rb);
+    static PerDeviceOnce once;
+    MDSIP_CUDA(once.run([] {
+        return cudaFuncSetAttribute(k_bk_persist64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQSmem);
+    }));
+    int per_sm = 0;
+    MDSIP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bk_persist64, Q_THREADS, kQSmem));
+    MDSIP_REQUIRE(per_sm >= 1, MDSIP_ERR_CUDA, "ldlt: persistent factorization does not fit an SM");
+    // one CTA per 16 rows below the first block or per two of its trailing
+    // tiles, whichever is more, at most one per SM
+    const int64_t rest = std::max<int64_t>(0, N - QN), nbr = (rest + 127) / 128;
+    const int64_t want = std::max<int64_t>({1, (rest + 15) / 16, nbr * (nbr + 1)});
+    const int G = (int)std::min<int64_t>(want, (int64_t)num_sms);
+    void *kargs[] = {&q};
+    MDSIP_CUDA(cudaLaunchCooperativeKernel((const void *)k_bk_persist64, dim3(G), dim3(Q_THREADS), kargs, kQSmem, s));
+    count_launch();
+}
+
+}  // namespace mdsip

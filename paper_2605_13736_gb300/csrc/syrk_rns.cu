@@ -33,55 +33,19 @@
 #include <climits>
 
 #include "internal.cuh"
+#include "rns.cuh"
 #include "tc.cuh"
 
 namespace mdsip {
 
 namespace {
 
+using namespace rns;
+
 constexpr int RN = 14;                 // moduli
-constexpr int LIMB = 14;               // bits per limb of |X| in the residue pass
-constexpr int CL = 5;                  // 30-bit limbs of the CRT constants
-
-struct RnsTab {
-    float p[RN], pinv[RN];
-    float c1[RN], c2[RN], c3[RN];      // 2^14, 2^28, 2^42 mod p, symmetric
-    int inv[RN];                       // (M / p)^-1 mod p, symmetric
-    int mhat[RN][CL];                  // M / p
-    int mod[CL];                       // M
-};
-
-constexpr int kModuli[RN] = {512, 511, 509, 507, 505, 503, 499, 493, 491, 487, 479, 473, 467, 463};
 constexpr int kModBits = 125;          // floor(log2 of their product)
 
-constexpr int sym(int v, int p) {
-    v %= p;
-    if (v < 0) v += p;
-    return v > p / 2 ? v - p : v;
-}
-
-constexpr RnsTab make_tab() {
-    RnsTab t{};
-    unsigned __int128 M = 1;
-    for (int l = 0; l < RN; ++l) M *= (unsigned)kModuli[l];
-    for (int j = 0; j < CL; ++j) t.mod[j] = (int)((M >> (30 * j)) & 0x3fffffffu);
-    for (int l = 0; l < RN; ++l) {
-        const int p = kModuli[l];
-        t.p[l] = (float)p;
-        t.pinv[l] = 1.0f / (float)p;
-        t.c1[l] = (float)sym((int)((1LL << LIMB) % p), p);
-        t.c2[l] = (float)sym((int)((1LL << (2 * LIMB)) % p), p);
-        t.c3[l] = (float)sym((int)((1LL << (3 * LIMB)) % p), p);
-        const unsigned __int128 h = M / (unsigned)p;
-        for (int j = 0; j < CL; ++j) t.mhat[l][j] = (int)((h >> (30 * j)) & 0x3fffffffu);
-        const int hm = (int)(h % (unsigned)p);
-        for (int v = 1; v < p; ++v)
-            if ((v * hm) % p == 1) t.inv[l] = sym(v, p);
-    }
-    return t;
-}
-
-__constant__ RnsTab c_tab = make_tab();
+__constant__ Tab<RN> c_tab = make_tab<RN>();
 
 constexpr int T_M = 128, T_N = 256;    // output tile: 128 rows p, 256 columns q
 constexpr int SLAB = 64;               // rows of A (K) per pipeline stage
@@ -91,7 +55,6 @@ constexpr int BOX_BYTES = (int)tc::kMnBoxBytes;    // one 64-column x 64-row TMA
 constexpr int STAGE_BYTES = (T_M + T_N) / 64 * BOX_BYTES;   // 48 KiB
 constexpr int MMA_THREADS = 384;       // warp 0 loads, warp 1 issues, warps 4-11 fold
 constexpr size_t kMmaSmem = 1024 + (size_t)STAGES * STAGE_BYTES + 256;
-constexpr float kMagic = 12582912.0f;  // 1.5 2^23: adding and subtracting it rounds to an integer
 
 // tile t of the lower triangle: row block P of 128, column block Q of 256, P >= 2 Q
 __device__ __forceinline__ void rns_tile(int t, int &P, int &Q) {
@@ -108,8 +71,7 @@ __host__ __device__ inline int rns_tiles(int64_t n) {
     return (int)(a * (a + 1) + (np & 1 ? a + 1 : 0));
 }
 
-// w_i^-1/2 = sm[i] 2^(se[i] - 63), sm accurate to about 63 bits (one Newton
-// correction of the FP64 value with exact residuals)
+// w_i^-1/2 = sm[i] 2^(se[i] - 63)
 __global__ void k_rns_rows(int64_t m, const double *__restrict__ w, unsigned long long *__restrict__ sm,
                            int *__restrict__ se, int *__restrict__ flag) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
@@ -118,16 +80,7 @@ __global__ void k_rns_rows(int64_t m, const double *__restrict__ w, unsigned lon
             atomicExch(flag, 1);
             continue;
         }
-        const double s = 1.0 / sqrt(v);
-        const double h = v * s, hl = fma(v, s, -h);
-        const double r = fma(-h, s, 1.0) - hl * s;             // 1 - w s^2
-        const int e = (int)((__double_as_longlong(s) >> 52) & 0x7ff) - 1023;
-        const unsigned long long mant =
-            (((unsigned long long)__double_as_longlong(s) & 0xfffffffffffffULL) | 0x10000000000000ULL) << 11;
-        const double cd = ldexp(0.5 * s * r, 63 - e);
-        long long c = __double2ll_rn(fmin(fmax(cd, -2047.0), 2047.0));
-        sm[i] = mant + (unsigned long long)c;
-        se[i] = e;
+        rsqrt64(v, sm[i], se[i]);
     }
 }
 
@@ -216,39 +169,20 @@ __global__ void __launch_bounds__(256) k_rns_residues(const double *__restrict__
                 }
             }
         }
-        float x0[8], x1[8], x2[8], x3[8];
+        Limbs x[8];
         unsigned sgn[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            const long long bits = __double_as_longlong(v[j]);
-            const int ef = (int)((bits >> 52) & 0x7ff);
-            unsigned long long X = 0;
-            if (ef != 0) {   // zero otherwise (subnormal entries raised the flag)
-                const unsigned long long mant = (((unsigned long long)bits & 0xfffffffffffffULL) | 0x10000000000000ULL)
-                                                << 11;
-                // a s = hi 2^(ea + es - 62); X = hi >> sh with rounding, sh >= 64 - b >= 8
-                const unsigned long long hi = __umul64hi(mant, s);
-                const int sh = 62 - b + __ldg(colE + q0 + j) - (ef - 1023 + es) - 1;
-                X = sh < 64 ? ((hi >> sh) + 1ULL) >> 1 : 0ULL;
-            }
-            auto lf = [](unsigned u) { return __uint_as_float(0x4B000000u | u) - 8388608.0f; };
-            x0[j] = lf((unsigned)X & 0x3fffu);
-            x1[j] = lf((unsigned)(X >> LIMB) & 0x3fffu);
-            x2[j] = lf((unsigned)(X >> (2 * LIMB)) & 0x3fffu);
-            x3[j] = lf((unsigned)(X >> (3 * LIMB)));
-            if (bits < 0) sgn[j >> 1] |= 0x8000u << (16 * (j & 1));
+            // (columns beyond n hold zeros; subnormal entries raised the flag)
+            x[j] = limbs(v[j] != 0.0 ? scaled_int(v[j], s, es, __ldg(colE + q0 + j), b) : 0ULL);
+            if (__double2hiint(v[j]) < 0) sgn[j >> 1] |= 0x8000u << (16 * (j & 1));
         }
         uint4 *out = R + (int64_t)k * groups + g;
 #pragma unroll
         for (int l = 0; l < RN; ++l) {
-            const float p = c_tab.p[l], pi = c_tab.pinv[l], c1 = c_tab.c1[l], c2 = c_tab.c2[l], c3 = c_tab.c3[l];
             uint32_t r[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const float t = fmaf(c3, x3[j], fmaf(c2, x2[j], fmaf(c1, x1[j], x0[j])));
-                const float qf = __fadd_rn(fmaf(t, pi, kMagic), -kMagic);
-                r[j] = __float_as_uint(fmaf(-p, qf, t));
-            }
+            for (int j = 0; j < 8; ++j) r[j] = __float_as_uint(residue(c_tab, l, x[j]));
             uint4 o;   // the BF16 of an integer of magnitude <= 256 is the upper half of its FP32
             o.x = __byte_perm(r[0], r[1], 0x7632) ^ sgn[0];
             o.y = __byte_perm(r[2], r[3], 0x7632) ^ sgn[1];
@@ -257,28 +191,6 @@ __global__ void __launch_bounds__(256) k_rns_residues(const double *__restrict__
             out[(int64_t)l * total] = o;
         }
     }
-}
-
-// packed FP32 pairs
-__device__ __forceinline__ uint64_t pk(float a, float b) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float2 upk(uint64_t v) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
 }
 
 struct MmaArgs {
@@ -490,9 +402,7 @@ __global__ void __launch_bounds__(256) k_rns_combine(int64_t n, int tile0, int n
         }
 #pragma unroll
         for (int l = 0; l < RN; ++l) {
-            const float t = (float)(r[l] * c_tab.inv[l]);         // |t| < 2^24
-            const float qf = __fadd_rn(fmaf(t, c_tab.pinv[l], kMagic), -kMagic);
-            const float y = fmaf(-c_tab.p[l], qf, t);
+            const float y = mod((float)r[l] * c_tab.inv[l], c_tab.p[l], c_tab.pinv[l]);   // the product < 2^24
             frac = fmaf(y, c_tab.pinv[l], frac);
             const int yi = (int)y;
 #pragma unroll
@@ -503,27 +413,7 @@ __global__ void __launch_bounds__(256) k_rns_combine(int64_t n, int tile0, int n
 #pragma unroll
         for (int j = CL - 1; j >= 0; --j)
             u = (u << 30) + (unsigned __int128)(__int128)(acc[j] - (long long)kq * c_tab.mod[j]);
-        double val = 0.0;
-        if (u != 0) {
-            const bool neg = (long long)(u >> 64) < 0;
-            if (neg) u = (unsigned __int128)0 - u;
-            unsigned long long hi = (unsigned long long)(u >> 64);
-            const int z = hi ? __clzll((long long)hi) : 64 + __clzll((long long)(unsigned long long)u);
-            u <<= z;
-            hi = (unsigned long long)(u >> 64);   // top bit set
-            const int ex = 127 - z + colE[p] + colE[q] - 2 * b;   // exponent of the value
-            if (ex > -1022 && ex < 1023) {
-                // round to nearest, ties to even, in integers (an FP64 instruction costs as
-                // much as 64 integer ones here)
-                unsigned long long mant = hi >> 11;
-                const unsigned rest = (unsigned)hi & 0x7ffu;
-                mant += rest > 0x400u || (rest == 0x400u && ((unsigned long long)u != 0ULL || (mant & 1ULL)));
-                val = __longlong_as_double((long long)(((unsigned long long)(ex + 1022) << 52) + mant));
-            } else {
-                val = scalbn((double)(hi | ((unsigned long long)u != 0ULL)), ex - 63);
-            }
-            if (neg) val = -val;
-        }
+        double val = to_double(u, colE[p] + colE[q] - 2 * b);
         double *out = C + p + q * ldc;
         if (poison) val = NAN;
         *out = (beta != 0.0 ? *out : 0.0) + val;

@@ -416,7 +416,7 @@ EncodeTiledFn encode_fn() {
 }  // namespace
 
 void encode_2d(CUtensorMap *map, const void *base, bool f32, uint64_t inner, uint64_t outer, uint64_t ld,
-               uint32_t box_inner, uint32_t box_outer, bool swizzle) {
+               uint32_t box_inner, uint32_t box_outer, int swizzle) {
     const size_t esz = f32 ? 4 : 2;
     MDSIP_REQUIRE(reinterpret_cast<uintptr_t>(base) % 16 == 0 && (ld * esz) % 16 == 0 && ld >= inner,
                   MDSIP_ERR_INVALID_ARG, "tensor map: base or row stride not 16-byte aligned");
@@ -427,7 +427,7 @@ void encode_2d(CUtensorMap *map, const void *base, bool f32, uint64_t inner, uin
     const CUresult r = encode_fn()(map, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
                                    const_cast<void *>(base), gdim, gstride, box, estride,
                                    CU_TENSOR_MAP_INTERLEAVE_NONE,
-                                   swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                                   swizzle == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
                                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     MDSIP_REQUIRE(r == CUDA_SUCCESS, MDSIP_ERR_CUDA, "cuTensorMapEncodeTiled failed");
 }

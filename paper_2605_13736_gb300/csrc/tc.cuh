@@ -53,6 +53,14 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, u
         : "memory");
 }
 
+// contiguous global -> shared, 16-byte aligned, a multiple of 16 bytes
+__device__ __forceinline__ void bulk_load(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                     smem_u32(dst)),
+                 "l"(src), "r"(bytes), "r"(smem_u32(bar))
+                 : "memory");
+}
+
 // shared -> global; the caller commits and waits the bulk group
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, const void *src, int x, int y) {
     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(
@@ -92,6 +100,19 @@ __device__ __forceinline__ uint64_t sw128_kmajor_desc(uint32_t saddr) {
     d |= (uint64_t)(1024 >> 4) << 32;            // stride byte offset: 8 rows x 128 B
     d |= (uint64_t)1 << 46;                      // descriptor version
     d |= (uint64_t)2 << 61;                      // 128-byte swizzle
+    return d;
+}
+
+// K-major operand of 32 BF16 per row in the 64-byte-swizzle layout (8-row x
+// 64-byte atoms, 512 bytes apart along M/N); a K step of 16 advances the start
+// address by 32 bytes.
+__device__ __forceinline__ uint64_t sw64_kmajor_desc(uint32_t saddr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)1 << 16;
+    d |= (uint64_t)(512 >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)4 << 61;                      // 64-byte swizzle
     return d;
 }
 
@@ -167,12 +188,18 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// 2 columns; the values are there after tmem_wait_ld
+__device__ __forceinline__ void tmem_ld2_async(uint32_t taddr, uint32_t (&r)[2]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
 // Host: 2-D tiled tensor map (inner extent `inner` elements of `esz` bytes,
 // `outer` rows `ld` elements apart; box `box_inner` x `box_outer`; 128-byte
-// swizzle, or rows of the box packed without one; out-of-range elements read
+// swizzle, or (0) rows of the box packed without one; out-of-range elements read
 // as zero and are not written).  Throws on failure.
 void encode_2d(CUtensorMap *map, const void *base, bool f32, uint64_t inner, uint64_t outer, uint64_t ld,
-               uint32_t box_inner, uint32_t box_outer, bool swizzle = true);
+               uint32_t box_inner, uint32_t box_outer, int swizzle = 128);
 
 }  // namespace tc
 }  // namespace mdsip
