@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <cmath>
 #include <mutex>
 #include <new>
@@ -199,39 +200,190 @@ enum Scalar : int {
 };
 
 // ---------------------------------------------------------------------------
-// Block-level reductions (deterministic for a fixed launch shape).
+// FP64 scalar pieces.  GB300 issues one FP64 instruction of a warp in 64
+// cycles per sub-partition, comparisons included, so the small kernels of a
+// step are bound by the number of FP64 instructions on their longest chain:
+// tests and maxima work on bit patterns, divisions on the short reciprocal.
 // ---------------------------------------------------------------------------
-template <int NT>
-__device__ __forceinline__ double block_sum(double v, double *sh) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) sh[wid] = v;
-    __syncthreads();
-    double r = 0.0;
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < NT / 32; ++i) r += sh[i];
-    }
-    return r;  // valid in thread 0
+// 1/d by Newton-Raphson iteration x <- x (2 - d x) (0 for d = 0): the first
+// step in FP32 and integers on the mantissa m of d -- hardware reciprocal q of
+// m's upper 24 bits, the residual 1 - m q with all of m, x = q + q (e + e^2) in
+// units of 2^-53, good to about 2^-46 -- and the last in FP64.  Two FP64
+// instructions, where the FP32 conversions and two FP64 steps were six: on
+// GB300 each occupies a warp's FP64 pipe for 64 cycles and every pivot waits
+// for this value.  d near the ends of the range goes through the division
+// operator.
+__device__ __forceinline__ double rcp_newton(double d) {
+    const int hi = __double2hiint(d);
+    const unsigned lo = (unsigned)__double2loint(d);
+    const int ef = (hi >> 20) & 0x7ff;
+    if (ef < 100 || ef > 1946) return d == 0.0 ? 0.0 : 1.0 / d;
+    const float mh = __uint_as_float(0x3f800000u | (((unsigned)hi & 0xfffffu) << 3) | (lo >> 29));
+    const float ml = (float)(lo & 0x1fffffffu) * 0x1p-52f;
+    float q;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(mh));
+    const float e = fmaf(-ml, q, fmaf(-mh, q, 1.0f));
+    const float qe = q * e;
+    const int c = __float2int_rn(fmaf(qe, e, qe) * 0x1p52f);       // |q e| < 2^-21
+    const unsigned qb = __float_as_uint(q);                        // 1/2 <= q <= 1
+    const long long X = ((long long)((qb & 0x7fffffu) | 0x800000u) << (29 + (int)(qb >> 23) - 126)) + 2LL * c;
+    const double x = __longlong_as_double((1021LL << 52) + X);     // 2^52 <= X <= 2^53 (as 1022 << 52 plus X - 2^52)
+    const double m = __hiloint2double((hi & 0xfffff) | 0x3ff00000, (int)lo);
+    const double y = fma(x, fma(-m, x, 1.0), x);                   // 1 / m
+    return __hiloint2double((__double2hiint(y) - ((ef - 1023) << 20)) | (hi & (int)0x80000000), __double2loint(y));
 }
 
-template <int NT>
-__device__ __forceinline__ double block_max(double v, double *sh) {
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) sh[wid] = v;
-    __syncthreads();
-    double r = -INFINITY;
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < NT / 32; ++i) r = fmax(r, sh[i]);
-    }
-    return r;
+// a / b: reciprocal, product and one residual correction (Markstein 1990), five
+// FP64 instructions; magnitudes outside 2^-500 .. 2^500 take the operator
+__device__ __forceinline__ double ddiv(double a, double b) {
+    const int ha = __double2hiint(a), hb = __double2hiint(b);
+    const bool zero = (((unsigned)ha << 1) | (unsigned)__double2loint(a)) == 0u;
+    const unsigned ea = (unsigned)((ha >> 20) & 0x7ff) - 523u, eb = (unsigned)((hb >> 20) & 0x7ff) - 523u;
+    if ((ea > 1000u && !zero) || eb > 1000u) return a / b;
+    const double r = rcp_newton(b);
+    const double q = a * r;
+    return fma(fma(-q, b, a), r, q);
 }
 
+__device__ __forceinline__ bool fin(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+
+// non-NaN doubles as integers of the same order
+__device__ __forceinline__ long long ord64(double v) {
+    const long long b = __double_as_longlong(v);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
+}
+
+// ---------------------------------------------------------------------------
+// Grid-wide reductions of up to 8 quantities in one kernel (deterministic for
+// a fixed launch shape): warps by shuffles, the block's warps by one warp per
+// quantity, and the last block to arrive combines the blocks' partials in
+// order.  The ticket counter returns to zero by itself, so any grid size may
+// follow; the kernels that share one run in turn on a stream.  (A separate
+// combining launch per operation took 4 to 8 us each, eleven a Newton step.)
+// ---------------------------------------------------------------------------
+struct RedOut {
+    double *partial;     // kRedBlocks per quantity
+    unsigned *ticket;
+    double *out;         // one per quantity
+};
+
+enum RedOp { R_SUM, R_MAX, R_MIN };
+
+__device__ __forceinline__ double red_identity(RedOp op) {
+    return op == R_SUM ? 0.0 : (op == R_MAX ? -INFINITY : INFINITY);
+}
+__device__ __forceinline__ double red_combine(RedOp op, double a, double b) {
+    if (op == R_SUM) return a + b;
+    return (op == R_MAX) == (ord64(b) > ord64(a)) ? b : a;
+}
+
+// whether this block is the last of the grid to get here (all threads)
+__device__ __forceinline__ bool red_last(unsigned *ticket) {
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
+    __syncthreads();
+    if (s_last) __threadfence();
+    return s_last;
+}
+
+template <int NT, RedOp... OPS>
+__device__ __forceinline__ void reduce_finish(double (&v)[sizeof...(OPS)], const RedOut &o) {
+    constexpr int K = sizeof...(OPS), W = NT / 32;
+    constexpr RedOp ops[K] = {OPS...};
+    static_assert(K <= W && W <= 32, "one warp per quantity");
+    __shared__ double sh[K][W];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1)
+#pragma unroll
+        for (int k = 0; k < K; ++k) v[k] = red_combine(ops[k], v[k], __shfl_xor_sync(0xffffffffu, v[k], s));
+    if (lane == 0)
+#pragma unroll
+        for (int k = 0; k < K; ++k) sh[k][wid] = v[k];
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+        if (wid == k) {
+            double x = lane < W ? sh[k][lane] : red_identity(ops[k]);
+#pragma unroll
+            for (int s = W / 2; s > 0; s >>= 1) x = red_combine(ops[k], x, __shfl_xor_sync(0xffffffffu, x, s));
+            if (lane == 0) *(gridDim.x == 1 ? o.out + k : o.partial + (size_t)k * kRedBlocks + blockIdx.x) = x;
+        }
+    if (gridDim.x == 1 || !red_last(o.ticket)) return;
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+        if (wid == k) {
+            double p[(kRedBlocks + 31) / 32];
+#pragma unroll
+            for (int i = 0; i < (kRedBlocks + 31) / 32; ++i)
+                p[i] = lane + 32 * i < (int)gridDim.x ? __ldcg(o.partial + (size_t)k * kRedBlocks + lane + 32 * i)
+                                                      : red_identity(ops[k]);
+            double x = p[0];
+#pragma unroll
+            for (int i = 1; i < (kRedBlocks + 31) / 32; ++i)
+                if (32 * i < (int)gridDim.x) x = red_combine(ops[k], x, p[i]);
+#pragma unroll
+            for (int s = 16; s > 0; s >>= 1) x = red_combine(ops[k], x, __shfl_xor_sync(0xffffffffu, x, s));
+            if (lane == 0) o.out[k] = x;
+        }
+}
+
+// the same for K counts (integers; out receives them as doubles)
+template <int NT, int K>
+__device__ __forceinline__ void count_finish(unsigned (&c)[K], const RedOut &o) {
+    constexpr int W = NT / 32;
+    __shared__ unsigned sh[K][W];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < K; ++k) c[k] = __reduce_add_sync(0xffffffffu, c[k]);
+    if (lane == 0)
+#pragma unroll
+        for (int k = 0; k < K; ++k) sh[k][wid] = c[k];
+    __syncthreads();
+    unsigned *part = reinterpret_cast<unsigned *>(o.partial);
+    if (wid < K) {
+        const unsigned x = __reduce_add_sync(0xffffffffu, lane < W ? sh[wid][lane] : 0u);
+        if (lane == 0) {
+            if (gridDim.x == 1) o.out[wid] = (double)x;
+            else part[(size_t)wid * kRedBlocks + blockIdx.x] = x;
+        }
+    }
+    if (gridDim.x == 1 || !red_last(o.ticket)) return;
+    if (wid < K) {
+        unsigned x = 0;
+        for (int i = lane; i < (int)gridDim.x; i += 32) x += __ldcg(part + (size_t)wid * kRedBlocks + i);
+        x = __reduce_add_sync(0xffffffffu, x);
+        if (lane == 0) o.out[wid] = (double)x;
+    }
+}
+
+// (J^T y)_k of 32 columns k0 .. k0 + 31 of a row-major m x n matrix, by a block
+// whose warps share the rows: returned to threads 0 .. 31 (every thread calls)
 template <int NT>
-__device__ __forceinline__ double block_min(double v, double *sh) {
-    return -block_max<NT>(-v, sh);
+__device__ __forceinline__ double colgroup_dot(const double *__restrict__ J, int64_t m, int64_t n, int64_t k0,
+                                               const double *__restrict__ y, double (*sp)[33]) {
+    if (m == 0) return 0.0;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t k = k0 + lane;
+    double s = 0.0;
+    if (k < n)
+#pragma unroll 4
+        for (int64_t j = wid; j < m; j += NT / 32) s = fma(J[j * n + k], y[j], s);
+    __syncthreads();                               // an earlier group's sums are read
+    sp[wid][lane] = s;
+    __syncthreads();
+    double t = 0.0;
+    if (wid == 0)
+#pragma unroll
+        for (int w = 0; w < NT / 32; ++w) t += sp[w][lane];
+    return t;
+}
+
+// blocks of a reduction kernel over `len` elements or more (one per thread)
+inline int red_grid(int64_t len) {
+    return (int)std::max<int64_t>(1, std::min<int64_t>(kRedBlocks, (len + kRedThreads - 1) / kRedThreads));
 }
 
 // ---------------------------------------------------------------------------
@@ -303,13 +455,9 @@ struct PerDeviceOnce {
 // ---------------------------------------------------------------------------
 // Kernel launchers (defined in the .cu files).
 // ---------------------------------------------------------------------------
-// reductions: partial[k * kRedBlocks + b] -> scalars[first + k] (sum / max / min)
 // probe.cu: blocks x 256 threads, each iters x 8 independent FP64 FMAs; sink
 // holds blocks x 256 doubles
 void launch_fp64_fma_probe(cudaStream_t s, int blocks, int64_t iters, double *sink);
-void launch_finalize_sum(cudaStream_t s, const double *partial, int nq, double *out);
-void launch_finalize_max(cudaStream_t s, const double *partial, int nq, double *out);
-void launch_finalize_min(cudaStream_t s, const double *partial, int nq, double *out);
 
 // A passes (row-major A, m x n, leading dimension lda)
 void launch_gemv_rows(cudaStream_t s, const double *A, int64_t m, int64_t n, int64_t lda,
@@ -406,8 +554,7 @@ void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, cons
 void launch_ldlt_solve(cudaStream_t s, int64_t N, const double *L, const double *Dd,
                        const double *Doff, const int32_t *perm, int64_t nrhs, double *B,
                        int64_t ldb);
-void launch_maxabs_lower(cudaStream_t s, int64_t N, const double *S, int64_t ld, double *partial,
-                         double *out);
+void launch_maxabs_lower(cudaStream_t s, int64_t N, const double *S, int64_t ld, double *out);
 size_t ldlt_solve_scratch_bytes(int64_t N);
 // tiles of L for the solve (FP64, or FP32 when fp32), into the solve scratch; after each factorization
 void launch_ldlt_solve_prepare(cudaStream_t s, int64_t N, const double *L, void *scratch, bool fp32);

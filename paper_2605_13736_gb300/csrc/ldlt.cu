@@ -534,13 +534,20 @@ k_ldlt_solve(int N, const double *__restrict__ L, const double *__restrict__ Dd,
     for (int i = tid; i < N; i += blockDim.x) b[perm[i]] = y[i];
 }
 
-__global__ void k_maxabs_lower(int64_t N, const double *S, int64_t ld, double *partial) {
-    __shared__ double sh[32];
-    double v = 0.0;
+// *out = max |S_ij| over the lower triangle (NaN entries ignored), as bit
+// patterns: out starts at zero, the order of the blocks does not matter
+__global__ void __launch_bounds__(kRedThreads) k_maxabs_lower(int64_t N, const double *__restrict__ S, int64_t ld,
+                                                              unsigned long long *out) {
+    unsigned long long v = 0ULL;
     for (int64_t j = blockIdx.x; j < N; j += gridDim.x)
-        for (int64_t i = j + threadIdx.x; i < N; i += blockDim.x) v = fmax(v, fabs(S[i + j * ld]));
-    v = block_max<kRedThreads>(v, sh);
-    if (threadIdx.x == 0) partial[blockIdx.x] = v;
+#pragma unroll 4
+        for (int64_t i = j + threadIdx.x; i < N; i += kRedThreads) {
+            const unsigned long long b = (unsigned long long)__double_as_longlong(S[i + j * ld]) & 0x7fffffffffffffffULL;
+            if (b > v && b <= 0x7ff0000000000000ULL) v = b;
+        }
+    const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(v >> 32));
+    const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(v >> 32) == hi ? (unsigned)v : 0u);
+    if ((threadIdx.x & 31) == 0 && (hi | lo)) atomicMax(out, ((unsigned long long)hi << 32) | lo);
 }
 
 }  // namespace
@@ -560,11 +567,12 @@ size_t ldlt_scratch_bytes(int64_t N) {
     return std::max(ldlt_unblocked_scratch_bytes(N), ldlt_blocked_scratch_bytes(N));
 }
 
-void launch_maxabs_lower(cudaStream_t s, int64_t N, const double *S, int64_t ld, double *partial,
-                         double *out) {
-    k_maxabs_lower<<<kRedBlocks, kRedThreads, 0, s>>>(N, S, ld, partial);
+void launch_maxabs_lower(cudaStream_t s, int64_t N, const double *S, int64_t ld, double *out) {
+    MDSIP_CUDA(cudaMemsetAsync(out, 0, sizeof(double), s));
+    if (N <= 0) return;
+    k_maxabs_lower<<<(unsigned)std::min<int64_t>(N, 4 * kRedBlocks), kRedThreads, 0, s>>>(
+        N, S, ld, reinterpret_cast<unsigned long long *>(out));
     MDSIP_LAUNCHED();
-    launch_finalize_max(s, partial, 1, out);
 }
 
 // S: lower triangle with leading dimension ld, overwritten.  scratch:
@@ -658,16 +666,15 @@ void launch_ldlt_solve(cudaStream_t s, int64_t N, const double *L, const double 
 // arena of a real-time controller), or a loop that must not pay the implicit
 // device synchronisation that allocating and freeing can cause.  For them
 // the factorization's scratch (the ping-pong copy of the trailing matrix, the
-// pivot hand-off slots, the barrier words, the error flag and the reduction
-// partials of the zero-pivot scale) lives in this fixed device array, which
+// pivot hand-off slots, the barrier words, the error flag and the zero-pivot
+// scale) lives in this fixed device array, which
 // every GPU that loads the library holds until the process exits.
 // ---------------------------------------------------------------------------
 constexpr int64_t kNoAllocMaxN = 1024;
 constexpr size_t kNoAllocBytes = (size_t)kNoAllocMaxN * kNoAllocMaxN * sizeof(double) + 16384;
 // the layout below: [factor scratch, rounded up to 256 | error flag (256) |
-// kRedBlocks partials | max |S|], for the largest accepted order
-static_assert(ldlt_unblocked_scratch_bytes(kNoAllocMaxN) + 256 + (size_t)(kRedBlocks + 1) * sizeof(double) <=
-                  kNoAllocBytes,
+// max |S|], for the largest accepted order
+static_assert(ldlt_unblocked_scratch_bytes(kNoAllocMaxN) + 256 + sizeof(double) <= kNoAllocBytes,
               "fixed scratch too small for the factorization's layout");
 static __device__ __align__(256) unsigned char g_ldlt_fixed_scratch[kNoAllocBytes];
 
@@ -710,17 +717,16 @@ void ldlt_factor_fixed_scratch(cudaStream_t s, int device, int num_sms, int64_t 
     MDSIP_REQUIRE(S && out.L && out.Dd && out.Doff && out.perm && out.kind, MDSIP_ERR_INVALID_ARG,
                   "ldlt: null pointer");
     char *base = static_cast<char *>(fixed_scratch_address(device));
-    // layout: [unblocked factor scratch | error flag | partials | max |S|]
+    // layout: [unblocked factor scratch | error flag | max |S|]
     const size_t fs = ldlt_unblocked_scratch_bytes(N);
     int *err = reinterpret_cast<int *>(base + fs);
-    double *partial = reinterpret_cast<double *>(base + fs + 256);
-    double *maxabs = partial + kRedBlocks;
-    MDSIP_REQUIRE(((reinterpret_cast<uintptr_t>(partial) | reinterpret_cast<uintptr_t>(base)) & 255) == 0,
+    double *maxabs = reinterpret_cast<double *>(base + fs + 256);
+    MDSIP_REQUIRE(((reinterpret_cast<uintptr_t>(maxabs) | reinterpret_cast<uintptr_t>(base)) & 255) == 0,
                   MDSIP_ERR_INVALID_ARG, "ldlt (fixed scratch): misaligned layout");
     // every call shares the array: clear what must start at zero (the factor
     // launch clears its own slots and barrier words)
     MDSIP_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
-    launch_maxabs_lower(s, N, S, ld, partial, maxabs);
+    launch_maxabs_lower(s, N, S, ld, maxabs);
     launch_ldlt_unblocked(s, num_sms, N, S, ld, maxabs, zero_tol, out, base, err);
     int herr = 0;
     MDSIP_CUDA(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s));

@@ -46,34 +46,6 @@ __device__ __forceinline__ unsigned long long absbits64(double v) {
     return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL;
 }
 
-// 1/d by Newton-Raphson iteration x <- x (2 - d x) (0 for d = 0): the first
-// step in FP32 and integers on the mantissa m of d -- hardware reciprocal q of
-// m's upper 24 bits, the residual 1 - m q with all of m, x = q + q (e + e^2) in
-// units of 2^-53, good to about 2^-46 -- and the last in FP64.  Two FP64
-// instructions, where the FP32 conversions and two FP64 steps were six: on
-// GB300 each occupies a warp's FP64 pipe for 64 cycles and every pivot waits
-// for this value.  d near the ends of the range goes through the division
-// operator.
-__device__ __forceinline__ double rcp_newton(double d) {
-    const int hi = __double2hiint(d);
-    const unsigned lo = (unsigned)__double2loint(d);
-    const int ef = (hi >> 20) & 0x7ff;
-    if (ef < 100 || ef > 1946) return d == 0.0 ? 0.0 : 1.0 / d;
-    const float mh = __uint_as_float(0x3f800000u | (((unsigned)hi & 0xfffffu) << 3) | (lo >> 29));
-    const float ml = (float)(lo & 0x1fffffffu) * 0x1p-52f;
-    float q;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(q) : "f"(mh));
-    const float e = fmaf(-ml, q, fmaf(-mh, q, 1.0f));
-    const float qe = q * e;
-    const int c = __float2int_rn(fmaf(qe, e, qe) * 0x1p52f);       // |q e| < 2^-21
-    const unsigned qb = __float_as_uint(q);                        // 1/2 <= q <= 1
-    const long long X = ((long long)((qb & 0x7fffffu) | 0x800000u) << (29 + (int)(qb >> 23) - 126)) + 2LL * c;
-    const double x = __longlong_as_double((1021LL << 52) + X);     // 2^52 <= X <= 2^53 (as 1022 << 52 plus X - 2^52)
-    const double m = __hiloint2double((hi & 0xfffff) | 0x3ff00000, (int)lo);
-    const double y = fma(x, fma(-m, x, 1.0), x);                   // 1 / m
-    return __hiloint2double((__double2hiint(y) - ((ef - 1023) << 20)) | (hi & (int)0x80000000), __double2loint(y));
-}
-
 __device__ __forceinline__ long long global_ns() {
     long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

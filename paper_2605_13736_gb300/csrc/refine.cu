@@ -18,22 +18,18 @@ namespace {
 
 constexpr int NT = kRedThreads;
 
-__device__ __forceinline__ double *slot(double *partial, int q) {
-    return partial + (size_t)q * kRedBlocks + blockIdx.x;
-}
-
 __device__ __forceinline__ double rN_x(const ModelView &M, const IterView &I, const double *gl, double mu,
                                        int64_t i) {
     double r = gl[i];
-    if (isfinite(M.xl[i])) r -= mu / (I.x[i] - M.xl[i]);
-    if (isfinite(M.xu[i])) r += mu / (M.xu[i] - I.x[i]);
+    if (fin(M.xl[i])) r -= ddiv(mu, I.x[i] - M.xl[i]);
+    if (fin(M.xu[i])) r += ddiv(mu, M.xu[i] - I.x[i]);
     return r;
 }
 
 __device__ __forceinline__ double r_dslack(const ModelView &M, const IterView &I, double mu, int64_t j) {
     double r = -I.yh[j];
-    if (isfinite(M.hl[j])) r -= mu / (I.d[j] - M.hl[j]);
-    if (isfinite(M.hu[j])) r += mu / (M.hu[j] - I.d[j]);
+    if (fin(M.hl[j])) r -= ddiv(mu, I.d[j] - M.hl[j]);
+    if (fin(M.hu[j])) r += ddiv(mu, M.hu[j] - I.d[j]);
     return r;
 }
 
@@ -45,7 +41,7 @@ __global__ void k_rhs_full(Dims D, ModelView M, IterView I, const double *__rest
     for (int64_t i = gtid; i < D.n; i += gsz) b[i] = -rN_x(M, I, gl, mu, i);
     for (int64_t i = gtid; i < D.m_E; i += gsz) b[D.n + i] = -cg[i];
     for (int64_t j = gtid; j < D.m_I; j += gsz)
-        b[D.n + D.m_E + j] = -(ch[j] + r_dslack(M, I, mu, j) / (sig_d[j] + dw));
+        b[D.n + D.m_E + j] = -(ch[j] + ddiv(r_dslack(M, I, mu, j), sig_d[j] + dw));
 }
 
 // bt_g = b_g - J_sg (b_s / q);  u = bt_g / w
@@ -55,10 +51,10 @@ __global__ void k_prep_g(Dims D, ModelView M, const double *__restrict__ b, cons
         double s = b[D.n + i];
         for (int e = M.csr_ptr[i]; e < M.csr_ptr[i + 1]; ++e) {
             const int c = M.csr_col[e];
-            s -= M.csr_val[e] * b[c] / q[c];
+            s -= ddiv(M.csr_val[e] * b[c], q[c]);
         }
         bt_g[i] = s;
-        u[i] = s / w[i];
+        u[i] = ddiv(s, w[i]);
     }
 }
 
@@ -78,12 +74,12 @@ __global__ void k_pre_bt(Dims D, ModelView M, const double *__restrict__ b, cons
             for (int f = M.csc_ptr[c]; f < M.csc_ptr[c + 1]; ++f) Ku += M.csc_val[f] * u[D.n + M.csc_row[f]];
             const double rs = b[c] - Ku;
             s -= M.csr_val[e] * u[c];
-            s -= M.csr_val[e] * rs / q[c];
+            s -= ddiv(M.csr_val[e] * rs, q[c]);
         }
         cpre[i] = s;
         const float h = (float)s;
         cw[i] = make_float2(h, (float)(s - (double)h));
-        wf[i] = (float)(1.0 / w[i]);
+        wf[i] = (float)ddiv(1.0, w[i]);
     }
 }
 
@@ -99,7 +95,7 @@ __global__ void k_rhs_S(Dims D, const double *__restrict__ b, const double *__re
 __global__ void k_sol_gdh(Dims D, const double *__restrict__ Adx, const double *__restrict__ bt_g,
                           const double *__restrict__ w, const double *__restrict__ rhsS, double *__restrict__ sol) {
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, gsz = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = gtid; i < D.m_E; i += gsz) sol[D.n + i] = (Adx[i] - bt_g[i]) / w[i];
+    for (int64_t i = gtid; i < D.m_E; i += gsz) sol[D.n + i] = ddiv(Adx[i] - bt_g[i], w[i]);
     for (int64_t k = gtid; k < D.n_d; k += gsz) sol[D.n_s + k] = rhsS[k];
     for (int64_t j = gtid; j < D.m_I; j += gsz) sol[D.n + D.m_E + j] = rhsS[D.n_d + j];
 }
@@ -109,7 +105,7 @@ __global__ void k_sol_gdh_pre(Dims D, const double *__restrict__ Adx, const doub
                               const double *__restrict__ Au, const double *__restrict__ w,
                               const double *__restrict__ rhsS, double *__restrict__ sol) {
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, gsz = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = gtid; i < D.m_E; i += gsz) sol[D.n + i] = (Adx[i] - (cpre[i] - Au[i])) / w[i];
+    for (int64_t i = gtid; i < D.m_E; i += gsz) sol[D.n + i] = ddiv(Adx[i] - (cpre[i] - Au[i]), w[i]);
     for (int64_t k = gtid; k < D.n_d; k += gsz) sol[D.n_s + k] = rhsS[k];
     for (int64_t j = gtid; j < D.m_I; j += gsz) sol[D.n + D.m_E + j] = rhsS[D.n_d + j];
 }
@@ -120,7 +116,7 @@ __global__ void k_sol_s(Dims D, ModelView M, const double *__restrict__ b, const
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < D.n_s; k += (int64_t)gridDim.x * blockDim.x) {
         double s = b[k];
         for (int e = M.csc_ptr[k]; e < M.csc_ptr[k + 1]; ++e) s -= M.csc_val[e] * sol[D.n + M.csc_row[e]];
-        sol[k] = s / q[k];
+        sol[k] = ddiv(s, q[k]);
     }
 }
 
@@ -155,8 +151,7 @@ __global__ void __launch_bounds__(NT) k_residual(Dims D, ModelView M, const doub
                                                  const double *__restrict__ sig_xd, const double *__restrict__ sig_d,
                                                  const double *__restrict__ Jdh, const double *__restrict__ Au,
                                                  const double *__restrict__ ATug, const double *__restrict__ Hu,
-                                                 double dw, double dc, double *__restrict__ r, double *partial) {
-    __shared__ double sh[32];
+                                                 double dw, double dc, double *__restrict__ r, RedOut red) {
     double rm = 0.0, bm = 0.0, km = 0.0, um = 0.0;
     const int64_t gtid = (int64_t)blockIdx.x * NT + threadIdx.x, gsz = (int64_t)gridDim.x * NT;
     const double *us = u, *ud = u + D.n_s, *ug = u + D.n, *uh = u + D.n + D.m_E;
@@ -174,10 +169,11 @@ __global__ void __launch_bounds__(NT) k_residual(Dims D, ModelView M, const doub
         for (int e = M.csc_ptr[k]; e < M.csc_ptr[k + 1]; ++e) Ku += M.csc_val[e] * ug[M.csc_row[e]];
         put(k, Ku);
     }
-    for (int64_t k = gtid; k < D.n_d; k += gsz) {
-        double Ku = Hu[k] + (sig_xd[k] + dw) * ud[k] + ATug[k];
-        for (int64_t j = 0; j < D.m_I; ++j) Ku += Jdh[j * D.n_d + k] * uh[j];
-        put(D.n_s + k, Ku);
+    __shared__ double sp[NT / 32][33];
+    for (int64_t k0 = (int64_t)blockIdx.x * 32; k0 < D.n_d; k0 += (int64_t)gridDim.x * 32) {
+        const double jt = colgroup_dot<NT>(Jdh, D.m_I, D.n_d, k0, uh, sp);
+        const int64_t k = k0 + threadIdx.x;
+        if (threadIdx.x < 32 && k < D.n_d) put(D.n_s + k, Hu[k] + (sig_xd[k] + dw) * ud[k] + ATug[k] + jt);
     }
     for (int64_t i = gtid; i < D.m_E; i += gsz) {
         double Ku = Au[i] - dc * ug[i];
@@ -185,14 +181,11 @@ __global__ void __launch_bounds__(NT) k_residual(Dims D, ModelView M, const doub
         put(D.n + i, Ku);
     }
     for (int64_t j = gtid; j < D.m_I; j += gsz) {
-        const double Ku = -(1.0 / (sig_d[j] + dw) + dc) * uh[j] + Hu[D.n_d + j];   // + (J_dh u_d)_j
+        const double Ku = -(ddiv(1.0, sig_d[j] + dw) + dc) * uh[j] + Hu[D.n_d + j];   // + (J_dh u_d)_j
         put(D.n + D.m_E + j, Ku);
     }
-    double x;
-    x = block_max<NT>(rm, sh); if (threadIdx.x == 0) *slot(partial, 0) = x;
-    x = block_max<NT>(bm, sh); if (threadIdx.x == 0) *slot(partial, 1) = x;
-    x = block_max<NT>(km, sh); if (threadIdx.x == 0) *slot(partial, 2) = x;
-    x = block_max<NT>(um, sh); if (threadIdx.x == 0) *slot(partial, 3) = x;
+    double v[4] = {rm, bm, km, um};
+    reduce_finish<NT, R_MAX, R_MAX, R_MAX, R_MAX>(v, red);
 }
 
 __global__ void k_axpy(int64_t n, const double *__restrict__ x, double *__restrict__ y) {
@@ -208,15 +201,15 @@ __global__ void k_dir_from_sol(Dims D, ModelView M, IterView I, DirView Dir, con
         const double dx = u[i];
         Dir.dx[i] = dx;
         const double xi = I.x[i];
-        if (isfinite(M.xl[i])) {
+        if (fin(M.xl[i])) {
             const double s = xi - M.xl[i];
-            Dir.dzl[i] = mu / s - I.zl[i] - I.zl[i] / s * dx;
+            Dir.dzl[i] = ddiv(mu, s) - I.zl[i] - ddiv(I.zl[i], s) * dx;
         } else {
             Dir.dzl[i] = 0.0;
         }
-        if (isfinite(M.xu[i])) {
+        if (fin(M.xu[i])) {
             const double s = M.xu[i] - xi;
-            Dir.dzu[i] = mu / s - I.zu[i] + I.zu[i] / s * dx;
+            Dir.dzu[i] = ddiv(mu, s) - I.zu[i] + ddiv(I.zu[i], s) * dx;
         } else {
             Dir.dzu[i] = 0.0;
         }
@@ -225,16 +218,16 @@ __global__ void k_dir_from_sol(Dims D, ModelView M, IterView I, DirView Dir, con
     for (int64_t j = gtid; j < D.m_I; j += gsz) {
         const double dyh = u[D.n + D.m_E + j];
         Dir.dyh[j] = dyh;
-        const double dd = (dyh - r_dslack(M, I, mu, j)) / (sig_d[j] + dw);
+        const double dd = ddiv(dyh - r_dslack(M, I, mu, j), sig_d[j] + dw);
         Dir.dd[j] = dd;
         const double dj = I.d[j];
-        if (isfinite(M.hl[j])) {
+        if (fin(M.hl[j])) {
             const double s = dj - M.hl[j];
             Dir.dvl[j] = mu / s - I.vl[j] - I.vl[j] / s * dd;
         } else {
             Dir.dvl[j] = 0.0;
         }
-        if (isfinite(M.hu[j])) {
+        if (fin(M.hu[j])) {
             const double s = M.hu[j] - dj;
             Dir.dvu[j] = mu / s - I.vu[j] + I.vu[j] / s * dd;
         } else {
@@ -314,10 +307,10 @@ void Refiner::residual(const double *b, const double *u, double dw, double dc, d
     k_hdd_gemv<<<std::max(1, std::min(4096, ceil_div((D.n_d + D.m_I) * 32, 256))), 256, 0, st>>>(
         D.n_d, D.m_I, Hdd, Jdh, u + D.n_s, tmp_nd2);
     MDSIP_LAUNCHED();
-    k_residual<<<kRedBlocks, NT, 0, st>>>(D, M, b, u, q, sig_xd, sig_d, Jdh, Au, tmp_nd, tmp_nd2, dw, dc,
-                                          r, partial);
+    k_residual<<<red_grid(std::max(std::max(D.n_s, D.m_E), (NT / 32) * D.n_d)), NT, 0, st>>>(
+        D, M, b, u, q, sig_xd, sig_d, Jdh, Au, tmp_nd, tmp_nd2, dw, dc, r,
+        RedOut{partial, reinterpret_cast<unsigned *>(partial + kRedBlocks * 8), out4});
     MDSIP_LAUNCHED();
-    launch_finalize_max(st, partial, 4, out4);
 }
 
 void Refiner::axpy(int64_t n, const double *x, double *y) {

@@ -376,7 +376,8 @@ static Problem *create_common(Ctx *ctx, int64_t n_d, int64_t n_s, int64_t m_E, i
         dvec(ctx, P->bATu, D.n_d);
         dvec(ctx, P->bAdx, D.m_E);
         dvec(ctx, P->bscal, SC_COUNT);
-        dvec(ctx, P->bpartial, (int64_t)kRedBlocks * 8);
+        dvec(ctx, P->bpartial, (int64_t)kRedBlocks * 8 + 1);   // partials and the reductions' ticket
+        MDSIP_CUDA(cudaMemsetAsync(P->bpartial.as<double>() + kRedBlocks * 8, 0, sizeof(double), st));
         dvec(ctx, P->bcolpart, (int64_t)kRedBlocks * std::max<int64_t>(D.n_d, 1));
         dvec(ctx, P->browtmp, std::max<int64_t>(D.m_E, 1));
         P->berr.get<int>(ctx, 4);
@@ -814,7 +815,7 @@ static int tuned_ldlt_width(Problem *P, bool fp32) {
         MDSIP_CUDA(cudaMemcpyAsync(Ssave, S, (size_t)N * N * sizeof(double), cudaMemcpyDeviceToDevice, st));
         v = tune_pick(P, cands, [&](int nb) {
             MDSIP_CUDA(cudaMemcpyAsync(S, Ssave, (size_t)N * N * sizeof(double), cudaMemcpyDeviceToDevice, st));
-            launch_maxabs_lower(st, N, S, N, P->V.partial, sc + SC_MAXABS);
+            launch_maxabs_lower(st, N, S, N, sc + SC_MAXABS);
             LdltOut o{P->bL.as<double>(), P->bDd.as<double>(), P->bDoff.as<double>(), P->bperm.as<int32_t>(),
                       P->bkind.as<int32_t>(), P->binertia.as<int32_t>()};
             launch_ldlt(st, P->ctx->num_sms, N, S, N, sc + SC_MAXABS, P->opt.zero_tol, o, P->bldlt_ws.ptr,
@@ -872,7 +873,7 @@ static Inertia factor_attempt(Problem *P, double dw, double dc, bool force_fp64 
     const int nb = tuned_ldlt_width(P, tc_factor);
     MDSIP_CUDA(cudaEventRecord(P->ev[10], st));   // the width's trial runs are not the factorization
     auto factor_phase = [&] {
-        launch_maxabs_lower(st, P->N, S, P->N, P->V.partial, sc + SC_MAXABS);
+        launch_maxabs_lower(st, P->N, S, P->N, sc + SC_MAXABS);
         MDSIP_CUDA(cudaMemsetAsync(P->berr.ptr, 0, sizeof(int), st));
         LdltOut o{P->bL.as<double>(), P->bDd.as<double>(), P->bDoff.as<double>(), P->bperm.as<int32_t>(),
                   P->bkind.as<int32_t>(), P->binertia.as<int32_t>()};
@@ -1998,15 +1999,14 @@ static mdsip_status ldlt_factor_impl(mdsip_ctx *hctx, int64_t N, double *S, int6
             return;
         }
         MDSIP_REQUIRE(S && L && Dd && Doff && perm && kind, MDSIP_ERR_INVALID_ARG, "ldlt: null pointer");
-        const size_t ws = ldlt_scratch_bytes(N) + 64 + 8 * kRedBlocks + 64;
+        const size_t ws = ldlt_scratch_bytes(N) + 64 + 64;
         char *w = static_cast<char *>(ctx->scratch_at_least(ws));
-        double *partial = reinterpret_cast<double *>(w + ldlt_scratch_bytes(N) + 64);
-        double *maxabs = partial + kRedBlocks;
+        double *maxabs = reinterpret_cast<double *>(w + ldlt_scratch_bytes(N) + 64);
         int *err = reinterpret_cast<int *>(w + ldlt_scratch_bytes(N));   // err, then two panel counts
-        MDSIP_REQUIRE((reinterpret_cast<uintptr_t>(partial) & 7) == 0, MDSIP_ERR_INVALID_ARG,
+        MDSIP_REQUIRE((reinterpret_cast<uintptr_t>(maxabs) & 7) == 0, MDSIP_ERR_INVALID_ARG,
                       "ldlt: misaligned scratch layout");
         MDSIP_CUDA(cudaMemsetAsync(err, 0, 3 * sizeof(int), ctx->stream));
-        launch_maxabs_lower(ctx->stream, N, S, ld, partial, maxabs);
+        launch_maxabs_lower(ctx->stream, N, S, ld, maxabs);
         LdltOut o{L, Dd, Doff, perm, kind, inertia, err + 1};
         launch_ldlt(ctx->stream, ctx->num_sms, N, S, ld, maxabs, zero_tol, o, w, err, fp32_update, 0, spec);
         int herr[3] = {0, 0, 0};

@@ -1,8 +1,8 @@
 // Fused vector kernels of one Newton step (Section 2.3, kernel classes K1 and
 // K2) and the evaluation of the benchmark model family (Section 2 problem
-// class).  All FP64.  Reductions are two-pass and deterministic: every
-// reduction kernel runs on kRedBlocks blocks and writes one partial per block;
-// a finalize kernel combines the partials in block order.
+// class).  All FP64.  Reductions are deterministic: every reduction kernel
+// runs on at most kRedBlocks blocks, one element per thread where there are
+// fewer, and its last block combines the blocks' partials in order.
 #include "internal.cuh"
 #include "vec.cuh"
 
@@ -12,36 +12,11 @@ namespace {
 
 constexpr int NT = kRedThreads;
 
-__device__ __forceinline__ bool fin(double v) { return isfinite(v); }
-
-// partial slot of quantity q for this block
-__device__ __forceinline__ double *slot(double *partial, int q) {
-    return partial + (size_t)q * kRedBlocks + blockIdx.x;
-}
-
-__global__ void k_finalize(const double *partial, int nq, double *out, int op) {
-    // one warp per quantity; fixed order inside the warp reduction
-    const int q = blockIdx.x;
-    if (q >= nq) return;
-    const double *p = partial + (size_t)q * kRedBlocks;
-    double v = op == 0 ? 0.0 : (op == 1 ? -INFINITY : INFINITY);
-    for (int b = threadIdx.x; b < kRedBlocks; b += 32) {
-        const double x = p[b];
-        v = op == 0 ? v + x : (op == 1 ? fmax(v, x) : fmin(v, x));
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        const double x = __shfl_down_sync(0xffffffffu, v, o);
-        v = op == 0 ? v + x : (op == 1 ? fmax(v, x) : fmin(v, x));
-    }
-    if (threadIdx.x == 0) out[q] = v;
-}
-
 // ---------------------------------------------------------------------------
 // Model: f and grad f.  f = 1/2 x_d^T Q x_d + sum 1/4 x_s^4 + c^T x
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(NT) k_eval_f(Dims D, ModelView M, const double *__restrict__ x,
-                                               double *__restrict__ grad, double *partial) {
-    __shared__ double sh[32];
+                                               double *__restrict__ grad, RedOut red) {
     double acc = 0.0;
     const int64_t gtid = (int64_t)blockIdx.x * NT + threadIdx.x;
     const int64_t gsz = (int64_t)gridDim.x * NT;
@@ -66,8 +41,8 @@ __global__ void __launch_bounds__(NT) k_eval_f(Dims D, ModelView M, const double
             if (grad) grad[D.n_s + p] = s + cp;
         }
     }
-    const double r = block_sum<NT>(acc, sh);
-    if (threadIdx.x == 0) *slot(partial, 0) = r;
+    double v[1] = {acc};
+    reduce_finish<NT, R_SUM>(v, red);
 }
 
 // ---------------------------------------------------------------------------
@@ -77,8 +52,7 @@ __global__ void __launch_bounds__(NT) k_eval_f(Dims D, ModelView M, const double
 __global__ void __launch_bounds__(NT) k_eval_cons(Dims D, ModelView M, const double *__restrict__ x,
                                                   const double *__restrict__ Axd, const double *__restrict__ d,
                                                   double *__restrict__ cg, double *__restrict__ ch,
-                                                  double *partial) {
-    __shared__ double sh[32];
+                                                  RedOut red) {
     const int lane = threadIdx.x & 31;
     const int64_t gw = ((int64_t)blockIdx.x * NT + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * NT) >> 5;
@@ -107,10 +81,8 @@ __global__ void __launch_bounds__(NT) k_eval_cons(Dims D, ModelView M, const dou
             mx = fmax(mx, fabs(r));
         }
     }
-    const double a = block_sum<NT>(s1, sh);
-    if (threadIdx.x == 0) *slot(partial, 0) = a;
-    const double b = block_max<NT>(mx, sh);
-    if (threadIdx.x == 0) *slot(partial, 1) = b;
+    double v[2] = {s1, mx};
+    reduce_finish<NT, R_SUM, R_MAX>(v, red);
 }
 
 // Jacobian of h (dense m_I x n_d row-major) and the Hessian blocks:
@@ -192,45 +164,53 @@ __global__ void __launch_bounds__(NT) k_gemv_rows(const double *__restrict__ A, 
     if (live && h == 0) out[i] = sum;
 }
 
-// partial[b][p] = sum over the rows of block b of A[i][p] u[i]
-constexpr int kGtCols = 8;  // columns per thread per pass
+// partial[b][p] = sum over the rows of block b of A[i][p] u[i].  tc threads (a
+// power of two) take the columns, C each, and the block's NT / tc groups its
+// rows, U in flight: 8 to 12 loads a thread cover the memory's latency (m =
+// 15053, n = 301: 54 us with one row pair in flight and 8 columns per thread of
+// which two were used, 21 us so; m = 1000, n = 32: 8 -> 6 us).
+template <int C, int U>
 __global__ void __launch_bounds__(NT) k_gemv_t(const double *__restrict__ A, int64_t m, int64_t n,
-                                               int64_t lda, const double *__restrict__ u,
+                                               int64_t lda, const double *__restrict__ u, int tc,
                                                double *__restrict__ partial) {
+    __shared__ double sh[NT];
+    const int col = threadIdx.x & (tc - 1), g = threadIdx.x / tc, G = NT / tc;
     const int64_t rows_per = (m + gridDim.x - 1) / gridDim.x;
     const int64_t r0 = (int64_t)blockIdx.x * rows_per;
     const int64_t r1 = min(m, r0 + rows_per);
-    for (int64_t c0 = 0; c0 < n; c0 += (int64_t)NT * kGtCols) {
-        double acc[kGtCols];
+    for (int64_t c0 = 0; c0 < n; c0 += (int64_t)tc * C) {
+        double acc[C];
 #pragma unroll
-        for (int c = 0; c < kGtCols; ++c) acc[c] = 0.0;
-        int64_t i = r0;
-        for (; i + 1 < r1; i += 2) {
-            const double u0 = u[i], u1 = u[i + 1];
-            const double *row0 = A + i * lda, *row1 = row0 + lda;
-            double a0[kGtCols], a1[kGtCols];
+        for (int c = 0; c < C; ++c) acc[c] = 0.0;
+        for (int64_t i = r0 + g; i < r1; i += (int64_t)U * G) {
+            double a[U][C], ui[U];
 #pragma unroll
-            for (int c = 0; c < kGtCols; ++c) {
-                const int64_t p = c0 + threadIdx.x + (int64_t)c * NT;
-                a0[c] = p < n ? __ldg(row0 + p) : 0.0;
-                a1[c] = p < n ? __ldg(row1 + p) : 0.0;
+            for (int x = 0; x < U; ++x) {
+                const int64_t r = i + (int64_t)x * G;
+                ui[x] = r < r1 ? __ldg(u + r) : 0.0;
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    const int64_t p = c0 + col + (int64_t)c * tc;
+                    a[x][c] = r < r1 && p < n ? __ldg(A + r * lda + p) : 0.0;
+                }
             }
 #pragma unroll
-            for (int c = 0; c < kGtCols; ++c) acc[c] = fma(a1[c], u1, fma(a0[c], u0, acc[c]));
-        }
-        for (; i < r1; ++i) {
-            const double ui = u[i];
-            const double *row = A + i * lda;
+            for (int x = 0; x < U; ++x)
+                if (i + (int64_t)x * G < r1)
 #pragma unroll
-            for (int c = 0; c < kGtCols; ++c) {
-                const int64_t p = c0 + threadIdx.x + (int64_t)c * NT;
-                if (p < n) acc[c] = fma(__ldg(row + p), ui, acc[c]);
+                    for (int c = 0; c < C; ++c) acc[c] = fma(a[x][c], ui[x], acc[c]);
+        }
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const int64_t p = c0 + col + (int64_t)c * tc;
+            double v = acc[c];
+            if (G > 1) {                       // tc < NT: one pass, one column per thread
+                sh[threadIdx.x] = v;
+                __syncthreads();
+                for (int x = 1; x < G; ++x)
+                    if (g == 0) v += sh[x * tc + col];
             }
-        }
-#pragma unroll
-        for (int c = 0; c < kGtCols; ++c) {
-            const int64_t p = c0 + threadIdx.x + (int64_t)c * NT;
-            if (p < n) partial[(size_t)blockIdx.x * n + p] = acc[c];
+            if (g == 0 && p < n) partial[(size_t)blockIdx.x * n + p] = v;
         }
     }
 }
@@ -269,7 +249,7 @@ __global__ void __launch_bounds__(256) k_colsum(const double *__restrict__ parti
 // ---------------------------------------------------------------------------
 // Gradient of the Lagrangian: gl = grad f + J_g^T y_g + J_h^T y_h
 // ---------------------------------------------------------------------------
-__global__ void k_lagrangian_grad(Dims D, ModelView M, const double *__restrict__ grad,
+__global__ void __launch_bounds__(NT) k_lagrangian_grad(Dims D, ModelView M, const double *__restrict__ grad,
                                   const double *__restrict__ yg, const double *__restrict__ yh,
                                   const double *__restrict__ Jdh, const double *__restrict__ ATy,
                                   double *__restrict__ gl) {
@@ -282,10 +262,11 @@ __global__ void k_lagrangian_grad(Dims D, ModelView M, const double *__restrict_
             for (int e = M.hsc_ptr[i]; e < M.hsc_ptr[i + 1]; ++e) s += M.hsc_val[e] * yh[M.hsc_row[e]];
         gl[i] = s;
     }
-    for (int64_t k = gtid; k < D.n_d; k += gsz) {
-        double s = grad[D.n_s + k] + ATy[k];
-        for (int64_t j = 0; j < D.m_I; ++j) s += Jdh[j * D.n_d + k] * yh[j];
-        gl[D.n_s + k] = s;
+    __shared__ double sp[NT / 32][33];
+    for (int64_t k0 = (int64_t)blockIdx.x * 32; k0 < D.n_d; k0 += (int64_t)gridDim.x * 32) {
+        const double jt = colgroup_dot<NT>(Jdh, D.m_I, D.n_d, k0, yh, sp);
+        const int64_t k = k0 + threadIdx.x;
+        if (threadIdx.x < 32 && k < D.n_d) gl[D.n_s + k] = grad[D.n_s + k] + ATy[k] + jt;
     }
 }
 
@@ -297,15 +278,14 @@ __global__ void k_lagrangian_grad(Dims D, ModelView M, const double *__restrict_
 __global__ void __launch_bounds__(NT) k_errors(Dims D, ModelView M, IterView I,
                                                const double *__restrict__ gl,
                                                const double *__restrict__ cg,
-                                               const double *__restrict__ ch, double *partial) {
-    __shared__ double sh[32];
+                                               const double *__restrict__ ch, RedOut red) {
     double du = 0.0, pr = 0.0, cmax = -INFINITY, cmin = INFINITY, y1 = 0.0, z1 = 0.0, lg = 0.0;
     const int64_t gtid = (int64_t)blockIdx.x * NT + threadIdx.x;
     const int64_t gsz = (int64_t)gridDim.x * NT;
     for (int64_t i = gtid; i < D.n; i += gsz) {
         const double xi = I.x[i];
         du = fmax(du, fabs(gl[i] - I.zl[i] + I.zu[i]));
-        if (isfinite(M.xl[i])) {
+        if (fin(M.xl[i])) {
             const double s = xi - M.xl[i];
             const double p = s * I.zl[i];
             cmax = fmax(cmax, p);
@@ -313,7 +293,7 @@ __global__ void __launch_bounds__(NT) k_errors(Dims D, ModelView M, IterView I,
             z1 += fabs(I.zl[i]);
             lg += log(s);
         }
-        if (isfinite(M.xu[i])) {
+        if (fin(M.xu[i])) {
             const double s = M.xu[i] - xi;
             const double p = s * I.zu[i];
             cmax = fmax(cmax, p);
@@ -327,7 +307,7 @@ __global__ void __launch_bounds__(NT) k_errors(Dims D, ModelView M, IterView I,
         pr = fmax(pr, fabs(ch[j]));
         y1 += fabs(I.yh[j]);
         const double dj = I.d[j];
-        if (isfinite(M.hl[j])) {
+        if (fin(M.hl[j])) {
             const double s = dj - M.hl[j];
             const double p = s * I.vl[j];
             cmax = fmax(cmax, p);
@@ -335,7 +315,7 @@ __global__ void __launch_bounds__(NT) k_errors(Dims D, ModelView M, IterView I,
             z1 += fabs(I.vl[j]);
             lg += log(s);
         }
-        if (isfinite(M.hu[j])) {
+        if (fin(M.hu[j])) {
             const double s = M.hu[j] - dj;
             const double p = s * I.vu[j];
             cmax = fmax(cmax, p);
@@ -348,14 +328,8 @@ __global__ void __launch_bounds__(NT) k_errors(Dims D, ModelView M, IterView I,
         pr = fmax(pr, fabs(cg[i]));
         y1 += fabs(I.yg[i]);
     }
-    double r;
-    r = block_max<NT>(du, sh);   if (threadIdx.x == 0) *slot(partial, 0) = r;
-    r = block_max<NT>(pr, sh);   if (threadIdx.x == 0) *slot(partial, 1) = r;
-    r = block_max<NT>(cmax, sh); if (threadIdx.x == 0) *slot(partial, 2) = r;
-    r = block_min<NT>(cmin, sh); if (threadIdx.x == 0) *slot(partial, 3) = r;
-    r = block_sum<NT>(y1, sh);   if (threadIdx.x == 0) *slot(partial, 4) = r;
-    r = block_sum<NT>(z1, sh);   if (threadIdx.x == 0) *slot(partial, 5) = r;
-    r = block_sum<NT>(lg, sh);   if (threadIdx.x == 0) *slot(partial, 6) = r;
+    double v[7] = {du, pr, cmax, cmin, y1, z1, lg};
+    reduce_finish<NT, R_MAX, R_MAX, R_MAX, R_MIN, R_SUM, R_SUM, R_SUM>(v, red);
 }
 
 // ---------------------------------------------------------------------------
@@ -363,10 +337,19 @@ __global__ void __launch_bounds__(NT) k_errors(Dims D, ModelView M, IterView I,
 // two-stage elimination.  q = H_ss + Sigma_xs + dw; Sigma_d; w = J_sg^2 q^-1 + dc.
 // quantities: 0..2 inertia of Q_s (pos, neg, zero), 3..5 inertia of -W.
 // ---------------------------------------------------------------------------
+// sign of a value by its bit pattern (NaN counts nowhere)
+__device__ __forceinline__ void count_sign(double v, unsigned &pos, unsigned &neg, unsigned &zero) {
+    const long long b = __double_as_longlong(v), m = b & 0x7fffffffffffffffLL;
+    if (m > 0x7ff0000000000000LL) return;
+    zero += m == 0;
+    pos += m != 0 && b > 0;
+    neg += m != 0 && b < 0;
+}
+
 __device__ __forceinline__ double sigma_x(const ModelView &M, const IterView &I, int64_t i) {
     double s = 0.0;
-    if (isfinite(M.xl[i])) s += I.zl[i] / (I.x[i] - M.xl[i]);
-    if (isfinite(M.xu[i])) s += I.zu[i] / (M.xu[i] - I.x[i]);
+    if (fin(M.xl[i])) s += ddiv(I.zl[i], I.x[i] - M.xl[i]);
+    if (fin(M.xu[i])) s += ddiv(I.zu[i], M.xu[i] - I.x[i]);
     return s;
 }
 
@@ -374,9 +357,8 @@ __global__ void __launch_bounds__(NT) k_newton_diag(Dims D, ModelView M, IterVie
                                                     const double *__restrict__ Hss, double dw,
                                                     double dc, int want_w, double *__restrict__ sig_x,
                                                     double *__restrict__ q, double *__restrict__ sig_d,
-                                                    double *__restrict__ w, double *partial) {
-    __shared__ double sh[32];
-    double qp = 0, qn = 0, qz = 0, wp = 0, wn = 0, wz = 0;
+                                                    double *__restrict__ w, RedOut red) {
+    unsigned c6[6] = {0, 0, 0, 0, 0, 0};   // In(Q_s), In(-W): positive, negative, zero
     const int64_t gtid = (int64_t)blockIdx.x * NT + threadIdx.x;
     const int64_t gsz = (int64_t)gridDim.x * NT;
     for (int64_t i = gtid; i < D.n; i += gsz) {
@@ -385,15 +367,13 @@ __global__ void __launch_bounds__(NT) k_newton_diag(Dims D, ModelView M, IterVie
         if (i < D.n_s) {
             const double qi = Hss[i] + s + dw;
             q[i] = qi;
-            qp += qi > 0.0;
-            qn += qi < 0.0;
-            qz += qi == 0.0;
+            count_sign(qi, c6[0], c6[1], c6[2]);
         }
     }
     for (int64_t j = gtid; j < D.m_I; j += gsz) {
         double s = 0.0;
-        if (isfinite(M.hl[j])) s += I.vl[j] / (I.d[j] - M.hl[j]);
-        if (isfinite(M.hu[j])) s += I.vu[j] / (M.hu[j] - I.d[j]);
+        if (fin(M.hl[j])) s += ddiv(I.vl[j], I.d[j] - M.hl[j]);
+        if (fin(M.hu[j])) s += ddiv(I.vu[j], M.hu[j] - I.d[j]);
         sig_d[j] = s;
     }
     if (want_w) {
@@ -402,30 +382,21 @@ __global__ void __launch_bounds__(NT) k_newton_diag(Dims D, ModelView M, IterVie
             for (int e = M.csr_ptr[i]; e < M.csr_ptr[i + 1]; ++e) {
                 const int64_t c = M.csr_col[e];
                 const double qc = Hss[c] + sigma_x(M, I, c) + dw;
-                s += M.csr_val[e] * M.csr_val[e] / qc;
+                s += ddiv(M.csr_val[e] * M.csr_val[e], qc);
             }
             w[i] = s;
-            // inertia of -W
-            wp += s < 0.0;
-            wn += s > 0.0;
-            wz += s == 0.0;
+            count_sign(s, c6[4], c6[3], c6[5]);   // of -W
         }
     }
-    double r;
-    r = block_sum<NT>(qp, sh); if (threadIdx.x == 0) *slot(partial, 0) = r;
-    r = block_sum<NT>(qn, sh); if (threadIdx.x == 0) *slot(partial, 1) = r;
-    r = block_sum<NT>(qz, sh); if (threadIdx.x == 0) *slot(partial, 2) = r;
-    r = block_sum<NT>(wp, sh); if (threadIdx.x == 0) *slot(partial, 3) = r;
-    r = block_sum<NT>(wn, sh); if (threadIdx.x == 0) *slot(partial, 4) = r;
-    r = block_sum<NT>(wz, sh); if (threadIdx.x == 0) *slot(partial, 5) = r;
+    count_finish<NT>(c6, red);
 }
 
 // barrier gradient of the Lagrangian at x: rN_i = gl_i - mu/s_l + mu/s_u
 __device__ __forceinline__ double rN_x(const ModelView &M, const IterView &I, const double *gl,
                                        double mu, int64_t i) {
     double r = gl[i];
-    if (isfinite(M.xl[i])) r -= mu / (I.x[i] - M.xl[i]);
-    if (isfinite(M.xu[i])) r += mu / (M.xu[i] - I.x[i]);
+    if (fin(M.xl[i])) r -= ddiv(mu, I.x[i] - M.xl[i]);
+    if (fin(M.xu[i])) r += ddiv(mu, M.xu[i] - I.x[i]);
     return r;
 }
 
@@ -433,8 +404,8 @@ __device__ __forceinline__ double rN_x(const ModelView &M, const IterView &I, co
 __device__ __forceinline__ double r_dslack(const ModelView &M, const IterView &I, double mu,
                                            int64_t j) {
     double r = -I.yh[j];
-    if (isfinite(M.hl[j])) r -= mu / (I.d[j] - M.hl[j]);
-    if (isfinite(M.hu[j])) r += mu / (M.hu[j] - I.d[j]);
+    if (fin(M.hl[j])) r -= ddiv(mu, I.d[j] - M.hl[j]);
+    if (fin(M.hu[j])) r += ddiv(mu, M.hu[j] - I.d[j]);
     return r;
 }
 
@@ -453,10 +424,10 @@ __global__ void k_rhs_y(Dims D, ModelView M, IterView I, const double *__restric
         double s = -cg[i];
         for (int e = M.csr_ptr[i]; e < M.csr_ptr[i + 1]; ++e) {
             const int64_t c = M.csr_col[e];
-            s += M.csr_val[e] * rN_x(M, I, gl, mu, c) / q[c];   // -J_sg (b_s/q), b_s = -rN_s
+            s += ddiv(M.csr_val[e] * rN_x(M, I, gl, mu, c), q[c]);   // -J_sg (b_s/q), b_s = -rN_s
         }
         bt_g[i] = s;
-        if (u) u[i] = s / w[i];
+        if (u) u[i] = ddiv(s, w[i]);
     }
 }
 
@@ -477,11 +448,11 @@ __global__ void k_rhs_reduced(Dims D, ModelView M, IterView I, const double *__r
     }
     const int64_t off_h = p1 ? D.n_d + D.m_E : D.n_d;
     for (int64_t j = gtid; j < D.m_I; j += gsz) {
-        double r = -(ch[j] + r_dslack(M, I, mu, j) / (sig_d[j] + dw));
+        double r = -(ch[j] + ddiv(r_dslack(M, I, mu, j), sig_d[j] + dw));
         if (p1 && M.hsr_ptr)
             for (int e = M.hsr_ptr[j]; e < M.hsr_ptr[j + 1]; ++e) {
                 const int64_t c = M.hsr_col[e];
-                r += M.hsr_val[e] * rN_x(M, I, gl, mu, c) / q[c];   // -J_sh (b_s/q), b_s = -rN_s
+                r += ddiv(M.hsr_val[e] * rN_x(M, I, gl, mu, c), q[c]);   // -J_sh (b_s/q), b_s = -rN_s
             }
         rhs[off_h + j] = r;
     }
@@ -494,7 +465,7 @@ __global__ void k_dyg_p2(int64_t m_E, const double *__restrict__ Adx, const doub
                          const double *__restrict__ w, double *__restrict__ dyg) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m_E;
          i += (int64_t)gridDim.x * blockDim.x)
-        dyg[i] = (Adx[i] - bt_g[i]) / w[i];
+        dyg[i] = ddiv(Adx[i] - bt_g[i], w[i]);
 }
 
 // Common back-substitution: dx_s = (b_s - J_sg^T dy_g)/q, dx_d, dy_h from the
@@ -514,21 +485,21 @@ __global__ void k_backsub(Dims D, ModelView M, IterView I, DirView Dir, const do
                 s -= M.csc_val[e] * Dir.dyg[M.csc_row[e]];
             if (M.hsc_ptr)   // J_sh^T dy_h (dy_h from the reduced solution: Dir.dyh is written below)
                 for (int e = M.hsc_ptr[i]; e < M.hsc_ptr[i + 1]; ++e) s -= M.hsc_val[e] * sol_dyh[M.hsc_row[e]];
-            dx = s / q[i];
+            dx = ddiv(s, q[i]);
         } else {
             dx = sol_dxd[i - D.n_s];
         }
         Dir.dx[i] = dx;
         const double xi = I.x[i];
-        if (isfinite(M.xl[i])) {
+        if (fin(M.xl[i])) {
             const double s = xi - M.xl[i];
-            Dir.dzl[i] = mu / s - I.zl[i] - I.zl[i] / s * dx;
+            Dir.dzl[i] = ddiv(mu, s) - I.zl[i] - ddiv(I.zl[i], s) * dx;
         } else {
             Dir.dzl[i] = 0.0;
         }
-        if (isfinite(M.xu[i])) {
+        if (fin(M.xu[i])) {
             const double s = M.xu[i] - xi;
-            Dir.dzu[i] = mu / s - I.zu[i] + I.zu[i] / s * dx;
+            Dir.dzu[i] = ddiv(mu, s) - I.zu[i] + ddiv(I.zu[i], s) * dx;
         } else {
             Dir.dzu[i] = 0.0;
         }
@@ -536,18 +507,18 @@ __global__ void k_backsub(Dims D, ModelView M, IterView I, DirView Dir, const do
     for (int64_t j = gtid; j < D.m_I; j += gsz) {
         const double dyh = sol_dyh[j];
         Dir.dyh[j] = dyh;
-        const double dd = (dyh - r_dslack(M, I, mu, j)) / (sig_d[j] + dw);
+        const double dd = ddiv(dyh - r_dslack(M, I, mu, j), sig_d[j] + dw);
         Dir.dd[j] = dd;
         const double dj = I.d[j];
-        if (isfinite(M.hl[j])) {
+        if (fin(M.hl[j])) {
             const double s = dj - M.hl[j];
-            Dir.dvl[j] = mu / s - I.vl[j] - I.vl[j] / s * dd;
+            Dir.dvl[j] = ddiv(mu, s) - I.vl[j] - ddiv(I.vl[j], s) * dd;
         } else {
             Dir.dvl[j] = 0.0;
         }
-        if (isfinite(M.hu[j])) {
+        if (fin(M.hu[j])) {
             const double s = M.hu[j] - dj;
-            Dir.dvu[j] = mu / s - I.vu[j] + I.vu[j] / s * dd;
+            Dir.dvu[j] = ddiv(mu, s) - I.vu[j] + ddiv(I.vu[j], s) * dd;
         } else {
             Dir.dvu[j] = 0.0;
         }
@@ -556,8 +527,7 @@ __global__ void k_backsub(Dims D, ModelView M, IterView I, DirView Dir, const do
 
 // Distance between two packed directions: quantities 0 = sum (a - b)^2,
 // 1 = sum b^2 over the eight blocks (dx, dd, dyg, dyh, dzl, dzu, dvl, dvu).
-__global__ void __launch_bounds__(NT) k_dir_diff(Dims D, DirView a, DirView b, double *partial) {
-    __shared__ double sh[32];
+__global__ void __launch_bounds__(NT) k_dir_diff(Dims D, DirView a, DirView b, RedOut red) {
     const double *pa[8] = {a.dx, a.dd, a.dyg, a.dyh, a.dzl, a.dzu, a.dvl, a.dvu};
     const double *pb[8] = {b.dx, b.dd, b.dyg, b.dyh, b.dzl, b.dzu, b.dvl, b.dvu};
     const int64_t len[8] = {D.n, D.m_I, D.m_E, D.m_I, D.n, D.n, D.m_I, D.m_I};
@@ -570,9 +540,8 @@ __global__ void __launch_bounds__(NT) k_dir_diff(Dims D, DirView a, DirView b, d
             dd += e * e;
             bb += y * y;
         }
-    double r;
-    r = block_sum<NT>(dd, sh); if (threadIdx.x == 0) *slot(partial, 0) = r;
-    r = block_sum<NT>(bb, sh); if (threadIdx.x == 0) *slot(partial, 1) = r;
+    double v[2] = {dd, bb};
+    reduce_finish<NT, R_SUM, R_SUM>(v, red);
 }
 
 __global__ void k_copy(const double *__restrict__ src, double *__restrict__ dst, int64_t n) {
@@ -587,54 +556,52 @@ __global__ void k_copy(const double *__restrict__ src, double *__restrict__ dst,
 // quantities: 0 alpha_max (min), 1 alpha_z (min), 2 gphi (sum)
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ double ftb(double v, double dv, double tau) {
-    return dv < 0.0 ? -tau * v / dv : INFINITY;
+    // dv < 0, by its bit pattern (a NaN's quotient is a NaN, which fmin passes over)
+    return (unsigned long long)__double_as_longlong(dv) > 0x8000000000000000ULL ? ddiv(-tau * v, dv) : INFINITY;
 }
 
 __global__ void __launch_bounds__(NT) k_step_scalars(Dims D, ModelView M, IterView I, DirView Dir,
                                                      const double *__restrict__ grad, double tau,
-                                                     double mu, double *partial) {
-    __shared__ double sh[32];
+                                                     double mu, RedOut red) {
     double ap = INFINITY, az = INFINITY, gp = 0.0;
     const int64_t gtid = (int64_t)blockIdx.x * NT + threadIdx.x;
     const int64_t gsz = (int64_t)gridDim.x * NT;
     for (int64_t i = gtid; i < D.n; i += gsz) {
         const double dx = Dir.dx[i];
         double g = grad[i];
-        if (isfinite(M.xl[i])) {
+        if (fin(M.xl[i])) {
             const double s = I.x[i] - M.xl[i];
             ap = fmin(ap, ftb(s, dx, tau));
             az = fmin(az, ftb(I.zl[i], Dir.dzl[i], tau));
-            g -= mu / s;
+            g -= ddiv(mu, s);
         }
-        if (isfinite(M.xu[i])) {
+        if (fin(M.xu[i])) {
             const double s = M.xu[i] - I.x[i];
             ap = fmin(ap, ftb(s, -dx, tau));
             az = fmin(az, ftb(I.zu[i], Dir.dzu[i], tau));
-            g += mu / s;
+            g += ddiv(mu, s);
         }
         gp += g * dx;
     }
     for (int64_t j = gtid; j < D.m_I; j += gsz) {
         const double dd = Dir.dd[j];
         double g = 0.0;
-        if (isfinite(M.hl[j])) {
+        if (fin(M.hl[j])) {
             const double s = I.d[j] - M.hl[j];
             ap = fmin(ap, ftb(s, dd, tau));
             az = fmin(az, ftb(I.vl[j], Dir.dvl[j], tau));
-            g -= mu / s;
+            g -= ddiv(mu, s);
         }
-        if (isfinite(M.hu[j])) {
+        if (fin(M.hu[j])) {
             const double s = M.hu[j] - I.d[j];
             ap = fmin(ap, ftb(s, -dd, tau));
             az = fmin(az, ftb(I.vu[j], Dir.dvu[j], tau));
-            g += mu / s;
+            g += ddiv(mu, s);
         }
         gp += g * dd;
     }
-    double r;
-    r = block_min<NT>(ap, sh); if (threadIdx.x == 0) *slot(partial, 0) = r;
-    r = block_min<NT>(az, sh); if (threadIdx.x == 0) *slot(partial, 1) = r;
-    r = block_sum<NT>(gp, sh); if (threadIdx.x == 0) *slot(partial, 2) = r;
+    double v[3] = {ap, az, gp};
+    reduce_finish<NT, R_MIN, R_MIN, R_SUM>(v, red);
 }
 
 // Trial point x_t = x + alpha dx, d_t = d + alpha dd; sum of log slacks and
@@ -642,19 +609,18 @@ __global__ void __launch_bounds__(NT) k_step_scalars(Dims D, ModelView M, IterVi
 // quantities: 0 sum log s (sum), 1 number of non-positive slacks (sum)
 __global__ void __launch_bounds__(NT) k_trial(Dims D, ModelView M, IterView I, DirView Dir,
                                               double alpha, double *__restrict__ xt,
-                                              double *__restrict__ dt, double *partial) {
-    __shared__ double sh[32];
+                                              double *__restrict__ dt, RedOut red) {
     double lg = 0.0, bad = 0.0;
     const int64_t gtid = (int64_t)blockIdx.x * NT + threadIdx.x;
     const int64_t gsz = (int64_t)gridDim.x * NT;
     for (int64_t i = gtid; i < D.n; i += gsz) {
         const double v = I.x[i] + alpha * Dir.dx[i];
         xt[i] = v;
-        if (isfinite(M.xl[i])) {
+        if (fin(M.xl[i])) {
             const double s = v - M.xl[i];
             if (s > 0.0) lg += log(s); else bad += 1.0;
         }
-        if (isfinite(M.xu[i])) {
+        if (fin(M.xu[i])) {
             const double s = M.xu[i] - v;
             if (s > 0.0) lg += log(s); else bad += 1.0;
         }
@@ -662,18 +628,17 @@ __global__ void __launch_bounds__(NT) k_trial(Dims D, ModelView M, IterView I, D
     for (int64_t j = gtid; j < D.m_I; j += gsz) {
         const double v = I.d[j] + alpha * Dir.dd[j];
         dt[j] = v;
-        if (isfinite(M.hl[j])) {
+        if (fin(M.hl[j])) {
             const double s = v - M.hl[j];
             if (s > 0.0) lg += log(s); else bad += 1.0;
         }
-        if (isfinite(M.hu[j])) {
+        if (fin(M.hu[j])) {
             const double s = M.hu[j] - v;
             if (s > 0.0) lg += log(s); else bad += 1.0;
         }
     }
-    double r;
-    r = block_sum<NT>(lg, sh);  if (threadIdx.x == 0) *slot(partial, 0) = r;
-    r = block_sum<NT>(bad, sh); if (threadIdx.x == 0) *slot(partial, 1) = r;
+    double v[2] = {lg, bad};
+    reduce_finish<NT, R_SUM, R_SUM>(v, red);
 }
 
 // Accept: y += alpha dy, z += alpha_z dz, then the kappa_Sigma safeguard
@@ -682,25 +647,25 @@ __global__ void k_accept(Dims D, ModelView M, IterView I, DirView Dir, double al
                          double alpha_z, double mu, double ks) {
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t gsz = (int64_t)gridDim.x * blockDim.x;
-    auto guard = [&](double z, double s) { return fmax(fmin(z, ks * mu / s), mu / (ks * s)); };
+    auto guard = [&](double z, double s) { return fmax(fmin(z, ddiv(ks * mu, s)), ddiv(mu, ks * s)); };
     for (int64_t i = gtid; i < D.m_E; i += gsz) I.yg[i] += alpha * Dir.dyg[i];
     for (int64_t j = gtid; j < D.m_I; j += gsz) {
         I.yh[j] += alpha * Dir.dyh[j];
         const double dj = I.d[j];
-        if (isfinite(M.hl[j])) I.vl[j] = guard(I.vl[j] + alpha_z * Dir.dvl[j], dj - M.hl[j]);
-        if (isfinite(M.hu[j])) I.vu[j] = guard(I.vu[j] + alpha_z * Dir.dvu[j], M.hu[j] - dj);
+        if (fin(M.hl[j])) I.vl[j] = guard(I.vl[j] + alpha_z * Dir.dvl[j], dj - M.hl[j]);
+        if (fin(M.hu[j])) I.vu[j] = guard(I.vu[j] + alpha_z * Dir.dvu[j], M.hu[j] - dj);
     }
     for (int64_t i = gtid; i < D.n; i += gsz) {
         const double xi = I.x[i];
-        if (isfinite(M.xl[i])) I.zl[i] = guard(I.zl[i] + alpha_z * Dir.dzl[i], xi - M.xl[i]);
-        if (isfinite(M.xu[i])) I.zu[i] = guard(I.zu[i] + alpha_z * Dir.dzu[i], M.xu[i] - xi);
+        if (fin(M.xl[i])) I.zl[i] = guard(I.zl[i] + alpha_z * Dir.dzl[i], xi - M.xl[i]);
+        if (fin(M.xu[i])) I.zu[i] = guard(I.zu[i] + alpha_z * Dir.dzu[i], M.xu[i] - xi);
     }
 }
 
 // W&B Section 3.6 starting point: push x0 (and d0 = h(x0)) inside the bounds;
 // multipliers of finite bounds 1, y = 0.
 __device__ double push_inside(double v, double lo, double hi, double k1, double k2) {
-    const bool hl = isfinite(lo), hu = isfinite(hi);
+    const bool hl = fin(lo), hu = fin(hi);
     const double width = (hl && hu) ? hi - lo : INFINITY;
     if (hl) {
         const double pl = fmin(k1 * fmax(1.0, fabs(lo)), k2 * width);
@@ -719,15 +684,15 @@ __global__ void k_init_x(Dims D, ModelView M, const double *__restrict__ x0, dou
     const int64_t gsz = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = gtid; i < D.n; i += gsz) {
         I.x[i] = push_inside(x0 ? x0[i] : 0.0, M.xl[i], M.xu[i], k1, k2);
-        I.zl[i] = isfinite(M.xl[i]) ? 1.0 : 0.0;
-        I.zu[i] = isfinite(M.xu[i]) ? 1.0 : 0.0;
+        I.zl[i] = fin(M.xl[i]) ? 1.0 : 0.0;
+        I.zu[i] = fin(M.xu[i]) ? 1.0 : 0.0;
     }
     for (int64_t i = gtid; i < D.m_E; i += gsz) I.yg[i] = 0.0;
     for (int64_t j = gtid; j < D.m_I; j += gsz) {
         I.yh[j] = 0.0;
         I.d[j] = 0.0;
-        I.vl[j] = isfinite(M.hl[j]) ? 1.0 : 0.0;
-        I.vu[j] = isfinite(M.hu[j]) ? 1.0 : 0.0;
+        I.vl[j] = fin(M.hl[j]) ? 1.0 : 0.0;
+        I.vu[j] = fin(M.hu[j]) ? 1.0 : 0.0;
     }
 }
 
@@ -754,8 +719,8 @@ __global__ void k_start_predicted(Dims D, ModelView M, const float *__restrict__
         const double lo = M.xl[i], hi = M.xu[i];
         const double x = push_inside((double)pred[i], lo, hi, push, push);
         I.x[i] = x;
-        I.zl[i] = isfinite(lo) ? fmax((double)pred[o_zl + i], mu0 / (x - lo)) : 0.0;
-        I.zu[i] = isfinite(hi) ? fmax((double)pred[o_zu + i], mu0 / (hi - x)) : 0.0;
+        I.zl[i] = fin(lo) ? fmax((double)pred[o_zl + i], mu0 / (x - lo)) : 0.0;
+        I.zu[i] = fin(hi) ? fmax((double)pred[o_zu + i], mu0 / (hi - x)) : 0.0;
     }
     for (int64_t i = gtid; i < D.m_E; i += gsz) I.yg[i] = (double)pred[o_yg + i];
     for (int64_t j = gtid; j < D.m_I; j += gsz) {
@@ -763,16 +728,15 @@ __global__ void k_start_predicted(Dims D, ModelView M, const float *__restrict__
         const double d = push_inside((double)pred[o_d + j], lo, hi, push, push);
         I.d[j] = d;
         I.yh[j] = (double)pred[o_yh + j];
-        I.vl[j] = isfinite(lo) ? fmax((double)pred[o_vl + j], mu0 / (d - lo)) : 0.0;
-        I.vu[j] = isfinite(hi) ? fmax((double)pred[o_vu + j], mu0 / (hi - d)) : 0.0;
+        I.vl[j] = fin(lo) ? fmax((double)pred[o_vl + j], mu0 / (d - lo)) : 0.0;
+        I.vu[j] = fin(hi) ? fmax((double)pred[o_vu + j], mu0 / (hi - d)) : 0.0;
     }
 }
 
 __global__ void __launch_bounds__(NT) k_cons_from_values(Dims D, ModelView M, const double *__restrict__ g,
                                                          const double *__restrict__ h, const double *__restrict__ d,
                                                          double *__restrict__ cg, double *__restrict__ ch,
-                                                         double *partial) {
-    __shared__ double sh[32];
+                                                         RedOut red) {
     double s1 = 0.0, mx = 0.0;
     const int64_t gtid = (int64_t)blockIdx.x * NT + threadIdx.x, gsz = (int64_t)gridDim.x * NT;
     for (int64_t i = gtid; i < D.m_E; i += gsz) {
@@ -787,10 +751,8 @@ __global__ void __launch_bounds__(NT) k_cons_from_values(Dims D, ModelView M, co
         s1 += fabs(r);
         mx = fmax(mx, fabs(r));
     }
-    const double a = block_sum<NT>(s1, sh);
-    if (threadIdx.x == 0) *slot(partial, 0) = a;
-    const double b = block_max<NT>(mx, sh);
-    if (threadIdx.x == 0) *slot(partial, 1) = b;
+    double v[2] = {s1, mx};
+    reduce_finish<NT, R_SUM, R_MAX>(v, red);
 }
 
 __global__ void k_gather(int64_t n, const double *__restrict__ src, const int32_t *__restrict__ idx,
@@ -804,19 +766,6 @@ __global__ void k_gather(int64_t n, const double *__restrict__ src, const int32_
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-void launch_finalize_sum(cudaStream_t s, const double *partial, int nq, double *out) {
-    k_finalize<<<nq, 32, 0, s>>>(partial, nq, out, 0);
-    MDSIP_LAUNCHED();
-}
-void launch_finalize_max(cudaStream_t s, const double *partial, int nq, double *out) {
-    k_finalize<<<nq, 32, 0, s>>>(partial, nq, out, 1);
-    MDSIP_LAUNCHED();
-}
-void launch_finalize_min(cudaStream_t s, const double *partial, int nq, double *out) {
-    k_finalize<<<nq, 32, 0, s>>>(partial, nq, out, 2);
-    MDSIP_LAUNCHED();
-}
-
 static int elem_grid(int64_t n) { return std::max(1, std::min(4096, ceil_div(n, 256))); }
 
 // A: rows 16-byte aligned (lda even, A 16-byte aligned); n <= 24560 (v staged in shared memory)
@@ -850,16 +799,21 @@ void launch_gemv_t(cudaStream_t s, const double *A, int64_t m, int64_t n, int64_
         MDSIP_CUDA(cudaMemsetAsync(out, 0, n * sizeof(double), s));
         return;
     }
-    k_gemv_t<<<kRedBlocks, NT, 0, s>>>(A, m, n, lda, u, partial);
+    // threads over columns first; with fewer than NT columns the rest of the block takes further rows
+    int tc = 32;
+    while (tc < NT && tc < n) tc *= 2;
+    const int grid = (int)std::min<int64_t>(kRedBlocks, ceil_div(m, (int64_t)8 * (NT / tc)));
+    if (n <= NT) k_gemv_t<1, 8><<<grid, NT, 0, s>>>(A, m, n, lda, u, tc, partial);
+    else if (n <= 2 * NT) k_gemv_t<2, 6><<<grid, NT, 0, s>>>(A, m, n, lda, u, tc, partial);
+    else k_gemv_t<4, 3><<<grid, NT, 0, s>>>(A, m, n, lda, u, tc, partial);
     MDSIP_LAUNCHED();
-    k_colsum<<<(unsigned)ceil_div(n, 32), 256, 0, s>>>(partial, kRedBlocks, n, out);
+    k_colsum<<<(unsigned)ceil_div(n, 32), 256, 0, s>>>(partial, grid, n, out);
     MDSIP_LAUNCHED();
 }
 
 void VecOps::eval_f(const double *x, double *grad, double *out_scalar) {
-    k_eval_f<<<kRedBlocks, NT, 0, st>>>(D, M, x, grad, partial);
+    k_eval_f<<<red_grid(std::max(D.n_s, 32 * D.n_d)), NT, 0, st>>>(D, M, x, grad, red(out_scalar));
     MDSIP_LAUNCHED();
-    launch_finalize_sum(st, partial, 1, out_scalar);
 }
 
 void VecOps::eval_cons(const double *x, const double *d, double *cg, double *ch, double *out2) {
@@ -867,18 +821,14 @@ void VecOps::eval_cons(const double *x, const double *d, double *cg, double *ch,
         if (Ahi) launch_gemv_rows_df(st, Ahi, Alo, D.m_E, D.n_d, D.lda, x + D.n_s, split, rowtmp);
         else launch_gemv_rows(st, M.A, D.m_E, D.n_d, D.lda, x + D.n_s, rowtmp);
     }
-    k_eval_cons<<<kRedBlocks, NT, 0, st>>>(D, M, x, rowtmp, d, cg, ch, partial);
+    k_eval_cons<<<red_grid(std::max(D.m_E, 32 * D.m_I)), NT, 0, st>>>(D, M, x, rowtmp, d, cg, ch, red(out2));
     MDSIP_LAUNCHED();
-    launch_finalize_sum(st, partial, 1, out2);
-    launch_finalize_max(st, partial + kRedBlocks, 1, out2 + 1);
 }
 
 void VecOps::eval_cons_ax(const double *x, const double *Ax, const double *d, double *cg, double *ch,
                           double *out2) {
-    k_eval_cons<<<kRedBlocks, NT, 0, st>>>(D, M, x, Ax, d, cg, ch, partial);
+    k_eval_cons<<<red_grid(std::max(D.m_E, 32 * D.m_I)), NT, 0, st>>>(D, M, x, Ax, d, cg, ch, red(out2));
     MDSIP_LAUNCHED();
-    launch_finalize_sum(st, partial, 1, out2);
-    launch_finalize_max(st, partial + kRedBlocks, 1, out2 + 1);
 }
 
 namespace {
@@ -904,33 +854,29 @@ void VecOps::lagrangian_grad(const IterView &I, const double *grad, const double
                              double *gl) {
     if (Ahi) launch_gemv_t_df(st, Ahi, Alo, D.m_E, D.n_d, D.lda, I.yg, split, colpart, ATy);
     else launch_gemv_t(st, M.A, D.m_E, D.n_d, D.lda, I.yg, colpart, ATy);
-    k_lagrangian_grad<<<elem_grid(std::max(D.n_s, D.n_d)), 256, 0, st>>>(D, M, grad, I.yg, I.yh, Jdh,
+    k_lagrangian_grad<<<elem_grid(std::max(D.n_s, (NT / 32) * D.n_d)), NT, 0, st>>>(D, M, grad, I.yg, I.yh, Jdh,
                                                                          ATy, gl);
     MDSIP_LAUNCHED();
 }
 
 void VecOps::lagrangian_grad_aty(const IterView &I, const double *grad, const double *Jdh, const double *ATy,
                                  double *gl) {
-    k_lagrangian_grad<<<elem_grid(std::max(D.n_s, D.n_d)), 256, 0, st>>>(D, M, grad, I.yg, I.yh, Jdh,
+    k_lagrangian_grad<<<elem_grid(std::max(D.n_s, (NT / 32) * D.n_d)), NT, 0, st>>>(D, M, grad, I.yg, I.yh, Jdh,
                                                                          ATy, gl);
     MDSIP_LAUNCHED();
 }
 
 void VecOps::errors(const IterView &I, const double *gl, const double *cg, const double *ch,
                     double *out7) {
-    k_errors<<<kRedBlocks, NT, 0, st>>>(D, M, I, gl, cg, ch, partial);
+    k_errors<<<red_grid(std::max(D.n, D.m_E)), NT, 0, st>>>(D, M, I, gl, cg, ch, red(out7));
     MDSIP_LAUNCHED();
-    launch_finalize_max(st, partial, 3, out7);                       // 0,1,2
-    launch_finalize_min(st, partial + 3 * kRedBlocks, 1, out7 + 3);  // 3
-    launch_finalize_sum(st, partial + 4 * kRedBlocks, 3, out7 + 4);  // 4,5,6
 }
 
 void VecOps::newton_diag(const IterView &I, const double *Hss, double dw, double dc, bool want_w,
                          double *sig_x, double *q, double *sig_d, double *w, double *out6) {
-    k_newton_diag<<<kRedBlocks, NT, 0, st>>>(D, M, I, Hss, dw, dc, want_w ? 1 : 0, sig_x, q, sig_d, w,
-                                             partial);
+    k_newton_diag<<<red_grid(std::max(D.n, D.m_E)), NT, 0, st>>>(D, M, I, Hss, dw, dc, want_w ? 1 : 0, sig_x, q, sig_d,
+                                                                 w, red(out6));
     MDSIP_LAUNCHED();
-    launch_finalize_sum(st, partial, 6, out6);
 }
 
 void VecOps::rhs_y(const IterView &I, const double *gl, const double *cg, const double *q,
@@ -967,17 +913,14 @@ void VecOps::backsub(const IterView &I, const DirView &Dir, const double *gl, co
 
 void VecOps::step_scalars(const IterView &I, const DirView &Dir, const double *grad, double tau,
                           double mu, double *out3) {
-    k_step_scalars<<<kRedBlocks, NT, 0, st>>>(D, M, I, Dir, grad, tau, mu, partial);
+    k_step_scalars<<<red_grid(D.n), NT, 0, st>>>(D, M, I, Dir, grad, tau, mu, red(out3));
     MDSIP_LAUNCHED();
-    launch_finalize_min(st, partial, 2, out3);
-    launch_finalize_sum(st, partial + 2 * kRedBlocks, 1, out3 + 2);
 }
 
 void VecOps::trial(const IterView &I, const DirView &Dir, double alpha, double *xt, double *dt,
                    double *out2) {
-    k_trial<<<kRedBlocks, NT, 0, st>>>(D, M, I, Dir, alpha, xt, dt, partial);
+    k_trial<<<red_grid(D.n), NT, 0, st>>>(D, M, I, Dir, alpha, xt, dt, red(out2));
     MDSIP_LAUNCHED();
-    launch_finalize_sum(st, partial, 2, out2);
 }
 
 void VecOps::accept(const IterView &I, const DirView &Dir, double alpha, double alpha_z, double mu,
@@ -1003,16 +946,13 @@ void VecOps::start_predicted(const float *pred, double push, double mu0, const I
 
 void VecOps::cons_from_values(const double *g, const double *h, const double *d, double *cg, double *ch,
                               double *out2) {
-    k_cons_from_values<<<kRedBlocks, NT, 0, st>>>(D, M, g, h, d, cg, ch, partial);
+    k_cons_from_values<<<red_grid(D.m_E), NT, 0, st>>>(D, M, g, h, d, cg, ch, red(out2));
     MDSIP_LAUNCHED();
-    launch_finalize_sum(st, partial, 1, out2);
-    launch_finalize_max(st, partial + kRedBlocks, 1, out2 + 1);
 }
 
 void VecOps::dir_diff(const DirView &a, const DirView &b, double *out2) {
-    k_dir_diff<<<kRedBlocks, NT, 0, st>>>(D, a, b, partial);
+    k_dir_diff<<<red_grid(D.n), NT, 0, st>>>(D, a, b, red(out2));
     MDSIP_LAUNCHED();
-    launch_finalize_sum(st, partial, 2, out2);
 }
 
 void VecOps::copy_dir(const DirView &src, const DirView &dst) {

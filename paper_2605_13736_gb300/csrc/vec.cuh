@@ -12,7 +12,8 @@ struct DirView {
     double *dx, *dd, *dyg, *dyh, *dzl, *dzu, *dvl, *dvu;
 };
 
-// All launches on one stream; `partial` holds kRedBlocks x 8 doubles and
+// All launches on one stream; `partial` holds kRedBlocks x 8 doubles, then the
+// reductions' ticket (zero between kernels), and
 // `colpart` kRedBlocks x n_d doubles of reduction scratch, `rowtmp` m_E doubles.
 struct VecOps {
     Dims D;
@@ -26,6 +27,8 @@ struct VecOps {
     // null on the plain FP64 path
     const float *Ahi = nullptr, *Alo = nullptr;
     float2 *split = nullptr;
+
+    RedOut red(double *out) const { return RedOut{partial, reinterpret_cast<unsigned *>(partial + kRedBlocks * 8), out}; }
 
     void eval_f(const double *x, double *grad, double *out_scalar);
     void eval_cons(const double *x, const double *d, double *cg, double *ch, double *out2);
