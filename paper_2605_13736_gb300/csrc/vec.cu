@@ -168,7 +168,9 @@ __global__ void __launch_bounds__(NT) k_gemv_rows(const double *__restrict__ A, 
 // power of two) take the columns, C each, and the block's NT / tc groups its
 // rows, U in flight: 8 to 12 loads a thread cover the memory's latency (m =
 // 15053, n = 301: 54 us with one row pair in flight and 8 columns per thread of
-// which two were used, 21 us so; m = 1000, n = 32: 8 -> 6 us).
+// which two were used, 20 us so; m = 1000, n = 32: 8 -> 6 us).  Above 1024
+// columns eight a thread stay: bound by the FP64 pipe, fewer columns repeat the
+// row's addresses (m = 100000, n = 2000: 363 us, with four columns 467).
 template <int C, int U>
 __global__ void __launch_bounds__(NT) k_gemv_t(const double *__restrict__ A, int64_t m, int64_t n,
                                                int64_t lda, const double *__restrict__ u, int tc,
@@ -182,23 +184,51 @@ __global__ void __launch_bounds__(NT) k_gemv_t(const double *__restrict__ A, int
         double acc[C];
 #pragma unroll
         for (int c = 0; c < C; ++c) acc[c] = 0.0;
-        for (int64_t i = r0 + g; i < r1; i += (int64_t)U * G) {
+        int64_t i = r0 + g;
+        if constexpr (C <= 2)                  // few rows a thread: the last batch stays whole
+            for (; i < r1; i += (int64_t)U * G) {
+                double a[U][C], ui[U];
+#pragma unroll
+                for (int x = 0; x < U; ++x) {
+                    const int64_t r = i + (int64_t)x * G;
+                    ui[x] = r < r1 ? __ldg(u + r) : 0.0;
+#pragma unroll
+                    for (int c = 0; c < C; ++c) {
+                        const int64_t p = c0 + col + (int64_t)c * tc;
+                        a[x][c] = r < r1 && p < n ? __ldg(A + r * lda + p) : 0.0;
+                    }
+                }
+#pragma unroll
+                for (int x = 0; x < U; ++x)
+                    if (i + (int64_t)x * G < r1)
+#pragma unroll
+                        for (int c = 0; c < C; ++c) acc[c] = fma(a[x][c], ui[x], acc[c]);
+            }
+        for (; i + (int64_t)(U - 1) * G < r1; i += (int64_t)U * G) {
             double a[U][C], ui[U];
 #pragma unroll
             for (int x = 0; x < U; ++x) {
-                const int64_t r = i + (int64_t)x * G;
-                ui[x] = r < r1 ? __ldg(u + r) : 0.0;
+                const double *row = A + (i + (int64_t)x * G) * lda;
+                ui[x] = __ldg(u + i + (int64_t)x * G);
 #pragma unroll
                 for (int c = 0; c < C; ++c) {
                     const int64_t p = c0 + col + (int64_t)c * tc;
-                    a[x][c] = r < r1 && p < n ? __ldg(A + r * lda + p) : 0.0;
+                    a[x][c] = p < n ? __ldg(row + p) : 0.0;
                 }
             }
 #pragma unroll
             for (int x = 0; x < U; ++x)
-                if (i + (int64_t)x * G < r1)
 #pragma unroll
-                    for (int c = 0; c < C; ++c) acc[c] = fma(a[x][c], ui[x], acc[c]);
+                for (int c = 0; c < C; ++c) acc[c] = fma(a[x][c], ui[x], acc[c]);
+        }
+        for (; i < r1; i += G) {
+            const double *row = A + i * lda;
+            const double ui = __ldg(u + i);
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                const int64_t p = c0 + col + (int64_t)c * tc;
+                if (p < n) acc[c] = fma(__ldg(row + p), ui, acc[c]);
+            }
         }
 #pragma unroll
         for (int c = 0; c < C; ++c) {
@@ -805,7 +835,8 @@ void launch_gemv_t(cudaStream_t s, const double *A, int64_t m, int64_t n, int64_
     const int grid = (int)std::min<int64_t>(kRedBlocks, ceil_div(m, (int64_t)8 * (NT / tc)));
     if (n <= NT) k_gemv_t<1, 8><<<grid, NT, 0, s>>>(A, m, n, lda, u, tc, partial);
     else if (n <= 2 * NT) k_gemv_t<2, 6><<<grid, NT, 0, s>>>(A, m, n, lda, u, tc, partial);
-    else k_gemv_t<4, 3><<<grid, NT, 0, s>>>(A, m, n, lda, u, tc, partial);
+    else if (n <= 4 * NT) k_gemv_t<4, 3><<<grid, NT, 0, s>>>(A, m, n, lda, u, tc, partial);
+    else k_gemv_t<8, 2><<<grid, NT, 0, s>>>(A, m, n, lda, u, tc, partial);
     MDSIP_LAUNCHED();
     k_colsum<<<(unsigned)ceil_div(n, 32), 256, 0, s>>>(partial, grid, n, out);
     MDSIP_LAUNCHED();
