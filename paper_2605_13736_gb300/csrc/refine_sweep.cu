@@ -1,0 +1,639 @@
+// One sweep of the iterative refinement in one read of A (path P2, FP32 tiles
+// of a tensor-core factor, n_d <= 4096).
+//
+// A sweep solves S~ sol = rhs, completes the correction on the eliminated rows
+// and columns, adds it to u and forms the residual b - K u and the first half
+// of the next approximate solve.  Written out per equality row i (P2: every
+// sparse column has at most one row, so all of it is the row's own):
+//
+//   sol_g,i = ((A_hi sol_d)_i - bt_i) / w_i          FP32 row product
+//   u_g,i += sol_g,i
+//   u_c   += (r_c - J_ic sol_g,i) / q_c              the row's sparse columns c
+//   (A u_d)_i                                        double-float row product
+//   bt_i   = b_i + dc u_g,i - sum J_ic u_c - sum J_ic (b_c - q_c u_c - J_ic u_g,i) / q_c - (A u_d)_i
+//   A^T u_g                                          double-float column product
+//   A_hi^T (bt / w)                                  FP32 column product
+//
+// Both row products need only sol_d and u_d, known before the pass; both
+// column products need the row's own results.  So a batch of rows stays in
+// shared memory between its two halves and A_hi, A_lo are read once a sweep, 8
+// bytes per entry (12 in the separate passes, with ten small launches more
+// around them).  A sweep's passes at m = 100000, n = 2000: 361 + 164 us apart,
+// 445 in one; m = 200000, n = 4000: 1275 + 800 + 498 apart, 1600; m = 25600,
+// n = 512: 78 + 23 apart, 43.
+#include "df.cuh"
+#include "internal.cuh"
+#include "refine.cuh"
+#include "tc.cuh"
+
+namespace mdsip {
+
+namespace {
+
+constexpr int NT = kRedThreads;
+constexpr int kSwC = 512;                     // column threads: 16 warps
+constexpr int kSwMaxSlots = 12;
+constexpr size_t kSwRing = 222 * 1024;        // half-batches in flight or in use
+constexpr size_t kSwMin = 48 * 1024;          // the groups' column sums meet in the ring at the end
+
+struct SweepArgs {
+    const float *Ahi, *Alo;
+    int64_t m, lda;
+    int n, T, S;           // columns, threads per row, half-batches of the ring
+    const float4 *xq;      // per column: u_d split (x, y), fl32(sol_d) (z)
+    const double *b_g, *winv;
+    const float *wf;
+    double *u_g, *bt, *sol_g, *Au;
+    double dc;
+    const int *csr_ptr, *csr_col;
+    const double *csr_val, *b_s, *u_s, *r_s, *q, *qinv;
+    int init;              // u = 0 and r = b before this sweep
+    double *pu;            // partial sums of A^T u_g, a row per CTA
+    float *pv;             // and of A_hi^T (bt / w)
+    int *err;
+};
+
+// the sparse column's new u_s: the same bits wherever it is formed
+__device__ __forceinline__ double new_us(double u, double r, double J, double sol, double qinv) {
+    return fma(fma(-J, sol, r), qinv, u);
+}
+
+// Warps 0 .. 15 compute, warp 16 loads, warps 17 .. finish rows.  T threads
+// (32 .. 512) take a row's columns, 4 CH each; the 512 / T groups take KBR rows
+// of a batch each, so a batch is about 64 KB at any width.  It comes as two
+// half-batches, each one bulk copy of A_hi and one of A_lo (the rows are
+// contiguous).  Per batch: row products, warp sums to shared memory, the
+// finishing warps' scalars in FP64, and one batch later, with the finished
+// rows, the column products.  Only mbarriers: no warp waits for the finishing
+// warps until it has done the next batch's row products.  Waits are bounded.
+template <int CH, int KBR>
+__global__ void __launch_bounds__(CH == 1 ? 608 : 576, 1) k_sweep(SweepArgs a) {
+    extern __shared__ __align__(128) unsigned char sw_smem[];
+    constexpr int NTW = KBR / 2;               // finishing warps: KBR * 16 / 32
+    constexpr int kVals = KBR * 16;            // (row, warp) sums of a batch
+    __shared__ float4 s_red[2][kVals];
+    __shared__ float4 s_y[2][kVals];
+    __shared__ __align__(8) uint64_t full[kSwMaxSlots], empty[kSwMaxSlots], rowdone[2], rowready[2];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int T = a.T, W = T / 32, G = kSwC / T, HR = G * KBR / 2, RB = G * KBR, S = a.S;
+    const int64_t lda = a.lda;
+    const size_t slot_bytes = (size_t)2 * HR * lda * sizeof(float);
+    const int64_t rows_per = (a.m + gridDim.x - 1) / gridDim.x;
+    const int64_t r0 = (int64_t)blockIdx.x * rows_per;
+    const int64_t r1 = min(a.m, r0 + rows_per);
+    const int nbat = r1 > r0 ? (int)((r1 - r0 + RB - 1) / RB) : 0;
+    if (tid == 0) {
+        for (int i = 0; i < S; ++i) {
+            tc::mbar_init(&full[i], 1);
+            tc::mbar_init(&empty[i], 16);
+        }
+        for (int i = 0; i < 2; ++i) {
+            tc::mbar_init(&rowdone[i], 16);
+            tc::mbar_init(&rowready[i], NTW);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    bool ok = true;
+    if (wid < 16) {
+        const int g = tid / T, t = tid - g * T, w = t >> 5;
+        float2 xh[2 * CH], xl[2 * CH], xs[2 * CH];
+        bool on[CH];
+#pragma unroll
+        for (int ch = 0; ch < CH; ++ch) {
+            const int p0 = 4 * t + ch * 4 * T;
+            on[ch] = p0 < a.n;
+            float4 v[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] = p0 + q < a.n ? __ldg(a.xq + p0 + q) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                xh[2 * ch + h] = make_float2(v[2 * h].x, v[2 * h + 1].x);
+                xl[2 * ch + h] = make_float2(v[2 * h].y, v[2 * h + 1].y);
+                xs[2 * ch + h] = make_float2(v[2 * h].z, v[2 * h + 1].z);
+            }
+        }
+        // column sums: a double-float pair per 16 rows, added into a second pair,
+        // which goes into FP64 every 256 rows (the FP64 pipe: 1/64 of the FP32 rate)
+        const float2 z2 = make_float2(0.0f, 0.0f);
+        float2 cs[2 * CH], cc[2 * CH], CS[2 * CH], CC[2 * CH], cv[2 * CH];
+        double cacc[CH == 1 ? 4 : 1] = {};
+        bool flushed = false;
+#pragma unroll
+        for (int j = 0; j < 2 * CH; ++j) cs[j] = cc[j] = CS[j] = CC[j] = cv[j] = z2;
+        int cnt = 0, cnt2 = 0;
+        int rslot = 0, cslot = 0;
+        uint32_t rph = 0;
+        for (int b = 0; b <= nbat; ++b) {
+            if (!__all_sync(0xffffffffu, ok)) break;   // a wait ran out: the whole warp stops
+            if (b < nbat) {   // ---- row products of batch b
+                float rs[KBR], rc[KBR], r2[KBR];
+                const int64_t i0 = r0 + (int64_t)b * RB;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    if (!tc::mbar_wait(&full[rslot], rph)) ok = false;
+                    const float *base = reinterpret_cast<const float *>(sw_smem + (size_t)rslot * slot_bytes);
+#pragma unroll
+                    for (int k = 0; k < KBR / 2; ++k) {
+                        const int rr = h * (KBR / 2) + k, rho = g * (KBR / 2) + k;
+                        float2 ps = z2, pc = z2, p2 = z2;
+                        if (i0 + h * HR + rho < r1) {
+                            const float *row = base + rho * lda + 4 * t;
+#pragma unroll
+                            for (int ch = 0; ch < CH; ++ch)
+                                if (on[ch]) {
+                                    const float4 ah = *reinterpret_cast<const float4 *>(row + ch * 4 * T);
+                                    const float4 al = *reinterpret_cast<const float4 *>(row + HR * lda + ch * 4 * T);
+                                    const float2 h0 = make_float2(ah.x, ah.y), h1 = make_float2(ah.z, ah.w);
+                                    df_acc2(h0, make_float2(al.x, al.y), xh[2 * ch], xl[2 * ch], ps, pc);
+                                    df_acc2(h1, make_float2(al.z, al.w), xh[2 * ch + 1], xl[2 * ch + 1], ps, pc);
+                                    p2 = __ffma2_rn(h0, xs[2 * ch], p2);
+                                    p2 = __ffma2_rn(h1, xs[2 * ch + 1], p2);
+                                }
+                        }
+                        rs[rr] = ps.x;
+                        rc[rr] = pc.x;
+                        df_add(rs[rr], rc[rr], ps.y, pc.y);
+                        r2[rr] = p2.x + p2.y;
+                    }
+                    if (++rslot == S) rslot = 0, rph ^= 1;
+                }
+                // the rows' sums over the warp by halving exchanges, then a butterfly
+                const bool u16 = (lane & 16) != 0, u8 = (lane & 8) != 0;
+                auto xch = [&](int o, bool up, int keep_lo, int keep_hi, float &s, float &c, float &d) {
+                    float es = up ? rs[keep_lo] : rs[keep_hi], ec = up ? rc[keep_lo] : rc[keep_hi];
+                    float ed = up ? r2[keep_lo] : r2[keep_hi];
+                    s = up ? rs[keep_hi] : rs[keep_lo];
+                    c = up ? rc[keep_hi] : rc[keep_lo];
+                    d = up ? r2[keep_hi] : r2[keep_lo];
+                    es = __shfl_xor_sync(0xffffffffu, es, o);
+                    ec = __shfl_xor_sync(0xffffffffu, ec, o);
+                    d += __shfl_xor_sync(0xffffffffu, ed, o);
+                    df_add(s, c, es, ec);
+                };
+                float s, c, d;
+                int rho;
+                bool lead;
+                if constexpr (KBR == 4) {
+                    float s0, c0, d0, s1, c1, d1;
+                    xch(16, u16, 0, 2, s0, c0, d0);
+                    xch(16, u16, 1, 3, s1, c1, d1);
+                    float es = u8 ? s0 : s1, ec = u8 ? c0 : c1, ed = u8 ? d0 : d1;
+                    s = u8 ? s1 : s0;
+                    c = u8 ? c1 : c0;
+                    d = u8 ? d1 : d0;
+                    es = __shfl_xor_sync(0xffffffffu, es, 8);
+                    ec = __shfl_xor_sync(0xffffffffu, ec, 8);
+                    d += __shfl_xor_sync(0xffffffffu, ed, 8);
+                    df_add(s, c, es, ec);
+                    rho = (u16 ? HR : 0) + 2 * g + (u8 ? 1 : 0);
+                    lead = (lane & 7) == 0;
+                } else {
+                    xch(16, u16, 0, 1, s, c, d);
+                    rho = (u16 ? HR : 0) + g;
+                    lead = (lane & 15) == 0;
+                }
+#pragma unroll
+                for (int o = KBR == 4 ? 4 : 8; o > 0; o >>= 1) {
+                    const float es = __shfl_xor_sync(0xffffffffu, s, o), ec = __shfl_xor_sync(0xffffffffu, c, o);
+                    d += __shfl_xor_sync(0xffffffffu, d, o);
+                    df_add(s, c, es, ec);
+                }
+                if (lead) s_red[b & 1][rho * W + w] = make_float4(s, c, d, 0.0f);
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&rowdone[b & 1]);
+            }
+            if (b == 0) continue;
+            // ---- column products of batch b - 1
+            const int e = b - 1;
+            const int64_t i0 = r0 + (int64_t)e * RB;
+            if (!tc::mbar_wait(&rowready[e & 1], (uint32_t)(e >> 1) & 1)) ok = false;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const float *base = reinterpret_cast<const float *>(sw_smem + (size_t)cslot * slot_bytes);
+#pragma unroll
+                for (int k = 0; k < KBR / 2; ++k) {
+                    const int rho = g * (KBR / 2) + k;
+                    if (i0 + h * HR + rho >= r1) continue;
+                    const float4 y = s_y[e & 1][h * HR + rho];
+                    const float2 yh = make_float2(y.x, y.x), yl = make_float2(y.y, y.y), yv = make_float2(y.z, y.z);
+                    const float *row = base + rho * lda + 4 * t;
+#pragma unroll
+                    for (int ch = 0; ch < CH; ++ch)
+                        if (on[ch]) {
+                            const float4 ah = *reinterpret_cast<const float4 *>(row + ch * 4 * T);
+                            const float4 al = *reinterpret_cast<const float4 *>(row + HR * lda + ch * 4 * T);
+                            const float2 h0 = make_float2(ah.x, ah.y), h1 = make_float2(ah.z, ah.w);
+                            df_acc2(h0, make_float2(al.x, al.y), yh, yl, cs[2 * ch], cc[2 * ch]);
+                            df_acc2(h1, make_float2(al.z, al.w), yh, yl, cs[2 * ch + 1], cc[2 * ch + 1]);
+                            cv[2 * ch] = __ffma2_rn(h0, yv, cv[2 * ch]);
+                            cv[2 * ch + 1] = __ffma2_rn(h1, yv, cv[2 * ch + 1]);
+                        }
+                }
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&empty[cslot]);
+                if (++cslot == S) cslot = 0;
+            }
+            if (++cnt == 16 / KBR) {   // every 16 rows
+                cnt = 0;
+#pragma unroll
+                for (int j = 0; j < 2 * CH; ++j) {
+                    df_add(CS[j].x, CC[j].x, cs[j].x, cc[j].x);
+                    df_add(CS[j].y, CC[j].y, cs[j].y, cc[j].y);
+                    cs[j] = cc[j] = z2;
+                }
+                if (++cnt2 == 16) {   // every 256 rows
+                    cnt2 = 0;
+                    if constexpr (CH == 1) {
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const float2 A = CS[q >> 1], B = CC[q >> 1];
+                            cacc[q] += (double)(q & 1 ? A.y : A.x) + (double)(q & 1 ? B.y : B.x);
+                        }
+                    } else {   // one group: this thread's columns of the CTA's partial row
+#pragma unroll
+                        for (int q = 0; q < 4 * CH; ++q) {
+                            const int p = 4 * t + (q >> 2) * 4 * T + (q & 3);
+                            const float2 A = CS[q >> 1], B = CC[q >> 1];
+                            const double v = (double)(q & 1 ? A.y : A.x) + (double)(q & 1 ? B.y : B.x);
+                            double *at = a.pu + (size_t)blockIdx.x * a.n + p;
+                            if (p < a.n) *at = flushed ? *at + v : v;
+                        }
+                    }
+                    flushed = true;
+#pragma unroll
+                    for (int j = 0; j < 2 * CH; ++j) CS[j] = CC[j] = z2;
+                }
+            }
+        }
+        if (!ok) atomicExch(a.err, 1);
+#pragma unroll
+        for (int j = 0; j < 2 * CH; ++j) {
+            df_add(CS[j].x, CC[j].x, cs[j].x, cc[j].x);
+            df_add(CS[j].y, CC[j].y, cs[j].y, cc[j].y);
+        }
+        if constexpr (CH == 1) {
+            if (G > 1) {   // the groups' sums meet in shared memory, group 0 adds them up in order
+                asm volatile("bar.sync 1, 512;" ::: "memory");   // every warp is through with the ring
+                float4 *gp = reinterpret_cast<float4 *>(sw_smem);            // [2][512]: pairs of columns
+                float4 *gv = gp + 2 * kSwC;                                  // [512]
+                double *ga = reinterpret_cast<double *>(gv + kSwC);          // [512][4]
+                gp[tid] = make_float4(CS[0].x, CC[0].x, CS[0].y, CC[0].y);
+                gp[kSwC + tid] = make_float4(CS[1].x, CC[1].x, CS[1].y, CC[1].y);
+                gv[tid] = make_float4(cv[0].x, cv[0].y, cv[1].x, cv[1].y);
+                if (flushed)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) ga[4 * tid + q] = cacc[q];
+                asm volatile("bar.sync 1, 512;" ::: "memory");
+                if (g == 0)
+                    for (int x = 1; x < G; ++x) {
+                        const int o = x * T + t;
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) {
+                            const float4 v = gp[j * kSwC + o];
+                            df_add(CS[j].x, CC[j].x, v.x, v.y);
+                            df_add(CS[j].y, CC[j].y, v.z, v.w);
+                        }
+                        const float4 v = gv[o];
+                        cv[0] = make_float2(cv[0].x + v.x, cv[0].y + v.y);
+                        cv[1] = make_float2(cv[1].x + v.z, cv[1].y + v.w);
+                        if (flushed)
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) cacc[q] += ga[4 * o + q];
+                    }
+            }
+        }
+        if (g == 0)
+#pragma unroll
+            for (int q = 0; q < 4 * CH; ++q) {
+                const int p = 4 * t + (q >> 2) * 4 * T + (q & 3);
+                if (p >= a.n) continue;
+                const float2 A = CS[q >> 1], B = CC[q >> 1], V = cv[q >> 1];
+                double v = (double)(q & 1 ? A.y : A.x) + (double)(q & 1 ? B.y : B.x);
+                const size_t at = (size_t)blockIdx.x * a.n + p;
+                if (flushed) {
+                    if constexpr (CH == 1) v += cacc[q];
+                    else v += a.pu[at];
+                }
+                a.pu[at] = v;
+                a.pv[at] = q & 1 ? V.y : V.x;
+            }
+    } else if (wid == 16) {
+        // ---- loads
+        int slot = 0;
+        uint32_t ph = 1;   // of the slot's previous use
+        int hs = 0;
+        for (; hs < 2 * nbat && ok; ++hs) {
+            if (hs >= S) ok = __all_sync(0xffffffffu, tc::mbar_wait(&empty[slot], ph));
+            if (!ok) break;
+            const int64_t i = r0 + (int64_t)hs * HR;
+            const int vr = (int)max((int64_t)0, min((int64_t)HR, r1 - i));
+            const uint32_t bytes = (uint32_t)(vr * lda * (int64_t)sizeof(float));
+            if (lane == 0) tc::mbar_expect_tx(&full[slot], 2 * bytes);
+            __syncwarp();
+            if (lane < 2 && vr > 0)
+                tc::bulk_load(sw_smem + (size_t)slot * slot_bytes + (size_t)lane * HR * lda * sizeof(float),
+                              (lane ? a.Alo : a.Ahi) + i * lda, bytes, &full[slot]);
+            if (++slot == S) slot = 0, ph ^= 1;
+        }
+        if (!ok && lane == 0) atomicExch(a.err, 1);
+        // no copy is in flight when the CTA leaves
+        for (int x = max(0, hs - S); x < hs; ++x) tc::mbar_wait(&full[x % S], (uint32_t)(x / S) & 1);
+    } else {
+        // ---- finishing warps: lane = (row, warp sum)
+        const int idx = 32 * (wid - 17) + lane, rho = idx / W, sub = idx - rho * W;
+        const bool lead = sub == 0;
+        for (int b = 0; b < nbat && ok; ++b) {
+            const int64_t i = r0 + (int64_t)b * RB + rho;
+            const bool live = i < r1;
+            double ug = 0.0, bt = 0.0, winv = 0.0, bg = 0.0;
+            float wf = 0.0f;
+            int e0 = 0, e1 = 0;
+            if (live) {
+                bg = __ldg(a.b_g + i);
+                winv = __ldg(a.winv + i);
+                wf = __ldg(a.wf + i);
+                bt = a.bt[i];
+                ug = a.init ? 0.0 : a.u_g[i];
+                e0 = __ldg(a.csr_ptr + i);
+                e1 = __ldg(a.csr_ptr + i + 1);
+            }
+            // the row's sparse entries over its lanes; the first one's data now
+            const int most = __reduce_max_sync(0xffffffffu, e1 - e0);
+            double J = 0.0, bc = 0.0, uc = 0.0, rcv = 0.0, q = 0.0, qi = 0.0;
+            auto entry = [&](int e) {
+                const int cidx = __ldg(a.csr_col + e);
+                J = __ldg(a.csr_val + e);
+                bc = __ldg(a.b_s + cidx);
+                q = __ldg(a.q + cidx);
+                qi = __ldg(a.qinv + cidx);
+                uc = a.init ? 0.0 : __ldg(a.u_s + cidx);
+                rcv = a.init ? bc : __ldg(a.r_s + cidx);
+            };
+            if (e0 + sub < e1) entry(e0 + sub);
+            ok = __all_sync(0xffffffffu, tc::mbar_wait(&rowdone[b & 1], (uint32_t)(b >> 1) & 1));
+            if (!ok) break;
+            const float4 v = s_red[b & 1][idx];
+            float s = v.x, c = v.y, d = v.z;
+            for (int o = 1; o < W; o <<= 1) {
+                const float es = __shfl_xor_sync(0xffffffffu, s, o), ec = __shfl_xor_sync(0xffffffffu, c, o);
+                d += __shfl_xor_sync(0xffffffffu, d, o);
+                df_add(s, c, es, ec);
+            }
+            const double sol = ((double)d - bt) * winv;
+            const double un = ug + sol;
+            double part = 0.0;
+            for (int e = e0 + sub; e < e1; e += W) {
+                if (e != e0 + sub) entry(e);
+                const double us = new_us(uc, rcv, J, sol, qi);
+                const double rs = bc - fma(J, un, q * us);
+                part = fma(-J, us, part);
+                part = fma(-(J * qi), rs, part);
+            }
+            for (int o = 1; o < W && o < most; o <<= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+            const double Au = (double)s + (double)c;
+            const double btn = (fma(a.dc, un, bg) + part) - Au;
+            const float uh = (float)un;
+            if (lead) {
+                s_y[b & 1][rho] = make_float4(uh, (float)(un - (double)uh), (float)btn * wf, 0.0f);
+                if (live) {
+                    a.u_g[i] = un;
+                    a.sol_g[i] = sol;
+                    a.bt[i] = btn;
+                    a.Au[i] = Au;
+                }
+            }
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&rowready[b & 1]);
+        }
+        if (!ok && lane == 0) atomicExch(a.err, 1);
+    }
+}
+
+// bt = b_g - J_sg (b_s / q), u = bt / w (first approximate solve); 1 / w in FP64 and FP32, 1 / q
+__global__ void k_sweep_start(Dims D, ModelView M, const double *__restrict__ b, const double *__restrict__ q,
+                              const double *__restrict__ w, double *__restrict__ bt, double *__restrict__ u,
+                              double *__restrict__ winv, float *__restrict__ wf, double *__restrict__ qinv) {
+    const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, gsz = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = gtid; i < D.m_E; i += gsz) {
+        double s = b[D.n + i];
+        for (int e = M.csr_ptr[i]; e < M.csr_ptr[i + 1]; ++e) {
+            const int c = M.csr_col[e];
+            s -= ddiv(M.csr_val[e] * b[c], q[c]);
+        }
+        bt[i] = s;
+        u[i] = ddiv(s, w[i]);
+        const double r = ddiv(1.0, w[i]);
+        winv[i] = r;
+        wf[i] = (float)r;
+    }
+    for (int64_t k = gtid; k < D.n_s; k += gsz) qinv[k] = ddiv(1.0, q[k]);
+}
+
+// x = u_d + sol_d, u_h + sol_h into xnew, x and sol_d as FP32 parts, and
+// Hu = [H_dd; J_dh] x, a warp per row with x in shared memory
+__global__ void __launch_bounds__(NT) k_sweep_x(int64_t n_d, int64_t m_I, const double *__restrict__ Hdd,
+                                                const double *__restrict__ Jdh, const double *__restrict__ ud,
+                                                const double *__restrict__ uh, const double *__restrict__ sol, int init,
+                                                float4 *__restrict__ xq, double *__restrict__ xnew,
+                                                double *__restrict__ Hu) {
+    extern __shared__ double xsh[];
+    for (int64_t k = threadIdx.x; k < n_d; k += NT) {
+        const double d = sol[k], x = init ? d : ud[k] + d;
+        xsh[k] = x;
+        if (k / NT == blockIdx.x) {   // the grid has a block per NT columns at least
+            const float h = (float)x;
+            xq[k] = make_float4(h, (float)(x - (double)h), (float)d, 0.0f);
+            xnew[k] = x;
+        }
+    }
+    for (int64_t j = (int64_t)blockIdx.x * NT + threadIdx.x; j < m_I; j += (int64_t)gridDim.x * NT)
+        xnew[n_d + j] = init ? sol[n_d + j] : uh[j] + sol[n_d + j];
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    for (int64_t p = (int64_t)blockIdx.x * (NT / 32) + (threadIdx.x >> 5); p < n_d + m_I; p += (int64_t)gridDim.x * (NT / 32)) {
+        const double *row = p < n_d ? Hdd + p * n_d : Jdh + (p - n_d) * n_d;
+        double s0 = 0.0, s1 = 0.0;
+        int64_t k = lane;
+        for (; k + 96 < n_d; k += 128) {
+            const double a0 = __ldg(row + k), a1 = __ldg(row + k + 32), a2 = __ldg(row + k + 64), a3 = __ldg(row + k + 96);
+            s0 = fma(a0, xsh[k], s0);
+            s1 = fma(a1, xsh[k + 32], s1);
+            s0 = fma(a2, xsh[k + 64], s0);
+            s1 = fma(a3, xsh[k + 96], s1);
+        }
+        for (; k < n_d; k += 32) s0 = fma(row[k], xsh[k], s0);
+        double s = s0 + s1;
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane == 0) Hu[p] = s;
+    }
+}
+
+// |v| by its bit pattern into a running maximum (NaN passed over, as fmax does)
+__device__ __forceinline__ void max_abs(unsigned long long &m, double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL;
+    if (b > m && b <= 0x7ff0000000000000ULL) m = b;
+}
+
+// The rest of the sweep: u_s, u_d, u_h, the residual r = b - K u with its norms
+// (||r||, ||b||, ||K u||, ||u|| in the maximum norm), A^T u_g and the next
+// right-hand side of the reduced system from the CTAs' partial column sums.
+__global__ void __launch_bounds__(NT) k_sweep_residual(
+    Dims D, ModelView M, const double *__restrict__ b, double *__restrict__ u, double *__restrict__ r,
+    const double *__restrict__ q, const double *__restrict__ qinv, const double *__restrict__ sig_xd,
+    const double *__restrict__ sig_d, const double *__restrict__ Jdh, const double *__restrict__ Au,
+    const double *__restrict__ sol_g, const double *__restrict__ Hu, const double *__restrict__ xnew,
+    const double *__restrict__ pu, const float *__restrict__ pv, int nparts, int init, double dw, double dc,
+    double *__restrict__ ATu, double *__restrict__ rhsS, RedOut red) {
+    __shared__ double sp[NT / 32][33], su[NT / 32][33];
+    __shared__ float2 sv[NT / 32][33];
+    unsigned long long rm = 0, bm = 0, km = 0, um = 0;
+    const int64_t gtid = (int64_t)blockIdx.x * NT + threadIdx.x, gsz = (int64_t)gridDim.x * NT;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    auto put = [&](int64_t idx, double Ku, double ui) -> double {
+        const double bi = b[idx], ri = bi - Ku;
+        r[idx] = ri;
+        max_abs(rm, ri);
+        max_abs(bm, bi);
+        max_abs(km, Ku);
+        max_abs(um, ui);
+        return ri;
+    };
+    for (int64_t k0 = (int64_t)blockIdx.x * 32; k0 < D.n_d; k0 += (int64_t)gridDim.x * 32) {
+        const double jt = colgroup_dot<NT>(Jdh, D.m_I, D.n_d, k0, xnew + D.n_d, sp);
+        const int64_t k = k0 + lane;
+        double s = 0.0;
+        float vs = 0.0f, vc = 0.0f;
+        if (k < D.n_d)
+#pragma unroll 4
+            for (int p = wid; p < nparts; p += NT / 32) {
+                s += pu[(size_t)p * D.n_d + k];
+                df_add(vs, vc, pv[(size_t)p * D.n_d + k], 0.0f);
+            }
+        __syncthreads();
+        su[wid][lane] = s;
+        sv[wid][lane] = make_float2(vs, vc);
+        __syncthreads();
+        if (wid == 0 && k < D.n_d) {
+            double at = 0.0;
+#pragma unroll
+            for (int x = 0; x < NT / 32; ++x) {
+                at += su[x][lane];
+                if (x) df_add(vs, vc, sv[x][lane].x, sv[x][lane].y);
+            }
+            const double x = xnew[k];
+            ATu[k] = at;
+            u[D.n_s + k] = x;
+            const double ri = put(D.n_s + k, Hu[k] + (sig_xd[k] + dw) * x + at + jt, x);
+            rhsS[k] = ri + ((double)vs + (double)vc);
+        }
+    }
+    // equality rows with their sparse columns
+    for (int64_t i = gtid; i < D.m_E; i += gsz) {
+        const double ug = u[D.n + i], sol = sol_g[i];
+        double Kg = Au[i] - dc * ug;
+        for (int e = M.csr_ptr[i]; e < M.csr_ptr[i + 1]; ++e) {
+            const int c = M.csr_col[e];
+            const double J = M.csr_val[e];
+            const double us = new_us(init ? 0.0 : u[c], init ? b[c] : r[c], J, sol, qinv[c]);
+            u[c] = us;
+            put(c, fma(J, ug, q[c] * us), us);
+            Kg = fma(J, us, Kg);
+        }
+        put(D.n + i, Kg, ug);
+    }
+    for (int64_t k = gtid; k < D.n_s; k += gsz)
+        if (M.csc_ptr[k] == M.csc_ptr[k + 1]) {   // a sparse variable of no equality row
+            const double us = new_us(init ? 0.0 : u[k], init ? b[k] : r[k], 0.0, 0.0, qinv[k]);
+            u[k] = us;
+            put(k, q[k] * us, us);
+        }
+    for (int64_t j = gtid; j < D.m_I; j += gsz) {
+        const double uh = xnew[D.n_d + j];
+        u[D.n + D.m_E + j] = uh;
+        rhsS[D.n_d + j] = put(D.n + D.m_E + j, Hu[D.n_d + j] - (ddiv(1.0, sig_d[j] + dw) + dc) * uh, uh);
+    }
+    double v[4] = {__longlong_as_double((long long)rm), __longlong_as_double((long long)bm),
+                   __longlong_as_double((long long)km), __longlong_as_double((long long)um)};
+    reduce_finish<NT, R_MAX, R_MAX, R_MAX, R_MAX>(v, red);
+}
+
+int grid_for(int64_t n) { return std::max(1, std::min(4096, ceil_div(std::max<int64_t>(n, 1), 256))); }
+
+template <int CH, int KBR>
+int launch_sweep_t(cudaStream_t st, int num_sms, SweepArgs a) {
+    a.T = 32;
+    while (a.T < kSwC && 4 * CH * a.T < a.n) a.T *= 2;
+    const int G = kSwC / a.T, HR = G * KBR / 2;
+    const size_t slot = (size_t)2 * HR * a.lda * sizeof(float);
+    a.S = (int)std::min<size_t>(kSwMaxSlots, kSwRing / slot);
+    MDSIP_REQUIRE(a.S >= 5, MDSIP_ERR_INVALID_ARG, "refinement sweep: rows too long");
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(num_sms, kRedBlocks / 2), ceil_div(a.m, 2 * HR)));
+    a.pv = reinterpret_cast<float *>(a.pu + (size_t)grid * a.n);
+    static PerDeviceOnce once;
+    MDSIP_CUDA(once.run([] {
+        return cudaFuncSetAttribute(k_sweep<CH, KBR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSwRing);
+    }));
+    k_sweep<CH, KBR><<<grid, 32 * (17 + KBR / 2), std::max(kSwMin, a.S * slot), st>>>(a);
+    MDSIP_LAUNCHED();
+    return grid;
+}
+
+}  // namespace
+
+// FP32 tiles of a tensor-core factor with the FP32 pair of A; above 4096
+// columns a batch and its predecessor no longer fit the shared memory together
+// (the separate passes of refine.cu take those)
+bool Refiner::sweep_path() const { return xq && Ahi && solve_fp32 && AfT && D.n_d > 0 && D.n_d <= 4096; }
+
+void Refiner::sweep_start(const double *b) {
+    k_sweep_start<<<grid_for(std::max(D.m_E, D.n_s)), 256, 0, st>>>(D, M, b, q, w, bt, tmp_m, winv, wf, qinv);
+    MDSIP_LAUNCHED();
+    launch_aft_dot(st, num_sms, AfT, ldt, D.m_E, D.n_d, tmp_m, vf, tmp_nd);
+    rhs_S(b, tmp_nd);
+}
+
+void Refiner::sweep(const double *b, double *u, double *r, bool init, double dw, double dc, double *out4) {
+    launch_ldlt_solve_coop(st, num_sms, N, Dd, Doff, perm, 1, rhsS, N, solve_ws, solve_err, solve_fp32);
+    static PerDeviceOnce once;
+    MDSIP_CUDA(once.run([] {
+        return cudaFuncSetAttribute(k_sweep_x, cudaFuncAttributeMaxDynamicSharedMemorySize, 4096 * (int)sizeof(double));
+    }));
+    k_sweep_x<<<std::max(1, std::min(4096, ceil_div(D.n_d + D.m_I, NT / 32))), NT, D.n_d * sizeof(double), st>>>(
+        D.n_d, D.m_I, Hdd, Jdh, u + D.n_s, u + D.n + D.m_E, rhsS, init ? 1 : 0, xq, xnew, tmp_nd2);
+    MDSIP_LAUNCHED();
+    SweepArgs a{};
+    a.Ahi = Ahi;
+    a.Alo = Alo;
+    a.m = D.m_E;
+    a.lda = D.lda;
+    a.n = (int)D.n_d;
+    a.xq = xq;
+    a.b_g = b + D.n;
+    a.winv = winv;
+    a.wf = wf;
+    a.u_g = u + D.n;
+    a.bt = bt;
+    a.sol_g = sol_g;
+    a.Au = tmp_m;
+    a.dc = dc;
+    a.csr_ptr = M.csr_ptr;
+    a.csr_col = M.csr_col;
+    a.csr_val = M.csr_val;
+    a.b_s = b;
+    a.u_s = u;
+    a.r_s = r;
+    a.q = q;
+    a.qinv = qinv;
+    a.init = init ? 1 : 0;
+    a.pu = colpart;
+    a.err = solve_err;
+    const int grid = D.n_d <= 4 * kSwC ? launch_sweep_t<1, 4>(st, num_sms, a) : launch_sweep_t<2, 2>(st, num_sms, a);
+    k_sweep_residual<<<red_grid(std::max(std::max(D.n_s, D.m_E), (NT / 32) * D.n_d)), NT, 0, st>>>(
+        D, M, b, u, r, q, qinv, sig_xd, sig_d, Jdh, tmp_m, sol_g, tmp_nd2, xnew, colpart,
+        reinterpret_cast<const float *>(colpart + (size_t)grid * D.n_d), grid, init ? 1 : 0, dw, dc, tmp_nd, rhsS,
+        RedOut{partial, reinterpret_cast<unsigned *>(partial + kRedBlocks * 8), out4});
+    MDSIP_LAUNCHED();
+}
+
+}  // namespace mdsip

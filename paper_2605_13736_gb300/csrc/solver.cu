@@ -114,7 +114,7 @@ struct Problem {
     bool rns_oom = false;   // the residue workspace did not fit once: the DFMA product from then on
     // tensor-core condensation and refinement
     DBuf bAfT, bvf, btc_ws, btc_err, bref_b, bref_u, bref_r, bref_d, btmp_nd2, bsolve_ws, bsolve_err, bAu_run;
-    DBuf bcpre, bcw, bwf, bATv, bAsd;   // the refinement's fused residual pass
+    DBuf bxq, bxnew, bqinv, bwinv, bwf, bsol_g;   // the refinement's one-pass sweeps
     bool aft_ready = false;
     DBuf bAhi, bAlo, bsplit;   // A as an FP32 pair (mixed path's double-float passes) and vector scratch
     // Products with A carried from step to step on the mixed path of a data-given
@@ -601,11 +601,12 @@ static void prepare_path(Problem *P) {
         dvec(ctx, P->bref_d, nm);
         dvec(ctx, P->btmp_nd2, D.n_d + D.m_I);
         dvec(ctx, P->bAu_run, D.m_E);
-        dvec(ctx, P->bcpre, D.m_E);
-        dvec(ctx, P->bcw, D.m_E);    // m_E float2
-        dvec(ctx, P->bwf, D.m_E);    // m_E floats (room for m_E doubles)
-        dvec(ctx, P->bATv, D.n_d);
-        dvec(ctx, P->bAsd, D.m_E);
+        dvec(ctx, P->bxq, 2 * D.n_d);   // n_d float4
+        dvec(ctx, P->bxnew, D.n_d + D.m_I);
+        dvec(ctx, P->bqinv, D.n_s);
+        dvec(ctx, P->bwinv, D.m_E);
+        dvec(ctx, P->bwf, D.m_E);       // m_E floats
+        dvec(ctx, P->bsol_g, D.m_E);
     }
 }
 
@@ -980,7 +981,7 @@ static RefineResult solve_direction_refined(Problem *P, double mu, double dw, do
     R.sig_d = P->bsig_d.as<double>();
     R.Jdh = P->bJdh.as<double>();
     R.Hdd = P->bHdd.as<double>();
-    R.bt_g = P->bbt_g.as<double>();
+    R.bt = P->bbt_g.as<double>();
     R.tmp_m = P->bAdx.as<double>();
     R.tmp_nd = P->bATu.as<double>();
     R.tmp_nd2 = P->btmp_nd2.as<double>();
@@ -991,31 +992,40 @@ static RefineResult solve_direction_refined(Problem *P, double mu, double dw, do
     R.Ahi = P->V.Ahi;
     R.Alo = P->V.Alo;
     R.split = P->V.split;
-    R.cpre = P->bcpre.as<double>();
-    R.cw = P->bcw.as<float2>();
+    R.xq = P->bxq.as<float4>();
+    R.xnew = P->bxnew.as<double>();
+    R.qinv = P->bqinv.as<double>();
+    R.winv = P->bwinv.as<double>();
     R.wf = P->bwf.as<float>();
-    R.ATv = P->bATv.as<double>();
-    R.Asd = P->bAsd.as<double>();
+    R.sol_g = P->bsol_g.as<double>();
     double *b = P->bref_b.as<double>(), *u = P->bref_u.as<double>(), *r = P->bref_r.as<double>(),
            *d = P->bref_d.as<double>();
     const double *h = P->hscal;
     MDSIP_CUDA(cudaEventRecord(P->ev[3], st));
     R.rhs(P->I, P->bgl.as<double>(), P->cg, P->ch, R.sig_d, mu, dw, b);
-    R.approx_solve(b, u);
-    R.track_Au(true);
+    const bool one_pass = R.sweep_path();
+    if (one_pass) {
+        R.sweep_start(b);
+    } else {
+        R.approx_solve(b, u);
+        R.track_Au(true);
+    }
     RefineResult out{false, 0, INFINITY};
     double rprev = INFINITY;
     while (true) {
-        R.residual(b, u, dw, dc, r, P->scal() + SC_REF);
+        if (one_pass) R.sweep(b, u, r, out.sweeps == 0, dw, dc, P->scal() + SC_REF);
+        else R.residual(b, u, dw, dc, r, P->scal() + SC_REF);
         P->sync_scalars();
         const double rinf = h[SC_REF], scale = h[SC_REF + 1] + h[SC_REF + 2];
         out.res = scale > 0 ? rinf / scale : 0.0;
         if (!std::isfinite(out.res)) break;
         if (rinf <= P->opt.refine_tol * scale) break;
         if (out.sweeps >= max_sweeps || (out.sweeps > 0 && rinf > 0.5 * rprev)) break;
-        R.approx_solve(r, d);
-        R.track_Au(false);
-        R.axpy(D.n + D.m, d, u);
+        if (!one_pass) {
+            R.approx_solve(r, d);
+            R.track_Au(false);
+            R.axpy(D.n + D.m, d, u);
+        }
         out.sweeps++;
         rprev = rinf;
     }
