@@ -4,6 +4,8 @@
 
 namespace mdsip {
 
+int64_t refine_sweep_parts(int64_t n);
+
 struct Refiner {
     Dims D;
     ModelView M;

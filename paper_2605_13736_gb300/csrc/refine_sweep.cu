@@ -19,8 +19,8 @@
 // shared memory between its two halves and A_hi, A_lo are read once a sweep, 8
 // bytes per entry (12 in the separate passes, with ten small launches more
 // around them).  A sweep's passes at m = 100000, n = 2000: 361 + 164 us apart,
-// 445 in one; m = 200000, n = 4000: 1275 + 800 + 498 apart, 1600; m = 25600,
-// n = 512: 78 + 23 apart, 43.
+// 358 in one; m = 200000, n = 4000: 1275 + 800 + 498 apart, 1360; m = 25600,
+// n = 512: 78 + 23 apart, 35.
 #include "df.cuh"
 #include "internal.cuh"
 #include "refine.cuh"
@@ -32,14 +32,15 @@ namespace {
 
 constexpr int NT = kRedThreads;
 constexpr int kSwC = 512;                     // column threads: 16 warps
+constexpr int kSwThreads = 640;               // 20 warps, five a sub-partition: 96 registers a thread
 constexpr int kSwMaxSlots = 12;
-constexpr size_t kSwRing = 222 * 1024;        // half-batches in flight or in use
+constexpr size_t kSwSmem = 224 * 1024;        // batches in flight or in use
 constexpr size_t kSwMin = 48 * 1024;          // the groups' column sums meet in the ring at the end
 
 struct SweepArgs {
     const float *Ahi, *Alo;
     int64_t m, lda;
-    int n, T, S;           // columns, threads per row, half-batches of the ring
+    int n, T, S;           // columns, threads per row, batches of the ring
     const float4 *xq;      // per column: u_d split (x, y), fl32(sol_d) (z)
     const double *b_g, *winv;
     const float *wf;
@@ -48,8 +49,8 @@ struct SweepArgs {
     const int *csr_ptr, *csr_col;
     const double *csr_val, *b_s, *u_s, *r_s, *q, *qinv;
     int init;              // u = 0 and r = b before this sweep
-    double *pu;            // partial sums of A^T u_g, a row per CTA
-    float *pv;             // and of A_hi^T (bt / w)
+    double *pu;            // partial sums of A^T u_g, a row per CTA and group (the CTA's in its first)
+    float *pv;             // and of A_hi^T (bt / w), a row per CTA
     int *err;
 };
 
@@ -58,45 +59,68 @@ __device__ __forceinline__ double new_us(double u, double r, double J, double so
     return fma(fma(-J, sol, r), qinv, u);
 }
 
-// Warps 0 .. 15 compute, warp 16 loads, warps 17 .. finish rows.  T threads
-// (32 .. 512) take a row's columns, 4 CH each; the 512 / T groups take KBR rows
-// of a batch each, so a batch is about 64 KB at any width.  It comes as two
-// half-batches, each one bulk copy of A_hi and one of A_lo (the rows are
-// contiguous).  Per batch: row products, warp sums to shared memory, the
-// finishing warps' scalars in FP64, and one batch later, with the finished
-// rows, the column products.  Only mbarriers: no warp waits for the finishing
-// warps until it has done the next batch's row products.  Waits are bounded.
-template <int CH, int KBR>
-__global__ void __launch_bounds__(CH == 1 ? 608 : 576, 1) k_sweep(SweepArgs a) {
+// v = hi + lo to 2^-49, hi to nearest: on the bits for ordinary magnitudes (four
+// FP64 conversions and a subtraction otherwise, 64 cycles each)
+__device__ __forceinline__ float2 split64(double v) {
+    const long long b = __double_as_longlong(v);
+    const int e = (int)((b >> 52) & 0x7ff);
+    if (e < 1023 - 60 || e > 1023 + 100) {
+        const float h = (float)v;
+        return make_float2(h, (float)(v - (double)h));
+    }
+    const long long t = (b + 0x10000000LL) & ~0x1fffffffLL;   // the magnitude's upper 24 bits, rounded
+    const unsigned sg = (unsigned)(b >> 32) & 0x80000000u;
+    const unsigned hi = sg | ((unsigned)(((t & 0x7fffffffffffffffLL) >> 29) - (896LL << 23)));
+    const float lo = (float)(int)(b - t) * __uint_as_float(sg | (unsigned)((e - 948) << 23));
+    return make_float2(__uint_as_float(hi), lo);
+}
+
+// Warps 0 .. 15 compute, warp 16 loads, warps 17 .. 19 finish rows in turn
+// (batch b by warp 17 + b mod 3).  T threads (32 .. 512) take a row's columns,
+// 4 CH each; the 512 / T groups take KBR rows of a batch each, so a batch is
+// 32 (CH = 1) or 64 KB at any width and comes as one bulk copy of A_hi and one
+// of A_lo (the rows are contiguous).  Per batch: row products, warp sums to
+// shared memory, the finishing warp's scalars in FP64 (some 20 instructions of
+// 64 cycles, its gathers a turn ahead), and kLag batches later, with the
+// finished rows, the column products.  Only mbarriers; waits are bounded.
+// What bounds it is the double-float arithmetic's dependent chains with the
+// five warps a sub-partition holds: the FP32 pipe is 49% busy, HBM at 4.7 of
+// 6.9 TB/s at n = 4000.  Eight columns and two rows a thread (CH = KBR = 2)
+// spread the row sums' shuffles over the most products: m = 100000, n = 2000
+// 358 us, with four columns and three batches of lag (whose row and column
+// parts interleave) 385, summing the rows in the finishing warps 377; m =
+// 200000, n = 4000 1360 us, with one row a batch 1770.
+template <int CH, int KBR, int kLag>
+__global__ void __launch_bounds__(kSwThreads, 1) k_sweep(SweepArgs a) {
     extern __shared__ __align__(128) unsigned char sw_smem[];
-    constexpr int NTW = KBR / 2;               // finishing warps: KBR * 16 / 32
     constexpr int kVals = KBR * 16;            // (row, warp) sums of a batch
-    __shared__ float4 s_red[2][kVals];
-    __shared__ float4 s_y[2][kVals];
-    __shared__ __align__(8) uint64_t full[kSwMaxSlots], empty[kSwMaxSlots], rowdone[2], rowready[2];
+    __shared__ float4 s_y[3][kVals];
+    __shared__ float2 s_red[3][kVals];
+    __shared__ float s_red2[3][kVals];
+    __shared__ __align__(8) uint64_t full[kSwMaxSlots], empty[kSwMaxSlots], rowdone[3], rowready[3];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    const int T = a.T, W = T / 32, G = kSwC / T, HR = G * KBR / 2, RB = G * KBR, S = a.S;
-    const int64_t lda = a.lda;
-    const size_t slot_bytes = (size_t)2 * HR * lda * sizeof(float);
+    const int T = a.T, W = T / 32, G = kSwC / T, RB = G * KBR, S = a.S;
+    const int lda = (int)a.lda;
+    const uint32_t slot_bytes = 2u * RB * lda * (uint32_t)sizeof(float);
     const int64_t rows_per = (a.m + gridDim.x - 1) / gridDim.x;
     const int64_t r0 = (int64_t)blockIdx.x * rows_per;
-    const int64_t r1 = min(a.m, r0 + rows_per);
-    const int nbat = r1 > r0 ? (int)((r1 - r0 + RB - 1) / RB) : 0;
+    const int nrow = (int)max((int64_t)0, min(a.m - r0, rows_per));
+    const int nbat = (nrow + RB - 1) / RB;
     if (tid == 0) {
         for (int i = 0; i < S; ++i) {
             tc::mbar_init(&full[i], 1);
             tc::mbar_init(&empty[i], 16);
         }
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < 3; ++i) {
             tc::mbar_init(&rowdone[i], 16);
-            tc::mbar_init(&rowready[i], NTW);
+            tc::mbar_init(&rowready[i], 1);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
     bool ok = true;
     if (wid < 16) {
-        const int g = tid / T, t = tid - g * T, w = t >> 5;
+        const int g = tid / T, t = tid - g * T;
         float2 xh[2 * CH], xl[2 * CH], xs[2 * CH];
         bool on[CH];
 #pragma unroll
@@ -117,122 +141,136 @@ __global__ void __launch_bounds__(CH == 1 ? 608 : 576, 1) k_sweep(SweepArgs a) {
         // which goes into FP64 every 256 rows (the FP64 pipe: 1/64 of the FP32 rate)
         const float2 z2 = make_float2(0.0f, 0.0f);
         float2 cs[2 * CH], cc[2 * CH], CS[2 * CH], CC[2 * CH], cv[2 * CH];
-        double cacc[CH == 1 ? 4 : 1] = {};
         bool flushed = false;
 #pragma unroll
         for (int j = 0; j < 2 * CH; ++j) cs[j] = cc[j] = CS[j] = CC[j] = cv[j] = z2;
         int cnt = 0, cnt2 = 0;
-        int rslot = 0, cslot = 0;
-        uint32_t rph = 0;
-        for (int b = 0; b <= nbat; ++b) {
+        int rslot = 0, cslot = 0, rb = 0, cb = 0;   // ring slots, result buffers (b mod 3) of the two halves
+        uint32_t rph = 0, cph = 0;
+        const uint32_t off = (uint32_t)(g * KBR * lda) * (uint32_t)sizeof(float), lo_off = (uint32_t)(RB * lda) * 4u;
+        // columns beyond n read the row's first ones: x is zero there, their sums are not stored
+        uint32_t coff[CH];
+#pragma unroll
+        for (int ch = 0; ch < CH; ++ch) coff[ch] = on[ch] ? (uint32_t)(4 * t + ch * 4 * T) * 4u : 0u;
+        float2 ps[KBR][CH], pc[KBR][CH], p2[KBR];
+        auto row_part = [&](const unsigned char *base, int k) {
+            p2[k] = z2;
+#pragma unroll
+            for (int ch = 0; ch < CH; ++ch) {
+                const unsigned char *at = base + (uint32_t)(k * lda) * 4u + coff[ch];
+                const float4 ah = *reinterpret_cast<const float4 *>(at);
+                const float4 al = *reinterpret_cast<const float4 *>(at + lo_off);
+                const float2 h0 = make_float2(ah.x, ah.y), h1 = make_float2(ah.z, ah.w);
+                ps[k][ch] = pc[k][ch] = z2;
+                df_acc2(h0, make_float2(al.x, al.y), xh[2 * ch], xl[2 * ch], ps[k][ch], pc[k][ch]);
+                df_acc2(h1, make_float2(al.z, al.w), xh[2 * ch + 1], xl[2 * ch + 1], ps[k][ch], pc[k][ch]);
+                p2[k] = __ffma2_rn(h0, xs[2 * ch], p2[k]);
+                p2[k] = __ffma2_rn(h1, xs[2 * ch + 1], p2[k]);
+            }
+        };
+        auto col_part = [&](const unsigned char *base, int k, float4 y) {
+            const float2 yh = make_float2(y.x, y.x), yl = make_float2(y.y, y.y), yv = make_float2(y.z, y.z);
+#pragma unroll
+            for (int ch = 0; ch < CH; ++ch) {
+                const unsigned char *at = base + (uint32_t)(k * lda) * 4u + coff[ch];
+                const float4 ah = *reinterpret_cast<const float4 *>(at);
+                const float4 al = *reinterpret_cast<const float4 *>(at + lo_off);
+                const float2 h0 = make_float2(ah.x, ah.y), h1 = make_float2(ah.z, ah.w);
+                df_acc2(h0, make_float2(al.x, al.y), yh, yl, cs[2 * ch], cc[2 * ch]);
+                df_acc2(h1, make_float2(al.z, al.w), yh, yl, cs[2 * ch + 1], cc[2 * ch + 1]);
+                cv[2 * ch] = __ffma2_rn(h0, yv, cv[2 * ch]);
+                cv[2 * ch + 1] = __ffma2_rn(h1, yv, cv[2 * ch + 1]);
+            }
+        };
+        for (int b = 0; b < nbat + kLag; ++b) {
             if (!__all_sync(0xffffffffu, ok)) break;   // a wait ran out: the whole warp stops
-            if (b < nbat) {   // ---- row products of batch b
-                float rs[KBR], rc[KBR], r2[KBR];
-                const int64_t i0 = r0 + (int64_t)b * RB;
+            if (b < nbat && !tc::mbar_wait(&full[rslot], rph)) ok = false;
+            if (kLag > 1 && b >= kLag && !tc::mbar_wait(&rowready[cb], cph)) ok = false;
+            const unsigned char *rbase = sw_smem + rslot * slot_bytes + off;
+            const unsigned char *cbase = sw_smem + cslot * slot_bytes + off;
+            auto rows = [&]() {
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    if (!tc::mbar_wait(&full[rslot], rph)) ok = false;
-                    const float *base = reinterpret_cast<const float *>(sw_smem + (size_t)rslot * slot_bytes);
+                for (int k = 0; k < KBR; ++k) {
+                    if (b * RB + g * KBR + k < nrow) {
+                        row_part(rbase, k);
+                    } else {
+                        p2[k] = z2;
 #pragma unroll
-                    for (int k = 0; k < KBR / 2; ++k) {
-                        const int rr = h * (KBR / 2) + k, rho = g * (KBR / 2) + k;
-                        float2 ps = z2, pc = z2, p2 = z2;
-                        if (i0 + h * HR + rho < r1) {
-                            const float *row = base + rho * lda + 4 * t;
-#pragma unroll
-                            for (int ch = 0; ch < CH; ++ch)
-                                if (on[ch]) {
-                                    const float4 ah = *reinterpret_cast<const float4 *>(row + ch * 4 * T);
-                                    const float4 al = *reinterpret_cast<const float4 *>(row + HR * lda + ch * 4 * T);
-                                    const float2 h0 = make_float2(ah.x, ah.y), h1 = make_float2(ah.z, ah.w);
-                                    df_acc2(h0, make_float2(al.x, al.y), xh[2 * ch], xl[2 * ch], ps, pc);
-                                    df_acc2(h1, make_float2(al.z, al.w), xh[2 * ch + 1], xl[2 * ch + 1], ps, pc);
-                                    p2 = __ffma2_rn(h0, xs[2 * ch], p2);
-                                    p2 = __ffma2_rn(h1, xs[2 * ch + 1], p2);
-                                }
-                        }
-                        rs[rr] = ps.x;
-                        rc[rr] = pc.x;
-                        df_add(rs[rr], rc[rr], ps.y, pc.y);
-                        r2[rr] = p2.x + p2.y;
+                        for (int ch = 0; ch < CH; ++ch) ps[k][ch] = pc[k][ch] = z2;
                     }
-                    if (++rslot == S) rslot = 0, rph ^= 1;
                 }
-                // the rows' sums over the warp by halving exchanges, then a butterfly
-                const bool u16 = (lane & 16) != 0, u8 = (lane & 8) != 0;
-                auto xch = [&](int o, bool up, int keep_lo, int keep_hi, float &s, float &c, float &d) {
-                    float es = up ? rs[keep_lo] : rs[keep_hi], ec = up ? rc[keep_lo] : rc[keep_hi];
-                    float ed = up ? r2[keep_lo] : r2[keep_hi];
-                    s = up ? rs[keep_hi] : rs[keep_lo];
-                    c = up ? rc[keep_hi] : rc[keep_lo];
-                    d = up ? r2[keep_hi] : r2[keep_lo];
-                    es = __shfl_xor_sync(0xffffffffu, es, o);
-                    ec = __shfl_xor_sync(0xffffffffu, ec, o);
-                    d += __shfl_xor_sync(0xffffffffu, ed, o);
+            };
+            auto cols = [&]() {
+#pragma unroll
+                for (int k = 0; k < KBR; ++k)
+                    if ((b - kLag) * RB + g * KBR + k < nrow) col_part(cbase, k, s_y[cb][g * KBR + k]);
+            };
+            auto release = [&]() {
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&empty[cslot]);
+                if (++cslot == S) cslot = 0;
+                if (++cb == 3) cb = 0, cph ^= 1;
+            };
+            if (kLag > 1 && b >= kLag && (b + 1) * RB <= nrow) {   // whole batches: both parts in one stream of instructions
+#pragma unroll
+                for (int k = 0; k < KBR; ++k) {
+                    row_part(rbase, k);
+                    col_part(cbase, k, s_y[cb][g * KBR + k]);
+                }
+            } else {
+                rows();
+                if (kLag > 1 && b >= kLag) cols();
+            }
+            if (kLag > 1 && b >= kLag) release();
+            if (b < nbat) {   // ---- the rows' sums over the warp: two rows exchange halves, then a butterfly
+                float rs[KBR], rc[KBR], r2[KBR];
+#pragma unroll
+                for (int k = 0; k < KBR; ++k) {
+                    float2 s = ps[k][0], c = pc[k][0];
+#pragma unroll
+                    for (int ch = 1; ch < CH; ++ch) {
+                        df_add(s.x, c.x, ps[k][ch].x, pc[k][ch].x);
+                        df_add(s.y, c.y, ps[k][ch].y, pc[k][ch].y);
+                    }
+                    df_add(s.x, c.x, s.y, c.y);
+                    rs[k] = s.x;
+                    rc[k] = c.x;
+                    r2[k] = p2[k].x + p2[k].y;
+                }
+                if (++rslot == S) rslot = 0, rph ^= 1;
+                float s = rs[0], c = rc[0], d = r2[0];
+                int row = g * KBR;
+                if constexpr (KBR == 2) {
+                    const bool up = (lane & 16) != 0;
+                    float es = up ? s : rs[1], ec = up ? c : rc[1], ed = up ? d : r2[1];
+                    s = up ? rs[1] : s;
+                    c = up ? rc[1] : c;
+                    d = up ? r2[1] : d;
+                    es = __shfl_xor_sync(0xffffffffu, es, 16);
+                    ec = __shfl_xor_sync(0xffffffffu, ec, 16);
+                    d += __shfl_xor_sync(0xffffffffu, ed, 16);
                     df_add(s, c, es, ec);
-                };
-                float s, c, d;
-                int rho;
-                bool lead;
-                if constexpr (KBR == 4) {
-                    float s0, c0, d0, s1, c1, d1;
-                    xch(16, u16, 0, 2, s0, c0, d0);
-                    xch(16, u16, 1, 3, s1, c1, d1);
-                    float es = u8 ? s0 : s1, ec = u8 ? c0 : c1, ed = u8 ? d0 : d1;
-                    s = u8 ? s1 : s0;
-                    c = u8 ? c1 : c0;
-                    d = u8 ? d1 : d0;
-                    es = __shfl_xor_sync(0xffffffffu, es, 8);
-                    ec = __shfl_xor_sync(0xffffffffu, ec, 8);
-                    d += __shfl_xor_sync(0xffffffffu, ed, 8);
-                    df_add(s, c, es, ec);
-                    rho = (u16 ? HR : 0) + 2 * g + (u8 ? 1 : 0);
-                    lead = (lane & 7) == 0;
-                } else {
-                    xch(16, u16, 0, 1, s, c, d);
-                    rho = (u16 ? HR : 0) + g;
-                    lead = (lane & 15) == 0;
+                    row += up ? 1 : 0;
                 }
 #pragma unroll
-                for (int o = KBR == 4 ? 4 : 8; o > 0; o >>= 1) {
+                for (int o = KBR == 2 ? 8 : 16; o > 0; o >>= 1) {
                     const float es = __shfl_xor_sync(0xffffffffu, s, o), ec = __shfl_xor_sync(0xffffffffu, c, o);
                     d += __shfl_xor_sync(0xffffffffu, d, o);
                     df_add(s, c, es, ec);
                 }
-                if (lead) s_red[b & 1][rho * W + w] = make_float4(s, c, d, 0.0f);
-                __syncwarp();
-                if (lane == 0) tc::mbar_arrive(&rowdone[b & 1]);
-            }
-            if (b == 0) continue;
-            // ---- column products of batch b - 1
-            const int e = b - 1;
-            const int64_t i0 = r0 + (int64_t)e * RB;
-            if (!tc::mbar_wait(&rowready[e & 1], (uint32_t)(e >> 1) & 1)) ok = false;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const float *base = reinterpret_cast<const float *>(sw_smem + (size_t)cslot * slot_bytes);
-#pragma unroll
-                for (int k = 0; k < KBR / 2; ++k) {
-                    const int rho = g * (KBR / 2) + k;
-                    if (i0 + h * HR + rho >= r1) continue;
-                    const float4 y = s_y[e & 1][h * HR + rho];
-                    const float2 yh = make_float2(y.x, y.x), yl = make_float2(y.y, y.y), yv = make_float2(y.z, y.z);
-                    const float *row = base + rho * lda + 4 * t;
-#pragma unroll
-                    for (int ch = 0; ch < CH; ++ch)
-                        if (on[ch]) {
-                            const float4 ah = *reinterpret_cast<const float4 *>(row + ch * 4 * T);
-                            const float4 al = *reinterpret_cast<const float4 *>(row + HR * lda + ch * 4 * T);
-                            const float2 h0 = make_float2(ah.x, ah.y), h1 = make_float2(ah.z, ah.w);
-                            df_acc2(h0, make_float2(al.x, al.y), yh, yl, cs[2 * ch], cc[2 * ch]);
-                            df_acc2(h1, make_float2(al.z, al.w), yh, yl, cs[2 * ch + 1], cc[2 * ch + 1]);
-                            cv[2 * ch] = __ffma2_rn(h0, yv, cv[2 * ch]);
-                            cv[2 * ch + 1] = __ffma2_rn(h1, yv, cv[2 * ch + 1]);
-                        }
+                if ((lane & (KBR == 2 ? 15 : 31)) == 0) {
+                    s_red[rb][row * W + (t >> 5)] = make_float2(s, c);
+                    s_red2[rb][row * W + (t >> 5)] = d;
                 }
                 __syncwarp();
-                if (lane == 0) tc::mbar_arrive(&empty[cslot]);
-                if (++cslot == S) cslot = 0;
+                if (lane == 0) tc::mbar_arrive(&rowdone[rb]);
+                if (++rb == 3) rb = 0;
+            }
+            if (b < kLag) continue;
+            if (kLag == 1) {
+                if (!tc::mbar_wait(&rowready[cb], cph)) ok = false;
+                cols();
+                release();
             }
             if (++cnt == 16 / KBR) {   // every 16 rows
                 cnt = 0;
@@ -244,21 +282,14 @@ __global__ void __launch_bounds__(CH == 1 ? 608 : 576, 1) k_sweep(SweepArgs a) {
                 }
                 if (++cnt2 == 16) {   // every 256 rows
                     cnt2 = 0;
-                    if constexpr (CH == 1) {
+                    // this group's row of sums, its own until the end
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const float2 A = CS[q >> 1], B = CC[q >> 1];
-                            cacc[q] += (double)(q & 1 ? A.y : A.x) + (double)(q & 1 ? B.y : B.x);
-                        }
-                    } else {   // one group: this thread's columns of the CTA's partial row
-#pragma unroll
-                        for (int q = 0; q < 4 * CH; ++q) {
-                            const int p = 4 * t + (q >> 2) * 4 * T + (q & 3);
-                            const float2 A = CS[q >> 1], B = CC[q >> 1];
-                            const double v = (double)(q & 1 ? A.y : A.x) + (double)(q & 1 ? B.y : B.x);
-                            double *at = a.pu + (size_t)blockIdx.x * a.n + p;
-                            if (p < a.n) *at = flushed ? *at + v : v;
-                        }
+                    for (int q = 0; q < 4 * CH; ++q) {
+                        const int p = 4 * t + (q >> 2) * 4 * T + (q & 3);
+                        const float2 A = CS[q >> 1], B = CC[q >> 1];
+                        const double v = (double)(q & 1 ? A.y : A.x) + (double)(q & 1 ? B.y : B.x);
+                        double *at = a.pu + ((size_t)blockIdx.x * G + g) * a.n + p;
+                        if (p < a.n) *at = flushed ? *at + v : v;
                     }
                     flushed = true;
 #pragma unroll
@@ -272,36 +303,32 @@ __global__ void __launch_bounds__(CH == 1 ? 608 : 576, 1) k_sweep(SweepArgs a) {
             df_add(CS[j].x, CC[j].x, cs[j].x, cc[j].x);
             df_add(CS[j].y, CC[j].y, cs[j].y, cc[j].y);
         }
-        if constexpr (CH == 1) {
-            if (G > 1) {   // the groups' sums meet in shared memory, group 0 adds them up in order
-                asm volatile("bar.sync 1, 512;" ::: "memory");   // every warp is through with the ring
-                float4 *gp = reinterpret_cast<float4 *>(sw_smem);            // [2][512]: pairs of columns
-                float4 *gv = gp + 2 * kSwC;                                  // [512]
-                double *ga = reinterpret_cast<double *>(gv + kSwC);          // [512][4]
-                gp[tid] = make_float4(CS[0].x, CC[0].x, CS[0].y, CC[0].y);
-                gp[kSwC + tid] = make_float4(CS[1].x, CC[1].x, CS[1].y, CC[1].y);
-                gv[tid] = make_float4(cv[0].x, cv[0].y, cv[1].x, cv[1].y);
-                if (flushed)
+        if (G > 1) {   // the groups' sums meet in shared memory, group 0 adds them up in order
+            asm volatile("bar.sync 1, 512;" ::: "memory");   // every warp is through with the ring
+            float4 *gp = reinterpret_cast<float4 *>(sw_smem);            // [2 CH][512]: pairs of columns
+            float4 *gv = gp + 2 * CH * kSwC;                             // [CH][512]
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) ga[4 * tid + q] = cacc[q];
-                asm volatile("bar.sync 1, 512;" ::: "memory");
-                if (g == 0)
-                    for (int x = 1; x < G; ++x) {
-                        const int o = x * T + t;
+            for (int j = 0; j < 2 * CH; ++j) gp[j * kSwC + tid] = make_float4(CS[j].x, CC[j].x, CS[j].y, CC[j].y);
 #pragma unroll
-                        for (int j = 0; j < 2; ++j) {
-                            const float4 v = gp[j * kSwC + o];
-                            df_add(CS[j].x, CC[j].x, v.x, v.y);
-                            df_add(CS[j].y, CC[j].y, v.z, v.w);
-                        }
-                        const float4 v = gv[o];
-                        cv[0] = make_float2(cv[0].x + v.x, cv[0].y + v.y);
-                        cv[1] = make_float2(cv[1].x + v.z, cv[1].y + v.w);
-                        if (flushed)
+            for (int ch = 0; ch < CH; ++ch)
+                gv[ch * kSwC + tid] = make_float4(cv[2 * ch].x, cv[2 * ch].y, cv[2 * ch + 1].x, cv[2 * ch + 1].y);
+            asm volatile("bar.sync 1, 512;" ::: "memory");
+            if (g == 0)
+                for (int x = 1; x < G; ++x) {
+                    const int o = x * T + t;
 #pragma unroll
-                            for (int q = 0; q < 4; ++q) cacc[q] += ga[4 * o + q];
+                    for (int j = 0; j < 2 * CH; ++j) {
+                        const float4 v = gp[j * kSwC + o];
+                        df_add(CS[j].x, CC[j].x, v.x, v.y);
+                        df_add(CS[j].y, CC[j].y, v.z, v.w);
                     }
-            }
+#pragma unroll
+                    for (int ch = 0; ch < CH; ++ch) {
+                        const float4 v = gv[ch * kSwC + o];
+                        cv[2 * ch] = make_float2(cv[2 * ch].x + v.x, cv[2 * ch].y + v.y);
+                        cv[2 * ch + 1] = make_float2(cv[2 * ch + 1].x + v.z, cv[2 * ch + 1].y + v.w);
+                    }
+                }
         }
         if (g == 0)
 #pragma unroll
@@ -310,56 +337,51 @@ __global__ void __launch_bounds__(CH == 1 ? 608 : 576, 1) k_sweep(SweepArgs a) {
                 if (p >= a.n) continue;
                 const float2 A = CS[q >> 1], B = CC[q >> 1], V = cv[q >> 1];
                 double v = (double)(q & 1 ? A.y : A.x) + (double)(q & 1 ? B.y : B.x);
-                const size_t at = (size_t)blockIdx.x * a.n + p;
-                if (flushed) {
-                    if constexpr (CH == 1) v += cacc[q];
-                    else v += a.pu[at];
-                }
-                a.pu[at] = v;
-                a.pv[at] = q & 1 ? V.y : V.x;
+                double *at = a.pu + (size_t)blockIdx.x * G * a.n + p;
+                if (flushed)
+                    for (int x = 0; x < G; ++x) v += at[(size_t)x * a.n];
+                *at = v;
+                a.pv[(size_t)blockIdx.x * a.n + p] = q & 1 ? V.y : V.x;
             }
     } else if (wid == 16) {
         // ---- loads
         int slot = 0;
         uint32_t ph = 1;   // of the slot's previous use
-        int hs = 0;
-        for (; hs < 2 * nbat && ok; ++hs) {
-            if (hs >= S) ok = __all_sync(0xffffffffu, tc::mbar_wait(&empty[slot], ph));
+        int b = 0;
+        for (; b < nbat; ++b) {
+            if (b >= S) ok = __all_sync(0xffffffffu, tc::mbar_wait(&empty[slot], ph));
             if (!ok) break;
-            const int64_t i = r0 + (int64_t)hs * HR;
-            const int vr = (int)max((int64_t)0, min((int64_t)HR, r1 - i));
-            const uint32_t bytes = (uint32_t)(vr * lda * (int64_t)sizeof(float));
+            const uint32_t bytes = (uint32_t)(min(RB, nrow - b * RB) * lda) * (uint32_t)sizeof(float);
             if (lane == 0) tc::mbar_expect_tx(&full[slot], 2 * bytes);
             __syncwarp();
-            if (lane < 2 && vr > 0)
-                tc::bulk_load(sw_smem + (size_t)slot * slot_bytes + (size_t)lane * HR * lda * sizeof(float),
-                              (lane ? a.Alo : a.Ahi) + i * lda, bytes, &full[slot]);
+            if (lane < 2)
+                tc::bulk_load(sw_smem + slot * slot_bytes + lane * (slot_bytes / 2),
+                              (lane ? a.Alo : a.Ahi) + (r0 + (int64_t)b * RB) * lda, bytes, &full[slot]);
             if (++slot == S) slot = 0, ph ^= 1;
         }
         if (!ok && lane == 0) atomicExch(a.err, 1);
         // no copy is in flight when the CTA leaves
-        for (int x = max(0, hs - S); x < hs; ++x) tc::mbar_wait(&full[x % S], (uint32_t)(x / S) & 1);
+        for (int x = max(0, b - S); x < b; ++x) tc::mbar_wait(&full[x % S], (uint32_t)(x / S) & 1);
     } else {
         // ---- finishing warps: lane = (row, warp sum)
-        const int idx = 32 * (wid - 17) + lane, rho = idx / W, sub = idx - rho * W;
-        const bool lead = sub == 0;
-        for (int b = 0; b < nbat && ok; ++b) {
-            const int64_t i = r0 + (int64_t)b * RB + rho;
-            const bool live = i < r1;
+        const int me = wid - 17, rho = lane / W, sub = lane - rho * W;
+        const bool mine = lane < kVals, lead = mine && sub == 0;
+        uint32_t ph = 0;
+        int e0 = 0, e1 = 0;
+        auto rows_entries = [&](int b) {   // the row's entries, loaded a turn ahead
+            const int x = b * RB + rho;
+            const bool live = mine && x < nrow && b < nbat;
+            e0 = live ? __ldg(a.csr_ptr + r0 + x) : 0;
+            e1 = live ? __ldg(a.csr_ptr + r0 + x + 1) : 0;
+        };
+        rows_entries(me);
+        for (int b = me; b < nbat; b += 3) {
+            const bool live = mine && b * RB + rho < nrow;
+            const int64_t i = r0 + b * RB + rho;
             double ug = 0.0, bt = 0.0, winv = 0.0, bg = 0.0;
             float wf = 0.0f;
-            int e0 = 0, e1 = 0;
-            if (live) {
-                bg = __ldg(a.b_g + i);
-                winv = __ldg(a.winv + i);
-                wf = __ldg(a.wf + i);
-                bt = a.bt[i];
-                ug = a.init ? 0.0 : a.u_g[i];
-                e0 = __ldg(a.csr_ptr + i);
-                e1 = __ldg(a.csr_ptr + i + 1);
-            }
             // the row's sparse entries over its lanes; the first one's data now
-            const int most = __reduce_max_sync(0xffffffffu, e1 - e0);
+            const int f0 = e0 + sub, f1 = e1, most = __reduce_max_sync(0xffffffffu, e1 - e0);
             double J = 0.0, bc = 0.0, uc = 0.0, rcv = 0.0, q = 0.0, qi = 0.0;
             auto entry = [&](int e) {
                 const int cidx = __ldg(a.csr_col + e);
@@ -370,11 +392,19 @@ __global__ void __launch_bounds__(CH == 1 ? 608 : 576, 1) k_sweep(SweepArgs a) {
                 uc = a.init ? 0.0 : __ldg(a.u_s + cidx);
                 rcv = a.init ? bc : __ldg(a.r_s + cidx);
             };
-            if (e0 + sub < e1) entry(e0 + sub);
-            ok = __all_sync(0xffffffffu, tc::mbar_wait(&rowdone[b & 1], (uint32_t)(b >> 1) & 1));
+            if (f0 < f1) entry(f0);
+            if (live) {
+                bg = __ldg(a.b_g + i);
+                winv = __ldg(a.winv + i);
+                wf = __ldg(a.wf + i);
+                bt = a.bt[i];
+                ug = a.init ? 0.0 : a.u_g[i];
+            }
+            rows_entries(b + 3);
+            ok = __all_sync(0xffffffffu, tc::mbar_wait(&rowdone[me], ph));
             if (!ok) break;
-            const float4 v = s_red[b & 1][idx];
-            float s = v.x, c = v.y, d = v.z;
+            ph ^= 1;
+            float s = mine ? s_red[me][lane].x : 0.0f, c = mine ? s_red[me][lane].y : 0.0f, d = mine ? s_red2[me][lane] : 0.0f;
             for (int o = 1; o < W; o <<= 1) {
                 const float es = __shfl_xor_sync(0xffffffffu, s, o), ec = __shfl_xor_sync(0xffffffffu, c, o);
                 d += __shfl_xor_sync(0xffffffffu, d, o);
@@ -383,8 +413,8 @@ __global__ void __launch_bounds__(CH == 1 ? 608 : 576, 1) k_sweep(SweepArgs a) {
             const double sol = ((double)d - bt) * winv;
             const double un = ug + sol;
             double part = 0.0;
-            for (int e = e0 + sub; e < e1; e += W) {
-                if (e != e0 + sub) entry(e);
+            for (int e = f0; e < f1; e += W) {
+                if (e != f0) entry(e);
                 const double us = new_us(uc, rcv, J, sol, qi);
                 const double rs = bc - fma(J, un, q * us);
                 part = fma(-J, us, part);
@@ -393,18 +423,18 @@ __global__ void __launch_bounds__(CH == 1 ? 608 : 576, 1) k_sweep(SweepArgs a) {
             for (int o = 1; o < W && o < most; o <<= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
             const double Au = (double)s + (double)c;
             const double btn = (fma(a.dc, un, bg) + part) - Au;
-            const float uh = (float)un;
             if (lead) {
-                s_y[b & 1][rho] = make_float4(uh, (float)(un - (double)uh), (float)btn * wf, 0.0f);
-                if (live) {
-                    a.u_g[i] = un;
-                    a.sol_g[i] = sol;
-                    a.bt[i] = btn;
-                    a.Au[i] = Au;
-                }
+                const float2 y = split64(un);
+                s_y[me][rho] = make_float4(y.x, y.y, (float)btn * wf, 0.0f);
             }
             __syncwarp();
-            if (lane == 0) tc::mbar_arrive(&rowready[b & 1]);
+            if (lane == 0) tc::mbar_arrive(&rowready[me]);
+            if (lead && live) {
+                a.u_g[i] = un;
+                a.sol_g[i] = sol;
+                a.bt[i] = btn;
+                a.Au[i] = Au;
+            }
         }
         if (!ok && lane == 0) atomicExch(a.err, 1);
     }
@@ -483,10 +513,10 @@ __global__ void __launch_bounds__(NT) k_sweep_residual(
     const double *__restrict__ q, const double *__restrict__ qinv, const double *__restrict__ sig_xd,
     const double *__restrict__ sig_d, const double *__restrict__ Jdh, const double *__restrict__ Au,
     const double *__restrict__ sol_g, const double *__restrict__ Hu, const double *__restrict__ xnew,
-    const double *__restrict__ pu, const float *__restrict__ pv, int nparts, int init, double dw, double dc,
+    const double *__restrict__ pu, const float *__restrict__ pv, int nparts, int pstep, int init, double dw, double dc,
     double *__restrict__ ATu, double *__restrict__ rhsS, RedOut red) {
-    __shared__ double sp[NT / 32][33], su[NT / 32][33];
-    __shared__ float2 sv[NT / 32][33];
+    __shared__ double su[NT / 32][8], sj[NT / 32][8];
+    __shared__ float2 sv[NT / 32][8];
     unsigned long long rm = 0, bm = 0, km = 0, um = 0;
     const int64_t gtid = (int64_t)blockIdx.x * NT + threadIdx.x, gsz = (int64_t)gridDim.x * NT;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -499,32 +529,45 @@ __global__ void __launch_bounds__(NT) k_sweep_residual(
         max_abs(um, ui);
         return ri;
     };
-    for (int64_t k0 = (int64_t)blockIdx.x * 32; k0 < D.n_d; k0 += (int64_t)gridDim.x * 32) {
-        const double jt = colgroup_dot<NT>(Jdh, D.m_I, D.n_d, k0, xnew + D.n_d, sp);
-        const int64_t k = k0 + lane;
-        double s = 0.0;
+    // eight dense columns per block at a time: 32 threads share a column's partial
+    // sums (five rows each for 152 CTAs) and its part of J_dh^T u_h
+    for (int64_t k0 = (int64_t)blockIdx.x * 8; k0 < D.n_d; k0 += (int64_t)gridDim.x * 8) {
+        const int64_t k = k0 + (threadIdx.x & 7);
+        double s = 0.0, jt = 0.0;
         float vs = 0.0f, vc = 0.0f;
-        if (k < D.n_d)
+        if (k < D.n_d) {
 #pragma unroll 4
-            for (int p = wid; p < nparts; p += NT / 32) {
-                s += pu[(size_t)p * D.n_d + k];
+            for (int p = threadIdx.x >> 3; p < nparts; p += NT / 8) {
+                s += pu[(size_t)p * pstep * D.n_d + k];
                 df_add(vs, vc, pv[(size_t)p * D.n_d + k], 0.0f);
             }
-        __syncthreads();
-        su[wid][lane] = s;
-        sv[wid][lane] = make_float2(vs, vc);
-        __syncthreads();
-        if (wid == 0 && k < D.n_d) {
-            double at = 0.0;
+            for (int64_t j = threadIdx.x >> 3; j < D.m_I; j += NT / 8) jt = fma(Jdh[j * D.n_d + k], xnew[D.n_d + j], jt);
+        }
 #pragma unroll
-            for (int x = 0; x < NT / 32; ++x) {
-                at += su[x][lane];
-                if (x) df_add(vs, vc, sv[x][lane].x, sv[x][lane].y);
+        for (int o = 8; o < 32; o <<= 1) {
+            s += __shfl_xor_sync(0xffffffffu, s, o);
+            jt += __shfl_xor_sync(0xffffffffu, jt, o);
+            const float es = __shfl_xor_sync(0xffffffffu, vs, o), ec = __shfl_xor_sync(0xffffffffu, vc, o);
+            df_add(vs, vc, es, ec);
+        }
+        __syncthreads();   // an earlier group's sums are read
+        if (lane < 8) {
+            su[wid][lane] = s;
+            sj[wid][lane] = jt;
+            sv[wid][lane] = make_float2(vs, vc);
+        }
+        __syncthreads();
+        if (threadIdx.x < 8 && k < D.n_d) {
+#pragma unroll
+            for (int x = 1; x < NT / 32; ++x) {
+                s += su[x][lane];
+                jt += sj[x][lane];
+                df_add(vs, vc, sv[x][lane].x, sv[x][lane].y);
             }
             const double x = xnew[k];
-            ATu[k] = at;
+            ATu[k] = s;
             u[D.n_s + k] = x;
-            const double ri = put(D.n_s + k, Hu[k] + (sig_xd[k] + dw) * x + at + jt, x);
+            const double ri = put(D.n_s + k, Hu[k] + (sig_xd[k] + dw) * x + s + jt, x);
             rhsS[k] = ri + ((double)vs + (double)vc);
         }
     }
@@ -560,26 +603,35 @@ __global__ void __launch_bounds__(NT) k_sweep_residual(
 
 int grid_for(int64_t n) { return std::max(1, std::min(4096, ceil_div(std::max<int64_t>(n, 1), 256))); }
 
-template <int CH, int KBR>
-int launch_sweep_t(cudaStream_t st, int num_sms, SweepArgs a) {
+struct SweepParts {
+    int n, step;       // rows of partial sums, and their distance in rows
+    const float *pv;
+};
+
+template <int CH, int KBR, int kLag>
+SweepParts launch_sweep_t(cudaStream_t st, int num_sms, SweepArgs a) {
     a.T = 32;
     while (a.T < kSwC && 4 * CH * a.T < a.n) a.T *= 2;
-    const int G = kSwC / a.T, HR = G * KBR / 2;
-    const size_t slot = (size_t)2 * HR * a.lda * sizeof(float);
-    a.S = (int)std::min<size_t>(kSwMaxSlots, kSwRing / slot);
-    MDSIP_REQUIRE(a.S >= 5, MDSIP_ERR_INVALID_ARG, "refinement sweep: rows too long");
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(num_sms, kRedBlocks / 2), ceil_div(a.m, 2 * HR)));
-    a.pv = reinterpret_cast<float *>(a.pu + (size_t)grid * a.n);
+    const int RB = kSwC / a.T * KBR;
+    const size_t slot = (size_t)2 * RB * a.lda * sizeof(float);
+    a.S = (int)std::min<size_t>(kSwMaxSlots, kSwSmem / slot);
+    MDSIP_REQUIRE(a.S > kLag + 1, MDSIP_ERR_INVALID_ARG, "refinement sweep: rows too long");
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(std::min(num_sms, kRedBlocks / 2), ceil_div(a.m, RB)));
+    const size_t groups = (size_t)(kSwC / a.T);
+    a.pv = reinterpret_cast<float *>(a.pu + grid * groups * a.n);
     static PerDeviceOnce once;
     MDSIP_CUDA(once.run([] {
-        return cudaFuncSetAttribute(k_sweep<CH, KBR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSwRing);
+        return cudaFuncSetAttribute(k_sweep<CH, KBR, kLag>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSwSmem);
     }));
-    k_sweep<CH, KBR><<<grid, 32 * (17 + KBR / 2), std::max(kSwMin, a.S * slot), st>>>(a);
+    k_sweep<CH, KBR, kLag><<<grid, kSwThreads, std::max(kSwMin, a.S * slot), st>>>(a);
     MDSIP_LAUNCHED();
-    return grid;
+    return SweepParts{grid, (int)groups, a.pv};
 }
 
 }  // namespace
+
+// doubles of Refiner::colpart that a sweep's partial sums take
+int64_t refine_sweep_parts(int64_t n) { return kRedBlocks / 2 * std::max<int64_t>(8192, 2 * n); }
 
 // FP32 tiles of a tensor-core factor with the FP32 pair of A; above 4096
 // columns a batch and its predecessor no longer fit the shared memory together
@@ -628,10 +680,11 @@ void Refiner::sweep(const double *b, double *u, double *r, bool init, double dw,
     a.init = init ? 1 : 0;
     a.pu = colpart;
     a.err = solve_err;
-    const int grid = D.n_d <= 4 * kSwC ? launch_sweep_t<1, 4>(st, num_sms, a) : launch_sweep_t<2, 2>(st, num_sms, a);
-    k_sweep_residual<<<red_grid(std::max(std::max(D.n_s, D.m_E), (NT / 32) * D.n_d)), NT, 0, st>>>(
+    // up to 128 columns a warp of four columns a thread holds a row; wider rows go by eight
+    const SweepParts pt = D.n_d <= 128 ? launch_sweep_t<1, 2, 3>(st, num_sms, a) : launch_sweep_t<2, 2, 1>(st, num_sms, a);
+    k_sweep_residual<<<red_grid(std::max(std::max(D.n_s, D.m_E), 32 * D.n_d)), NT, 0, st>>>(
         D, M, b, u, r, q, qinv, sig_xd, sig_d, Jdh, tmp_m, sol_g, tmp_nd2, xnew, colpart,
-        reinterpret_cast<const float *>(colpart + (size_t)grid * D.n_d), grid, init ? 1 : 0, dw, dc, tmp_nd, rhsS,
+        pt.pv, pt.n, pt.step, init ? 1 : 0, dw, dc, tmp_nd, rhsS,
         RedOut{partial, reinterpret_cast<unsigned *>(partial + kRedBlocks * 8), out4});
     MDSIP_LAUNCHED();
 }

@@ -378,7 +378,7 @@ static Problem *create_common(Ctx *ctx, int64_t n_d, int64_t n_s, int64_t m_E, i
         dvec(ctx, P->bscal, SC_COUNT);
         dvec(ctx, P->bpartial, (int64_t)kRedBlocks * 8 + 1);   // partials and the reductions' ticket
         MDSIP_CUDA(cudaMemsetAsync(P->bpartial.as<double>() + kRedBlocks * 8, 0, sizeof(double), st));
-        dvec(ctx, P->bcolpart, (int64_t)kRedBlocks * std::max<int64_t>(D.n_d, 1));
+        dvec(ctx, P->bcolpart, std::max<int64_t>((int64_t)kRedBlocks * std::max<int64_t>(D.n_d, 1), refine_sweep_parts(D.n_d)));
         dvec(ctx, P->browtmp, std::max<int64_t>(D.m_E, 1));
         P->berr.get<int>(ctx, 4);
         MDSIP_CUDA(cudaMallocHost(&P->hscal, SC_COUNT * sizeof(double)));
