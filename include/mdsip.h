@@ -176,9 +176,8 @@ void mdsip_problem_destroy(mdsip_problem *p);
  *           shape; 0: the analytic choices),
  *           ldlt_spec (1, default: the mixed-precision factorization's
  *           panels first try the verified no-interchange path described at
- *           mdsip_ldlt_factor_ex, and from order 2048 on the persistent
- *           no-interchange kernel runs first in either precision; 2: that
- *           kernel at every order; 0: every panel pivots),
+ *           mdsip_ldlt_factor_ex, whose persistent kernel runs first in
+ *           either precision; 2: the same; 0: every panel pivots),
  *           direction_check (0, default; 1: every step of a mixed-precision
  *           solve also computes the FP64 direction from the same iterate and
  *           shifts and logs the relative gap as dir_err_fp64 -- an extra FP64
@@ -398,12 +397,11 @@ mdsip_status mdsip_ldlt_factor(mdsip_ctx *ctx, int64_t N, double *S, int64_t ld,
  * every column of the panel (and no pivot is below zero_tol times the
  * largest |S_ij|); otherwise the pivoting panel factors it from the
  * unchanged matrix.  The flag makes every panel take the pivoting kernel.
- * From order 2048 on (and wherever the pivoting panel does not fit shared
- * memory, N above about 16 000), and at any order with MDSIP_LDLT_PERSISTENT,
- * the no-interchange panels of either precision run in one persistent
- * cooperative kernel that stops at the first panel the rule would not keep;
- * the pivoting panels take over from there (beyond the pivoting panel's
- * limit such a panel is an INVALID_ARG error).  With FP32 updates that
+ * The no-interchange panels of either precision first run in one persistent
+ * cooperative kernel (with or without MDSIP_LDLT_PERSISTENT) that stops at the
+ * first panel the rule would not keep; the panels above take over from there
+ * (where the pivoting panel does not fit shared memory, N above about 16 000,
+ * such a panel is an INVALID_ARG error).  With FP32 updates that
  * kernel works on an FP32 copy of S (the FP32 updates are written back into
  * S before a hand-over; large trailing matrices are updated on the tensor
  * cores with a three-product TF32 split, about FP32 accuracy).  The call then
@@ -418,8 +416,8 @@ mdsip_status mdsip_ldlt_factor_ex(mdsip_ctx *ctx, int64_t N, double *S, int64_t 
 /* Panel counts of the last mdsip_ldlt_factor / mdsip_ldlt_factor_ex call on
  * ctx (host array of 2): out2[0] = panels kept by the verified
  * no-interchange path, out2[1] = panels it handed to the pivoting kernel.
- * Both are 0 when that path did not run (FP64 updates, MDSIP_LDLT_NO_SPECULATION,
- * or the unblocked kernel). */
+ * Both are 0 when that path did not run (MDSIP_LDLT_NO_SPECULATION or the
+ * unblocked kernel). */
 mdsip_status mdsip_ldlt_panel_counts(mdsip_ctx *ctx, int32_t *out2);
 
 /* Allocation-free variant of mdsip_ldlt_factor (same arguments, same

@@ -1850,9 +1850,12 @@ void launch_persist32(cudaStream_t s, int num_sms, int N, const PersistArgs &pa)
     int per_sm = 0;
     MDSIP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kPThreads, persist32_smem()));
     MDSIP_REQUIRE(per_sm >= 1, MDSIP_ERR_CUDA, "ldlt: persistent factorization does not fit an SM");
-    // about three trailing tiles per CTA after the first panel, at most one CTA per SM
+    // the first panel's trailing tiles twice over or four CTAs per tile column,
+    // whichever is more (rows per CTA set the panel's pace), at most one per SM
+    // (a third as many CTAs as tiles / so: N = 114 100 / 83 us, 200 157 / 121,
+    // 562 283 / 232, 1100 471 / 413, equal from 2050 on)
     const int64_t nt = std::max<int64_t>(1, (N - 64 + kUT - 1) / kUT);
-    const int64_t want = std::max<int64_t>(1, (nt * (nt + 1) / 2 + 2) / 3);
+    const int64_t want = std::max<int64_t>(4 * nt, nt * (nt + 1));
     const int G = (int)std::min<int64_t>(want, (int64_t)num_sms);
     PersistArgs args = pa;
     void *kargs[] = {&args};
@@ -1885,17 +1888,14 @@ std::vector<int> ldlt_blocked_widths(int64_t N, bool f32) {
 bool ldlt_blocked_available(int64_t N) { return blocked_config(N, true).C > 0 && blocked_config(N, false).C > 0; }
 
 // The persistent no-interchange factorization runs first (and the host reads
-// back where it stopped) in mode 2, in mode 1 at every order with FP64 updates
-// and from kPersistentMinOrder on with FP32 updates, and wherever the pivoting
-// panel does not fit shared memory: it needs no pivoting panel unless a panel
-// fails the column test, and a first panel that fails costs one short launch.
-// FP64, convex Newton-step shape, persistent / per-panel launches: N = 33
-// 0.10 / 0.14 ms, 351 0.46 / 1.47, 1036 1.31 / 4.46, 2050 2.83 / 11.1.
-// FP32 updates (the many small instances of a batch among them, whose
-// per-panel launches replay as one graph): N = 2050 0.82 / 1.73 ms.
-bool ldlt_persistent_path(int64_t N, int spec, bool fp32_update) {
-    if (spec == 0 || N <= 0 || N > (int64_t)0x7fffffff / 2) return false;
-    return spec == 2 || !fp32_update || N >= kPersistentMinOrder || !ldlt_blocked_available(N);
+// back where it stopped) at every order: it needs no pivoting panel unless a
+// panel fails the column test, and a first panel that fails costs one short
+// launch.  Convex Newton-step shape, persistent / per-panel launches, FP64: N =
+// 33 0.10 / 0.14 ms, 351 0.46 / 1.47, 1036 1.31 / 4.46, 2050 2.83 / 11.1; FP32
+// updates (whose per-panel launches replayed as one graph): N = 562 0.23 / 0.49, 2050
+// 0.82 / 1.73 ms; 24 solves of 114 to 350 at once 79 / 84 ms in all.
+bool ldlt_persistent_path(int64_t N, int spec) {
+    return spec != 0 && N > 0 && N <= (int64_t)0x7fffffff / 2;
 }
 
 // S (lower, ld N) is overwritten.  scratch: ldlt_blocked_scratch_bytes(N),
@@ -1909,7 +1909,7 @@ void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, cons
     }
     BlockedConfig cfg = blocked_config(N, fp32_update, nb);
     if (cfg.C == 0) cfg = blocked_config(N, fp32_update);
-    const bool persist = ldlt_persistent_path(N, spec, fp32_update);
+    const bool persist = ldlt_persistent_path(N, spec);
     MDSIP_REQUIRE(cfg.C > 0 || persist, MDSIP_ERR_INVALID_ARG, "ldlt: N too large for the blocked factorization");
     char *w = static_cast<char *>(scratch);
     MDSIP_REQUIRE((reinterpret_cast<uintptr_t>(w) & 255) == 0, MDSIP_ERR_INVALID_ARG, "ldlt: misaligned scratch");

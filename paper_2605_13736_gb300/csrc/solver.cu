@@ -758,7 +758,7 @@ static void run_factor_phase(Problem *P, int slot, F &&enqueue) {
     ++g.uses;
     // the persistent factorization reads back where it stopped: nothing to capture
     if (!P->opt.graphs || g.disabled || g.uses < 2 || !ldlt_blocked_available(P->N) ||
-        ldlt_persistent_path(P->N, (int)P->opt.ldlt_spec, slot == 1)) {
+        ldlt_persistent_path(P->N, (int)P->opt.ldlt_spec)) {
         enqueue();
         return;
     }
@@ -803,7 +803,7 @@ static void run_factor_phase(Problem *P, int slot, F &&enqueue) {
 static int tuned_ldlt_width(Problem *P, bool fp32) {
     const int64_t N = P->N;
     if (!P->opt.autotune || !ldlt_blocked_available(N)) return 0;
-    if (ldlt_persistent_path(N, (int)P->opt.ldlt_spec, fp32)) return 0;   // no panel launches to tune
+    if (ldlt_persistent_path(N, (int)P->opt.ldlt_spec)) return 0;   // no panel launches to tune
     int v = 0;
     if (tune_get(TUNE_LDLT_PANEL, N, fp32 ? 1 : 0, &v)) return v;
     const std::vector<int> cands = ldlt_blocked_widths(N, fp32);
