@@ -205,14 +205,15 @@ enum Scalar : int {
 // step are bound by the number of FP64 instructions on their longest chain:
 // tests and maxima work on bit patterns, divisions on the short reciprocal.
 // ---------------------------------------------------------------------------
-// 1/d by Newton-Raphson iteration x <- x (2 - d x) (0 for d = 0): the first
-// step in FP32 and integers on the mantissa m of d -- hardware reciprocal q of
-// m's upper 24 bits, the residual 1 - m q with all of m, x = q + q (e + e^2) in
-// units of 2^-53, good to about 2^-46 -- and the last in FP64.  Two FP64
-// instructions, where the FP32 conversions and two FP64 steps were six: on
-// GB300 each occupies a warp's FP64 pipe for 64 cycles and every pivot waits
-// for this value.  d near the ends of the range goes through the division
-// operator.
+// 1/d by Newton-Raphson iteration x <- x (2 - d x) (0 for d = 0), on FP32 and
+// integers alone: hardware reciprocal q of the upper 24 bits of d's mantissa m,
+// the residual 1 - m q with all of m, x = q + q (e + e^2) as an integer X of
+// units 2^-53, good to about 2^-46; then the second step with M = 2^52 m: E =
+// 2^105 - M X fits 64 bits, and X + X E / 2^105 rounded is 1/m to 0.51 units in
+// the last place.  An FP64 instruction occupies a warp's pipe for 64 cycles and
+// every pivot waits for this value: the two that the second step took, and six
+// with conversions, were most of its latency.  d near the ends of the range
+// goes through the division operator.
 __device__ __forceinline__ double rcp_newton(double d) {
     const int hi = __double2hiint(d);
     const unsigned lo = (unsigned)__double2loint(d);
@@ -227,10 +228,12 @@ __device__ __forceinline__ double rcp_newton(double d) {
     const int c = __float2int_rn(fmaf(qe, e, qe) * 0x1p52f);       // |q e| < 2^-21
     const unsigned qb = __float_as_uint(q);                        // 1/2 <= q <= 1
     const long long X = ((long long)((qb & 0x7fffffu) | 0x800000u) << (29 + (int)(qb >> 23) - 126)) + 2LL * c;
-    const double x = __longlong_as_double((1021LL << 52) + X);     // 2^52 <= X <= 2^53 (as 1022 << 52 plus X - 2^52)
-    const double m = __hiloint2double((hi & 0xfffff) | 0x3ff00000, (int)lo);
-    const double y = fma(x, fma(-m, x, 1.0), x);                   // 1 / m
-    return __hiloint2double((__double2hiint(y) - ((ef - 1023) << 20)) | (hi & (int)0x80000000), __double2loint(y));
+    const unsigned long long M = ((unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32) | lo;
+    const long long E = -(long long)(M * (unsigned long long)X);   // |E| < 2^60
+    const long long t = (long long)(int)(E >> 30) * (long long)(int)(X >> 23);
+    const long long Y = X + ((t + (1LL << 51)) >> 52);             // 2^52 <= Y <= 2^53
+    const long long y = (1021LL << 52) + Y;                        // as 1022 << 52 plus Y - 2^52
+    return __hiloint2double(((int)(y >> 32) - ((ef - 1023) << 20)) | (hi & (int)0x80000000), (int)y);
 }
 
 // a / b: reciprocal, product and one residual correction (Markstein 1990), five

@@ -12,9 +12,9 @@
 // off that pipe altogether.  Per panel:
 //   A  every CTA factors the 32 x 32 diagonal block and its own rows below it
 //      in shared memory, in two 16-column sub-panels: the 16 x 16 sub-block one
-//      lower-triangle element per thread (one multiply, one FMA and a
-//      reciprocal per column and warp), the rows four threads each, then a
-//      rank-16 update of the rest; L, D, the column maxima;
+//      lower-triangle element per thread (one multiply and one FMA per column
+//      and warp) with the rows beside it, four threads each, then a rank-16
+//      update of the rest; L, D, the column maxima;
 //   R  the rows' W scaled by |d|^-1/2 and rounded once to 54-bit integers per
 //      row, as residues modulo 13 coprime moduli in BF16 (rns.cuh);
 //   B  grid barrier, the column test, the same decision in every CTA;
@@ -24,11 +24,11 @@
 //      subtraction per entry): sum_j sign(d_j) X_ij X_cj <= 32 2^108 in exact
 //      integers, an error below that of a 32-term FP64 dot product; grid barrier.
 // Against the 64-column form with DFMA trailing tiles (its first panel's tiles
-// alone took 215 us): N = 2050 7.90 -> 2.83 ms, 4050 30.6 -> 8.9 ms.  Of the 45
-// us a panel takes at N = 2050 the pivot chain is 10 (32 columns of three
-// dependent FP64 instructions, a reciprocal's FP32 part and a barrier), the
-// rows and the rank-16 update 8, the tiles 16, grid barriers with the skew
-// between CTAs 5.
+// alone took 215 us): N = 2050 7.90 -> 2.42 ms, 4050 30.6 -> 8.1 ms.  A panel
+// takes 30 us at N = 351 to 1036, its pivot chain about 12 of them (32 columns
+// of an FP64 multiply and FMA, a reciprocal, an exchange); at N = 2050 37 us, 16
+// of them the tiles, whose read-back (13 residues to 128-bit integers per
+// entry) is bound by the integer pipes.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -47,11 +47,11 @@ using bf16 = __nv_bfloat16;
 constexpr int RL = 13;                  // moduli: log2 of their product 116.3
 constexpr int QB = 54;                  // 2 QB + 5 + 2 <= 116
 constexpr int QN = 32;                  // panel width
-constexpr int Q_THREADS = 576;          // warps 0-7 factor; 0-15 update, 16 loads, 17 issues
+constexpr int Q_THREADS = 544;          // warps 0-7 factor; 0-15 update, 0-12 issue a modulus each, 16 loads
 constexpr int Q_COMP = 256;             // threads of the factorization
 constexpr int Q_EPI = 16;               // warps of the trailing update
 constexpr int Q_OWN = 96;               // rows below the block staged at a time
-constexpr int VP = 33, LP = 17;         // shared-memory row pitches (doubles)
+constexpr int VP = 33, LP = 33;         // shared-memory row pitches (doubles)
 constexpr int QA_BYTES = 128 * 64, QB_BYTES = 32 * 64;   // residues of 128 rows / 32 rows, 32 BF16 each
 constexpr int Q_STAGE = QA_BYTES + QB_BYTES;             // one modulus; a tile's 13 are loaded together
 constexpr size_t kQSmem = 1024 + (size_t)RL * Q_STAGE + (size_t)(QN + Q_OWN) * (VP + LP) * sizeof(double);
@@ -71,36 +71,82 @@ struct P64Args {
 __device__ __forceinline__ void bar_comp() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 __device__ __forceinline__ void bar_chain() { asm volatile("bar.sync 2, 128;" ::: "memory"); }
 
-// The 16 x 16 diagonal sub-block at c0 (threads 0 .. 127): thread = one element
-// (ei, ej) of the lower triangle, ej >= 1.  Column j goes through `col` (two
-// buffers, one barrier per column); v_it -= (w_i w_t) / d.
-__device__ void q_chain(double *V, double *col, double *s_rc, int c0, int cw, int ei, int ej) {
-    const int tid = threadIdx.x;
-    double v = ei < cw && ej > 0 ? V[(c0 + ei) * VP + c0 + ej] : 0.0;
-    for (int j = 0; j < cw; ++j) {
-        double *cb = col + (j & 1) * 16;
-        if (j == 0) {
-            if (tid < 16) cb[tid] = V[(c0 + tid) * VP + c0];
-        } else if (ej == j) {
-            cb[ei] = v;
-            V[(c0 + ei) * VP + c0 + j] = v;
+// The 16 x 16 diagonal sub-block at c0 and up to 32 rows below it, together.
+// Warps 0 .. 3 hold one element (ei, ej), ej >= 1, of the block's lower
+// triangle per lane, 30 lanes each; column j goes through `col` (two buffers of
+// 17, one barrier per column); v_it -= (w_i w_t) / d.  Lane 31 of each also
+// forms the next pivot from its value before the column (col[16]), so that its
+// reciprocal is under way while the column's elements are exchanged: a column
+// is one FMA, a reciprocal and two shuffles of latency.  Warps 4 .. 7 take the
+// rows on the FP64 pipes that the chain leaves idle, four threads each with
+// columns strided by four.  (Chain and rows one after the other, with the
+// second Newton step on the FP64 pipe, took 31 of a panel's 77 thousand cycles.)
+__device__ bool q_chain_rows(double *V, double *Ls, double *col, double *s_rc, uint64_t *colbar, uint32_t phase, int c0,
+                             int cw, int ei, int ej, int nblk, int nr) {
+    bool ok = true;
+    const int tid = threadIdx.x, lane = tid & 31;
+    if (tid < 128) {
+        const bool elem = lane < 30;
+        double v = elem && ei < cw ? V[(c0 + ei) * VP + c0 + ej] : 0.0;
+        double r = rcp_newton(V[c0 * VP + c0]);
+        for (int j = 0; j < cw; ++j) {
+            double *cb = col + (j & 1) * 17;
+            if (j == 0) {
+                if (tid < 16) cb[tid] = V[(c0 + tid) * VP + c0];
+                if (tid == 16) cb[16] = V[(c0 + 1) * VP + c0 + 1];
+            } else if (elem && ej == j) {
+                cb[ei] = v;
+                V[(c0 + ei) * VP + c0 + j] = v;
+            }
+            if (j > 0 && elem && ei == j + 1 && ej == j + 1) cb[16] = v;
+            if (tid == 0) s_rc[c0 + j] = r;
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(&colbar[j]);
+            bar_chain();
+            if (j + 1 < cw) {
+                const bool nd = lane == 31;
+                const double wi = cb[nd ? j + 1 : ei], wt = cb[nd ? j + 1 : ej];
+                const double nv = fma(-(wi * wt), r, nd ? cb[16] : v);
+                if (ej > j) v = nv;
+                r = rcp_newton(__shfl_sync(0xffffffffu, nv, 31));
+            }
         }
-        bar_chain();
-        const double d = cb[j];
-        const double u = ej > j ? cb[ei] * cb[ej] : 0.0;
-        const double r = rcp_newton(d);
-        if (tid == 0) s_rc[c0 + j] = r;
-        if (ej > j) v = fma(-u, r, v);
+    } else {
+        const int q = lane & 3, x = (tid - 128) >> 2, total = min(32, nblk + nr);
+        const bool live = x < total;
+        const int row = live ? (x < nblk ? c0 + 16 + x : QN + x - nblk) : c0;
+        double v[4];
+#pragma unroll
+        for (int s = 0; s < 4; ++s) v[s] = live ? V[row * VP + c0 + q + 4 * s] : 0.0;
+        const bool any = __any_sync(0xffffffffu, live);
+        for (int j = 0; j < cw; ++j) {
+            if (!any) break;
+            if (!tc::mbar_wait(&colbar[j], phase)) ok = false;   // column j and its reciprocal are there
+            const int sl = j >> 2;
+            const double own = sl == 0 ? v[0] : sl == 1 ? v[1] : sl == 2 ? v[2] : v[3];
+            const double l = __shfl_sync(0xffffffffu, own, (lane & ~3) | (j & 3)) * s_rc[c0 + j];
+            if (live && (j & 3) == q) Ls[row * LP + c0 + j] = l;
+#pragma unroll
+            for (int s = 0; s < 4; ++s)
+                if (4 * s + 3 > j) {
+                    const int t = q + 4 * s;
+                    v[s] = fma(-l, t > j ? V[(c0 + t) * VP + c0 + j] : 0.0, v[s]);
+                }
+        }
+        if (live) {
+#pragma unroll
+            for (int s = 0; s < 4; ++s) V[row * VP + c0 + q + 4 * s] = v[s];
+        }
     }
+    return ok;
 }
 
-// Rows below the sub-block at c0 (block rows c0 + 16 .. nb - 1 when blk, then
-// the nr staged own rows): four threads per row, columns strided by four.
-__device__ void q_rows(double *V, double *Ls, const double *s_rc, int c0, int nb, bool blk, int nr) {
-    const int nblk = blk ? max(0, nb - c0 - 16) : 0;
+// Rows x0 .. of those below the sub-block at c0 (nblk block rows from c0 + 16 on,
+// then the nr staged own rows): four threads per row, columns strided by four.
+__device__ void q_rows(double *V, double *Ls, const double *s_rc, int c0, int first, int nblk, int nr) {
     const int total = nblk + nr;
     const int lane = threadIdx.x & 31, q = lane & 3;
-    for (int x0 = 0; x0 < total; x0 += Q_COMP / 4) {
+    for (int x0 = first; x0 < total; x0 += Q_COMP / 4) {
         const int x = x0 + (threadIdx.x >> 2);
         const bool live = x < total;
         if (!__any_sync(0xffffffffu, live)) break;   // warp-uniform: no row in this warp
@@ -112,7 +158,7 @@ __device__ void q_rows(double *V, double *Ls, const double *s_rc, int c0, int nb
         for (int j = 0; j < 16; ++j) {
             const double w = __shfl_sync(0xffffffffu, v[j >> 2], (lane & ~3) | (j & 3));
             const double l = w * s_rc[c0 + j];
-            if (live && (j & 3) == q) Ls[row * LP + j] = l;
+            if (live && (j & 3) == q) Ls[row * LP + c0 + j] = l;
             if (j < 15) {
 #pragma unroll
                 for (int s = j >> 2; s < 4; ++s) {
@@ -162,12 +208,13 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
     extern __shared__ uint8_t psm_raw[];
     uint8_t *ring = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(psm_raw) + 1023) & ~uintptr_t(1023));
     double *V = reinterpret_cast<double *>(ring + RL * Q_STAGE);   // [32 + Q_OWN][VP]: block rows, own rows
-    double *Ls = V + (QN + Q_OWN) * VP;                                  // [32 + Q_OWN][LP]: L of the first sub-panel
-    __shared__ double s_d[QN], s_rc[QN], s_col[32];
+    double *Ls = V + (QN + Q_OWN) * VP;                            // [32 + Q_OWN][LP]: L below the 16 x 16 sub-blocks
+    __shared__ double s_d[QN], s_rc[QN], s_col[34];
     __shared__ unsigned long long s_cmax[QN], s_sm[QN];
     __shared__ int s_se[QN];
     __shared__ uint4 s_km[16];   // -(bias + k M) modulo 2^128, k = -8 .. 7 at k + 8
-    __shared__ __align__(8) uint64_t full, tfull, tempty;   // operands loaded, products done, accumulators read
+    __shared__ __align__(8) uint64_t full[RL], tfull, tempty;   // a modulus loaded, products done, accumulators read
+    __shared__ __align__(8) uint64_t colbar[16];   // the chain's columns
     __shared__ uint32_t s_tmem;
     const int N = a.N, G = (int)gridDim.x, g = (int)blockIdx.x, tid = threadIdx.x;
     const int lane = tid & 31, wid = tid >> 5;
@@ -176,8 +223,9 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
     // pivoting panels take such a matrix (st->k stays where it is)
     if (!(maxabs > 0x1p-900)) return;
     if (tid == 0) {
-        tc::mbar_init(&full, 1);
-        tc::mbar_init(&tfull, 1);
+        for (int l = 0; l < RL; ++l) tc::mbar_init(&full[l], 1);
+        for (int j = 0; j < 16; ++j) tc::mbar_init(&colbar[j], 4);
+        tc::mbar_init(&tfull, RL);
         tc::mbar_init(&tempty, Q_EPI);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -197,20 +245,22 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
     const uint32_t tmem = s_tmem;
     int tl = 0;   // tiles this warp's role has gone through
     auto release = [&]() {
-        if (wid == Q_EPI && tl > 0) tc::mbar_wait(&full, (tl - 1) & 1);   // no copy is in flight when the CTA leaves
+        if (wid == Q_EPI && tl > 0 && lane < RL) tc::mbar_wait(&full[lane], (tl - 1) & 1);   // no copy is in flight when the CTA leaves
+        __syncwarp();
         tc::fence_before();
         __syncthreads();
         if (wid == 0) tc::tmem_dealloc(tmem, 512);
     };
     // this thread's element of a 16 x 16 lower triangle without its first column
     int ei = 0, ej = 0;
-    if (tid < 120) {
-        int e = tid;
+    if (tid < 128 && lane < 30) {
+        int e = 30 * wid + lane;
         for (ej = 1; e >= 16 - ej; ++ej) e -= 16 - ej;
         ei = ej + e;
     }
 
     unsigned epoch = 0;   // grid barriers passed (thread 0)
+    uint32_t sub = 0;     // sub-panels gone through
     int p = 0;
     for (int k = a.st->k; k < N; k += QN, ++p) {
         const int nb = min(QN, N - k);
@@ -223,36 +273,57 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
             for (int cb = r_begin, first = 1; first || cb < r_end; cb += Q_OWN, first = 0) {
                 const int nr = max(0, min(Q_OWN, r_end - cb));
                 // ---- stage the block (first time) and the own rows
-                if (first) {
-                    for (int e = tid; e < QN * QN; e += Q_COMP) {
-                        const int c = e >> 5, r = e & 31;
-                        V[r * VP + c] = (r < nb && c <= r) ? __ldcg(a.A + (int64_t)(k + r) + (int64_t)(k + c) * N) : 0.0;
-                    }
-                    if (tid < QN) {
-                        s_cmax[tid] = 0ULL;
-                        s_rc[tid] = 0.0;    // columns beyond a narrow last panel stay zero
-                    }
-                }
+                {
+                    double sb[QN * QN / Q_COMP], so[QN / 8];   // every load in flight before the first store
 #pragma unroll
+                    for (int x = 0; x < QN * QN / Q_COMP; ++x) {
+                        const int c = wid + 8 * x;
+                        sb[x] = first && lane < nb && c <= lane ? __ldcg(a.A + (int64_t)(k + lane) + (int64_t)(k + c) * N) : 0.0;
+                    }
+#pragma unroll
+                    for (int x = 0; x < QN / 8; ++x) {
+                        const int c = wid + 8 * x;
+                        so[x] = lane < nr && c < nb ? __ldcg(a.A + (int64_t)(cb + lane) + (int64_t)(k + c) * N) : 0.0;
+                    }
+                    if (first) {
+#pragma unroll
+                        for (int x = 0; x < QN * QN / Q_COMP; ++x) V[lane * VP + wid + 8 * x] = sb[x];
+                        if (tid < QN) {
+                            s_cmax[tid] = 0ULL;
+                            s_rc[tid] = 0.0;    // columns beyond a narrow last panel stay zero
+                        }
+                    }
+                    if (lane < nr)
+#pragma unroll
+                        for (int x = 0; x < QN / 8; ++x) V[(QN + lane) * VP + wid + 8 * x] = so[x];
+                }
                 for (int c = wid; c < QN; c += 8)
-                    for (int r = lane; r < nr; r += 32)
+                    for (int r = lane + 32; r < nr; r += 32)
                         V[(QN + r) * VP + c] = c < nb ? __ldcg(a.A + (int64_t)(cb + r) + (int64_t)(k + c) * N) : 0.0;
                 bar_comp();
                 // ---- factor and solve
                 for (int c0 = 0; c0 < nb; c0 += 16) {
+                    const int nblk = first ? max(0, nb - c0 - 16) : 0;
                     if (first) {
-                        if (tid < 128) q_chain(V, s_col, s_rc, c0, min(16, nb - c0), ei, ej);
+                        if (!q_chain_rows(V, Ls, s_col, s_rc, colbar, sub & 1, c0, min(16, nb - c0), ei, ej, nblk, nr))
+                            atomicExch(&a.bar->err, 1);
+                        ++sub;
                         bar_comp();
                     }
-                    q_rows(V, Ls, s_rc, c0, nb, first, nr);
-                    bar_comp();
+                    if (!first || nblk + nr > 32) {
+                        q_rows(V, Ls, s_rc, c0, first ? 32 : 0, nblk, nr);
+                        bar_comp();
+                    }
                     if (c0 == 0 && nb > 16) {
                         q_rank16(V, Ls, nb, first, nr);
                         bar_comp();
                     }
                 }
-                if (first) {
-                    if (wid == 0) {   // pivots and their scaling |d|^-1/2
+                // ---- pivots and their scaling |d|^-1/2 (warp 0); the block's L and D and the
+                // column maxima of its rows, column c by CTA c mod G; the own rows' L and column
+                // maxima; a warp per column, lanes over rows
+                if (wid == 0) {
+                    if (first) {
                         const double d = lane < nb ? V[lane * VP + lane] : 0.0;
                         s_d[lane] = d;
                         unsigned long long m = 0ULL;
@@ -261,39 +332,32 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
                         if (ad > 0x1p-1000 && isfinite(ad)) rns::rsqrt64(ad, m, e);   // else the panel is rejected
                         s_sm[lane] = m;
                         s_se[lane] = e;
-                    } else {
-                        // the block's L and D and the column maxima of its rows: column c by
-                        // CTA c mod G, one warp per column, lanes over rows
-                        for (int c = g + G * (wid - 1); c < nb; c += G * 7) {
-                            const int r = lane;
-                            unsigned long long bm = 0ULL;
-                            if (r >= c && r < nb) {
-                                const int64_t o = (int64_t)(k + r) + (int64_t)(k + c) * N;
-                                const double w = V[r * VP + c];
-                                if (r == c) {
-                                    a.L[o] = 1.0;
-                                    a.Dd[k + c] = w;
-                                } else {
-                                    a.L[o] = w * s_rc[c];
-                                    bm = absbits64(w);
-                                }
-                            }
-                            q_colmax(bm, &s_cmax[c], lane);
+                    }
+                } else {
+                    for (int c = wid - 1; c < nb; c += 7) {
+                        unsigned long long bm = 0ULL;
+                        for (int r = lane; r < nr; r += 32) {
+                            const double w = V[(QN + r) * VP + c];
+                            a.L[(int64_t)(cb + r) + (int64_t)(k + c) * N] = Ls[(QN + r) * LP + c];
+                            const unsigned long long bw = absbits64(w);
+                            bm = bw > bm ? bw : bm;
                         }
+                        if (first && c % G == g && lane >= c && lane < nb) {
+                            const int64_t o = (int64_t)(k + lane) + (int64_t)(k + c) * N;
+                            const double w = V[lane * VP + c];
+                            if (lane == c) {
+                                a.L[o] = 1.0;
+                                a.Dd[k + c] = w;
+                            } else {
+                                a.L[o] = w * s_rc[c];
+                                const unsigned long long bw = absbits64(w);
+                                bm = bw > bm ? bw : bm;
+                            }
+                        }
+                        q_colmax(bm, &s_cmax[c], lane);
                     }
-                    bar_comp();
                 }
-                // ---- own rows: L, column maxima (a warp per column)
-                for (int c = wid; c < nb; c += 8) {
-                    unsigned long long bm = 0ULL;
-                    for (int r = lane; r < nr; r += 32) {
-                        const double w = V[(QN + r) * VP + c];
-                        a.L[(int64_t)(cb + r) + (int64_t)(k + c) * N] = w * s_rc[c];
-                        const unsigned long long bw = absbits64(w);
-                        bm = bw > bm ? bw : bm;
-                    }
-                    q_colmax(bm, &s_cmax[c], lane);
-                }
+                bar_comp();
                 // ---- own rows: residues (a warp per row, lane = panel column)
                 for (int r = wid; r < nr; r += 8) {
                     const double w = lane < nb ? V[(QN + r) * VP + lane] : 0.0;
@@ -365,14 +429,16 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
         if (k + nb >= N) break;
         // ---------------- trailing update: 128 x 32 tiles of the lower triangle
         const int base = k + nb, nbr = (N - base + 127) / 128;
-        const int tiles = 2 * nbr * (nbr + 1);
+        // 16 columns a tile when that still is one tile per CTA: half the read-back
+        const int tw = 4 * nbr * (nbr + 1) <= G ? 16 : 32, per = 64 / tw;
+        const int tiles = per * nbr * (nbr + 1);
         bool ok = true;
         auto tile_at = [&](int t, int &i0, int &c0) {   // false: beyond the last column
-            int tr = (int)((sqrtf(2.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
-            while (2 * (tr + 1) * (tr + 2) <= t) ++tr;
-            while (2 * tr * (tr + 1) > t) --tr;
+            int tr = (int)(sqrtf((float)t / (float)per + 0.25f) - 0.5f);
+            while (per * (tr + 1) * (tr + 2) <= t) ++tr;
+            while (per * tr * (tr + 1) > t) --tr;
             i0 = base + 128 * tr;
-            c0 = base + 32 * (t - 2 * tr * (tr + 1));
+            c0 = base + tw * (t - per * tr * (tr + 1));
             return c0 < N;
         };
         if (wid == Q_EPI) {   // loads: lane l takes modulus l (one thread issuing all 26 copies took 750 cycles each)
@@ -385,42 +451,34 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
                     break;
                 }
                 ++tl;
-                if (lane == 0) tc::mbar_expect_tx(&full, RL * Q_STAGE);
-                __syncwarp();
                 if (lane < RL) {
                     uint8_t *d = ring + lane * Q_STAGE;
-                    tc::bulk_load(d, q.RA + ((int64_t)lane * q.npad + i0) * QN, QA_BYTES, &full);
-                    tc::bulk_load(d + QA_BYTES, q.RB + ((int64_t)lane * q.npad + c0) * QN, QB_BYTES, &full);
+                    tc::mbar_expect_tx(&full[lane], QA_BYTES + tw * 64);
+                    tc::bulk_load(d, q.RA + ((int64_t)lane * q.npad + i0) * QN, QA_BYTES, &full[lane]);
+                    tc::bulk_load(d + QA_BYTES, q.RB + ((int64_t)lane * q.npad + c0) * QN, tw * 64, &full[lane]);
                 }
                 __syncwarp();
-            }
-        } else if (wid == Q_EPI + 1 && lane == 0) {
-            for (int t = g; t < tiles && ok; t += G) {
-                int i0, c0;
-                if (!tile_at(t, i0, c0)) continue;
-                if (!tc::mbar_wait(&tempty, (tl & 1) ^ 1) || !tc::mbar_wait(&full, tl & 1)) {
-                    ok = false;
-                    break;
-                }
-                ++tl;
-                tc::fence_after();
-                const uint32_t ab0 = tc::smem_u32(ring);
-#pragma unroll
-                for (int l = 0; l < RL; ++l) {
-                    const uint32_t ab = ab0 + l * Q_STAGE, bb = ab + QA_BYTES;
-#pragma unroll
-                    for (int s = 0; s < 2; ++s)
-                        tc::mma<false, tc::instr_desc(false, 128, 32)>(tmem + 32 * l, tc::sw64_kmajor_desc(ab + 32 * s),
-                                                                       tc::sw64_kmajor_desc(bb + 32 * s), s ? 1u : 0u);
-                }
-                tc::commit(&tfull);
             }
         } else if (wid < Q_EPI) {
             const int quad = wid & 3, quarter = wid >> 2;
             for (int t = g; t < tiles && ok; t += G) {
                 int i0, c0;
                 if (!tile_at(t, i0, c0)) continue;
-                const int i = i0 + 32 * quad + lane, cb = c0 + 8 * quarter;
+                if (wid < RL && lane == 0) {   // this warp's modulus, as soon as it is there
+                    if (tc::mbar_wait(&tempty, (tl & 1) ^ 1) && tc::mbar_wait(&full[wid], tl & 1)) {
+                        tc::fence_after();
+                        const uint32_t ab = tc::smem_u32(ring + wid * Q_STAGE), bb = ab + QA_BYTES;
+#pragma unroll
+                        for (int s = 0; s < 2; ++s) {
+                            const uint64_t da = tc::sw64_kmajor_desc(ab + 32 * s), db = tc::sw64_kmajor_desc(bb + 32 * s);
+                            if (tw == 32) tc::mma<false, tc::instr_desc(false, 128, 32)>(tmem + 32 * wid, da, db, s ? 1u : 0u);
+                            else tc::mma<false, tc::instr_desc(false, 128, 16)>(tmem + 32 * wid, da, db, s ? 1u : 0u);
+                        }
+                        tc::commit(&tfull);
+                    }
+                }
+                __syncwarp();
+                const int i = i0 + 32 * quad + lane, cb = c0 + (tw / 4) * quarter;
                 const int Ei = i < N ? __ldcg(q.rowE + i) : 0;
                 const int Ecl = lane < 8 && cb + lane < N ? __ldcg(q.rowE + cb + lane) : 0;
                 // two entries of A in use, the next two in flight
@@ -438,18 +496,18 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
                 ++tl;
                 tc::fence_after();
                 // parts of the tile above the diagonal or beyond N: nothing to do (warp-uniform)
-                const int nbatch = i0 + 32 * quad < N && cb <= i0 + 32 * quad + 31 ? 4 : 0;
+                const int nbatch = i0 + 32 * quad < N && cb <= i0 + 32 * quad + 31 ? tw / 8 : 0;
 #pragma unroll 1
                 for (int b = 0; b < nbatch; ++b) {
                     const int c = cb + 2 * b;
 #pragma unroll
                     for (int j = 0; j < 2; ++j) old[j] = nxt[j];
-                    if (b < 3) fetch(nxt, c + 2);
+                    if (b + 1 < nbatch) fetch(nxt, c + 2);
                     uint32_t r[RL][2];
                     __syncwarp();
 #pragma unroll
                     for (int l = 0; l < RL; ++l)
-                        tc::tmem_ld2_async(tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(32 * l + 8 * quarter + 2 * b), r[l]);
+                        tc::tmem_ld2_async(tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(32 * l + (tw / 4) * quarter + 2 * b), r[l]);
                     tc::tmem_wait_ld();
 #pragma unroll
                     for (int l = 0; l < RL; ++l)   // the values exist only after the wait
@@ -532,10 +590,10 @@ void launch_persist64(cudaStream_t s, int num_sms, int64_t N, const PersistArgs 
     int per_sm = 0;
     MDSIP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_bk_persist64, Q_THREADS, kQSmem));
     MDSIP_REQUIRE(per_sm >= 1, MDSIP_ERR_CUDA, "ldlt: persistent factorization does not fit an SM");
-    // one CTA per 16 rows below the first block or per two of its trailing
-    // tiles, whichever is more, at most one per SM
+    // one CTA per 16 rows below the first block or per 128 x 16 part of the first
+    // trailing update, whichever is more, at most one per SM
     const int64_t rest = std::max<int64_t>(0, N - QN), nbr = (rest + 127) / 128;
-    const int64_t want = std::max<int64_t>({1, (rest + 15) / 16, nbr * (nbr + 1)});
+    const int64_t want = std::max<int64_t>({1, (rest + 15) / 16, 4 * nbr * (nbr + 1)});
     const int G = (int)std::min<int64_t>(want, (int64_t)num_sms);
     void *kargs[] = {&q};
     MDSIP_CUDA(cudaLaunchCooperativeKernel((const void *)k_bk_persist64, dim3(G), dim3(Q_THREADS), kargs, kQSmem, s));
