@@ -1104,6 +1104,20 @@ static void eval_derivatives(Problem *P) {
 // alpha A dx) and the next iterate's A^T y_g need no pass over A.
 static bool carry_products(const Problem *P) { return P->model_kind == 0 && P->V.Ahi != nullptr && P->D.m_E > 0; }
 
+// Constraints at the first point of a solve or a direction; true when A^T y_g
+// came with A x_d (in bATy), both from one pass over A: n = 512 78 us for both,
+// 35 + 82 apart; 2000 361 for 311 + 337; 4000 1275 for 1315 + 1312.
+static bool start_cons(Problem *P) {
+    double *out2 = P->scal() + SC_THETA;
+    if (!carry_products(P) || P->D.n_d == 0) {
+        model_cons(P, P->I.x, P->I.d, P->cg, P->ch, out2);
+        return false;
+    }
+    P->V.both_products(P->I, P->bATy.as<double>(), P->bsolve_err.as<int>());
+    P->V.eval_cons_ax(P->I.x, P->V.rowtmp, P->I.d, P->cg, P->ch, out2);
+    return true;
+}
+
 struct Errs {
     double E, dual, primal, comp;
 };
@@ -1182,8 +1196,8 @@ static mdsip_status run_ipm(Problem *P) {
     double mu = (P->has_start && P->start_mu0 > 0) ? P->start_mu0 : o.mu0;
     double tau = std::max(o.tau_min, 1.0 - mu);
     model_f(P, P->I.x, P->grad, sc + SC_F);
-    model_cons(P, P->I.x, P->I.d, P->cg, P->ch, sc + SC_THETA);
-    P->lin_ax = P->lin_aty = P->dir_prod = false;
+    P->lin_ax = P->dir_prod = false;
+    P->lin_aty = start_cons(P);
     if (carry_products(P)) {
         P->ax_cur = P->bAx_a.get<double>(P->ctx, D.m_E);
         P->ax_t = P->bAx_b.get<double>(P->ctx, D.m_E);
@@ -1456,9 +1470,10 @@ static void debug_direction(Problem *P, const double *packed, double mu, double 
     double *sc = P->scal();
     MDSIP_REQUIRE(P->bounds_set, MDSIP_ERR_INVALID_ARG, "bounds not set (mdsip_set_bounds)");
     model_f(P, P->I.x, P->grad, sc + SC_F);
-    model_cons(P, P->I.x, P->I.d, P->cg, P->ch, sc + SC_THETA);
-    P->lin_ax = P->lin_aty = P->dir_prod = false;   // the carried products belong to a solve
+    P->lin_ax = P->dir_prod = false;   // the carried products belong to a solve
+    P->lin_aty = start_cons(P);
     eval_derivatives(P);
+    P->lin_aty = false;
     Inertia in = factor_attempt(P, dw, dc);
     const int64_t saved = P->opt.refine_max;
     if (refine > 0) P->opt.refine_max = refine;

@@ -890,6 +890,10 @@ void VecOps::lagrangian_grad(const IterView &I, const double *grad, const double
     MDSIP_LAUNCHED();
 }
 
+void VecOps::both_products(const IterView &I, double *ATy, int *err) {
+    launch_gemv_both_df(st, Ahi, Alo, D.m_E, D.n_d, D.lda, I.x + D.n_s, I.yg, split + D.m_E, split, colpart, rowtmp, ATy,
+                        err, nullptr);
+}
 void VecOps::lagrangian_grad_aty(const IterView &I, const double *grad, const double *Jdh, const double *ATy,
                                  double *gl) {
     k_lagrangian_grad<<<elem_grid(std::max(D.n_s, (NT / 32) * D.n_d)), NT, 0, st>>>(D, M, grad, I.yg, I.yh, Jdh,

@@ -34,6 +34,8 @@ struct VecOps {
     void eval_cons(const double *x, const double *d, double *cg, double *ch, double *out2);
     // the same with A x_d given (Ax, m_E doubles) instead of formed from x
     void eval_cons_ax(const double *x, const double *Ax, const double *d, double *cg, double *ch, double *out2);
+    // rowtmp = A x_d and ATy = A^T y_g in one pass over the FP32 pair of A
+    void both_products(const IterView &I, double *ATy, int *err);
     // y = a + alpha b (n doubles)
     void axpby(int64_t n, const double *a, double alpha, const double *b, double *y);
     void jac_hess(const double *x, const double *yh, double *Jdh, double *Hss, double *Hdd);
