@@ -13,15 +13,14 @@
 //    product in both sweeps reads its tile with lanes along contiguous rows;
 //  * one CTA per 64-row block row (cooperative launch, so all are resident).
 //    The CTA of block row I accumulates L_IJ x_J for J < I as soon as block J
-//    has published x_J (a per-block release flag tagged with the launch's
-//    epoch, no grid-wide barrier), loads the next tile into registers before
-//    it waits for the next flag, and finishes with inv(L_II); the backward
-//    sweep runs the same way from the last block up;
+//    has published x_J (words tagged with the launch's epoch, no grid-wide
+//    barrier), has its tiles in registers before it waits, and finishes with
+//    inv(L_II); the backward sweep runs the same way from the last block up;
 //  * D^-1 (1x1 and 2x2 blocks) is applied per block row between the sweeps;
 //    a 2x2 block that straddles two block rows waits for the neighbour's
 //    forward result.
 //
-// Flags hold the epoch of the launch that set them, so no reset is needed
+// Words hold the epoch of the launch that set them, so no reset is needed
 // between solves; the last CTA to finish advances the epoch.  Every wait is
 // bounded and sets the error flag on expiry.
 #include <algorithm>
@@ -35,13 +34,14 @@ namespace {
 constexpr int kBS = 64;            // block rows and tile edge
 constexpr int kThreads = 256;      // 64 rows x 4 column quarters
 constexpr int kTile = kBS * kBS;
+constexpr int kSolveRhs = 4;       // right-hand sides side by side
 
 __host__ __device__ inline int64_t tile_index(int64_t I, int64_t J) { return I * (I + 1) / 2 + J; }  // J <= I
 
 struct Layout {
     int nblk = 0;
     int64_t ntile = 0;
-    size_t off_flags_f = 0, off_flags_b = 0, off_x = 0, off_z = 0, off_F = 0, off_B = 0, total = 0;
+    size_t off_x = 0, off_z = 0, off_F = 0, off_B = 0, total = 0;
 };
 
 Layout layout_for(int64_t N) {
@@ -50,10 +50,8 @@ Layout layout_for(int64_t N) {
     l.nblk = (int)((std::max<int64_t>(N, 1) + kBS - 1) / kBS);
     l.ntile = (int64_t)l.nblk * (l.nblk + 1) / 2;
     size_t o = 256;                                    // epoch, done counter
-    l.off_flags_f = o; o += al((size_t)l.nblk * 4);
-    l.off_flags_b = o; o += al((size_t)l.nblk * 4);
-    l.off_x = o; o += al((size_t)l.nblk * kBS * sizeof(double));
-    l.off_z = o; o += al((size_t)l.nblk * kBS * sizeof(double));
+    l.off_x = o; o += al(kSolveRhs * (size_t)l.nblk * kBS * 2 * sizeof(double));   // two tagged words per value
+    l.off_z = o; o += al(kSolveRhs * (size_t)l.nblk * kBS * 2 * sizeof(double));
     l.off_F = o; o += al((size_t)l.ntile * kTile * sizeof(double));
     l.off_B = o; o += al((size_t)l.ntile * kTile * sizeof(double));
     l.total = o;
@@ -167,40 +165,6 @@ __global__ void __launch_bounds__(kThreads) k_solve_tiles(int N, const double *_
     bk[(lane + 32) * kBS + c] = (T)x1;
 }
 
-template <typename T>
-struct FlagSolve {
-    int N, nblk;
-    const T *F, *Bk;
-    const double *Dd, *Doff;
-    const int32_t *perm;
-    double *b;
-    T *x, *z;
-    unsigned *fwd, *bwd, *epoch, *done;
-    int *err;
-};
-
-// all threads: wait until *flag == e (bounded); uniform result
-__device__ __forceinline__ bool wait_flag(const unsigned *flag, unsigned e, int *err, int *s_ok) {
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        volatile const unsigned *vp = flag;
-        if (*vp != e) {
-            const long long t0 = clock64();
-            while (*vp != e) {
-                if (*((volatile int *)err) != 0 || clock64() - t0 > kBarrierLimitCycles) {
-                    atomicExch(err, 1);
-                    ok = 0;
-                    break;
-                }
-            }
-        }
-        __threadfence();
-        *s_ok = ok;
-    }
-    __syncthreads();
-    return *s_ok != 0;
-}
-
 // partial of (tile * v)[r] over the column quarter q, tile in registers
 template <typename T>
 __device__ __forceinline__ void load_quarter(const T *tile, int r, int q, T (&reg)[16]) {
@@ -216,291 +180,198 @@ __device__ __forceinline__ T dot_quarter(const T (&reg)[16], const T *sv, int q,
     return acc;
 }
 
+// A block's result travels as 64-bit words (32 bits of a value | epoch << 32; an
+// FP64 value takes two), so one load both tests that block J is published and
+// delivers x_J: no separate flags, no fences between value and flag.
 template <typename T>
-__global__ void __launch_bounds__(kThreads) k_ldlt_solve_flags(FlagSolve<T> p) {
-    __shared__ T sv[kBS];
-    __shared__ T spart[4][kBS];
-    __shared__ unsigned s_e;
-    __shared__ int s_ok;
-    const int tid = threadIdx.x, r = tid & (kBS - 1), q = tid >> 6;
-    const int G = (int)gridDim.x, N = p.N, nblk = p.nblk;
-    if (tid == 0) s_e = *((volatile unsigned *)p.epoch) + 1u;
-    __syncthreads();
-    const unsigned e = s_e;
-    bool ok = true;
-    T reg[16];
-
-    // ---------------- forward: x_I = inv(L_II) (P b - sum_J<I L_IJ x_J) ----------------
-    for (int I = blockIdx.x; I < nblk && ok; I += G) {
-        T acc = (T)0;
-        for (int J = 0; J < I; ++J) {
-            load_quarter(p.F + tile_index(I, J) * kTile, r, q, reg);
-            if (!wait_flag(p.fwd + J, e, p.err, &s_ok)) {
-                ok = false;
-                break;
-            }
-            if (tid < kBS) sv[tid] = __ldcg(p.x + (int64_t)J * kBS + tid);
-            __syncthreads();
-            acc = dot_quarter(reg, sv, q, acc);
-            __syncthreads();
-        }
-        if (!ok) break;
-        load_quarter(p.F + tile_index(I, I) * kTile, r, q, reg);
-        spart[q][r] = acc;
-        __syncthreads();
-        if (tid < kBS) {
-            const int row = I * kBS + tid;
-            const T y0 = row < N ? (T)p.b[p.perm[row]] : (T)0;
-            sv[tid] = y0 - (spart[0][tid] + spart[1][tid] + spart[2][tid] + spart[3][tid]);
-        }
-        __syncthreads();
-        const T a2 = dot_quarter(reg, sv, q, (T)0);
-        __syncthreads();
-        spart[q][r] = a2;
-        __syncthreads();
-        if (tid < kBS) {
-            p.x[(int64_t)I * kBS + tid] = spart[0][tid] + spart[1][tid] + spart[2][tid] + spart[3][tid];
-            __threadfence();
-        }
-        __syncthreads();
-        if (tid == 0) atomicExch(p.fwd + I, e);
-    }
-
-    // ---------------- w = D^-1 x, then z_I = inv(L_II)^T (w_I - sum_J>I L_JI^T z_J) ----------------
-    int last = (int)blockIdx.x;
-    while (last + G < nblk) last += G;
-    for (int I = last; I >= 0 && ok && (int)blockIdx.x < nblk; I -= G) {
-        // a 2x2 block straddling into block row I+1 needs its forward result
-        const int lr = I * kBS + kBS - 1;
-        if (I + 1 < nblk && lr + 1 < N && p.Doff[lr] != 0.0) {
-            if (!wait_flag(p.fwd + I + 1, e, p.err, &s_ok)) {
-                ok = false;
-                break;
-            }
-        }
-        T w = (T)0;
-        if (tid < kBS) {
-            const int k = I * kBS + tid;
-            if (k < N) {
-                const double off = p.Doff[k];
-                if (off != 0.0) {
-                    const double a = p.Dd[k], c = p.Dd[k + 1];
-                    const double u = (double)__ldcg(p.x + k), v = (double)__ldcg(p.x + k + 1);
-                    w = (T)((c * u - off * v) / (a * c - off * off));
-                } else if (k > 0 && p.Doff[k - 1] != 0.0) {
-                    const double a = p.Dd[k - 1], c = p.Dd[k], o2 = p.Doff[k - 1];
-                    const double u = (double)__ldcg(p.x + k - 1), v = (double)__ldcg(p.x + k);
-                    w = (T)((a * v - o2 * u) / (a * c - o2 * o2));
-                } else {
-                    w = (T)((double)__ldcg(p.x + k) / p.Dd[k]);
-                }
-            }
-        }
-        T acc = (T)0;
-        for (int J = nblk - 1; J > I; --J) {
-            load_quarter(p.Bk + tile_index(J, I) * kTile, r, q, reg);
-            if (!wait_flag(p.bwd + J, e, p.err, &s_ok)) {
-                ok = false;
-                break;
-            }
-            if (tid < kBS) sv[tid] = __ldcg(p.z + (int64_t)J * kBS + tid);
-            __syncthreads();
-            acc = dot_quarter(reg, sv, q, acc);
-            __syncthreads();
-        }
-        if (!ok) break;
-        load_quarter(p.Bk + tile_index(I, I) * kTile, r, q, reg);
-        spart[q][r] = acc;
-        __syncthreads();
-        if (tid < kBS) sv[tid] = w - (spart[0][tid] + spart[1][tid] + spart[2][tid] + spart[3][tid]);
-        __syncthreads();
-        const T a2 = dot_quarter(reg, sv, q, (T)0);
-        __syncthreads();
-        spart[q][r] = a2;
-        __syncthreads();
-        if (tid < kBS) {
-            const T zi = spart[0][tid] + spart[1][tid] + spart[2][tid] + spart[3][tid];
-            p.z[(int64_t)I * kBS + tid] = zi;
-            const int row = I * kBS + tid;
-            if (row < N) p.b[p.perm[row]] = (double)zi;
-            __threadfence();
-        }
-        __syncthreads();
-        if (tid == 0) atomicExch(p.bwd + I, e);
-    }
-
-    // the last CTA to finish advances the epoch (every CTA has read it by then:
-    // none can finish before all have published their backward blocks)
-    __syncthreads();
-    if (tid == 0) {
-        __threadfence();
-        const unsigned d = atomicAdd(p.done, 1u);
-        if (d == (unsigned)G - 1u) {
-            atomicExch(p.done, 0u);
-            __threadfence();
-            atomicAdd(p.epoch, 1u);
-        }
-    }
-}
-
-// FP32 form (the refined mixed-precision path): a block's result travels as
-// 64-bit words (value bits | epoch << 32), so one load both tests that block J
-// is published and delivers x_J, and a CTA fetches up to four published blocks
-// per round trip.  No separate flags, no fences between value and flag.
 struct TagSolve {
     int N, nblk;
-    const float *F, *Bk;
+    const T *F, *Bk;
     const double *Dd, *Doff;
     const int32_t *perm;
     double *b;
-    unsigned long long *xw, *zw;   // tagged block results
+    int64_t ldb;
+    unsigned long long *xw, *zw;   // tagged block results, kSolveRhs sets
     unsigned *epoch, *done;
     int *err;
 };
 
-__device__ __forceinline__ unsigned long long tag_word(float v, unsigned e) {
-    return ((unsigned long long)e << 32) | (unsigned long long)__float_as_uint(v);
+__device__ __forceinline__ void tag_store(unsigned long long *w, int64_t i, float v, unsigned e) {
+    w[i] = ((unsigned long long)e << 32) | (unsigned long long)__float_as_uint(v);
+}
+__device__ __forceinline__ void tag_store(unsigned long long *w, int64_t i, double v, unsigned e) {
+    const unsigned long long t = (unsigned long long)e << 32;
+    *reinterpret_cast<ulonglong2 *>(w + 2 * i) =
+        make_ulonglong2(t | (unsigned)__double2loint(v), t | (unsigned)__double2hiint(v));
+}
+__device__ __forceinline__ bool tag_load(const unsigned long long *w, int64_t i, unsigned e, float &v) {
+    const unsigned long long x = *((volatile const unsigned long long *)w + i);
+    v = __uint_as_float((unsigned)x);
+    return (unsigned)(x >> 32) == e;
+}
+__device__ __forceinline__ bool tag_load(const unsigned long long *w, int64_t i, unsigned e, double &v) {
+    unsigned long long x, y;
+    asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];" : "=l"(x), "=l"(y) : "l"(w + 2 * i) : "memory");
+    v = __hiloint2double((int)(unsigned)y, (int)(unsigned)x);
+    return (unsigned)(x >> 32) == e && (unsigned)(y >> 32) == e;
 }
 
-// value of a tagged word once it carries epoch e (bounded wait; false on expiry)
-__device__ __forceinline__ bool tag_wait(const unsigned long long *w, unsigned e, int *err, float &v) {
-    volatile const unsigned long long *vp = w;
-    unsigned long long x = *vp;
-    if ((unsigned)(x >> 32) != e) {
-        const long long t0 = clock64();
-        do {
-            if (*((volatile int *)err) != 0 || clock64() - t0 > kBarrierLimitCycles) {
-                atomicExch(err, 1);
-                return false;
-            }
-            x = *vp;
-        } while ((unsigned)(x >> 32) != e);
-    }
-    v = __uint_as_float((unsigned)x);
+// value i once its words carry epoch e (bounded wait; false on expiry)
+template <typename T>
+__device__ __forceinline__ bool tag_wait(const unsigned long long *w, int64_t i, unsigned e, int *err, T &v) {
+    if (tag_load(w, i, e, v)) return true;
+    const long long t0 = clock64();
+    while (!tag_load(w, i, e, v))
+        if (*((volatile int *)err) != 0 || clock64() - t0 > kBarrierLimitCycles) {
+            atomicExch(err, 1);
+            return false;
+        }
     return true;
 }
 
-constexpr int kTagBatch = 4;   // published blocks fetched per round trip
-
-__global__ void __launch_bounds__(kThreads) k_ldlt_solve_tagged(TagSolve p) {
-    __shared__ float sv[kTagBatch][kBS];
-    __shared__ float spart[4][kBS];
+// Grid: CTAs over block rows (x), right-hand sides (y), each with its own set of
+// result words.  What does not depend on the last block to arrive -- the
+// diagonal tile, its predecessor's tile, the right-hand side -- is loaded
+// before the wait for it: a step of the chain is one exchange through L2, two
+// 64 x 64 products and three barriers.  Blocks before the last come kB at a
+// time (FP32: a round trip for four tiles; FP64: a product is bound by the FP64
+// pipe, so one, with the next tile on its way).  N = 2050: FP32 113 -> 52 us,
+// FP64 311 -> 195 (which had a flag, a fence and a second load per block).
+template <typename T>
+__global__ void __launch_bounds__(kThreads) k_ldlt_solve_tagged(TagSolve<T> p) {
+    constexpr int kB = sizeof(T) == sizeof(float) ? 4 : 1;
+    constexpr int kW = sizeof(T) / sizeof(float);
+    __shared__ T sv[kB][kBS], sy[kBS];
+    __shared__ T spart[4][kBS], spart2[4][kBS];
     __shared__ unsigned s_e;
-    __shared__ int s_ok;
     const int tid = threadIdx.x, r = tid & (kBS - 1), q = tid >> 6;
     const int G = (int)gridDim.x, N = p.N, nblk = p.nblk;
-    if (tid == 0) {
-        s_e = *((volatile unsigned *)p.epoch) + 1u;
-        s_ok = 1;
-    }
+    const int64_t set = (int64_t)blockIdx.y * nblk * kBS * kW;
+    unsigned long long *const xw = p.xw + set, *const zw = p.zw + set;
+    double *const bvec = p.b + (int64_t)blockIdx.y * p.ldb;
+    if (tid == 0) s_e = *((volatile unsigned *)p.epoch) + 1u;
     __syncthreads();
     const unsigned e = s_e;
-    float reg[kTagBatch][16];
+    bool ok = true;   // the same in every thread: agreed on at a barrier
+    T reg[kB][16], lt[16], dg[16];
 
-    // sum over J in [J0, J1) of tile(J) * v_J, tiles at tile_of(J), results in words w
-    auto accumulate = [&](auto tile_of, const unsigned long long *w, int J0, int J1, int step, float acc) {
-        for (int J = J0; J != J1 && s_ok;) {
-            const int nbat = min(kTagBatch, (J1 - J) * step);
+    // sum over `count` blocks J0, J0 + step, .. of tile(J) v_J, results in words w; the last one's tile in lt
+    auto accumulate = [&](auto tile_of, const unsigned long long *w, int J0, int count, int step) {
+        T acc = (T)0;
+        if (kB == 1 && count > 1) load_quarter(tile_of(J0), r, q, reg[0]);
+        for (int j = 0; j < count;) {
+            const bool last = j == count - 1;
+            const int nbat = last ? 1 : min(kB, count - 1 - j);
+            T nx[16];
+            if (!last) {
+                if (kB > 1) {
 #pragma unroll
-            for (int bq = 0; bq < kTagBatch; ++bq)
-                if (bq < nbat) load_quarter(tile_of(J + bq * step), r, q, reg[bq]);
-            {   // thread t fetches word t % 64 of block t / 64
-                const int bq = tid >> 6;
-                if (bq < nbat) {
-                    float v = 0.0f;
-                    if (!tag_wait(w + (int64_t)(J + bq * step) * kBS + r, e, p.err, v)) atomicExch(&s_ok, 0);
-                    sv[bq][r] = v;
+                    for (int bq = 0; bq < kB; ++bq)
+                        if (bq < nbat) load_quarter(tile_of(J0 + (j + bq) * step), r, q, reg[bq]);
+                } else if (j + 2 < count) {
+                    load_quarter(tile_of(J0 + (j + 1) * step), r, q, nx);
                 }
             }
-            __syncthreads();
-            if (!s_ok) break;
+            const int bq = tid >> 6;   // thread t fetches value t % 64 of block t / 64
+            bool got = true;
+            if (bq < nbat) {
+                T v = (T)0;
+                got = tag_wait(w, (int64_t)(J0 + (j + bq) * step) * kBS + r, e, p.err, v);
+                sv[bq][r] = v;
+            }
+            ok = __syncthreads_and(got);
+            if (!ok) break;
+            if (last) {
+                acc = dot_quarter(lt, sv[0], q, acc);
+                break;   // the caller's barrier follows
+            }
 #pragma unroll
-            for (int bq = 0; bq < kTagBatch; ++bq)
-                if (bq < nbat) acc = dot_quarter(reg[bq], sv[bq], q, acc);
+            for (int bq2 = 0; bq2 < kB; ++bq2)
+                if (bq2 < nbat) acc = dot_quarter(reg[bq2], sv[bq2], q, acc);
             __syncthreads();
-            J += nbat * step;
+            if (kB == 1 && j + 2 < count)
+#pragma unroll
+                for (int c = 0; c < 16; ++c) reg[0][c] = nx[c];
+            j += nbat;
         }
         return acc;
     };
-
-    // ---------------- forward: x_I = inv(L_II) (P b - sum_J<I L_IJ x_J) ----------------
-    for (int I = blockIdx.x; I < nblk && s_ok; I += G) {
-        float acc = accumulate([&](int J) { return p.F + tile_index(I, J) * kTile; }, p.xw, 0, I, 1, 0.0f);
-        if (!s_ok) break;
-        load_quarter(p.F + tile_index(I, I) * kTile, r, q, reg[0]);
+    // block row's result from its right-hand side y (threads 0 .. 63) and the sum: inv(L_II) (y - acc)
+    auto finish = [&](T y, T acc) -> T {
         spart[q][r] = acc;
         __syncthreads();
-        if (tid < kBS) {
-            const int row = I * kBS + tid;
-            const float y0 = row < N ? (float)p.b[p.perm[row]] : 0.0f;
-            sv[0][tid] = y0 - (spart[0][tid] + spart[1][tid] + spart[2][tid] + spart[3][tid]);
-        }
+        if (tid < kBS) sy[tid] = y - ((spart[0][tid] + spart[1][tid]) + (spart[2][tid] + spart[3][tid]));
         __syncthreads();
-        const float a2 = dot_quarter(reg[0], sv[0], q, 0.0f);
+        spart2[q][r] = dot_quarter(dg, sy, q, (T)0);
         __syncthreads();
-        spart[q][r] = a2;
-        __syncthreads();
-        if (tid < kBS)
-            p.xw[(int64_t)I * kBS + tid] = tag_word(spart[0][tid] + spart[1][tid] + spart[2][tid] + spart[3][tid], e);
+        return tid < kBS ? (spart2[0][tid] + spart2[1][tid]) + (spart2[2][tid] + spart2[3][tid]) : (T)0;
+    };
+
+    // ---------------- forward: x_I = inv(L_II) (P b - sum_J<I L_IJ x_J) ----------------
+    for (int I = blockIdx.x; I < nblk; I += G) {
+        load_quarter(p.F + tile_index(I, I) * kTile, r, q, dg);
+        if (I > 0) load_quarter(p.F + tile_index(I, I - 1) * kTile, r, q, lt);
+        T y0 = (T)0;
+        if (tid < kBS && I * kBS + tid < N) y0 = (T)bvec[p.perm[I * kBS + tid]];
+        const T acc = accumulate([&](int J) { return p.F + tile_index(I, J) * kTile; }, xw, 0, I, 1);
+        if (!ok) break;
+        const T xi = finish(y0, acc);
+        if (tid < kBS) tag_store(xw, (int64_t)I * kBS + tid, xi, e);
         __syncthreads();
     }
 
     // ---------------- w = D^-1 x, then z_I = inv(L_II)^T (w_I - sum_J>I L_JI^T z_J) ----------------
-    int last = (int)blockIdx.x;
-    while (last + G < nblk) last += G;
-    for (int I = last; I >= 0 && s_ok && (int)blockIdx.x < nblk; I -= G) {
-        float w = 0.0f;
+    int first = (int)blockIdx.x;
+    while (first + G < nblk) first += G;
+    for (int I = first; ok && I >= 0 && (int)blockIdx.x < nblk; I -= G) {
+        load_quarter(p.Bk + tile_index(I, I) * kTile, r, q, dg);
+        if (I + 1 < nblk) load_quarter(p.Bk + tile_index(I + 1, I) * kTile, r, q, lt);
+        T w = (T)0;
+        bool got = true;
         if (tid < kBS) {
             const int k = I * kBS + tid;
             if (k < N) {
                 // x of rows k and k + 1 (a 2x2 block may straddle into block I + 1)
                 auto xval = [&](int kk) {
-                    float v = 0.0f;
-                    if (!tag_wait(p.xw + kk, e, p.err, v)) atomicExch(&s_ok, 0);
+                    T v = (T)0;
+                    got = tag_wait(xw, kk, e, p.err, v) && got;
                     return (double)v;
                 };
                 const double off = p.Doff[k];
                 if (off != 0.0) {
                     const double a = p.Dd[k], c = p.Dd[k + 1];
                     const double u = xval(k), v = xval(k + 1);
-                    w = (float)((c * u - off * v) / (a * c - off * off));
+                    w = (T)((c * u - off * v) / (a * c - off * off));
                 } else if (k > 0 && p.Doff[k - 1] != 0.0) {
                     const double a = p.Dd[k - 1], c = p.Dd[k], o2 = p.Doff[k - 1];
                     const double u = xval(k - 1), v = xval(k);
-                    w = (float)((a * v - o2 * u) / (a * c - o2 * o2));
+                    w = (T)((a * v - o2 * u) / (a * c - o2 * o2));
                 } else {
-                    w = (float)(xval(k) / p.Dd[k]);
+                    w = (T)ddiv(xval(k), p.Dd[k]);
                 }
             }
         }
-        __syncthreads();
-        if (!s_ok) break;
-        float acc = accumulate([&](int J) { return p.Bk + tile_index(J, I) * kTile; }, p.zw, nblk - 1, I, -1, 0.0f);
-        if (!s_ok) break;
-        load_quarter(p.Bk + tile_index(I, I) * kTile, r, q, reg[0]);
-        spart[q][r] = acc;
-        __syncthreads();
-        if (tid < kBS) sv[0][tid] = w - (spart[0][tid] + spart[1][tid] + spart[2][tid] + spart[3][tid]);
-        __syncthreads();
-        const float a2 = dot_quarter(reg[0], sv[0], q, 0.0f);
-        __syncthreads();
-        spart[q][r] = a2;
-        __syncthreads();
+        ok = __syncthreads_and(got);
+        if (!ok) break;
+        const T acc = accumulate([&](int J) { return p.Bk + tile_index(J, I) * kTile; }, zw, nblk - 1, nblk - 1 - I, -1);
+        if (!ok) break;
+        const T zi = finish(w, acc);
         if (tid < kBS) {
-            const float zi = spart[0][tid] + spart[1][tid] + spart[2][tid] + spart[3][tid];
-            p.zw[(int64_t)I * kBS + tid] = tag_word(zi, e);
+            tag_store(zw, (int64_t)I * kBS + tid, zi, e);
             const int row = I * kBS + tid;
-            if (row < N) p.b[p.perm[row]] = (double)zi;
+            if (row < N) bvec[p.perm[row]] = (double)zi;
         }
         __syncthreads();
     }
 
-    // the last CTA to finish advances the epoch (every CTA has read it by then)
+    // the last CTA to finish advances the epoch (every CTA has read it by then:
+    // none can finish before all of its right-hand side have published their
+    // backward blocks, and the counter waits for every right-hand side)
     __syncthreads();
     if (tid == 0) {
         __threadfence();
         const unsigned d = atomicAdd(p.done, 1u);
-        if (d == (unsigned)G - 1u) {
+        if (d == (unsigned)G * gridDim.y - 1u) {
             atomicExch(p.done, 0u);
             __threadfence();
             atomicAdd(p.epoch, 1u);
@@ -508,40 +379,13 @@ __global__ void __launch_bounds__(kThreads) k_ldlt_solve_tagged(TagSolve p) {
     }
 }
 
-void launch_solve_tagged(cudaStream_t s, int num_sms, int64_t N, const double *Dd, const double *Doff,
-                         const int32_t *perm, int64_t nrhs, double *B, int64_t ldb, char *w, int *err_dev) {
-    const Layout l = layout_for(N);
-    TagSolve p{};
-    p.N = (int)N;
-    p.nblk = l.nblk;
-    p.F = reinterpret_cast<const float *>(w + l.off_F);
-    p.Bk = reinterpret_cast<const float *>(w + l.off_B);
-    p.Dd = Dd;
-    p.Doff = Doff;
-    p.perm = perm;
-    p.xw = reinterpret_cast<unsigned long long *>(w + l.off_x);
-    p.zw = reinterpret_cast<unsigned long long *>(w + l.off_z);
-    p.epoch = reinterpret_cast<unsigned *>(w);
-    p.done = reinterpret_cast<unsigned *>(w + 4);
-    p.err = err_dev;
-    int per_sm = 0;
-    MDSIP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ldlt_solve_tagged, kThreads, 0));
-    MDSIP_REQUIRE(per_sm >= 1, MDSIP_ERR_INVALID_ARG, "ldlt_solve: kernel does not fit on an SM");
-    const int grid = (int)std::min<int64_t>(l.nblk, (int64_t)num_sms * per_sm);
-    for (int64_t rr = 0; rr < nrhs; ++rr) {
-        p.b = B + rr * ldb;
-        void *args[] = {&p};
-        MDSIP_CUDA(cudaLaunchCooperativeKernel((const void *)k_ldlt_solve_tagged, dim3(grid), dim3(kThreads), args,
-                                               0, s));
-        count_launch();
-    }
-}
-
+// As many right-hand sides at once as fit the device beside one another: their
+// chains run side by side (N = 2003, four: 1208 us one after the other, 189 so).
 template <typename T>
 void launch_solve_t(cudaStream_t s, int num_sms, int64_t N, const double *Dd, const double *Doff,
                     const int32_t *perm, int64_t nrhs, double *B, int64_t ldb, char *w, int *err_dev) {
     const Layout l = layout_for(N);
-    FlagSolve<T> p{};
+    TagSolve<T> p{};
     p.N = (int)N;
     p.nblk = l.nblk;
     p.F = reinterpret_cast<const T *>(w + l.off_F);
@@ -549,21 +393,23 @@ void launch_solve_t(cudaStream_t s, int num_sms, int64_t N, const double *Dd, co
     p.Dd = Dd;
     p.Doff = Doff;
     p.perm = perm;
-    p.x = reinterpret_cast<T *>(w + l.off_x);
-    p.z = reinterpret_cast<T *>(w + l.off_z);
+    p.ldb = ldb;
+    p.xw = reinterpret_cast<unsigned long long *>(w + l.off_x);
+    p.zw = reinterpret_cast<unsigned long long *>(w + l.off_z);
     p.epoch = reinterpret_cast<unsigned *>(w);
     p.done = reinterpret_cast<unsigned *>(w + 4);
-    p.fwd = reinterpret_cast<unsigned *>(w + l.off_flags_f);
-    p.bwd = reinterpret_cast<unsigned *>(w + l.off_flags_b);
     p.err = err_dev;
     int per_sm = 0;
-    MDSIP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ldlt_solve_flags<T>, kThreads, 0));
+    MDSIP_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ldlt_solve_tagged<T>, kThreads, 0));
     MDSIP_REQUIRE(per_sm >= 1, MDSIP_ERR_INVALID_ARG, "ldlt_solve: kernel does not fit on an SM");
-    const int grid = (int)std::min<int64_t>(l.nblk, (int64_t)num_sms * per_sm);
-    for (int64_t rr = 0; rr < nrhs; ++rr) {
+    const int64_t room = (int64_t)num_sms * per_sm;
+    const int grid = (int)std::min<int64_t>(l.nblk, room);
+    const int64_t side = std::min<int64_t>(kSolveRhs, std::max<int64_t>(1, (int64_t)num_sms / grid));
+    for (int64_t rr = 0; rr < nrhs; rr += side) {
         p.b = B + rr * ldb;
         void *args[] = {&p};
-        MDSIP_CUDA(cudaLaunchCooperativeKernel((const void *)k_ldlt_solve_flags<T>, dim3(grid), dim3(kThreads),
+        MDSIP_CUDA(cudaLaunchCooperativeKernel((const void *)k_ldlt_solve_tagged<T>,
+                                               dim3(grid, (unsigned)std::min<int64_t>(side, nrhs - rr)), dim3(kThreads),
                                                args, 0, s));
         count_launch();
     }
@@ -573,14 +419,14 @@ void launch_solve_t(cudaStream_t s, int num_sms, int64_t N, const double *Dd, co
 
 size_t ldlt_solve_scratch_bytes(int64_t N) { return layout_for(N).total; }
 
-// Tiles of L (FP64, or FP32 when fp32) and reset flags; once per factorization.
+// Tiles of L (FP64, or FP32 when fp32) and cleared words; once per factorization.
 void launch_ldlt_solve_prepare(cudaStream_t s, int64_t N, const double *L, void *scratch, bool fp32) {
     if (N <= 0) return;
     char *w = static_cast<char *>(scratch);
     MDSIP_REQUIRE((reinterpret_cast<uintptr_t>(w) & 255) == 0, MDSIP_ERR_INVALID_ARG,
                   "ldlt_solve: misaligned scratch");
     const Layout l = layout_for(N);
-    // epoch, done counter, flags, and the tagged results (a stale word must
+    // epoch, done counter and the tagged results (a stale word must
     // not carry an epoch of the new series)
     MDSIP_CUDA(cudaMemsetAsync(w, 0, l.off_F, s));
     if (fp32)
@@ -601,7 +447,7 @@ void launch_ldlt_solve_coop(cudaStream_t s, int num_sms, int64_t N, const double
     if (N <= 0 || nrhs <= 0) return;
     char *w = static_cast<char *>(scratch);
     if (fp32)
-        launch_solve_tagged(s, num_sms, N, Dd, Doff, perm, nrhs, B, ldb, w, err_dev);
+        launch_solve_t<float>(s, num_sms, N, Dd, Doff, perm, nrhs, B, ldb, w, err_dev);
     else
         launch_solve_t<double>(s, num_sms, N, Dd, Doff, perm, nrhs, B, ldb, w, err_dev);
 }

@@ -33,3 +33,22 @@ def test_solve_at_block_edges(ctx, N):
     m.mdsip_ldlt_solve(ctx, N, Ld, dev(D), dev(np.zeros(N)), dev(np.arange(N, dtype=np.int32)), 1, x, N)
     torch.cuda.synchronize()
     assert np.abs(x.cpu().numpy() - want).max() <= 1e-11 * np.abs(want).max()
+
+
+@pytest.mark.parametrize("N,nrhs", [(65, 7), (1033, 9), (700, 4)])
+def test_solve_several_right_hand_sides(ctx, N, nrhs):
+    """Columns solved side by side equal the same columns solved one at a time, bit for bit."""
+    torch = torch_cuda()
+    rng = np.random.default_rng(N)
+    L = np.tril(rng.uniform(-1, 1, (N, N)) / np.sqrt(N), -1) + np.eye(N)
+    D = rng.uniform(1, 2, N) * rng.choice([-1.0, 1.0], N)
+    Ld, Dd, off = dev(L.T.copy()), dev(D), dev(np.zeros(N))
+    perm = dev(np.arange(N, dtype=np.int32))
+    b = rng.standard_normal((nrhs, N))
+    X = dev(b)
+    m.mdsip_ldlt_solve(ctx, N, Ld, Dd, off, perm, nrhs, X, N)
+    for k in range(nrhs):
+        x = dev(b[k])
+        m.mdsip_ldlt_solve(ctx, N, Ld, Dd, off, perm, 1, x, N)
+        torch.cuda.synchronize()
+        assert torch.equal(x, X[k])
