@@ -551,7 +551,7 @@ bool ldlt_persistent_path(int64_t N, int spec);
 std::vector<int> ldlt_blocked_widths(int64_t N, bool f32);
 void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, const double *maxabs_dev,
                          double zero_tol, LdltOut out, void *scratch, bool fp32_update, int nb = 0,
-                         int spec = 1);
+                         int spec = 1, int *err_dev = nullptr);
 void launch_ldlt_solve(cudaStream_t s, int64_t N, const double *L, const double *Dd,
                        const double *Doff, const int32_t *perm, int64_t nrhs, double *B,
                        int64_t ldb);

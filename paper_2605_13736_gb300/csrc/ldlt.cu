@@ -638,7 +638,7 @@ void launch_ldlt(cudaStream_t s, int num_sms, int64_t N, const double *S, int64_
                  int *err_dev, bool fp32_update, int nb, int spec) {
     if (N > 0 && ld == N && (ldlt_blocked_available(N) || ldlt_persistent_path(N, spec))) {
         launch_ldlt_blocked(s, num_sms, N, const_cast<double *>(S), maxabs_dev, zero_tol, out, scratch,
-                            fp32_update, nb, spec);
+                            fp32_update, nb, spec, err_dev);
         return;
     }
     launch_ldlt_unblocked(s, num_sms, N, S, ld, maxabs_dev, zero_tol, out, scratch, err_dev);

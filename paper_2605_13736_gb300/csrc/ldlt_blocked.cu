@@ -50,13 +50,6 @@ constexpr int kPanelThreads = 512;
 constexpr int kUpdThreads = 256;
 constexpr int kUT = 64;   // trailing-update tile edge
 
-// Programmatic dependent launch: the kernels of the panel loop are launched
-// with programmatic stream serialization, so a kernel's launch overlaps the
-// tail of the one before it.  Each waits for its predecessor's completion (and
-// memory) before touching data, then lets its own successor launch.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 struct Cand {                  // one CTA's candidate of a cluster-wide arg-max
     unsigned long long bits;   // |v| bit pattern
     int idx;                   // global row (first index on ties)
@@ -162,7 +155,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_bk_panel(PanelArgs a) {
     pdl_release();
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank();
-    const int C = a.C, N = a.N, NB = a.NB, S = NB + 1;
+    const int C = a.C, N = a.N, NB = a.NB, S = (NB + 1) | 1;   // an odd pitch: lanes over rows meet no bank twice
     const int tid = threadIdx.x;
     extern __shared__ double smem[];
     double *Ap = smem;                       // R x S: raw A columns, then L columns
@@ -204,10 +197,14 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_bk_panel(PanelArgs a) {
     int npos = 0, nneg = 0, nzero = 0;
     cl.sync();
 
-    // tpr threads per row for the row-times-W-row products (a power of two,
-    // as many as fit one pass over the owned rows)
+    // tpr threads per row for the row-times-W-row products (a power of two): FP32
+    // as many as fit one pass over the owned rows; FP64 one warp per
+    // sub-partition, since another warp's share of a row costs the FP64 pipe its
+    // shuffles' additions on top of the same products (125 rows, 16 columns: 4
+    // threads a row 1950 cycles, one 1100)
+    constexpr int kWide = F32 ? kPanelThreads : 128;
     int tpr = 1;
-    while (tpr < 32 && 2 * tpr * R <= kPanelThreads) tpr *= 2;
+    while (tpr < 32 && 2 * tpr * R <= kWide) tpr *= 2;
     const int q4 = tid & (tpr - 1), rsub = tid / tpr, rpp = kPanelThreads / tpr;
     int jj = 0, it = 0;
     while (jj < NB && k + jj < N) {
@@ -224,6 +221,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_bk_panel(PanelArgs a) {
         int bi = 0x7fffffff;
         for (int lr0 = 0; lr0 < r1 - r0; lr0 += rpp) {
             const int lr = lr0 + rsub, i = r0 + lr;
+            if (!F32 && !__any_sync(0xffffffffu, lr < r1 - r0 && i >= j)) continue;   // a warp without rows
             double s;
             if constexpr (F32) {
                 float sf = 0.0f;
@@ -285,7 +283,16 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_bk_panel(PanelArgs a) {
             for (int lr0 = 0; lr0 < r1 - r0; lr0 += rpp) {
                 const int lr = lr0 + rsub, i = r0 + lr;
                 const bool act = lr < r1 - r0 && i >= j;
+                if (!F32 && !__any_sync(0xffffffffu, act)) continue;   // a warp without rows
                 double s;
+                // column r's entry: its load passes under the products
+                double air = 0.0;
+                if (act && q4 == 0) {
+                    if (i < r)
+                        air = (i - k < S) ? rAp(r)[i - k] : a.A[r + (int64_t)i * N];
+                    else
+                        air = r_in_panel ? Ap[(size_t)lr * S + (r - k)] : a.A[i + (int64_t)r * N];
+                }
                 if constexpr (F32) {
                     float sf = 0.0f;
                     if (act)
@@ -299,11 +306,6 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_bk_panel(PanelArgs a) {
                     for (int o = 1; o < tpr; o <<= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
                 }
                 if (act && q4 == 0) {
-                    double air;
-                    if (i < r)
-                        air = (i - k < S) ? rAp(r)[i - k] : a.A[r + (int64_t)i * N];
-                    else
-                        air = r_in_panel ? Ap[(size_t)lr * S + (r - k)] : a.A[i + (int64_t)r * N];
                     const double v = air - s;
                     Wp[(size_t)lr * S + jj + 1] = v;
                     if (i != r) cand_combine(b2, bi2, absbits64(v), i);
@@ -317,7 +319,7 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_bk_panel(PanelArgs a) {
                 if (cluster_cand(cl, cpair, 1, C, owner(r), res)) {
                     const double absakk = s_sc[0], colmax = s_sc[1];
                     const double rowmax = __longlong_as_double((long long)res.bits);
-                    if (absakk >= alpha * colmax * (colmax / rowmax)) s_dec[2] = 0;   // 1x1, no interchange
+                    if (absakk >= alpha * colmax * ddiv(colmax, rowmax)) s_dec[2] = 0;   // 1x1, no interchange
                     else if (fabs(res.val) >= alpha * rowmax) s_dec[2] = 1;         // 1x1 on V, interchange
                     else s_dec[2] = 2;                                              // 2x2, interchange
                 }
@@ -408,10 +410,12 @@ __global__ void __launch_bounds__(kPanelThreads, 1) k_bk_panel(PanelArgs a) {
                 s_d[3] = rcp_newton(d11);
                 s_d[4] = s_d[5] = 0.0;
             } else {
-                const double inv = rcp_newton(d11 * d22 - d21 * d21);
-                s_d[3] = d22 * inv;
-                s_d[4] = -d21 * inv;
-                s_d[5] = d11 * inv;
+                // in units of d21, so that no product leaves the range the entries are in
+                const double r = rcp_newton(d21), a11 = d11 * r, a22 = d22 * r;
+                const double t = r * rcp_newton(fma(a11, a22, -1.0));
+                s_d[3] = a22 * t;
+                s_d[4] = -t;
+                s_d[5] = a11 * t;
             }
         }
         if (!d_ready) __syncthreads();
@@ -1776,33 +1780,6 @@ BlockedConfig blocked_config(int64_t N, bool f32, int nb_want = 0) {
     return c;
 }
 
-// launch with programmatic stream serialization (and a cluster when cluster > 1)
-template <typename... KArgs, typename... Args>
-void launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, int cluster,
-                Args... args) {
-    cudaLaunchConfig_t c{};
-    c.gridDim = dim3(grid);
-    c.blockDim = dim3(block);
-    c.dynamicSmemBytes = smem;
-    c.stream = s;
-    cudaLaunchAttribute at[2];
-    int na = 0;
-    at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[na].val.programmaticStreamSerializationAllowed = 1;
-    ++na;
-    if (cluster > 1) {
-        at[na].id = cudaLaunchAttributeClusterDimension;
-        at[na].val.clusterDim.x = (unsigned)cluster;
-        at[na].val.clusterDim.y = 1;
-        at[na].val.clusterDim.z = 1;
-        ++na;
-    }
-    c.attrs = at;
-    c.numAttrs = na;
-    MDSIP_CUDA(cudaLaunchKernelEx(&c, kern, args...));
-    count_launch();
-}
-
 // scratch layout: W of the last panel (N x 65 doubles), the panel state, the
 // FP32 L and W columns of the last panel (N x 65 floats each; FP32-update
 // form), and for the verified no-interchange panels the per-column maxima
@@ -1898,11 +1875,18 @@ bool ldlt_persistent_path(int64_t N, int spec) {
     return spec != 0 && N > 0 && N <= (int64_t)0x7fffffff / 2;
 }
 
+// Pivoting FP64 panels: columns left from which they are 31 wide with
+// tensor-core trailing updates (64 wide with DFMA tiles / so: N = 64 227 / 238 us,
+// 114 448 / 366, 350 1473 / 1028, 1100 4798 / 3297, 2050 11.1 / 7.0 ms), and from
+// which such a panel's update takes them (a DFMA tile takes 38 us of the FP64
+// pipe however few there are, rows and update 7 + 12).
+constexpr int64_t kRnsPanelMin = 96, kRnsTrailingMin = 32;
+
 // S (lower, ld N) is overwritten.  scratch: ldlt_blocked_scratch_bytes(N),
 // 256-byte aligned.  fp32_update: trailing products in FP32.  spec (with
 // fp32_update): each panel first tries the verified no-interchange path.
 void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, const double *maxabs_dev,
-                         double zero_tol, LdltOut out, void *scratch, bool fp32_update, int nb, int spec) {
+                         double zero_tol, LdltOut out, void *scratch, bool fp32_update, int nb, int spec, int *err_dev) {
     if (N <= 0) {
         MDSIP_CUDA(cudaMemsetAsync(out.inertia, 0, 3 * sizeof(int32_t), s));
         return;
@@ -1952,6 +1936,13 @@ void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, cons
         if (k0 < N) MDSIP_CUDA(cudaMemsetAsync(w + lay.cmax, 0, 192 * sizeof(unsigned long long), s));
     }
 
+    // FP64 panels without a width asked for: 31 columns (32 with a 2x2 pivot at
+    // the end), whose trailing updates go through the tensor cores
+    const bool rns = !fp32_update && nb == 0 && N - k0 > kRnsPanelMin && cfg.NB >= 32;
+    if (rns) {
+        cfg = blocked_config(N, false, 32);
+        cfg.NB = 31;
+    }
     PanelArgs a{};
     a.N = (int)N;
     a.NB = cfg.NB;
@@ -2026,7 +2017,10 @@ void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, cons
         const float *cLf = a.Lf, *cWf = a.Wf;
         const double *cL = out.L, *cWg = Wg;
         const PanelState *cst = st;
-        if (fp32_update)
+        if (rns && rest > kRnsTrailingMin)
+            launch_rns_trailing(s, num_sms, N, rest, p, S, out.L, out.Dd, out.Doff, Wg, maxabs_dev, st,
+                                err_dev ? err_dev : &bar->err, w + lay.p64);
+        else if (fp32_update)
             launch_pdl(k_bk_trailing<float>, tiles, kUpdThreads, usm, s, 1, (int)N, cfg.NB, S, cL, cWg, cLf, cWf, cst);
         else
             launch_pdl(k_bk_trailing<double>, tiles, kUpdThreads, usm, s, 1, (int)N, cfg.NB, S, cL, cWg, cLf, cWf, cst);

@@ -42,6 +42,13 @@ struct PersistArgs {
 
 namespace {
 
+// Programmatic dependent launch: the kernels of the panel loop are launched
+// with programmatic stream serialization, so a kernel's launch overlaps the
+// tail of the one before it.  Each waits for its predecessor's completion (and
+// memory) before touching data, then lets its own successor launch.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ unsigned long long absbits64(double v) {
     return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL;
 }
@@ -92,6 +99,33 @@ __device__ bool panel_barrier(PanelBar *b, unsigned &epoch, long long wait_ns) {
     return s_ok != 0;
 }
 
+// launch with programmatic stream serialization (and a cluster when cluster > 1)
+template <typename... KArgs, typename... Args>
+void launch_pdl(void (*kern)(KArgs...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, int cluster,
+                Args... args) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(block);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    cudaLaunchAttribute at[2];
+    int na = 0;
+    at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[na].val.programmaticStreamSerializationAllowed = 1;
+    ++na;
+    if (cluster > 1) {
+        at[na].id = cudaLaunchAttributeClusterDimension;
+        at[na].val.clusterDim.x = (unsigned)cluster;
+        at[na].val.clusterDim.y = 1;
+        at[na].val.clusterDim.z = 1;
+        ++na;
+    }
+    c.attrs = at;
+    c.numAttrs = na;
+    MDSIP_CUDA(cudaLaunchKernelEx(&c, kern, args...));
+    count_launch();
+}
+
 }  // namespace
 
 // ldlt_persist64.cu: the persistent no-interchange factorization, FP64.  One
@@ -99,5 +133,9 @@ __device__ bool panel_barrier(PanelBar *b, unsigned &epoch, long long wait_ns) {
 // panel the rule's column test rejects.  scratch: persist64_scratch_bytes(N).
 size_t persist64_scratch_bytes(int64_t N);
 void launch_persist64(cudaStream_t s, int num_sms, int64_t N, const PersistArgs &pa, void *scratch);
+// and the trailing update after a pivoting FP64 panel of at most 32 columns
+void launch_rns_trailing(cudaStream_t s, int num_sms, int64_t N, int64_t rest, int panel, double *A, const double *L,
+                         const double *Dd, const double *Doff, const double *Wg, const double *maxabs,
+                         const PanelState *st, int *err, void *scratch);
 
 }  // namespace mdsip

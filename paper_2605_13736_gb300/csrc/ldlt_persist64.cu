@@ -203,6 +203,176 @@ __device__ __forceinline__ void q_colmax(unsigned long long bm, unsigned long lo
     if (lane == 0 && (hi | lo)) atomicMax(dst, ((unsigned long long)hi << 32) | lo);
 }
 
+// mbarriers of q_update, and -(bias + k M) modulo 2^128 in s_km (threads 0 .. 15)
+__device__ void q_update_init(uint64_t *full, uint64_t *tfull, uint64_t *tempty, uint4 *s_km) {
+    const int tid = threadIdx.x;
+    if (tid == 0) {
+        for (int l = 0; l < RL; ++l) tc::mbar_init(&full[l], 1);
+        tc::mbar_init(tfull, RL);
+        tc::mbar_init(tempty, Q_EPI);
+    }
+    if (tid < 16) {
+        unsigned __int128 M = 0, B = 0;
+        for (int m = 3; m >= 0; --m) {
+            M = (M << 32) | c_tab13.mod32[m];
+            B = (B << 32) | c_tab13.bias32[m];
+        }
+        const unsigned __int128 v = (unsigned __int128)0 - B - M * (unsigned __int128)(__int128)(tid - 8);
+        s_km[tid] = make_uint4((unsigned)v, (unsigned)(v >> 32), (unsigned)(v >> 64), (unsigned)(v >> 96));
+    }
+}
+
+// the residues of one row's scaled value (lane = column) at the tensor core's layout
+__device__ __forceinline__ int64_t q_at(int64_t row, int lane) {
+    return row * QN + ((((lane >> 3) ^ (int)(row >> 1)) & 3) << 3) + (lane & 7);
+}
+
+// The trailing update A(i, c) -= sum_t X(i, t) Y(c, t), first <= c <= i < N, from
+// residues of X in RA and of Y in RB, by this CTA g of G: tiles of 128 rows from
+// `base` (a multiple of 8, at most 7 below `first`) and tw columns of the lower
+// triangle.  tl counts the tiles this warp's role has gone through.
+struct QUpdate {
+    double *A;
+    const bf16 *RA, *RB;
+    const int *EA, *EB;   // row exponents
+    int N, npad, base, first;
+};
+
+__device__ bool q_update(const QUpdate &u, int G, int g, uint8_t *ring, uint32_t tmem, uint64_t *full, uint64_t *tfull,
+                         uint64_t *tempty, const uint4 *s_km, int &tl) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, N = u.N, base = u.base;
+    const int nbr = (N - base + 127) / 128;
+    // 16 columns a tile when that still is one tile per CTA: half the read-back
+    const int tw = 4 * nbr * (nbr + 1) <= G ? 16 : 32, per = 64 / tw;
+    const int tiles = per * nbr * (nbr + 1);
+            bool ok = true;
+            auto tile_at = [&](int t, int &i0, int &c0) {   // false: beyond the last column
+                int tr = (int)(sqrtf((float)t / (float)per + 0.25f) - 0.5f);
+                while (per * (tr + 1) * (tr + 2) <= t) ++tr;
+                while (per * tr * (tr + 1) > t) --tr;
+                i0 = base + 128 * tr;
+                c0 = base + tw * (t - per * tr * (tr + 1));
+                return c0 < N;
+            };
+            if (wid == Q_EPI) {   // loads: lane l takes modulus l (one thread issuing all 26 copies took 750 cycles each)
+                asm volatile("fence.proxy.async;" ::: "memory");
+                for (int t = g; t < tiles && ok; t += G) {
+                    int i0, c0;
+                    if (!tile_at(t, i0, c0)) continue;
+                    if (tl > 0 && !tc::mbar_wait(tfull, (tl - 1) & 1)) {   // the previous tile's operands are read
+                        ok = false;
+                        break;
+                    }
+                    ++tl;
+                    if (lane < RL) {
+                        uint8_t *d = ring + lane * Q_STAGE;
+                        tc::mbar_expect_tx(&full[lane], QA_BYTES + tw * 64);
+                        tc::bulk_load(d, u.RA + ((int64_t)lane * u.npad + i0) * QN, QA_BYTES, &full[lane]);
+                        tc::bulk_load(d + QA_BYTES, u.RB + ((int64_t)lane * u.npad + c0) * QN, tw * 64, &full[lane]);
+                    }
+                    __syncwarp();
+                }
+            } else if (wid < Q_EPI) {
+                const int quad = wid & 3, quarter = wid >> 2;
+                for (int t = g; t < tiles && ok; t += G) {
+                    int i0, c0;
+                    if (!tile_at(t, i0, c0)) continue;
+                    if (wid < RL && lane == 0) {   // this warp's modulus, as soon as it is there
+                        if (tc::mbar_wait(tempty, (tl & 1) ^ 1) && tc::mbar_wait(&full[wid], tl & 1)) {
+                            tc::fence_after();
+                            const uint32_t ab = tc::smem_u32(ring + wid * Q_STAGE), bb = ab + QA_BYTES;
+    #pragma unroll
+                            for (int s = 0; s < 2; ++s) {
+                                const uint64_t da = tc::sw64_kmajor_desc(ab + 32 * s), db = tc::sw64_kmajor_desc(bb + 32 * s);
+                                if (tw == 32) tc::mma<false, tc::instr_desc(false, 128, 32)>(tmem + 32 * wid, da, db, s ? 1u : 0u);
+                                else tc::mma<false, tc::instr_desc(false, 128, 16)>(tmem + 32 * wid, da, db, s ? 1u : 0u);
+                            }
+                            tc::commit(tfull);
+                        }
+                    }
+                    __syncwarp();
+                    const int i = i0 + 32 * quad + lane, cb = c0 + (tw / 4) * quarter;
+                    const int Ei = i < N ? __ldcg(u.EA + i) : 0;
+                    const int Ecl = lane < 8 && cb + lane < N ? __ldcg(u.EB + cb + lane) : 0;
+                    // two entries of A in use, the next two in flight
+                    double old[2], nxt[2];
+                    auto fetch = [&](double (&d)[2], int c) {
+    #pragma unroll
+                        for (int j = 0; j < 2; ++j)
+                            d[j] = i < N && c + j <= i && c + j >= u.first ? __ldcg(u.A + i + (int64_t)(c + j) * N) : 0.0;
+                    };
+                    fetch(nxt, cb);
+                    if (!tc::mbar_wait(tfull, tl & 1)) {
+                        ok = false;
+                        break;
+                    }
+                    ++tl;
+                    tc::fence_after();
+                    // parts of the tile above the diagonal or beyond N: nothing to do (warp-uniform)
+                    const int nbatch = i0 + 32 * quad < N && cb <= i0 + 32 * quad + 31 ? tw / 8 : 0;
+    #pragma unroll 1
+                    for (int b = 0; b < nbatch; ++b) {
+                        const int c = cb + 2 * b;
+    #pragma unroll
+                        for (int j = 0; j < 2; ++j) old[j] = nxt[j];
+                        if (b + 1 < nbatch) fetch(nxt, c + 2);
+                        uint32_t r[RL][2];
+                        __syncwarp();
+    #pragma unroll
+                        for (int l = 0; l < RL; ++l)
+                            tc::tmem_ld2_async(tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(32 * l + (tw / 4) * quarter + 2 * b), r[l]);
+                        tc::tmem_wait_ld();
+    #pragma unroll
+                        for (int l = 0; l < RL; ++l)   // the values exist only after the wait
+                            asm volatile("" : "+r"(r[l][0]), "+r"(r[l][1]));
+                        unsigned long long acc[2][4] = {};   // per entry, 32-bit limbs
+                        uint64_t yp = 0;                     // the pair's first residues
+    #pragma unroll
+                        for (int l = 0; l < RL; ++l) {
+                            const float pf = c_tab13.p[l], pi = c_tab13.pinv[l];
+                            const uint64_t x = rns::pk(__uint_as_float(r[l][0]), __uint_as_float(r[l][1]));
+                            const uint64_t qq = rns::add2(rns::fma2(x, rns::pk(pi, pi), rns::pk(rns::kMagic, rns::kMagic)),
+                                                          rns::pk(-rns::kMagic, -rns::kMagic));
+                            const uint64_t y = rns::fma2(rns::pk(-pf, -pf), qq, x);   // x mod p
+                            if (l % 2 == 0 && l + 1 < RL) {
+                                yp = y;
+                                continue;
+                            }
+                            // z = y_p q + y_q p (exact); z + 2^19 is the low 23 bits of z + 2^23 + 2^19
+                            const uint64_t zb = rns::pk(8912896.0f, 8912896.0f);
+                            const float pp = c_tab13.p[l > 0 ? l - 1 : 0];
+                            const uint64_t z =
+                                l % 2 ? rns::add2(rns::fma2(yp, rns::pk(pf, pf), rns::mul2(y, rns::pk(pp, pp))), zb) : rns::add2(y, zb);
+                            const float2 zf = rns::upk(z);
+                            const uint32_t u0 = __float_as_uint(zf.x) & 0x7fffffu, u1 = __float_as_uint(zf.y) & 0x7fffffu;
+    #pragma unroll
+                            for (int m = 0; m < 4; ++m) {
+                                acc[0][m] += (unsigned long long)u0 * c_tab13.mpair32[l / 2][m];
+                                acc[1][m] += (unsigned long long)u1 * c_tab13.mpair32[l / 2][m];
+                            }
+                        }
+    #pragma unroll
+                        for (int j = 0; j < 2; ++j) {
+                            // T = sum z M/(p q) + bias; X = T - bias - k M with k = rint((T - bias) / M)
+                            unsigned __int128 T = ((unsigned __int128)acc[j][3] << 96) + ((unsigned __int128)acc[j][2] << 64) +
+                                                  ((unsigned __int128)acc[j][1] << 32) + acc[j][0];
+                            const float f = fmaf((float)(uint32_t)(T >> 96), c_tab13.top, -c_tab13.btop) + rns::kMagic;
+                            const uint4 km = s_km[(__float_as_uint(f) + 8u) & 15u];   // kMagic's low bits are zero
+                            T += ((unsigned __int128)(((unsigned long long)km.w << 32) | km.z) << 64) |
+                                 (((unsigned long long)km.y << 32) | km.x);
+                            const int Ec = __shfl_sync(0xffffffffu, Ecl, 2 * b + j);
+                            if (i < N && c + j <= i && c + j >= u.first)
+                                u.A[i + (int64_t)(c + j) * N] = old[j] - rns::to_double(T, Ei + Ec - 2 * QB);
+                        }
+                    }
+                    tc::fence_before();
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(tempty);
+                }
+            }
+    return ok;
+}
+
 __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
     const PersistArgs &a = q.p;
     extern __shared__ uint8_t psm_raw[];
@@ -223,21 +393,10 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
     // pivoting panels take such a matrix (st->k stays where it is)
     if (!(maxabs > 0x1p-900)) return;
     if (tid == 0) {
-        for (int l = 0; l < RL; ++l) tc::mbar_init(&full[l], 1);
         for (int j = 0; j < 16; ++j) tc::mbar_init(&colbar[j], 4);
-        tc::mbar_init(&tfull, RL);
-        tc::mbar_init(&tempty, Q_EPI);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (tid < 16) {
-        unsigned __int128 M = 0, B = 0;
-        for (int m = 3; m >= 0; --m) {
-            M = (M << 32) | c_tab13.mod32[m];
-            B = (B << 32) | c_tab13.bias32[m];
-        }
-        const unsigned __int128 v = (unsigned __int128)0 - B - M * (unsigned __int128)(__int128)(tid - 8);
-        s_km[tid] = make_uint4((unsigned)v, (unsigned)(v >> 32), (unsigned)(v >> 64), (unsigned)(v >> 96));
-    }
+    q_update_init(full, &tfull, &tempty, s_km);
+    if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     if (wid == 0) tc::tmem_alloc(&s_tmem, 512);
     tc::fence_before();
     __syncthreads();
@@ -369,7 +528,7 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
                     const uint32_t sa = w < 0.0 ? 0x8000u : 0u, sb = sa ^ (s_d[lane] < 0.0 ? 0x8000u : 0u);
                     const int64_t row = cb + r;
                     if (lane == 0) q.rowE[row] = E;
-                    const int64_t at = row * QN + ((((lane >> 3) ^ (int)(row >> 1)) & 3) << 3) + (lane & 7);
+                    const int64_t at = q_at(row, lane);
                     uint16_t *ra = reinterpret_cast<uint16_t *>(q.RA) + at;
                     uint16_t *rb = reinterpret_cast<uint16_t *>(q.RB) + at;
                     const int64_t ls = (int64_t)q.npad * QN;
@@ -427,141 +586,116 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
             }
         }
         if (k + nb >= N) break;
-        // ---------------- trailing update: 128 x 32 tiles of the lower triangle
-        const int base = k + nb, nbr = (N - base + 127) / 128;
-        // 16 columns a tile when that still is one tile per CTA: half the read-back
-        const int tw = 4 * nbr * (nbr + 1) <= G ? 16 : 32, per = 64 / tw;
-        const int tiles = per * nbr * (nbr + 1);
-        bool ok = true;
-        auto tile_at = [&](int t, int &i0, int &c0) {   // false: beyond the last column
-            int tr = (int)(sqrtf((float)t / (float)per + 0.25f) - 0.5f);
-            while (per * (tr + 1) * (tr + 2) <= t) ++tr;
-            while (per * tr * (tr + 1) > t) --tr;
-            i0 = base + 128 * tr;
-            c0 = base + tw * (t - per * tr * (tr + 1));
-            return c0 < N;
-        };
-        if (wid == Q_EPI) {   // loads: lane l takes modulus l (one thread issuing all 26 copies took 750 cycles each)
-            asm volatile("fence.proxy.async;" ::: "memory");
-            for (int t = g; t < tiles && ok; t += G) {
-                int i0, c0;
-                if (!tile_at(t, i0, c0)) continue;
-                if (tl > 0 && !tc::mbar_wait(&tfull, (tl - 1) & 1)) {   // the previous tile's operands are read
-                    ok = false;
-                    break;
-                }
-                ++tl;
-                if (lane < RL) {
-                    uint8_t *d = ring + lane * Q_STAGE;
-                    tc::mbar_expect_tx(&full[lane], QA_BYTES + tw * 64);
-                    tc::bulk_load(d, q.RA + ((int64_t)lane * q.npad + i0) * QN, QA_BYTES, &full[lane]);
-                    tc::bulk_load(d + QA_BYTES, q.RB + ((int64_t)lane * q.npad + c0) * QN, tw * 64, &full[lane]);
-                }
-                __syncwarp();
-            }
-        } else if (wid < Q_EPI) {
-            const int quad = wid & 3, quarter = wid >> 2;
-            for (int t = g; t < tiles && ok; t += G) {
-                int i0, c0;
-                if (!tile_at(t, i0, c0)) continue;
-                if (wid < RL && lane == 0) {   // this warp's modulus, as soon as it is there
-                    if (tc::mbar_wait(&tempty, (tl & 1) ^ 1) && tc::mbar_wait(&full[wid], tl & 1)) {
-                        tc::fence_after();
-                        const uint32_t ab = tc::smem_u32(ring + wid * Q_STAGE), bb = ab + QA_BYTES;
-#pragma unroll
-                        for (int s = 0; s < 2; ++s) {
-                            const uint64_t da = tc::sw64_kmajor_desc(ab + 32 * s), db = tc::sw64_kmajor_desc(bb + 32 * s);
-                            if (tw == 32) tc::mma<false, tc::instr_desc(false, 128, 32)>(tmem + 32 * wid, da, db, s ? 1u : 0u);
-                            else tc::mma<false, tc::instr_desc(false, 128, 16)>(tmem + 32 * wid, da, db, s ? 1u : 0u);
-                        }
-                        tc::commit(&tfull);
-                    }
-                }
-                __syncwarp();
-                const int i = i0 + 32 * quad + lane, cb = c0 + (tw / 4) * quarter;
-                const int Ei = i < N ? __ldcg(q.rowE + i) : 0;
-                const int Ecl = lane < 8 && cb + lane < N ? __ldcg(q.rowE + cb + lane) : 0;
-                // two entries of A in use, the next two in flight
-                double old[2], nxt[2];
-                auto fetch = [&](double (&d)[2], int c) {
-#pragma unroll
-                    for (int j = 0; j < 2; ++j)
-                        d[j] = i < N && c + j <= i ? __ldcg(a.A + i + (int64_t)(c + j) * N) : 0.0;
-                };
-                fetch(nxt, cb);
-                if (!tc::mbar_wait(&tfull, tl & 1)) {
-                    ok = false;
-                    break;
-                }
-                ++tl;
-                tc::fence_after();
-                // parts of the tile above the diagonal or beyond N: nothing to do (warp-uniform)
-                const int nbatch = i0 + 32 * quad < N && cb <= i0 + 32 * quad + 31 ? tw / 8 : 0;
-#pragma unroll 1
-                for (int b = 0; b < nbatch; ++b) {
-                    const int c = cb + 2 * b;
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) old[j] = nxt[j];
-                    if (b + 1 < nbatch) fetch(nxt, c + 2);
-                    uint32_t r[RL][2];
-                    __syncwarp();
-#pragma unroll
-                    for (int l = 0; l < RL; ++l)
-                        tc::tmem_ld2_async(tmem + ((uint32_t)(32 * quad) << 16) + (uint32_t)(32 * l + (tw / 4) * quarter + 2 * b), r[l]);
-                    tc::tmem_wait_ld();
-#pragma unroll
-                    for (int l = 0; l < RL; ++l)   // the values exist only after the wait
-                        asm volatile("" : "+r"(r[l][0]), "+r"(r[l][1]));
-                    unsigned long long acc[2][4] = {};   // per entry, 32-bit limbs
-                    uint64_t yp = 0;                     // the pair's first residues
-#pragma unroll
-                    for (int l = 0; l < RL; ++l) {
-                        const float pf = c_tab13.p[l], pi = c_tab13.pinv[l];
-                        const uint64_t x = rns::pk(__uint_as_float(r[l][0]), __uint_as_float(r[l][1]));
-                        const uint64_t qq = rns::add2(rns::fma2(x, rns::pk(pi, pi), rns::pk(rns::kMagic, rns::kMagic)),
-                                                      rns::pk(-rns::kMagic, -rns::kMagic));
-                        const uint64_t y = rns::fma2(rns::pk(-pf, -pf), qq, x);   // x mod p
-                        if (l % 2 == 0 && l + 1 < RL) {
-                            yp = y;
-                            continue;
-                        }
-                        // z = y_p q + y_q p (exact); z + 2^19 is the low 23 bits of z + 2^23 + 2^19
-                        const uint64_t zb = rns::pk(8912896.0f, 8912896.0f);
-                        const float pp = c_tab13.p[l > 0 ? l - 1 : 0];
-                        const uint64_t z =
-                            l % 2 ? rns::add2(rns::fma2(yp, rns::pk(pf, pf), rns::mul2(y, rns::pk(pp, pp))), zb) : rns::add2(y, zb);
-                        const float2 zf = rns::upk(z);
-                        const uint32_t u0 = __float_as_uint(zf.x) & 0x7fffffu, u1 = __float_as_uint(zf.y) & 0x7fffffu;
-#pragma unroll
-                        for (int m = 0; m < 4; ++m) {
-                            acc[0][m] += (unsigned long long)u0 * c_tab13.mpair32[l / 2][m];
-                            acc[1][m] += (unsigned long long)u1 * c_tab13.mpair32[l / 2][m];
-                        }
-                    }
-#pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        // T = sum z M/(p q) + bias; X = T - bias - k M with k = rint((T - bias) / M)
-                        unsigned __int128 T = ((unsigned __int128)acc[j][3] << 96) + ((unsigned __int128)acc[j][2] << 64) +
-                                              ((unsigned __int128)acc[j][1] << 32) + acc[j][0];
-                        const float f = fmaf((float)(uint32_t)(T >> 96), c_tab13.top, -c_tab13.btop) + rns::kMagic;
-                        const uint4 km = s_km[(__float_as_uint(f) + 8u) & 15u];   // kMagic's low bits are zero
-                        T += ((unsigned __int128)(((unsigned long long)km.w << 32) | km.z) << 64) |
-                             (((unsigned long long)km.y << 32) | km.x);
-                        const int Ec = __shfl_sync(0xffffffffu, Ecl, 2 * b + j);
-                        if (i < N && c + j <= i)
-                            a.A[i + (int64_t)(c + j) * N] = old[j] - rns::to_double(T, Ei + Ec - 2 * QB);
-                    }
-                }
-                tc::fence_before();
-                __syncwarp();
-                if (lane == 0) tc::mbar_arrive(&tempty);
-            }
-        }
+        // ---------------- trailing update
+        const int base = k + nb;
+        const QUpdate up{a.A, q.RA, q.RB, q.rowE, q.rowE, N, q.npad, base, base};
+        const bool ok = q_update(up, G, g, ring, tmem, full, &tfull, &tempty, s_km, tl);
         if (!ok) atomicExch(&a.bar->err, 1);
         __threadfence();
         if (!panel_barrier(a.bar, epoch, a.wait_ns)) break;
     }
     release();
+}
+
+// ---------------------------------------------------------------------------
+// The same update after a pivoting panel of at most 32 columns with 1x1 and 2x2
+// pivots: X = L with column t scaled by 2^h_t, Y = W by 2^-h_t, 2 h_t the
+// exponent of the pivot (block), which balances the two as |d|^1/2 does above.
+// (N = 2003: 64-column panels with DFMA tiles 3.9 ms of updates, 31-column ones
+// so 1.65, and the panels' own FP64 products halved.)
+// ---------------------------------------------------------------------------
+struct RnsTrailing {
+    int N, npad;
+    double *A;
+    const double *L, *Dd, *Doff, *Wg, *maxabs;
+    const PanelState *st;
+    bf16 *RA, *RB;
+    int *EA, *EB, *flag, *err;
+    int tag;   // of this panel: *flag == tag when its update has to be done term by term
+};
+
+constexpr int RT_THREADS = 256;
+
+// residues of the rows below the panel, a warp per row, lane = panel column
+__global__ void __launch_bounds__(RT_THREADS) k_bk_rns_rows(RnsTrailing a) {
+    pdl_wait();
+    pdl_release();
+    __shared__ int s_h[QN];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, N = a.N, kb = a.st->kb, first = a.st->k, k = first - kb;
+    if (first >= N || kb <= 0) return;
+    if (threadIdx.x < QN) {
+        int h = 0;
+        if (lane < kb) {
+            double d = fabs(a.Dd[k + lane]);
+            const double o = a.Doff[k + lane], p = lane > 0 ? a.Doff[k + lane - 1] : 0.0;
+            if (o != 0.0) d = fmax(fmax(d, fabs(o)), fabs(a.Dd[k + lane + 1]));
+            else if (p != 0.0) d = fmax(fmax(d, fabs(p)), fabs(a.Dd[k + lane - 1]));
+            const int ef = (int)((__double_as_longlong(d) >> 52) & 0x7ff);
+            if (ef != 0 && ef != 0x7ff) h = (ef - 1023) >> 1;
+        }
+        s_h[lane] = h;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0 && !(__ldg(a.maxabs) > 0x1p-900)) atomicExch(a.flag, a.tag);
+    __syncthreads();
+    const int h = s_h[lane];
+    const int64_t ls = (int64_t)a.npad * QN;
+    for (int i = first + (int)blockIdx.x * (RT_THREADS / 32) + wid; i < N; i += (int)gridDim.x * (RT_THREADS / 32)) {
+        const int64_t at = q_at(i, lane);
+#pragma unroll
+        for (int side = 0; side < 2; ++side) {
+            const double v = lane < kb ? (side ? a.Wg[i + (int64_t)lane * N] : a.L[i + (int64_t)(k + lane) * N]) : 0.0;
+            const int se = side ? -h : h;
+            const int ef = (int)((__double_as_longlong(v) >> 52) & 0x7ff);
+            if (ef == 0x7ff) atomicExch(a.flag, a.tag);
+            const int E = __reduce_max_sync(0xffffffffu, ef != 0 ? ef - 1023 + se : -100000) + 2;
+            const rns::Limbs x = rns::limbs(rns::scaled_int(v, 1ULL << 63, se, E, QB));
+            const uint32_t sg = v < 0.0 ? 0x8000u : 0u;
+            if (lane == 0) (side ? a.EB : a.EA)[i] = E;
+            uint16_t *out = reinterpret_cast<uint16_t *>(side ? a.RB : a.RA) + at;
+#pragma unroll
+            for (int l = 0; l < RL; ++l) {
+                float r = rns::residue(c_tab13, l, x);
+                if (side) r = rns::mod(r * c_tab13.inv[l], c_tab13.p[l], c_tab13.pinv[l]);
+                out[l * ls] = (uint16_t)((__float_as_uint(r) >> 16) ^ sg);
+            }
+        }
+    }
+}
+
+__global__ void __launch_bounds__(Q_THREADS, 1) k_bk_rns_trailing(RnsTrailing a) {
+    pdl_wait();
+    pdl_release();
+    extern __shared__ uint8_t psm_raw[];
+    uint8_t *ring = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(psm_raw) + 1023) & ~uintptr_t(1023));
+    __shared__ uint4 s_km[16];
+    __shared__ __align__(8) uint64_t full[RL], tfull, tempty;
+    __shared__ uint32_t s_tmem;
+    const int N = a.N, kb = a.st->kb, first = a.st->k, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    if (first >= N || kb <= 0) return;
+    if (*a.flag == a.tag) {   // entries that the integer form does not hold: term by term
+        for (int64_t e = (int64_t)blockIdx.x * Q_THREADS + tid; e < (int64_t)(N - first) * (N - first);
+             e += (int64_t)gridDim.x * Q_THREADS) {
+            const int i = first + (int)(e % (N - first)), c = first + (int)(e / (N - first));
+            if (c > i) continue;
+            double s = 0.0;
+            for (int t = 0; t < kb; ++t) s = fma(a.L[i + (int64_t)(first - kb + t) * N], a.Wg[c + (int64_t)t * N], s);
+            a.A[i + (int64_t)c * N] -= s;
+        }
+        return;
+    }
+    q_update_init(full, &tfull, &tempty, s_km);
+    if (tid == 0) asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (wid == 0) tc::tmem_alloc(&s_tmem, 512);
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    int tl = 0;
+    const QUpdate up{a.A, a.RA, a.RB, a.EA, a.EB, N, a.npad, first & ~7, first};
+    if (!q_update(up, (int)gridDim.x, (int)blockIdx.x, ring, s_tmem, full, &tfull, &tempty, s_km, tl)) atomicExch(a.err, 1);
+    if (wid == Q_EPI && tl > 0 && lane < RL) tc::mbar_wait(&full[lane], (tl - 1) & 1);   // no copy in flight on the way out
+    tc::fence_before();
+    __syncthreads();
+    if (wid == 0) tc::tmem_dealloc(s_tmem, 512);
 }
 
 int64_t q_npad(int64_t N) { return (N + 127) / 128 * 128 + 128; }
@@ -571,7 +705,7 @@ size_t al256(size_t b) { return (b + 255) / 256 * 256; }
 
 size_t persist64_scratch_bytes(int64_t N) {
     const size_t np = (size_t)q_npad(std::max<int64_t>(N, 1));
-    return 2 * al256(RL * np * QN * sizeof(bf16)) + al256(np * sizeof(int));
+    return 2 * al256(RL * np * QN * sizeof(bf16)) + 2 * al256(np * sizeof(int)) + 256;
 }
 
 void launch_persist64(cudaStream_t s, int num_sms, int64_t N, const PersistArgs &pa, void *scratch) {
@@ -598,6 +732,42 @@ void launch_persist64(cudaStream_t s, int num_sms, int64_t N, const PersistArgs 
     void *kargs[] = {&q};
     MDSIP_CUDA(cudaLaunchCooperativeKernel((const void *)k_bk_persist64, dim3(G), dim3(Q_THREADS), kargs, kQSmem, s));
     count_launch();
+}
+
+// Trailing update after the pivoting panel numbered `panel` (from 0) of at most
+// 32 columns; rest: at most this many columns are left (the panel state says how
+// many).  scratch: the persistent kernel's.
+void launch_rns_trailing(cudaStream_t s, int num_sms, int64_t N, int64_t rest, int panel, double *A, const double *L,
+                         const double *Dd, const double *Doff, const double *Wg, const double *maxabs,
+                         const PanelState *st, int *err, void *scratch) {
+    RnsTrailing a{};
+    a.N = (int)N;
+    a.npad = (int)q_npad(N);
+    a.A = A;
+    a.L = L;
+    a.Dd = Dd;
+    a.Doff = Doff;
+    a.Wg = Wg;
+    a.maxabs = maxabs;
+    a.st = st;
+    const size_t rb = al256((size_t)RL * a.npad * QN * sizeof(bf16)), eb = al256((size_t)a.npad * sizeof(int));
+    char *w = static_cast<char *>(scratch);
+    a.RA = reinterpret_cast<bf16 *>(w);
+    a.RB = reinterpret_cast<bf16 *>(w + rb);
+    a.EA = reinterpret_cast<int *>(w + 2 * rb);
+    a.EB = reinterpret_cast<int *>(w + 2 * rb + eb);
+    a.flag = reinterpret_cast<int *>(w + 2 * rb + 2 * eb);
+    a.err = err;
+    a.tag = panel + 1;
+    static PerDeviceOnce once;
+    MDSIP_CUDA(once.run([] {
+        return cudaFuncSetAttribute(k_bk_rns_trailing, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kQSmem);
+    }));
+    if (panel == 0) MDSIP_CUDA(cudaMemsetAsync(a.flag, 0, sizeof(int), s));
+    const int64_t nbr = (rest + 7 + 127) / 128;
+    launch_pdl(k_bk_rns_rows, (unsigned)std::min<int64_t>(4 * num_sms, ceil_div(rest, RT_THREADS / 32)), RT_THREADS, 0, s, 1, a);
+    launch_pdl(k_bk_rns_trailing, (unsigned)std::min<int64_t>(num_sms, 4 * nbr * (nbr + 1)), Q_THREADS,
+               (size_t)1024 + RL * Q_STAGE, s, 1, a);
 }
 
 }  // namespace mdsip
