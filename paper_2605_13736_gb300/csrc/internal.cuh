@@ -518,6 +518,8 @@ const int *launch_syrk_rns(cudaStream_t s, int num_sms, const double *A, int64_t
 // Tensor-core SYRK (syrk_tc.cu)
 struct TcPlan {
     int tiles, nsplit, slabs_per_split, total_slabs, elems_per_slab;
+    int nt, blocks;   // 128-row blocks; 256 x 256 blocks of the lower triangle (wide)
+    bool wide;
     int64_t ldt;
     size_t work_floats;
 };

@@ -16,8 +16,8 @@
 //     tcgen05.commit on its mbarrier;
 //   * all four warps read the accumulator with tcgen05.ld (32 lanes each)
 //     and write the partial tile, transposed for coalesced reduction.
-// Every mbarrier wait is bounded; on expiry the kernel raises an error flag
-// instead of hanging.
+// Wide products take 256 x 256 blocks (k_syrk_tc_wide).  Every mbarrier wait is
+// bounded; on expiry the kernel raises an error flag instead of hanging.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -57,6 +57,7 @@ __device__ __forceinline__ void tile_of(int t, int &tp, int &tq) {
 
 struct TcArgs {
     int tiles;            // lower-triangle tiles
+    int nt;               // 128-row blocks
     int slabs_per_split;  // K slabs per split
     int total_slabs;      // K slabs overall
     int elems_per_slab;   // 64 (BF16) or 32 (TF32)
@@ -155,6 +156,113 @@ __global__ void __launch_bounds__(TC_THREADS, 2) k_syrk_tc(const __grid_constant
     __syncthreads();
     if (warp == 0)
         tc::tmem_dealloc(tmem, TMEM_COLS);
+}
+
+// The same for wide products: one CTA = one 256 x 256 block of the lower
+// triangle (four tiles, all 512 TMEM columns) x one K range.  With M = N = 128
+// an instruction reads 8 KB of operands from shared memory per 64 (TF32) cycles
+// of the tensor core and TMA writes as much per slab: twice the shared memory's
+// 128 B a cycle, which held the 128 x 128 kernel to 500 TFLOP/s in TF32.  M = 128,
+// N = 256 over a 256-row block asks for 160.  Diagonal blocks take both operands
+// from one copy and leave out the tile above the diagonal.  n = 4000, m = 200000
+// TF32: 6.9 -> 4.05 ms; n = 2000, m = 100000 BF16: 317 -> 253 us.
+constexpr int WT_THREADS = 256, WT_STAGES = 3;
+constexpr int WT_STAGE = 4 * TILE_BYTES;               // two row blocks of each operand
+constexpr size_t kWideSmem = 1024 + (size_t)WT_STAGES * WT_STAGE;
+
+template <bool TF32>
+__global__ void __launch_bounds__(WT_THREADS, 1) k_syrk_tc_wide(const __grid_constant__ CUtensorMap tmap, TcArgs a) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    __shared__ __align__(8) uint64_t full[WT_STAGES], empty[WT_STAGES], accum;
+    __shared__ uint32_t s_tmem;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int P, Q;
+    tile_of(blockIdx.x, P, Q);
+    const bool diag = P == Q;
+    const int split = blockIdx.y;
+    const int s0 = split * a.slabs_per_split;
+    const int s1 = min(a.total_slabs, s0 + a.slabs_per_split);
+    const int nslab = max(0, s1 - s0);
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < WT_STAGES; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(&accum, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmap)) : "memory");
+    }
+    if (warp == 0) tc::tmem_alloc(&s_tmem, 512);
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const uint32_t tmem = s_tmem;
+    if (warp == 0 && lane == 0) {
+        int it = 0;
+        for (; it < nslab; ++it) {
+            const int st = it % WT_STAGES, rnd = it / WT_STAGES;
+            if (!mbar_wait(&empty[st], (rnd & 1) ^ 1)) {
+                atomicExch(a.err, 1);
+                break;
+            }
+            mbar_expect_tx(&full[st], diag ? WT_STAGE / 2 : WT_STAGE);
+            const int kx = (s0 + it) * a.elems_per_slab;
+            uint8_t *d = smem + st * WT_STAGE;
+            tma_load_2d(d, &tmap, &full[st], kx, P * 256);
+            tma_load_2d(d + TILE_BYTES, &tmap, &full[st], kx, P * 256 + TC_TILE);
+            if (!diag) {
+                tma_load_2d(d + 2 * TILE_BYTES, &tmap, &full[st], kx, Q * 256);
+                tma_load_2d(d + 3 * TILE_BYTES, &tmap, &full[st], kx, Q * 256 + TC_TILE);
+            }
+        }
+        // no copy is in flight when the CTA leaves
+        for (int x = max(0, it - WT_STAGES); x < it; ++x) mbar_wait(&full[x % WT_STAGES], (x / WT_STAGES) & 1);
+    } else if (warp == 1 && lane == 0) {
+        for (int it = 0; it < nslab; ++it) {
+            const int st = it % WT_STAGES, rnd = it / WT_STAGES;
+            if (!mbar_wait(&full[st], rnd & 1)) {
+                atomicExch(a.err, 1);
+                break;
+            }
+            fence_after();
+            const uint32_t ab = smem_u32(smem + st * WT_STAGE), bb = diag ? ab : ab + 2 * TILE_BYTES;
+#pragma unroll
+            for (int k = 0; k < SLAB_BYTES / 32; ++k) {
+                const uint32_t on = (it > 0 || k > 0) ? 1u : 0u;
+                const uint64_t db = sw128_kmajor_desc(bb + 32 * k);
+                if (diag)
+                    tc::mma<TF32, tc::instr_desc(TF32, TC_TILE, 128)>(tmem, sw128_kmajor_desc(ab + 32 * k), db, on);
+                else
+                    tc::mma<TF32, tc::instr_desc(TF32, TC_TILE, 256)>(tmem, sw128_kmajor_desc(ab + 32 * k), db, on);
+                tc::mma<TF32, tc::instr_desc(TF32, TC_TILE, 256)>(tmem + 256, sw128_kmajor_desc(ab + TILE_BYTES + 32 * k), db, on);
+            }
+            commit(&empty[st]);
+        }
+        commit(&accum);
+    }
+    __syncwarp();
+    // warps 0-3: the upper row block's lanes, 4-7: the lower one's
+    const bool ok = mbar_wait(&accum, 0);
+    fence_after();
+    const int h = warp >> 2, quad = warp & 3, row = quad * 32 + lane, tp = 2 * P + h;
+    if (!ok) atomicExch(a.err, 1);
+    for (int b = 0; b < 2; ++b) {
+        const int tq = 2 * Q + b;
+        if (tp >= a.nt || tq > tp) continue;
+        float *out = a.work + ((size_t)split * a.tiles + (size_t)tp * (tp + 1) / 2 + tq) * (TC_TILE * TC_TILE);
+#pragma unroll 1
+        for (int c = 0; c < TC_TILE / 32; ++c) {
+            uint32_t r[32];
+            __syncwarp();
+            tmem_ld32(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(256 * h + 128 * b + c * 32), r);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) out[(size_t)(c * 32 + j) * TC_TILE + row] = ok && nslab > 0 ? __uint_as_float(r[j]) : 0.0f;
+        }
+    }
+    fence_before();
+    __syncthreads();
+    if (warp == 0) tc::tmem_dealloc(tmem, 512);
 }
 
 // AfT[p][i] = (float) A[i][p]  (transposed FP32 copy, zero padded to ldt)
@@ -304,6 +412,10 @@ void launch_transpose_f32(cudaStream_t s, const double *A, int64_t m, int64_t n,
     MDSIP_LAUNCHED();
 }
 
+// Columns above which the product takes 256 x 256 blocks: there the two meet (n =
+// 1200, m = 60000 BF16 with the sum of the splits 96 us narrow, 94 wide).
+constexpr int64_t kWideMin = 1024;
+
 TcPlan syrk_tc_plan(int64_t m, int64_t n, int num_sms, int precision) {
     TcPlan pl{};
     const int64_t ldt = syrk_tc_ld(m);
@@ -311,18 +423,41 @@ TcPlan syrk_tc_plan(int64_t m, int64_t n, int num_sms, int precision) {
     pl.tiles = (int)(nt * (nt + 1) / 2);
     pl.elems_per_slab = precision == MDSIP_PREC_TF32 ? 32 : 64;
     pl.total_slabs = (int)(ldt / pl.elems_per_slab);
-    // split-K so that (tile, split) items fill whole waves of two CTAs per SM
-    double best = 0.0;
+    pl.nt = (int)nt;
     pl.nsplit = 1;
-    for (int s = 1; s <= 64; ++s) {
-        if (s > 1 && pl.total_slabs / s < 8) break;
-        const double waves = (double)pl.tiles * s / (2.0 * num_sms);
-        const double eff = waves / std::ceil(waves);
-        if (eff > best + 0.005) {
-            best = eff;
-            pl.nsplit = s;
+    const int64_t mt = (nt + 1) / 2;   // 256-row blocks
+    pl.wide = n > kWideMin;
+    {
+        // split-K so that (tile, split) items fill whole waves of two CTAs per SM
+        double best = 0.0;
+        for (int s = 1; s <= 64; ++s) {
+            if (s > 1 && pl.total_slabs / s < 8) break;
+            const double waves = (double)pl.tiles * s / (2.0 * num_sms);
+            const double eff = waves / std::ceil(waves);
+            if (eff > best + 0.005) {
+                best = eff;
+                pl.nsplit = s;
+            }
+            if (eff >= 0.985) break;
         }
-        if (eff >= 0.985) break;
+    }
+    if (pl.wide) {
+        // one CTA per SM; no fewer splits than above, so that no FP32 sum is longer:
+        // the product at about 80% of its tensor rate over the fill of the last wave,
+        // plus the partials' way out and back
+        pl.blocks = (int)(mt * (mt + 1) / 2);
+        const double flop = (double)pl.blocks * 256 * 256 * 2 * (double)ldt;
+        const double t0 = flop / (precision == MDSIP_PREC_TF32 ? 0.8e15 : 1.5e15);
+        double best = 1e30;
+        for (int s = pl.nsplit, first = s; s <= 64; ++s) {
+            if (s > first && pl.total_slabs / s < 16) break;
+            const double waves = (double)pl.blocks * s / num_sms;
+            const double t = t0 * std::ceil(waves) / waves + 2.0 * s * pl.tiles * (TC_TILE * TC_TILE * 4.0) / 5e12;
+            if (t < 0.99 * best) {
+                best = t;
+                pl.nsplit = s;
+            }
+        }
     }
     pl.slabs_per_split = (pl.total_slabs + pl.nsplit - 1) / pl.nsplit;
     pl.nsplit = (pl.total_slabs + pl.slabs_per_split - 1) / pl.slabs_per_split;  // no empty split
@@ -370,12 +505,13 @@ void launch_syrk_tc(cudaStream_t s, int num_sms, int precision, const float *AfT
 
     TcArgs a{};
     a.tiles = pl.tiles;
+    a.nt = pl.nt;
     a.slabs_per_split = pl.slabs_per_split;
     a.total_slabs = pl.total_slabs;
     a.elems_per_slab = pl.elems_per_slab;
     a.work = work;
     a.err = err_dev;
-    const dim3 grid((unsigned)pl.tiles, (unsigned)pl.nsplit);
+    const dim3 grid((unsigned)(pl.wide ? pl.blocks : pl.tiles), (unsigned)pl.nsplit);
     static PerDeviceOnce once;
     MDSIP_CUDA(once.run([] {
         cudaError_t e =
@@ -383,9 +519,17 @@ void launch_syrk_tc(cudaStream_t s, int num_sms, int precision, const float *AfT
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_syrk_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)kTcSmemBytes);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_syrk_tc_wide<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWideSmem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_syrk_tc_wide<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWideSmem);
         return e;
     }));
-    if (tf32)
+    if (pl.wide && tf32)
+        k_syrk_tc_wide<true><<<grid, WT_THREADS, kWideSmem, s>>>(tmap, a);
+    else if (pl.wide)
+        k_syrk_tc_wide<false><<<grid, WT_THREADS, kWideSmem, s>>>(tmap, a);
+    else if (tf32)
         k_syrk_tc<true><<<grid, TC_THREADS, kTcSmemBytes, s>>>(tmap, a);
     else
         k_syrk_tc<false><<<grid, TC_THREADS, kTcSmemBytes, s>>>(tmap, a);
