@@ -256,6 +256,49 @@ __device__ __forceinline__ long long ord64(double v) {
     return b ^ ((b >> 63) & 0x7fffffffffffffffLL);
 }
 
+// |v| by its bit pattern into a running maximum (NaN passed over, as fmax does)
+__device__ __forceinline__ void max_abs(unsigned long long &m, double v) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL;
+    if (b > m && b <= 0x7ff0000000000000ULL) m = b;
+}
+
+// running maximum and minimum of v as ordered integers (NaN passed over)
+struct MinMax {
+    long long hi = (long long)0x800fffffffffffffULL, lo = 0x7ff0000000000000LL;   // of -inf and inf
+    __device__ __forceinline__ void add(double v) {
+        const long long k = ord64(v);
+        if (((unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL) > 0x7ff0000000000000ULL) return;
+        hi = k > hi ? k : hi;
+        lo = k < lo ? k : lo;
+    }
+    static __device__ __forceinline__ double value(long long k) {
+        return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffLL));
+    }
+};
+
+// sum of logarithms of positive values: the mantissas' product and the
+// exponents' sum, one logarithm in the end (some 35 FP64 instructions each)
+struct LogSum {
+    double m = 1.0, rest = 0.0;
+    int e = 0;
+    __device__ __forceinline__ void add(double v) {
+        const long long b = __double_as_longlong(v);
+        const int ef = (int)(b >> 52);   // sign included
+        if (ef <= 0 || ef >= 0x7ff) {    // not a positive normal number
+            rest += log(v);
+            return;
+        }
+        const double p = m * __longlong_as_double((b & 0xfffffffffffffLL) | (1023LL << 52));   // in [1, 4)
+        const long long q = __double_as_longlong(p);
+        const int ep = (int)(q >> 52) - 1023;
+        e += ef - 1023 + ep;
+        m = __longlong_as_double(q - ((long long)ep << 52));
+    }
+    __device__ __forceinline__ double value() const {
+        return fma((double)e, 0.69314718055994530942, log(m)) + rest;
+    }
+};
+
 // ---------------------------------------------------------------------------
 // Grid-wide reductions of up to 8 quantities in one kernel (deterministic for
 // a fixed launch shape): warps by shuffles, the block's warps by one warp per
@@ -295,7 +338,7 @@ template <int NT, RedOp... OPS>
 __device__ __forceinline__ void reduce_finish(double (&v)[sizeof...(OPS)], const RedOut &o) {
     constexpr int K = sizeof...(OPS), W = NT / 32;
     constexpr RedOp ops[K] = {OPS...};
-    static_assert(K <= W && W <= 32, "one warp per quantity");
+    static_assert(W <= 32, "a quantity's warp sums fit a warp");
     __shared__ double sh[K][W];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
 #pragma unroll
@@ -308,7 +351,7 @@ __device__ __forceinline__ void reduce_finish(double (&v)[sizeof...(OPS)], const
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < K; ++k)
-        if (wid == k) {
+        if (wid == k % W) {
             double x = lane < W ? sh[k][lane] : red_identity(ops[k]);
 #pragma unroll
             for (int s = W / 2; s > 0; s >>= 1) x = red_combine(ops[k], x, __shfl_xor_sync(0xffffffffu, x, s));
@@ -317,7 +360,7 @@ __device__ __forceinline__ void reduce_finish(double (&v)[sizeof...(OPS)], const
     if (gridDim.x == 1 || !red_last(o.ticket)) return;
 #pragma unroll
     for (int k = 0; k < K; ++k)
-        if (wid == k) {
+        if (wid == k % W) {
             double p[(kRedBlocks + 31) / 32];
 #pragma unroll
             for (int i = 0; i < (kRedBlocks + 31) / 32; ++i)
@@ -346,19 +389,19 @@ __device__ __forceinline__ void count_finish(unsigned (&c)[K], const RedOut &o) 
         for (int k = 0; k < K; ++k) sh[k][wid] = c[k];
     __syncthreads();
     unsigned *part = reinterpret_cast<unsigned *>(o.partial);
-    if (wid < K) {
-        const unsigned x = __reduce_add_sync(0xffffffffu, lane < W ? sh[wid][lane] : 0u);
+    for (int k = wid; k < K; k += W) {
+        const unsigned x = __reduce_add_sync(0xffffffffu, lane < W ? sh[k][lane] : 0u);
         if (lane == 0) {
-            if (gridDim.x == 1) o.out[wid] = (double)x;
-            else part[(size_t)wid * kRedBlocks + blockIdx.x] = x;
+            if (gridDim.x == 1) o.out[k] = (double)x;
+            else part[(size_t)k * kRedBlocks + blockIdx.x] = x;
         }
     }
     if (gridDim.x == 1 || !red_last(o.ticket)) return;
-    if (wid < K) {
+    for (int k = wid; k < K; k += W) {
         unsigned x = 0;
-        for (int i = lane; i < (int)gridDim.x; i += 32) x += __ldcg(part + (size_t)wid * kRedBlocks + i);
+        for (int i = lane; i < (int)gridDim.x; i += 32) x += __ldcg(part + (size_t)k * kRedBlocks + i);
         x = __reduce_add_sync(0xffffffffu, x);
-        if (lane == 0) o.out[wid] = (double)x;
+        if (lane == 0) o.out[k] = (double)x;
     }
 }
 
@@ -385,8 +428,8 @@ __device__ __forceinline__ double colgroup_dot(const double *__restrict__ J, int
 }
 
 // blocks of a reduction kernel over `len` elements or more (one per thread)
-inline int red_grid(int64_t len) {
-    return (int)std::max<int64_t>(1, std::min<int64_t>(kRedBlocks, (len + kRedThreads - 1) / kRedThreads));
+inline int red_grid(int64_t len, int threads = kRedThreads) {
+    return (int)std::max<int64_t>(1, std::min<int64_t>(kRedBlocks, (len + threads - 1) / threads));
 }
 
 // ---------------------------------------------------------------------------

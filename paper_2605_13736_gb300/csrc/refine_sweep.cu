@@ -499,12 +499,6 @@ __global__ void __launch_bounds__(NT) k_sweep_x(int64_t n_d, int64_t m_I, const 
     }
 }
 
-// |v| by its bit pattern into a running maximum (NaN passed over, as fmax does)
-__device__ __forceinline__ void max_abs(unsigned long long &m, double v) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL;
-    if (b > m && b <= 0x7ff0000000000000ULL) m = b;
-}
-
 // The rest of the sweep: u_s, u_d, u_h, the residual r = b - K u with its norms
 // (||r||, ||b||, ||K u||, ||u|| in the maximum norm), A^T u_g and the next
 // right-hand side of the reduced system from the CTAs' partial column sums.

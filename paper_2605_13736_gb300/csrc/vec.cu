@@ -15,6 +15,7 @@ constexpr int NT = kRedThreads;
 // ---------------------------------------------------------------------------
 // Model: f and grad f.  f = 1/2 x_d^T Q x_d + sum 1/4 x_s^4 + c^T x
 // ---------------------------------------------------------------------------
+template <int NT>
 __global__ void __launch_bounds__(NT) k_eval_f(Dims D, ModelView M, const double *__restrict__ x,
                                                double *__restrict__ grad, RedOut red) {
     double acc = 0.0;
@@ -49,6 +50,7 @@ __global__ void __launch_bounds__(NT) k_eval_f(Dims D, ModelView M, const double
 // Model: constraint residuals cg = g(x) - g_E (warp per row: sparse part plus
 // the dense row of A), ch = h(x) - d.  Reductions: sum |c|, max |c|.
 // ---------------------------------------------------------------------------
+template <int NT>
 __global__ void __launch_bounds__(NT) k_eval_cons(Dims D, ModelView M, const double *__restrict__ x,
                                                   const double *__restrict__ Axd, const double *__restrict__ d,
                                                   double *__restrict__ cg, double *__restrict__ ch,
@@ -305,60 +307,57 @@ __global__ void __launch_bounds__(NT) k_lagrangian_grad(Dims D, ModelView M, con
 // quantities: 0 max|dual| (max), 1 max|c| (max), 2 max s*z (max),
 //             3 min s*z (min), 4 ||y||_1 (sum), 5 ||z||_1 (sum), 6 sum log s (sum)
 // ---------------------------------------------------------------------------
+template <int NT>
 __global__ void __launch_bounds__(NT) k_errors(Dims D, ModelView M, IterView I,
                                                const double *__restrict__ gl,
                                                const double *__restrict__ cg,
                                                const double *__restrict__ ch, RedOut red) {
-    double du = 0.0, pr = 0.0, cmax = -INFINITY, cmin = INFINITY, y1 = 0.0, z1 = 0.0, lg = 0.0;
+    unsigned long long du = 0, pr = 0;
+    MinMax comp;
+    LogSum lg;
+    double y1 = 0.0, z1 = 0.0;
     const int64_t gtid = (int64_t)blockIdx.x * NT + threadIdx.x;
     const int64_t gsz = (int64_t)gridDim.x * NT;
     for (int64_t i = gtid; i < D.n; i += gsz) {
         const double xi = I.x[i];
-        du = fmax(du, fabs(gl[i] - I.zl[i] + I.zu[i]));
+        max_abs(du, gl[i] - I.zl[i] + I.zu[i]);
         if (fin(M.xl[i])) {
             const double s = xi - M.xl[i];
-            const double p = s * I.zl[i];
-            cmax = fmax(cmax, p);
-            cmin = fmin(cmin, p);
+            comp.add(s * I.zl[i]);
             z1 += fabs(I.zl[i]);
-            lg += log(s);
+            lg.add(s);
         }
         if (fin(M.xu[i])) {
             const double s = M.xu[i] - xi;
-            const double p = s * I.zu[i];
-            cmax = fmax(cmax, p);
-            cmin = fmin(cmin, p);
+            comp.add(s * I.zu[i]);
             z1 += fabs(I.zu[i]);
-            lg += log(s);
+            lg.add(s);
         }
     }
     for (int64_t j = gtid; j < D.m_I; j += gsz) {
-        du = fmax(du, fabs(-I.yh[j] - I.vl[j] + I.vu[j]));
-        pr = fmax(pr, fabs(ch[j]));
+        max_abs(du, -I.yh[j] - I.vl[j] + I.vu[j]);
+        max_abs(pr, ch[j]);
         y1 += fabs(I.yh[j]);
         const double dj = I.d[j];
         if (fin(M.hl[j])) {
             const double s = dj - M.hl[j];
-            const double p = s * I.vl[j];
-            cmax = fmax(cmax, p);
-            cmin = fmin(cmin, p);
+            comp.add(s * I.vl[j]);
             z1 += fabs(I.vl[j]);
-            lg += log(s);
+            lg.add(s);
         }
         if (fin(M.hu[j])) {
             const double s = M.hu[j] - dj;
-            const double p = s * I.vu[j];
-            cmax = fmax(cmax, p);
-            cmin = fmin(cmin, p);
+            comp.add(s * I.vu[j]);
             z1 += fabs(I.vu[j]);
-            lg += log(s);
+            lg.add(s);
         }
     }
     for (int64_t i = gtid; i < D.m_E; i += gsz) {
-        pr = fmax(pr, fabs(cg[i]));
+        max_abs(pr, cg[i]);
         y1 += fabs(I.yg[i]);
     }
-    double v[7] = {du, pr, cmax, cmin, y1, z1, lg};
+    double v[7] = {__longlong_as_double((long long)du), __longlong_as_double((long long)pr), MinMax::value(comp.hi),
+                   MinMax::value(comp.lo), y1, z1, lg.value()};
     reduce_finish<NT, R_MAX, R_MAX, R_MAX, R_MIN, R_SUM, R_SUM, R_SUM>(v, red);
 }
 
@@ -383,6 +382,7 @@ __device__ __forceinline__ double sigma_x(const ModelView &M, const IterView &I,
     return s;
 }
 
+template <int NT>
 __global__ void __launch_bounds__(NT) k_newton_diag(Dims D, ModelView M, IterView I,
                                                     const double *__restrict__ Hss, double dw,
                                                     double dc, int want_w, double *__restrict__ sig_x,
@@ -585,11 +585,14 @@ __global__ void k_copy(const double *__restrict__ src, double *__restrict__ dst,
 // the farthest bound-feasible point) and grad phi^T d.
 // quantities: 0 alpha_max (min), 1 alpha_z (min), 2 gphi (sum)
 // ---------------------------------------------------------------------------
+// alpha such that v + alpha dv = (1 - tau) v, where that is below 1 (larger ones
+// do not bind: the caller caps alpha at 1)
 __device__ __forceinline__ double ftb(double v, double dv, double tau) {
-    // dv < 0, by its bit pattern (a NaN's quotient is a NaN, which fmin passes over)
-    return (unsigned long long)__double_as_longlong(dv) > 0x8000000000000000ULL ? ddiv(-tau * v, dv) : INFINITY;
+    const double t = tau * v;
+    return -dv > t ? ddiv(-t, dv) : INFINITY;
 }
 
+template <int NT>
 __global__ void __launch_bounds__(NT) k_step_scalars(Dims D, ModelView M, IterView I, DirView Dir,
                                                      const double *__restrict__ grad, double tau,
                                                      double mu, RedOut red) {
@@ -637,10 +640,12 @@ __global__ void __launch_bounds__(NT) k_step_scalars(Dims D, ModelView M, IterVi
 // Trial point x_t = x + alpha dx, d_t = d + alpha dd; sum of log slacks and
 // "strictly inside" count at the trial point.
 // quantities: 0 sum log s (sum), 1 number of non-positive slacks (sum)
+template <int NT>
 __global__ void __launch_bounds__(NT) k_trial(Dims D, ModelView M, IterView I, DirView Dir,
                                               double alpha, double *__restrict__ xt,
                                               double *__restrict__ dt, RedOut red) {
-    double lg = 0.0, bad = 0.0;
+    LogSum lg;
+    unsigned bad = 0;
     const int64_t gtid = (int64_t)blockIdx.x * NT + threadIdx.x;
     const int64_t gsz = (int64_t)gridDim.x * NT;
     for (int64_t i = gtid; i < D.n; i += gsz) {
@@ -648,11 +653,11 @@ __global__ void __launch_bounds__(NT) k_trial(Dims D, ModelView M, IterView I, D
         xt[i] = v;
         if (fin(M.xl[i])) {
             const double s = v - M.xl[i];
-            if (s > 0.0) lg += log(s); else bad += 1.0;
+            if (s > 0.0) lg.add(s); else ++bad;
         }
         if (fin(M.xu[i])) {
             const double s = M.xu[i] - v;
-            if (s > 0.0) lg += log(s); else bad += 1.0;
+            if (s > 0.0) lg.add(s); else ++bad;
         }
     }
     for (int64_t j = gtid; j < D.m_I; j += gsz) {
@@ -660,14 +665,14 @@ __global__ void __launch_bounds__(NT) k_trial(Dims D, ModelView M, IterView I, D
         dt[j] = v;
         if (fin(M.hl[j])) {
             const double s = v - M.hl[j];
-            if (s > 0.0) lg += log(s); else bad += 1.0;
+            if (s > 0.0) lg.add(s); else ++bad;
         }
         if (fin(M.hu[j])) {
             const double s = M.hu[j] - v;
-            if (s > 0.0) lg += log(s); else bad += 1.0;
+            if (s > 0.0) lg.add(s); else ++bad;
         }
     }
-    double v[2] = {lg, bad};
+    double v[2] = {lg.value(), (double)bad};
     reduce_finish<NT, R_SUM, R_SUM>(v, red);
 }
 
@@ -796,7 +801,23 @@ __global__ void k_gather(int64_t n, const double *__restrict__ src, const int32_
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-static int elem_grid(int64_t n) { return std::max(1, std::min(4096, ceil_div(n, 256))); }
+// Up to one element per thread of kRedBlocks blocks of 128 a kernel is one chain
+// of FP64 instructions per thread, 64 cycles each for a warp alone on its
+// sub-partition: such blocks spread them over twice the SMs (2032 variables,
+// with the logarithms and maxima above: k_errors 15.6 -> 11.3 us, k_trial 13.5 ->
+// 9.9).  Longer vectors keep 256: at 51712 a second round took k_newton_diag
+// from 14.7 to 18.6.
+constexpr int64_t kSmallLen = (int64_t)128 * kRedBlocks;
+#define MDSIP_RED(kern, len, ...)                                                      \
+    do {                                                                               \
+        const int64_t len_ = (len);                                                    \
+        if (len_ <= kSmallLen) kern<128><<<red_grid(len_, 128), 128, 0, st>>>(__VA_ARGS__); \
+        else kern<NT><<<red_grid(len_), NT, 0, st>>>(__VA_ARGS__);                     \
+        MDSIP_LAUNCHED();                                                              \
+    } while (0)
+
+static int elem_grid(int64_t n, int threads = 256) { return std::max(1, std::min(4096, ceil_div(n, threads))); }
+static int elem_threads(int64_t n) { return n <= kSmallLen ? 128 : 256; }
 
 // A: rows 16-byte aligned (lda even, A 16-byte aligned); n <= 24560 (v staged in shared memory)
 void launch_gemv_rows(cudaStream_t s, const double *A, int64_t m, int64_t n, int64_t lda,
@@ -843,8 +864,7 @@ void launch_gemv_t(cudaStream_t s, const double *A, int64_t m, int64_t n, int64_
 }
 
 void VecOps::eval_f(const double *x, double *grad, double *out_scalar) {
-    k_eval_f<<<red_grid(std::max(D.n_s, 32 * D.n_d)), NT, 0, st>>>(D, M, x, grad, red(out_scalar));
-    MDSIP_LAUNCHED();
+    MDSIP_RED(k_eval_f, std::max(D.n_s, 32 * D.n_d), D, M, x, grad, red(out_scalar));
 }
 
 void VecOps::eval_cons(const double *x, const double *d, double *cg, double *ch, double *out2) {
@@ -852,14 +872,12 @@ void VecOps::eval_cons(const double *x, const double *d, double *cg, double *ch,
         if (Ahi) launch_gemv_rows_df(st, Ahi, Alo, D.m_E, D.n_d, D.lda, x + D.n_s, split, rowtmp);
         else launch_gemv_rows(st, M.A, D.m_E, D.n_d, D.lda, x + D.n_s, rowtmp);
     }
-    k_eval_cons<<<red_grid(std::max(D.m_E, 32 * D.m_I)), NT, 0, st>>>(D, M, x, rowtmp, d, cg, ch, red(out2));
-    MDSIP_LAUNCHED();
+    MDSIP_RED(k_eval_cons, std::max(D.m_E, 32 * D.m_I), D, M, x, rowtmp, d, cg, ch, red(out2));
 }
 
 void VecOps::eval_cons_ax(const double *x, const double *Ax, const double *d, double *cg, double *ch,
                           double *out2) {
-    k_eval_cons<<<red_grid(std::max(D.m_E, 32 * D.m_I)), NT, 0, st>>>(D, M, x, Ax, d, cg, ch, red(out2));
-    MDSIP_LAUNCHED();
+    MDSIP_RED(k_eval_cons, std::max(D.m_E, 32 * D.m_I), D, M, x, Ax, d, cg, ch, red(out2));
 }
 
 namespace {
@@ -903,27 +921,24 @@ void VecOps::lagrangian_grad_aty(const IterView &I, const double *grad, const do
 
 void VecOps::errors(const IterView &I, const double *gl, const double *cg, const double *ch,
                     double *out7) {
-    k_errors<<<red_grid(std::max(D.n, D.m_E)), NT, 0, st>>>(D, M, I, gl, cg, ch, red(out7));
-    MDSIP_LAUNCHED();
+    MDSIP_RED(k_errors, std::max(D.n, D.m_E), D, M, I, gl, cg, ch, red(out7));
 }
 
 void VecOps::newton_diag(const IterView &I, const double *Hss, double dw, double dc, bool want_w,
                          double *sig_x, double *q, double *sig_d, double *w, double *out6) {
-    k_newton_diag<<<red_grid(std::max(D.n, D.m_E)), NT, 0, st>>>(D, M, I, Hss, dw, dc, want_w ? 1 : 0, sig_x, q, sig_d,
-                                                                 w, red(out6));
-    MDSIP_LAUNCHED();
+    MDSIP_RED(k_newton_diag, std::max(D.n, D.m_E), D, M, I, Hss, dw, dc, want_w ? 1 : 0, sig_x, q, sig_d, w, red(out6));
 }
 
 void VecOps::rhs_y(const IterView &I, const double *gl, const double *cg, const double *q,
                    const double *w, double mu, double *bt_g, double *u) {
-    k_rhs_y<<<elem_grid(D.m_E), 256, 0, st>>>(D, M, I, gl, cg, q, w, mu, bt_g, u);
+    k_rhs_y<<<elem_grid(D.m_E, elem_threads(D.m_E)), elem_threads(D.m_E), 0, st>>>(D, M, I, gl, cg, q, w, mu, bt_g, u);
     MDSIP_LAUNCHED();
 }
 
 void VecOps::rhs_reduced(const IterView &I, const double *gl, const double *ch, const double *sig_d,
                          const double *ATu, const double *bt_g, const double *q, double mu, double dw, bool p1,
                          double *rhs) {
-    k_rhs_reduced<<<elem_grid(std::max(D.n_d, D.m_E)), 256, 0, st>>>(D, M, I, gl, ch, sig_d, ATu, bt_g, q,
+    k_rhs_reduced<<<elem_grid(std::max(D.n_d, D.m_E), elem_threads(std::max(D.n_d, D.m_E))), elem_threads(std::max(D.n_d, D.m_E)), 0, st>>>(D, M, I, gl, ch, sig_d, ATu, bt_g, q,
                                                                      mu, dw, p1 ? 1 : 0, rhs);
     MDSIP_LAUNCHED();
 }
@@ -942,25 +957,23 @@ void VecOps::copy(const double *src, double *dst, int64_t n) {
 void VecOps::backsub(const IterView &I, const DirView &Dir, const double *gl, const double *q,
                      const double *sig_d, const double *sol_dxd, const double *sol_dyh, double mu,
                      double dw) {
-    k_backsub<<<elem_grid(D.n), 256, 0, st>>>(D, M, I, Dir, gl, q, sig_d, sol_dxd, sol_dyh, mu, dw);
+    k_backsub<<<elem_grid(D.n, elem_threads(D.n)), elem_threads(D.n), 0, st>>>(D, M, I, Dir, gl, q, sig_d, sol_dxd, sol_dyh, mu, dw);
     MDSIP_LAUNCHED();
 }
 
 void VecOps::step_scalars(const IterView &I, const DirView &Dir, const double *grad, double tau,
                           double mu, double *out3) {
-    k_step_scalars<<<red_grid(D.n), NT, 0, st>>>(D, M, I, Dir, grad, tau, mu, red(out3));
-    MDSIP_LAUNCHED();
+    MDSIP_RED(k_step_scalars, D.n, D, M, I, Dir, grad, tau, mu, red(out3));
 }
 
 void VecOps::trial(const IterView &I, const DirView &Dir, double alpha, double *xt, double *dt,
                    double *out2) {
-    k_trial<<<red_grid(D.n), NT, 0, st>>>(D, M, I, Dir, alpha, xt, dt, red(out2));
-    MDSIP_LAUNCHED();
+    MDSIP_RED(k_trial, D.n, D, M, I, Dir, alpha, xt, dt, red(out2));
 }
 
 void VecOps::accept(const IterView &I, const DirView &Dir, double alpha, double alpha_z, double mu,
                     double ks) {
-    k_accept<<<elem_grid(std::max(D.n, D.m_E)), 256, 0, st>>>(D, M, I, Dir, alpha, alpha_z, mu, ks);
+    k_accept<<<elem_grid(std::max(D.n, D.m_E), elem_threads(std::max(D.n, D.m_E))), elem_threads(std::max(D.n, D.m_E)), 0, st>>>(D, M, I, Dir, alpha, alpha_z, mu, ks);
     MDSIP_LAUNCHED();
 }
 
