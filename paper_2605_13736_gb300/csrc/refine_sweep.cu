@@ -440,10 +440,12 @@ __global__ void __launch_bounds__(kSwThreads, 1) k_sweep(SweepArgs a) {
     }
 }
 
-// bt = b_g - J_sg (b_s / q), u = bt / w (first approximate solve); 1 / w in FP64 and FP32, 1 / q
+// bt = b_g - J_sg (b_s / q), u = fl32(bt / w) padded to ldt (first approximate solve); 1 / w
+// in FP64 and FP32, 1 / q; the inequalities' part of the first right-hand side
 __global__ void k_sweep_start(Dims D, ModelView M, const double *__restrict__ b, const double *__restrict__ q,
-                              const double *__restrict__ w, double *__restrict__ bt, double *__restrict__ u,
-                              double *__restrict__ winv, float *__restrict__ wf, double *__restrict__ qinv) {
+                              const double *__restrict__ w, double *__restrict__ bt, float *__restrict__ u,
+                              double *__restrict__ winv, float *__restrict__ wf, double *__restrict__ qinv,
+                              int64_t ldt, double *__restrict__ rhsS) {
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, gsz = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = gtid; i < D.m_E; i += gsz) {
         double s = b[D.n + i];
@@ -452,12 +454,14 @@ __global__ void k_sweep_start(Dims D, ModelView M, const double *__restrict__ b,
             s -= ddiv(M.csr_val[e] * b[c], q[c]);
         }
         bt[i] = s;
-        u[i] = ddiv(s, w[i]);
+        u[i] = (float)ddiv(s, w[i]);
         const double r = ddiv(1.0, w[i]);
         winv[i] = r;
         wf[i] = (float)r;
     }
+    for (int64_t i = D.m_E + gtid; i < ldt; i += gsz) u[i] = 0.0f;
     for (int64_t k = gtid; k < D.n_s; k += gsz) qinv[k] = ddiv(1.0, q[k]);
+    for (int64_t j = gtid; j < D.m_I; j += gsz) rhsS[D.n_d + j] = b[D.n + D.m_E + j];
 }
 
 // x = u_d + sol_d, u_h + sol_h into xnew, x and sol_d as FP32 parts, and
@@ -633,10 +637,9 @@ int64_t refine_sweep_parts(int64_t n) { return kRedBlocks / 2 * std::max<int64_t
 bool Refiner::sweep_path() const { return xq && Ahi && solve_fp32 && AfT && D.n_d > 0 && D.n_d <= 4096; }
 
 void Refiner::sweep_start(const double *b) {
-    k_sweep_start<<<grid_for(std::max(D.m_E, D.n_s)), 256, 0, st>>>(D, M, b, q, w, bt, tmp_m, winv, wf, qinv);
+    k_sweep_start<<<grid_for(std::max(D.m_E, D.n_s)), 256, 0, st>>>(D, M, b, q, w, bt, vf, winv, wf, qinv, ldt, rhsS);
     MDSIP_LAUNCHED();
-    launch_aft_dot(st, num_sms, AfT, ldt, D.m_E, D.n_d, tmp_m, vf, tmp_nd);
-    rhs_S(b, tmp_nd);
+    launch_aft_dot_add(st, num_sms, AfT, ldt, D.n_d, vf, b + D.n_s, rhsS);   // b_d + A_hi^T u
 }
 
 void Refiner::sweep(const double *b, double *u, double *r, bool init, double dw, double dc, double *out4) {

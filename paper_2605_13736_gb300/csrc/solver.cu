@@ -1308,15 +1308,19 @@ static mdsip_status run_ipm(Problem *P) {
         rec.n_refine = rr.sweeps;
         rec.fp64_fallback = (rr.ok && !fp64) ? 0 : 1;
         rec.refine_res = rr.res;
-        // the direction's products with A, kept before anything else uses the
-        // refinement's buffers (the FP64 check below computes a direction of its own)
+        // the direction's products with A, in the refinement's buffers until the next
+        // direction (the FP64 check below computes one of its own)
         const bool lin_step = carry_products(P) && P->lin_ax && P->dir_prod;
-        if (lin_step) {
-            P->V.copy(P->bAdx.as<double>(), P->bdAx.as<double>(), D.m_E);
-            P->V.copy(P->bATu.as<double>(), P->bdATy.as<double>(), D.n_d);
-        }
-        if (o.direction_check && use_refined(P) && P->opt.precision != MDSIP_PREC_FP64 && !fp64 && !rr.fell_back)
+        const double *dAx = P->bAdx.as<double>(), *dATy = P->bATu.as<double>();
+        if (o.direction_check && use_refined(P) && P->opt.precision != MDSIP_PREC_FP64 && !fp64 && !rr.fell_back) {
+            if (lin_step) {
+                P->V.copy(dAx, P->bdAx.as<double>(), D.m_E);
+                P->V.copy(dATy, P->bdATy.as<double>(), D.n_d);
+                dAx = P->bdAx.as<double>();
+                dATy = P->bdATy.as<double>();
+            }
             rec.dir_err_fp64 = fp64_direction_error(P, mu, dw, dc);
+        }
         // A.5 line search
         P->V.step_scalars(P->I, P->Dir, P->grad, tau, mu, sc + SC_STEP);
         P->sync_scalars();
@@ -1348,8 +1352,7 @@ static mdsip_status run_ipm(Problem *P) {
             P->V.trial(P->I, P->Dir, alpha, P->xt, P->dt, sc + SC_TRIAL);
             model_f(P, P->xt, P->grad_t, sc + SC_TF);
             if (lin_step) {   // A x_t = A x + alpha A dx (the same trial point)
-                P->V.axpby(D.m_E, P->ax_cur, alpha, P->bdAx.as<double>(), P->ax_t);
-                P->V.eval_cons_ax(P->xt, P->ax_t, P->dt, P->cg_t, P->ch_t, sc + SC_TTHETA);
+                P->V.eval_cons_ax(P->xt, P->ax_cur, P->dt, P->cg_t, P->ch_t, sc + SC_TTHETA, alpha, dAx, P->ax_t);
             } else {
                 model_cons(P, P->xt, P->dt, P->cg_t, P->ch_t, sc + SC_TTHETA);
             }
@@ -1397,10 +1400,9 @@ static mdsip_status run_ipm(Problem *P) {
             filt.emplace_back((1 - o.gamma_theta) * th_k, phi_k - o.gamma_phi * th_k);
         // A.6 accept: the trial becomes the iterate
         swap_trial(P);
-        P->V.accept(P->I, P->Dir, alpha, alpha_z, mu, o.kappa_sigma);
-        if (lin_step) {   // y_g moved by alpha dy_g (k_accept): A^T y_g and A x_d follow
+        P->V.accept(P->I, P->Dir, alpha, alpha_z, mu, o.kappa_sigma, P->bATy.as<double>(), lin_step ? dATy : nullptr);
+        if (lin_step) {   // y_g moved by alpha dy_g: A^T y_g with it in the same kernel, and A x_d
             std::swap(P->ax_cur, P->ax_t);
-            P->V.axpby(D.n_d, P->bATy.as<double>(), alpha, P->bdATy.as<double>(), P->bATy.as<double>());
         } else if (carry_products(P)) {   // the accepted trial's constraints were formed from x_t
             P->V.copy(P->V.rowtmp, P->ax_cur, D.m_E);
             P->lin_ax = true;

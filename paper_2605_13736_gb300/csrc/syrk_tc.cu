@@ -344,10 +344,11 @@ __global__ void k_to_f32_padded(int64_t m, int64_t ldt, const double *__restrict
         vf[i] = i < m ? (float)v[i] : 0.0f;
 }
 
-// out[p] = sum_i AfT[p][i] vf[i] (FP32 products and sums, one block per row of
+// out[p] = (add[p] +) sum_i AfT[p][i] vf[i] (FP32 products and sums, one block per row of
 // AfT, i.e. per column of A; 16-byte loads)
 __global__ void __launch_bounds__(256) k_aft_dot(const float *__restrict__ AfT, int64_t ldt, int64_t n,
-                                                 const float *__restrict__ vf, double *__restrict__ out) {
+                                                 const float *__restrict__ vf, const double *__restrict__ add,
+                                                 double *__restrict__ out) {
     __shared__ float red[8];
     const int64_t q = ldt / 4;
     const float4 *v4 = reinterpret_cast<const float4 *>(vf);
@@ -383,7 +384,7 @@ __global__ void __launch_bounds__(256) k_aft_dot(const float *__restrict__ AfT, 
         if (threadIdx.x == 0) {
             float u = 0.f;
             for (int w = 0; w < 8; ++w) u += red[w];
-            out[p] = (double)u;
+            out[p] = add ? add[p] + (double)u : (double)u;
         }
         __syncthreads();
     }
@@ -398,7 +399,15 @@ void launch_aft_dot(cudaStream_t s, int num_sms, const float *AfT, int64_t ldt, 
     if (n <= 0) return;
     k_to_f32_padded<<<std::max(1, std::min(4096, ceil_div(ldt, 256))), 256, 0, s>>>(m, ldt, v, vf);
     MDSIP_LAUNCHED();
-    k_aft_dot<<<(unsigned)std::min<int64_t>(n, (int64_t)num_sms * 8), 256, 0, s>>>(AfT, ldt, n, vf, out);
+    k_aft_dot<<<(unsigned)std::min<int64_t>(n, (int64_t)num_sms * 8), 256, 0, s>>>(AfT, ldt, n, vf, nullptr, out);
+    MDSIP_LAUNCHED();
+}
+
+// out = add + AfT vf, vf given in FP32 with zeros up to ldt
+void launch_aft_dot_add(cudaStream_t s, int num_sms, const float *AfT, int64_t ldt, int64_t n, const float *vf,
+                        const double *add, double *out) {
+    if (n <= 0) return;
+    k_aft_dot<<<(unsigned)std::min<int64_t>(n, (int64_t)num_sms * 8), 256, 0, s>>>(AfT, ldt, n, vf, add, out);
     MDSIP_LAUNCHED();
 }
 

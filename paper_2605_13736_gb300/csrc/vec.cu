@@ -53,7 +53,8 @@ __global__ void __launch_bounds__(NT) k_eval_f(Dims D, ModelView M, const double
 template <int NT>
 __global__ void __launch_bounds__(NT) k_eval_cons(Dims D, ModelView M, const double *__restrict__ x,
                                                   const double *__restrict__ Axd, const double *__restrict__ d,
-                                                  double *__restrict__ cg, double *__restrict__ ch,
+                                                  double *__restrict__ cg, double *__restrict__ ch, double alpha,
+                                                  const double *__restrict__ dAx, double *__restrict__ Ax_out,
                                                   RedOut red) {
     const int lane = threadIdx.x & 31;
     const int64_t gw = ((int64_t)blockIdx.x * NT + threadIdx.x) >> 5;
@@ -63,6 +64,10 @@ __global__ void __launch_bounds__(NT) k_eval_cons(Dims D, ModelView M, const dou
     // equalities: the dense part A x_d comes from the row-block pass (Axd)
     for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < D.m_E; i += (int64_t)gridDim.x * NT) {
         double s = Axd[i];
+        if (dAx) {   // a step of alpha from where Axd was formed
+            s = fma(alpha, dAx[i], s);
+            Ax_out[i] = s;
+        }
         for (int e = M.csr_ptr[i]; e < M.csr_ptr[i + 1]; ++e) s += M.csr_val[e] * x[M.csr_col[e]];
         const double r = s - M.gE[i];
         cg[i] = r;
@@ -679,11 +684,14 @@ __global__ void __launch_bounds__(NT) k_trial(Dims D, ModelView M, IterView I, D
 // Accept: y += alpha dy, z += alpha_z dz, then the kappa_Sigma safeguard
 // (W&B eq. (16)) against the new slacks (x, d already hold the new point).
 __global__ void k_accept(Dims D, ModelView M, IterView I, DirView Dir, double alpha,
-                         double alpha_z, double mu, double ks) {
+                         double alpha_z, double mu, double ks, double *__restrict__ ATy,
+                         const double *__restrict__ dATy) {
     const int64_t gtid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t gsz = (int64_t)gridDim.x * blockDim.x;
     auto guard = [&](double z, double s) { return fmax(fmin(z, ddiv(ks * mu, s)), ddiv(mu, ks * s)); };
     for (int64_t i = gtid; i < D.m_E; i += gsz) I.yg[i] += alpha * Dir.dyg[i];
+    if (dATy)   // A^T y_g follows y_g
+        for (int64_t k = gtid; k < D.n_d; k += gsz) ATy[k] = fma(alpha, dATy[k], ATy[k]);
     for (int64_t j = gtid; j < D.m_I; j += gsz) {
         I.yh[j] += alpha * Dir.dyh[j];
         const double dj = I.d[j];
@@ -872,26 +880,12 @@ void VecOps::eval_cons(const double *x, const double *d, double *cg, double *ch,
         if (Ahi) launch_gemv_rows_df(st, Ahi, Alo, D.m_E, D.n_d, D.lda, x + D.n_s, split, rowtmp);
         else launch_gemv_rows(st, M.A, D.m_E, D.n_d, D.lda, x + D.n_s, rowtmp);
     }
-    MDSIP_RED(k_eval_cons, std::max(D.m_E, 32 * D.m_I), D, M, x, rowtmp, d, cg, ch, red(out2));
+    MDSIP_RED(k_eval_cons, std::max(D.m_E, 32 * D.m_I), D, M, x, rowtmp, d, cg, ch, 0.0, nullptr, nullptr, red(out2));
 }
 
 void VecOps::eval_cons_ax(const double *x, const double *Ax, const double *d, double *cg, double *ch,
-                          double *out2) {
-    MDSIP_RED(k_eval_cons, std::max(D.m_E, 32 * D.m_I), D, M, x, Ax, d, cg, ch, red(out2));
-}
-
-namespace {
-__global__ void k_axpby(int64_t n, const double *__restrict__ a, double alpha, const double *__restrict__ b,
-                        double *__restrict__ y) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        y[i] = a[i] + alpha * b[i];
-}
-}  // namespace
-
-void VecOps::axpby(int64_t n, const double *a, double alpha, const double *b, double *y) {
-    if (n <= 0) return;
-    k_axpby<<<elem_grid(n), 256, 0, st>>>(n, a, alpha, b, y);
-    MDSIP_LAUNCHED();
+                          double *out2, double alpha, const double *dAx, double *Ax_out) {
+    MDSIP_RED(k_eval_cons, std::max(D.m_E, 32 * D.m_I), D, M, x, Ax, d, cg, ch, alpha, dAx, Ax_out, red(out2));
 }
 
 void VecOps::jac_hess(const double *x, const double *yh, double *Jdh, double *Hss, double *Hdd) {
@@ -972,8 +966,8 @@ void VecOps::trial(const IterView &I, const DirView &Dir, double alpha, double *
 }
 
 void VecOps::accept(const IterView &I, const DirView &Dir, double alpha, double alpha_z, double mu,
-                    double ks) {
-    k_accept<<<elem_grid(std::max(D.n, D.m_E), elem_threads(std::max(D.n, D.m_E))), elem_threads(std::max(D.n, D.m_E)), 0, st>>>(D, M, I, Dir, alpha, alpha_z, mu, ks);
+                    double ks, double *ATy, const double *dATy) {
+    k_accept<<<elem_grid(std::max(D.n, D.m_E), elem_threads(std::max(D.n, D.m_E))), elem_threads(std::max(D.n, D.m_E)), 0, st>>>(D, M, I, Dir, alpha, alpha_z, mu, ks, ATy, dATy);
     MDSIP_LAUNCHED();
 }
 

@@ -33,11 +33,11 @@ struct VecOps {
     void eval_f(const double *x, double *grad, double *out_scalar);
     void eval_cons(const double *x, const double *d, double *cg, double *ch, double *out2);
     // the same with A x_d given (Ax, m_E doubles) instead of formed from x
-    void eval_cons_ax(const double *x, const double *Ax, const double *d, double *cg, double *ch, double *out2);
+    // (Ax + alpha dAx with dAx non-null: then also stored in Ax_out)
+    void eval_cons_ax(const double *x, const double *Ax, const double *d, double *cg, double *ch, double *out2,
+                      double alpha = 0.0, const double *dAx = nullptr, double *Ax_out = nullptr);
     // rowtmp = A x_d and ATy = A^T y_g in one pass over the FP32 pair of A
     void both_products(const IterView &I, double *ATy, int *err);
-    // y = a + alpha b (n doubles)
-    void axpby(int64_t n, const double *a, double alpha, const double *b, double *y);
     void jac_hess(const double *x, const double *yh, double *Jdh, double *Hss, double *Hdd);
     void lagrangian_grad(const IterView &I, const double *grad, const double *Jdh, double *ATy,
                          double *gl);
@@ -62,8 +62,9 @@ struct VecOps {
                       double mu, double *out3);
     void trial(const IterView &I, const DirView &Dir, double alpha, double *xt, double *dt,
                double *out2);
+    // dATy non-null: ATy += alpha dATy as well
     void accept(const IterView &I, const DirView &Dir, double alpha, double alpha_z, double mu,
-                double ks);
+                double ks, double *ATy = nullptr, const double *dATy = nullptr);
     void init_x(const double *x0, double k1, double k2, const IterView &I);
     void init_d(const double *ch, double k1, double k2, const IterView &I);
     // Warm start from a predicted packed point `pred` (FP32): x and d pushed
