@@ -49,11 +49,9 @@ UNIT = "Newton steps/s"
 # microbenchmark reached 1.20 TFLOP/s at ~1.97 GHz on this machine.
 FP64_PEAK_TFLOPS = 152 * 4 * 2.07e9 / 1e12
 FP32_PEAK_TFLOPS = 152 * 256 * 2.07e9 / 1e12   # 128 FP32 lanes per SM, 2 flop per FMA
-# DRAM bytes per launch of the FP64 condensation kernel at n_d = 2000,
-# m_E = 100000, scaled from an ncu capture of the current kernel at m = 20000
-# (profiles/syrk_fp64_m20000_n2000.md): reads of A grow with m, the split
-# partial writes do not.
-SYRK_TRAFFIC_BYTES = 5 * 326.793216e6 + 183.695104e6
+# The FP64 product and the FP64 factorization's trailing updates run on the
+# BF16 tensor cores as exact contractions modulo this many coprime integers.
+SYRK_MODULI, LDLT_MODULI = 14, 13
 
 
 def measured_peak(key):
@@ -567,24 +565,25 @@ def run_warmstart(args, m, torch, local):
 def cond_ldlt_roofline(inst, syrk_ms, ldlt_ms, precision):
     """Roofline fraction of condensation + LDL^T together: (F_syrk / P_syrk +
     F_ldlt / P_ldlt) / (measured product + factorization time), F_syrk =
-    n_d (n_d + 1) m_E flop, F_ldlt = N^3 / 3 flop (N = n_d + m_I); P_syrk the FP64
-    ALU peak, the measured BF16 peak, or TF32 at half of it; P_ldlt the peak of
-    the arithmetic the factorization's updates use: FP64 on the FP64 path, FP32
-    (derived: 152 SMs x 128 lanes x 2 flop x 2.07 GHz) on the mixed-precision
-    path.  `ldlt_time_vs_fp64_peak` compares the factorization with the time
-    its flops take at the FP64 peak."""
+    n_d (n_d + 1) m_E flop, F_ldlt = N^3 / 3 flop (N = n_d + m_I); P_syrk the
+    measured BF16 peak, over the number of moduli on the FP64 path, or TF32 at
+    half of it; P_ldlt the peak of the arithmetic the factorization's updates
+    use: BF16 over the number of moduli on the FP64 path, FP32 (derived: 152
+    SMs x 128 lanes x 2 flop x 2.07 GHz) on the mixed-precision path.
+    `ldlt_time_vs_fp64_peak` compares the factorization with the time its
+    flops take at the FP64 ALU peak."""
     N = inst.n_d + inst.m_I
     f_syrk = inst.n_d * (inst.n_d + 1) * inst.m_E * 1.0
     f_ldlt = N ** 3 / 3.0
     p64 = FP64_PEAK_TFLOPS * 1e12
     bf16 = (measured_peak("bf16_tflops") or 1900.0) * 1e12
-    p_syrk = {"fp64": p64, "bf16": bf16, "tf32": bf16 / 2.0}[precision]
-    p_ldlt = p64 if precision == "fp64" else FP32_PEAK_TFLOPS * 1e12
+    p_syrk = {"fp64": bf16 / SYRK_MODULI, "bf16": bf16, "tf32": bf16 / 2.0}[precision]
+    p_ldlt = bf16 / LDLT_MODULI if precision == "fp64" else FP32_PEAK_TFLOPS * 1e12
     t_roof = f_syrk / p_syrk + f_ldlt / p_ldlt
     t_meas = (syrk_ms + ldlt_ms) / 1e3
     return {"t_roof_ms": 1e3 * t_roof, "t_measured_ms": 1e3 * t_meas, "frac": t_roof / t_meas if t_meas else None,
             "peaks": f"product at {p_syrk / 1e12:.1f} TFLOP/s ({precision}), LDL^T at {p_ldlt / 1e12:.1f} TFLOP/s "
-                     f"({'FP64' if precision == 'fp64' else 'FP32, derived'})",
+                     f"({f'BF16 over {LDLT_MODULI} moduli' if precision == 'fp64' else 'FP32, derived'})",
             "ldlt_time_vs_fp64_peak": (f_ldlt / p64) / (ldlt_ms / 1e3) if ldlt_ms else None}
 
 
@@ -880,14 +879,21 @@ def run_gpu(args):
     wstart = run_warmstart(args, m, torch, local) if (args.ws_train > 0 and world == 1) else None
     flops = D["n_d"] * (D["n_d"] + 1) / 2 * D["m_E"] * 2.0
     syrk_ms = acc["t_syrk_ms"] / max(1, acc["n_syrk"])
-    achieved = flops / (syrk_ms / 1e3) / 1e12 if acc["n_syrk"] else None
-    roofline = {"kernel": "k_syrk_fp64 (A^T W^-1 A, FP64 DFMA)", "bound": "alu",
-                "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                "frac": achieved / FP64_PEAK_TFLOPS if achieved else None,
-                "traffic": SYRK_TRAFFIC_BYTES if (D["n_d"], D["m_E"]) == (2000, 100000) else None,
-                "peak_source": "derived: 152 SMs x 4 FP64 flop/clk x 2.07 GHz (FP64 is not in MEASURED_PEAKS.json)",
+    fp64_rate = flops / (syrk_ms / 1e3) / 1e12 if acc["n_syrk"] else None
+    bf16_peak = measured_peak("bf16_tflops")
+    rns = D["m_E"] >= 256 and D["m_E"] * D["n_d"] ** 2 >= 3e7   # large enough for the tensor-core form
+    achieved = SYRK_MODULI * fp64_rate if (fp64_rate and rns) else fp64_rate
+    prod_peak = bf16_peak if rns else FP64_PEAK_TFLOPS
+    roofline = {"kernel": ("k_rns_rows/colmax/residues/mma/combine (A^T W^-1 A in FP64 by exact BF16 tensor products "
+                           f"modulo {SYRK_MODULI} integers)") if rns else "k_syrk_fp64 (A^T W^-1 A, FP64 DFMA)",
+                "bound": "tensor" if rns else "alu",
+                "achieved": achieved, "peak": prod_peak, "unit": "TFLOP/s",
+                "frac": achieved / prod_peak if achieved and prod_peak else None,
+                "traffic": None,
+                "peak_source": ("measured BF16 (MEASURED_PEAKS.json); achieved counts every modulus" if rns else
+                                "derived: 152 SMs x 4 FP64 flop/clk x 2.07 GHz (FP64 is not in MEASURED_PEAKS.json)"),
+                "fp64_tflops": fp64_rate, "fp64_alu_peak_tflops": FP64_PEAK_TFLOPS,
                 "peak_probe": probe,
-                "frac_of_probe": achieved / probe["tflops"] if (achieved and probe) else None,
                 "flops_per_launch": flops, "avg_launch_ms": syrk_ms, "launches": int(acc["n_syrk"]),
                 "share_of_step": acc["t_syrk_ms"] / (1e3 * elapsed) if elapsed else None}
     line = {

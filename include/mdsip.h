@@ -51,10 +51,10 @@ enum { MDSIP_MEM_HOST = 0, MDSIP_MEM_DEVICE = 1 };
  *   AUTO: P2 when applicable, else P1. */
 enum { MDSIP_PATH_AUTO = 0, MDSIP_PATH_P1 = 1, MDSIP_PATH_P2 = 2 };
 
-/* Arithmetic of the condensation product (option "precision"): FP64 on the
- * DFMA pipe, or tensor cores (tcgen05) with TF32 / BF16 operands and FP32
- * accumulation, the Newton direction then refined in FP64 on the unreduced
- * system. */
+/* Arithmetic of the condensation product (option "precision"): FP64 (as at
+ * mdsip_syrk_scaled), or tensor cores (tcgen05) with TF32 / BF16 operands and
+ * FP32 accumulation, the Newton direction then refined in FP64 on the
+ * unreduced system. */
 enum { MDSIP_PREC_FP64 = 0, MDSIP_PREC_TF32 = 1, MDSIP_PREC_BF16 = 2 };
 
 typedef struct mdsip_ctx mdsip_ctx;
@@ -322,7 +322,10 @@ mdsip_status mdsip_probe_fp64_fma(mdsip_ctx *ctx, int32_t blocks, int64_t iters,
  *   C[p][q] = beta * C[p][q] + sum_i A[i][p] * A[i][q] / w[i]   for p >= q,
  * A: m x n row-major with leading dimension lda (lda >= n, lda % 2 == 0),
  * w: m (nonzero), C: n x n column-major, leading dimension ldc; only the lower
- * triangle (p >= q) is written.  beta is 0 or 1.  FP64 throughout. */
+ * triangle (p >= q) is written.  beta is 0 or 1.  An FP64 product: small ones
+ * on the FP64 pipe, larger ones as exact integer products on the tensor cores
+ * (operands scaled and rounded once to 53 bits or more per column, the sum
+ * rounded once to FP64), with errors no larger. */
 mdsip_status mdsip_syrk_scaled(mdsip_ctx *ctx, int64_t m, int64_t n, const double *A, int64_t lda,
                                const double *w, double beta, double *C, int64_t ldc);
 
