@@ -1906,8 +1906,8 @@ void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, cons
         reinterpret_cast<unsigned *>(w + lay.colcnt));
     MDSIP_LAUNCHED();
     int k0 = 0;   // first column left to the panel loop below
+    PersistArgs pa{};
     if (persist) {
-        PersistArgs pa{};
         pa.N = (int)N;
         pa.A = S;
         pa.L = out.L;
@@ -1931,35 +1931,56 @@ void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, cons
         k0 = persist_stopped_at(s, st, bar);
         MDSIP_REQUIRE(k0 >= N || cfg.C > 0, MDSIP_ERR_INVALID_ARG,
                       "ldlt: a panel needs interchanges and N is too large for the pivoting panel");
-        // the panel loop's no-interchange kernels expect their column maxima and
-        // arg-max keys at zero; the rejected panel left its maxima there
-        if (k0 < N) MDSIP_CUDA(cudaMemsetAsync(w + lay.cmax, 0, 192 * sizeof(unsigned long long), s));
     }
 
+    auto panel_args = [&](const BlockedConfig &c) {
+        PanelArgs a{};
+        a.N = (int)N;
+        a.NB = c.NB;
+        a.C = c.C;
+        a.R = c.R;
+        a.A = S;
+        a.L = out.L;
+        a.Dd = out.Dd;
+        a.Doff = out.Doff;
+        a.perm = out.perm;
+        a.kind = out.kind;
+        a.Wg = Wg;
+        a.Lf = reinterpret_cast<float *>(w + lay.lf);
+        a.Wf = reinterpret_cast<float *>(w + lay.wf);
+        a.st = st;
+        a.maxabs = maxabs_dev;
+        a.zero_tol = zero_tol;
+        return a;
+    };
     // FP64 panels without a width asked for: 31 columns (32 with a 2x2 pivot at
     // the end), whose trailing updates go through the tensor cores
-    const bool rns = !fp32_update && nb == 0 && N - k0 > kRnsPanelMin && cfg.NB >= 32;
-    if (rns) {
-        cfg = blocked_config(N, false, 32);
-        cfg.NB = 31;
+    int npanel = 0;   // such panels so far
+    BlockedConfig cfg31 = blocked_config(N, false, 32);
+    cfg31.NB = 31;
+    const bool may31 = !fp32_update && nb == 0 && cfg31.C > 0 && cfg.NB >= 32;
+    // A matrix that needs an interchange here and there: one pivoting panel, then
+    // the persistent kernel again, as long as it keeps two panels or more each time
+    // (a run that keeps none costs some 60 us).  N = 1036 without an interchange 0.97
+    // ms, with one half way 1.09, with three 1.32; on pivoting panels to the end the
+    // first of them cost a one-stage direction 1.1 ms.
+    for (int kept = k0; persist && may31 && k0 < N && kept >= 64 && N - k0 > kRnsPanelMin; ++npanel) {
+        MDSIP_CUDA(cudaMemsetAsync(w + lay.cmax, 0, 192 * sizeof(unsigned long long), s));
+        launch_pdl(k_bk_panel<false>, (unsigned)cfg31.C, kPanelThreads, cfg31.smem, s, cfg31.C, panel_args(cfg31));
+        launch_rns_trailing(s, num_sms, N, N - k0 - 31, npanel, S, out.L, out.Dd, out.Doff, Wg, maxabs_dev, st,
+                            err_dev ? err_dev : &bar->err, w + lay.p64);
+        MDSIP_CUDA(cudaMemsetAsync(&bar->count, 0, sizeof(unsigned), s));
+        launch_persist64(s, num_sms, N, pa, w + lay.p64);
+        const int k1 = persist_stopped_at(s, st, bar);
+        kept = k1 - (k0 + 32);
+        k0 = k1;
     }
-    PanelArgs a{};
-    a.N = (int)N;
-    a.NB = cfg.NB;
-    a.C = cfg.C;
-    a.R = cfg.R;
-    a.A = S;
-    a.L = out.L;
-    a.Dd = out.Dd;
-    a.Doff = out.Doff;
-    a.perm = out.perm;
-    a.kind = out.kind;
-    a.Wg = Wg;
-    a.Lf = reinterpret_cast<float *>(w + lay.lf);
-    a.Wf = reinterpret_cast<float *>(w + lay.wf);
-    a.st = st;
-    a.maxabs = maxabs_dev;
-    a.zero_tol = zero_tol;
+    // the panel loop's no-interchange kernels expect their column maxima and
+    // arg-max keys at zero; the rejected panel left its maxima there
+    if (persist && k0 < N) MDSIP_CUDA(cudaMemsetAsync(w + lay.cmax, 0, 192 * sizeof(unsigned long long), s));
+    const bool rns = may31 && N - k0 > kRnsPanelMin;
+    if (rns) cfg = cfg31;
+    const PanelArgs a = panel_args(cfg);
 
     const size_t usm = 2 * (size_t)(cfg.NB + 1) * kUT * (fp32_update ? sizeof(float) : sizeof(double));
     static PerDeviceOnce once;
@@ -2018,7 +2039,7 @@ void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, cons
         const double *cL = out.L, *cWg = Wg;
         const PanelState *cst = st;
         if (rns && rest > kRnsTrailingMin)
-            launch_rns_trailing(s, num_sms, N, rest, p, S, out.L, out.Dd, out.Doff, Wg, maxabs_dev, st,
+            launch_rns_trailing(s, num_sms, N, rest, npanel + p, S, out.L, out.Dd, out.Doff, Wg, maxabs_dev, st,
                                 err_dev ? err_dev : &bar->err, w + lay.p64);
         else if (fp32_update)
             launch_pdl(k_bk_trailing<float>, tiles, kUpdThreads, usm, s, 1, (int)N, cfg.NB, S, cL, cWg, cLf, cWf, cst);

@@ -229,13 +229,14 @@ __device__ __forceinline__ int64_t q_at(int64_t row, int lane) {
 
 // The trailing update A(i, c) -= sum_t X(i, t) Y(c, t), first <= c <= i < N, from
 // residues of X in RA and of Y in RB, by this CTA g of G: tiles of 128 rows from
-// `base` (a multiple of 8, at most 7 below `first`) and tw columns of the lower
+// `base` (at most 7 below `first`) and tw columns of the lower
 // triangle.  tl counts the tiles this warp's role has gone through.
 struct QUpdate {
     double *A;
     const bf16 *RA, *RB;
     const int *EA, *EB;   // row exponents
     int N, npad, base, first;
+    int off;              // row i's residues are at i - off: a multiple of 8 for base
 };
 
 __device__ bool q_update(const QUpdate &u, int G, int g, uint8_t *ring, uint32_t tmem, uint64_t *full, uint64_t *tfull,
@@ -267,8 +268,8 @@ __device__ bool q_update(const QUpdate &u, int G, int g, uint8_t *ring, uint32_t
                     if (lane < RL) {
                         uint8_t *d = ring + lane * Q_STAGE;
                         tc::mbar_expect_tx(&full[lane], QA_BYTES + tw * 64);
-                        tc::bulk_load(d, u.RA + ((int64_t)lane * u.npad + i0) * QN, QA_BYTES, &full[lane]);
-                        tc::bulk_load(d + QA_BYTES, u.RB + ((int64_t)lane * u.npad + c0) * QN, tw * 64, &full[lane]);
+                        tc::bulk_load(d, u.RA + ((int64_t)lane * u.npad + i0 - u.off) * QN, QA_BYTES, &full[lane]);
+                        tc::bulk_load(d + QA_BYTES, u.RB + ((int64_t)lane * u.npad + c0 - u.off) * QN, tw * 64, &full[lane]);
                     }
                     __syncwarp();
                 }
@@ -421,7 +422,8 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
     unsigned epoch = 0;   // grid barriers passed (thread 0)
     uint32_t sub = 0;     // sub-panels gone through
     int p = 0;
-    for (int k = a.st->k; k < N; k += QN, ++p) {
+    const int kfirst = a.st->k;   // any column: a pivoting panel may have come before
+    for (int k = kfirst; k < N; k += QN, ++p) {
         const int nb = min(QN, N - k);
         const int buf = p & 1;
         // own rows: multiples of 8 per CTA
@@ -528,7 +530,7 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
                     const uint32_t sa = w < 0.0 ? 0x8000u : 0u, sb = sa ^ (s_d[lane] < 0.0 ? 0x8000u : 0u);
                     const int64_t row = cb + r;
                     if (lane == 0) q.rowE[row] = E;
-                    const int64_t at = q_at(row, lane);
+                    const int64_t at = q_at(row - (kfirst & 31), lane);
                     uint16_t *ra = reinterpret_cast<uint16_t *>(q.RA) + at;
                     uint16_t *rb = reinterpret_cast<uint16_t *>(q.RB) + at;
                     const int64_t ls = (int64_t)q.npad * QN;
@@ -581,14 +583,14 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
                     a.st->k = k + nb;
                     a.st->kb = nb;
                     // counted in panels of 64 columns, as the panel loop's
-                    if (k + nb >= N || (k + nb) % 64 == 0) a.st->nacc += 1;
+                    if (k + nb >= N || (k + nb - kfirst) % 64 == 0) a.st->nacc += 1;
                 }
             }
         }
         if (k + nb >= N) break;
         // ---------------- trailing update
         const int base = k + nb;
-        const QUpdate up{a.A, q.RA, q.RB, q.rowE, q.rowE, N, q.npad, base, base};
+        const QUpdate up{a.A, q.RA, q.RB, q.rowE, q.rowE, N, q.npad, base, base, kfirst & 31};
         const bool ok = q_update(up, G, g, ring, tmem, full, &tfull, &tempty, s_km, tl);
         if (!ok) atomicExch(&a.bar->err, 1);
         __threadfence();
@@ -690,7 +692,7 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_rns_trailing(RnsTrailing a)
     __syncthreads();
     tc::fence_after();
     int tl = 0;
-    const QUpdate up{a.A, a.RA, a.RB, a.EA, a.EB, N, a.npad, first & ~7, first};
+    const QUpdate up{a.A, a.RA, a.RB, a.EA, a.EB, N, a.npad, first & ~7, first, 0};
     if (!q_update(up, (int)gridDim.x, (int)blockIdx.x, ring, s_tmem, full, &tfull, &tempty, s_km, tl)) atomicExch(a.err, 1);
     if (wid == Q_EPI && tl > 0 && lane < RL) tc::mbar_wait(&full[lane], (tl - 1) & 1);   // no copy in flight on the way out
     tc::fence_before();

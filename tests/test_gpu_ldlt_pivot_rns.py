@@ -61,3 +61,33 @@ def test_reconstruction(ctx, N, kind, scale):
     b = ((np.abs(Lh) * h) ** 2).sum(axis=1) + ((np.abs(W) / h) ** 2).sum(axis=1)
     tol = 2 * N * np.longdouble(2.0) ** -52 * np.sqrt(np.outer(b, b))
     assert (R <= tol).all(), float((R / tol).max())
+
+
+@pytest.mark.parametrize("N,spots", [(300, (70,)), (705, (333,)), (1036, (500,)), (1036, (100, 431, 800)), (417, (64, 380))])
+def test_persistent_form_resumes_after_an_interchange(ctx, N, spots):
+    """A convex matrix with a few zero diagonals that only an interchange (a 2x2
+    pivot) gets past: the persistent kernel goes on behind each pivoting panel,
+    from whatever column that ends at."""
+    torch = torch_cuda()
+    rng = np.random.default_rng(N + len(spots))
+    g = rng.standard_normal((N, N)) / np.sqrt(N)
+    K = 0.1 * (g + g.T) / np.sqrt(N) + np.diag(rng.uniform(1.0, 2.0, N))
+    for j in spots:                            # [[0, 3], [3, 0]] coupled weakly to the rest
+        K[j, j] = K[j + 5, j + 5] = 0.0
+        K[j, j + 5] = K[j + 5, j] = 3.0
+    S = dev(np.tril(K).T.copy())
+    L = torch.zeros((N, N), dtype=torch.float64, device="cuda")
+    Dd, Doff = (torch.zeros(N, dtype=torch.float64, device="cuda") for _ in range(2))
+    perm, kd = (torch.zeros(N, dtype=torch.int32, device="cuda") for _ in range(2))
+    inr = torch.zeros(3, dtype=torch.int32, device="cuda")
+    m.mdsip_ldlt_factor(ctx, N, S, N, 1e-14, L, Dd, Doff, perm, kd, inr)
+    torch.cuda.synchronize()
+    assert tuple(inr.cpu().numpy()) == (N - len(spots), len(spots), 0)
+    assert int((kd == 2).sum()) == len(spots)
+    # all but two panels of 64 columns per interchange stay with the persistent kernel
+    assert m.mdsip_ldlt_panel_counts(ctx)[0] >= N // 64 - 2 * len(spots) - 1
+    Lh = np.tril(L.cpu().numpy().T)
+    d, o = Dd.cpu().numpy(), Doff.cpu().numpy()
+    p = perm.cpu().numpy()
+    R = K[np.ix_(p, p)] - Lh @ (np.diag(d) + np.diag(o[:-1], -1) + np.diag(o[:-1], 1)) @ Lh.T
+    assert np.abs(R).max() <= 1e-13 * N        # N 2^-53 times entries of at most 3 and a few roundings each
