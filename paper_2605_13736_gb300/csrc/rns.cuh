@@ -13,7 +13,6 @@ namespace rns {
 
 constexpr int kModuli[14] = {512, 511, 509, 507, 505, 503, 499, 493, 491, 487, 479, 473, 467, 463};
 constexpr int LIMB = 14;               // bits per limb of |X| when residues are formed
-constexpr int CL = 5;                  // 30-bit limbs of the CRT constants
 constexpr float kMagic = 12582912.0f;  // 1.5 2^23: adding and subtracting it rounds to an integer
 
 template <int RN>
@@ -21,8 +20,6 @@ struct Tab {
     float p[RN], pinv[RN];
     float c1[RN], c2[RN], c3[RN];      // 2^14, 2^28, 2^42 mod p, symmetric
     float inv[RN];                     // (M / p)^-1 mod p, symmetric
-    int mhat[RN][CL];                  // M / p in 30-bit limbs
-    int mod[CL];                       // M in 30-bit limbs
     // moduli taken in pairs (a last one alone): sum_l y_l M/p_l is the sum over
     // pairs of z M/(p q), z = y_p q + y_q p, |z| < 2^19
     uint32_t mpair32[(RN + 1) / 2][4], mod32[4], bias32[4];   // M/(p q), M, 2^19 sum of M/(p q), 32-bit limbs
@@ -40,7 +37,6 @@ constexpr Tab<RN> make_tab() {
     Tab<RN> t{};
     unsigned __int128 M = 1, bias = 0;
     for (int l = 0; l < RN; ++l) M *= (unsigned)kModuli[l];
-    for (int j = 0; j < CL; ++j) t.mod[j] = (int)((M >> (30 * j)) & 0x3fffffffu);
     for (int l = 0; l < RN; ++l) {
         const int p = kModuli[l];
         t.p[l] = (float)p;
@@ -49,7 +45,6 @@ constexpr Tab<RN> make_tab() {
         t.c2[l] = (float)sym((int)((1LL << (2 * LIMB)) % p), p);
         t.c3[l] = (float)sym((int)((1LL << (3 * LIMB)) % p), p);
         const unsigned __int128 h = M / (unsigned)p;
-        for (int j = 0; j < CL; ++j) t.mhat[l][j] = (int)((h >> (30 * j)) & 0x3fffffffu);
         const int hm = (int)(h % (unsigned)p);
         for (int v = 1; v < p; ++v)
             if ((v * hm) % p == 1) t.inv[l] = (float)sym(v, p);

@@ -374,7 +374,10 @@ __global__ void __launch_bounds__(MMA_THREADS, 1) k_rns_mma(const __grid_constan
 // residues of the splits added, y_l = r_l (M/p_l)^-1 mod p_l, the sum
 // X = sum_l y_l M/p_l - k M with k = rint(sum_l y_l / p_l) (|X| < M / 4, so FP32
 // finds k), rounded once to FP64.  A raised err word (a wait that expired in
-// k_rns_mma) poisons the result with NaN.
+// k_rns_mma) poisons the result with NaN.  Bound by the latency of its loads: a
+// thread loads its next column's 14 residues under the arithmetic of this one,
+// whose 14 terms of five 30-bit limbs are seven pairs of four 32-bit ones (n =
+// 2000, 72 tiles: 98 us with a column a thread and three splits, 46 so).
 __global__ void __launch_bounds__(256) k_rns_combine(int64_t n, int tile0, int ntile, int nsplit, int b,
                                                      const int16_t *__restrict__ W, const int *__restrict__ colE,
                                                      double beta, double *__restrict__ C, int64_t ldc,
@@ -386,39 +389,60 @@ __global__ void __launch_bounds__(256) k_rns_combine(int64_t n, int tile0, int n
     const int row = threadIdx.x & 127;
     const int64_t p = (int64_t)P * T_M + row;
     const size_t per_item = (size_t)T_M * T_N;
-    for (int c = blockIdx.y * 2 + (threadIdx.x >> 7); c < T_N; c += gridDim.y * 2) {
+    const size_t ls = (size_t)ntile * per_item;   // one split; nsplit of them per modulus
+    const int16_t *wp = W + (size_t)blockIdx.x * per_item + row;
+    const int step = gridDim.y * 2;
+    const int c0 = blockIdx.y * 2 + (threadIdx.x >> 7);
+    // columns this row has: c < T_N, q <= p < n
+    const int cend = p < n ? (int)min((int64_t)T_N, p - (int64_t)Q * T_N + 1) : 0;
+    int nx[RN];   // the next column's residues of the first split, loaded under this one's arithmetic
+    auto fetch = [&](int c) {
+        if (c < cend)
+#pragma unroll
+            for (int l = 0; l < RN; ++l) nx[l] = __ldg(wp + (size_t)(l * nsplit) * ls + (size_t)c * T_M);
+    };
+    fetch(c0);
+    for (int c = c0; c < cend; c += step) {
         const int64_t q = (int64_t)Q * T_N + c;
-        if (p >= n || q > p) continue;
-        long long acc[CL] = {0, 0, 0, 0, 0};
-        float frac = 0.0f;
-        const int16_t *wp = W + (size_t)blockIdx.x * per_item + (size_t)c * T_M + row;
-        const size_t ls = (size_t)ntile * per_item;   // one split; nsplit of them per modulus
         int r[RN];
 #pragma unroll
-        for (int l = 0; l < RN; ++l) r[l] = wp[(size_t)(l * nsplit) * ls];
+        for (int l = 0; l < RN; ++l) r[l] = nx[l];
+        double *out = C + p + q * ldc;
+        const double old = beta != 0.0 ? *out : 0.0;
+        const int e = __ldg(colE + p) + __ldg(colE + q) - 2 * b;
+        fetch(c + step);
         for (int s = 1; s < nsplit; ++s) {   // the 14 loads of a split in flight together
 #pragma unroll
-            for (int l = 0; l < RN; ++l) r[l] += wp[(size_t)(l * nsplit + s) * ls];
+            for (int l = 0; l < RN; ++l) r[l] += wp[(size_t)(l * nsplit + s) * ls + (size_t)c * T_M];
         }
+        // pairs of moduli: z = y_p q + y_q p (exact, |z| < 2^19), X = sum z M/(p q) - k M
+        // modulo 2^128 in 32-bit limbs, z + 2^19 against the bias
+        unsigned long long acc[4] = {0, 0, 0, 0};
+        float frac = 0.0f;
 #pragma unroll
-        for (int l = 0; l < RN; ++l) {
-            const float y = mod((float)r[l] * c_tab.inv[l], c_tab.p[l], c_tab.pinv[l]);   // the product < 2^24
-            frac = fmaf(y, c_tab.pinv[l], frac);
-            const int yi = (int)y;
+        for (int l = 0; l < RN; l += 2) {
+            const float y0 = mod((float)r[l] * c_tab.inv[l], c_tab.p[l], c_tab.pinv[l]);   // the product < 2^24
+            const float y1 = mod((float)r[l + 1] * c_tab.inv[l + 1], c_tab.p[l + 1], c_tab.pinv[l + 1]);
+            frac = fmaf(y0, c_tab.pinv[l], fmaf(y1, c_tab.pinv[l + 1], frac));
+            const unsigned z = (unsigned)((int)fmaf(y0, c_tab.p[l + 1], y1 * c_tab.p[l]) + (1 << 19));
 #pragma unroll
-            for (int j = 0; j < CL; ++j) acc[j] += (long long)yi * c_tab.mhat[l][j];
+            for (int j = 0; j < 4; ++j) acc[j] += (unsigned long long)z * c_tab.mpair32[l / 2][j];
         }
         const int kq = (int)rintf(frac);
-        unsigned __int128 u = 0;   // X modulo 2^128
+        unsigned __int128 M = 0, B = 0, u = 0;   // X modulo 2^128
 #pragma unroll
-        for (int j = CL - 1; j >= 0; --j)
-            u = (u << 30) + (unsigned __int128)(__int128)(acc[j] - (long long)kq * c_tab.mod[j]);
-        double val = to_double(u, colE[p] + colE[q] - 2 * b);
-        double *out = C + p + q * ldc;
-        if (poison) val = NAN;
-        *out = (beta != 0.0 ? *out : 0.0) + val;
+        for (int j = 3; j >= 0; --j) {
+            M = (M << 32) | c_tab.mod32[j];
+            B = (B << 32) | c_tab.bias32[j];
+            u = (u << 32) + acc[j];
+        }
+        u -= B + M * (unsigned __int128)(__int128)kq;
+        const double val = poison ? (double)NAN : to_double(u, e);
+        *out = old + val;
     }
 }
+
+static_assert(RN % 2 == 0, "moduli are taken in pairs");
 
 struct RnsPlan {
     int64_t ldn, kc, chunks;
@@ -445,17 +469,19 @@ RnsPlan rns_plan(int64_t m, int64_t n, int num_sms) {
     // K splits so that the items fill whole waves of one CTA per SM, each at
     // least 512 rows: two 256-row folds
     const int nslab = (int)(pl.kc / SLAB);
-    double best = 0.0;
+    // (products at their rate over the fill of the last wave, plus the sums'
+    // residues written and read once per split)
+    double best = 1e30;
     pl.nsplit = 1;
+    const double t0 = 2.0 * pl.tiles * RN * T_M * T_N * (double)pl.kc / 1.35e15;
     for (int s = 1; s <= 16; ++s) {
         if (s > 1 && nslab / s < 2 * FOLD) break;
         const double waves = (double)pl.tiles * RN * s / num_sms;
-        const double eff = waves / std::ceil(waves);
-        if (eff > best + 0.02) {
-            best = eff;
+        const double t = t0 * std::ceil(waves) / waves + 2.0 * s * pl.tiles * RN * T_M * T_N * sizeof(int16_t) / 5e12;
+        if (t < 0.99 * best) {
+            best = t;
             pl.nsplit = s;
         }
-        if (eff >= 0.95) break;
     }
     pl.slabs_per_split = ((nslab + pl.nsplit - 1) / pl.nsplit + FOLD - 1) / FOLD * FOLD;
     pl.nsplit = (nslab + pl.slabs_per_split - 1) / pl.slabs_per_split;
@@ -542,7 +568,9 @@ const int *launch_syrk_rns(cudaStream_t st, int num_sms, const double *A, int64_
             MmaArgs a{t0, nt, nsplit, nslab, pl.slabs_per_split, kpad, W, flag, err};
             k_rns_mma<<<std::min(num_sms, RN * nsplit * nt), MMA_THREADS, kMmaSmem, st>>>(rmap, a);
             MDSIP_LAUNCHED();
-            k_rns_combine<<<dim3((unsigned)nt, T_N / 2), 256, 0, st>>>(n, t0, nt, nsplit, b, W, colE + c * n,
+            // four columns a thread where there are blocks enough, fewer for few tiles
+            const int yb = nt >= 32 ? T_N / 8 : nt >= 8 ? T_N / 4 : T_N / 2;
+            k_rns_combine<<<dim3((unsigned)nt, (unsigned)yb), 256, 0, st>>>(n, t0, nt, nsplit, b, W, colE + c * n,
                                                                   c == 0 ? beta : 1.0, C, ldc, flag, err);
             MDSIP_LAUNCHED();
         }
