@@ -74,7 +74,9 @@ __device__ __forceinline__ void bar_chain() { asm volatile("bar.sync 2, 128;" ::
 // The 16 x 16 diagonal sub-block at c0 and up to 32 rows below it, together.
 // Warps 0 .. 3 hold one element (ei, ej), ej >= 1, of the block's lower
 // triangle per lane, 30 lanes each; column j goes through `col` (two buffers of
-// 17, one barrier per column); v_it -= (w_i w_t) / d.  Lane 31 of each also
+// 17, one barrier per column); v_it -= (w_i / d) w_t, in that order: w_i w_t
+// leaves the range below 2^-511 and above 2^512, and w_i / d is the L that the
+// rows below use.  Lane 31 of each also
 // forms the next pivot from its value before the column (col[16]), so that its
 // reciprocal is under way while the column's elements are exchanged: a column
 // is one FMA, a reciprocal and two shuffles of latency.  Warps 4 .. 7 take the
@@ -106,7 +108,7 @@ __device__ bool q_chain_rows(double *V, double *Ls, double *col, double *s_rc, u
             if (j + 1 < cw) {
                 const bool nd = lane == 31;
                 const double wi = cb[nd ? j + 1 : ei], wt = cb[nd ? j + 1 : ej];
-                const double nv = fma(-(wi * wt), r, nd ? cb[16] : v);
+                const double nv = fma(-(wi * r), wt, nd ? cb[16] : v);
                 if (ej > j) v = nv;
                 r = rcp_newton(__shfl_sync(0xffffffffu, nv, 31));
             }
