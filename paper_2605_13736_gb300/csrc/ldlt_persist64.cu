@@ -492,7 +492,7 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
                         unsigned long long m = 0ULL;
                         int e = 0;
                         const double ad = fabs(d);
-                        if (ad > 0x1p-1000 && isfinite(ad)) rns::rsqrt64(ad, m, e);   // else the panel is rejected
+                        if (ad > 0x1p-1000 && isfinite(ad)) rns::rsqrt64(ad, m, e);   // else the column test rejects the panel
                         s_sm[lane] = m;
                         s_se[lane] = e;
                     }
@@ -558,7 +558,9 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
             if (tid < nb) {
                 const double d = s_d[tid];
                 const double colmax = __longlong_as_double((long long)__ldcg(&a.cmax[buf * 64 + tid]));
-                if (absbits64(d) < absbits64(alpha * colmax) || d == 0.0 || fabs(d) <= ztol || !isfinite(d) ||
+                // (a pivot below 2^-1000 has no scaling |d|^-1/2 in the integer form: its panel
+                // goes to the pivoting kernel, as one that needs an interchange)
+                if (absbits64(d) < absbits64(alpha * colmax) || fabs(d) <= fmax(ztol, 0x1p-1000) || !isfinite(d) ||
                     !isfinite(colmax))
                     keep = 0;
             }

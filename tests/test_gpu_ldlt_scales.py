@@ -70,3 +70,20 @@ def test_blocks_of_different_scales(ctx, n1, n2, e):
     assert inertia == (N, 0, 0)
     tol = 2 * N * np.longdouble(2.0) ** -52 * np.sqrt(np.outer(b, b))
     assert (R <= tol).all(), float((R / np.where(tol > 0, tol, 1)).max())
+
+
+@pytest.mark.parametrize("i,j", [(3, 9), (31, 40), (5, 70)])
+def test_pivots_below_the_integer_form(ctx, i, j):
+    """Without a zero tolerance a pivot below 2^-1000 is a pivot like any other:
+    its column's update counts although |d|^-1/2 is outside the integer form."""
+    N = 96
+    K = np.eye(N)
+    t = 2.0 ** -1010
+    K[i, i], K[j, j] = 4 * t, 3 * t
+    K[i, j] = K[j, i] = 2 * t                                 # d_j = 3 t - (2 t)^2 / 4 t = 2 t
+    R, _, inertia, _, d = _factor(ctx, K, 0.0)
+    assert inertia == (N, 0, 0)
+    assert not R.any()                                        # powers of two: exact
+    want = np.ones(N)
+    want[i], want[j] = 4 * t, 2 * t
+    np.testing.assert_array_equal(np.sort(d.astype(float)), np.sort(want))
