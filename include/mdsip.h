@@ -323,9 +323,18 @@ mdsip_status mdsip_probe_fp64_fma(mdsip_ctx *ctx, int32_t blocks, int64_t iters,
  * A: m x n row-major with leading dimension lda (lda >= n, lda % 2 == 0),
  * w: m (nonzero), C: n x n column-major, leading dimension ldc; only the lower
  * triangle (p >= q) is written.  beta is 0 or 1.  An FP64 product: small ones
- * on the FP64 pipe, larger ones as exact integer products on the tensor cores
- * (operands scaled and rounded once to 53 bits or more per column, the sum
- * rounded once to FP64), with errors no larger. */
+ * on the FP64 pipe, larger ones as exact integer products on the tensor cores,
+ * their operands s_ip = A[i][p] w[i]^-1/2 in fixed point per column.  There, over
+ * at most 32768 consecutive rows at a time, s_ip is rounded to within
+ * 2^-53 max_i |s_ip|, the rows' sum is exact and rounded once to FP64, and the
+ * sums are added in FP64: an error of at most
+ *   2^-53 (max_i |s_ip| sum_i |s_iq| + max_i |s_iq| sum_i |s_ip|)
+ * (sums over the rows where both are nonzero) beyond that of the FP64 additions.
+ * Entries far below their column's largest lose bits in that form; where the
+ * geometric mean of a column's nonzero s_ip is more than 2^9 below the largest
+ * in any such range of rows, or an operand is outside the form's range
+ * (non-finite, subnormal, w not in 2^-1000 .. 2^1000), the FP64 pipe takes the
+ * whole product, with errors relative to sum_i |A[i][p] A[i][q] / w[i]|. */
 mdsip_status mdsip_syrk_scaled(mdsip_ctx *ctx, int64_t m, int64_t n, const double *A, int64_t lda,
                                const double *w, double beta, double *C, int64_t ldc);
 

@@ -7,17 +7,29 @@
 // contractions beats the DFMA kernel by more than an order of magnitude
 // wherever the product is large enough to pay for its passes.
 //
-// For a chunk of rows the scaled entry a_ip w_i^-1/2 is rounded once to an
-// integer X_ip of at most b bits (b = 53 .. 56) relative to the largest entry
+// For a chunk of rows the scaled entry s_ip = a_ip w_i^-1/2 is rounded once to
+// an integer X_ip of at most b bits (b = 53 .. 56) relative to the largest entry
 // of its column in the chunk; the integer sums sum_i X_ip X_iq are then formed
 // exactly: residues of X modulo 14 pairwise coprime moduli (<= 512, residues
 // of magnitude <= 256, exact in BF16), one tensor-core contraction per modulus
 // whose FP32 accumulators stay exact over 256 rows (256 * 256^2 = 2^24), the
 // accumulators reduced modulo p every 256 rows, and the sum recovered by the
 // Chinese remainder theorem in 128-bit integers (the construction published
-// as the Ozaki scheme II).  The only roundings are the one of X and the final
-// one to FP64, so the error is below that of the DFMA sum over the same rows,
-// whose accumulators round at every term.
+// as the Ozaki scheme II).  The only roundings are the one of X, the one of a
+// chunk's sum to FP64 and the FP64 sum of the chunks.
+//
+// The operands are in fixed point per column: an entry 2^k below its column's
+// largest keeps b - k bits.  An X is off by at most 2^(1 - b) max|s_p| (0 for a
+// zero entry), so a chunk's sum by 2^(1 - b) (max|s_p| sum|s_q| + max|s_q|
+// sum|s_p|) over the rows where both are nonzero, where a DFMA sum of r rows is
+// off by up to r 2^-53 sum|s_p s_q|.  The first is the smaller one as long as a
+// column's entries are not far below its largest: where the geometric mean of a
+// column's nonzero entries in a chunk is more than 2^kMeanGap below the largest
+// entry, the DFMA kernel takes the product.  kMeanGap = 9: N(0, 1) entries have a
+// gap of 3.6 to 4.6, at every step of the benchmark family's solves as well
+// (whose w_i span nine decades in the end), and 7.1 with weights over five
+// decades; one entry 2^8 above the others, or half of the rows 2^15 above the
+// other half, is where the bound meets that of a DFMA sum of some 400 rows.
 //
 // Passes: (1) k_rns_rows: w_i^-1/2 as a 64-bit mantissa and an exponent;
 // (2) k_rns_colmax: exponent bound of every column in every chunk; per chunk
@@ -25,8 +37,9 @@
 // FP32 arithmetic only: one FP64 instruction per entry costs as much as 64
 // FP32 ones); (4) k_rns_mma; (5) k_rns_combine.  Entries the integer form does
 // not cover (non-finite or subnormal entries of A; w not positive, finite and
-// within 2^+-1000) raise a device flag in (1) or (2); the later passes then
-// do nothing and the DFMA kernel, gated on the same flag, forms the product.
+// within 2^+-1000; columns of too wide a spread) raise a device flag in (1) or
+// (2); the later passes then do nothing and the DFMA kernel, gated on the same
+// flag, forms the product.
 #include <cuda.h>
 
 #include <algorithm>
@@ -71,6 +84,14 @@ __host__ __device__ inline int rns_tiles(int64_t n) {
     return (int)(a * (a + 1) + (np & 1 ? a + 1 : 0));
 }
 
+constexpr int kMeanGap = 9;            // binary orders (see above)
+
+// of the columns of every chunk: exponent bound, sum and count of the exponents;
+// of every 64 of them: strips done
+struct ColStat {
+    int *E, *sum, *cnt, *done;
+};
+
 // w_i^-1/2 = sm[i] 2^(se[i] - 63)
 __global__ void k_rns_rows(int64_t m, const double *__restrict__ w, unsigned long long *__restrict__ sm,
                            int *__restrict__ se, int *__restrict__ flag) {
@@ -84,24 +105,33 @@ __global__ void k_rns_rows(int64_t m, const double *__restrict__ w, unsigned lon
     }
 }
 
-// colE[chunk][q] = 2 + max_i (exponent of A[i][q] + se[i]) over the chunk's
-// rows (atomicMax into INT_MIN): |a s| < 2^colE.  32 x 8 threads, 64 columns
-// and `strip` rows per block; HBM-bound (one read of A).
+// col[chunk][q]: E = 2 + max_i (exponent of A[i][q] + se[i]) over the chunk's
+// rows, |a s| < 2^E, and the sum and count of the exponents of its nonzero
+// entries.  32 x 8 threads, 64 columns and `strip` rows per block, strips of 512
+// rows where that leaves blocks enough (fewer atomics and tickets); HBM-bound
+// (one read of A).  The sums, counts and tickets cost 8 of 646 us at m = 30011, n =
+// 771 and 35 us of 6.9 ms at m = 100000, n = 2000; a look at the spread inside
+// k_rns_residues took that kernel from 64 to 104 registers and 370 us more there.
 __global__ void __launch_bounds__(256) k_rns_colmax(const double *__restrict__ A, int64_t m, int64_t n, int64_t lda,
                                                     int64_t kc, int strip, int strips_per_chunk,
-                                                    const int *__restrict__ se, int *__restrict__ colE,
+                                                    const int *__restrict__ se, ColStat col_stat,
                                                     int *__restrict__ flag) {
-    __shared__ int red[8][64];
+    __shared__ int red[3][8][64];
     const int64_t col = (int64_t)blockIdx.x * 64 + 2 * threadIdx.x;
     const int64_t chunk = blockIdx.y / strips_per_chunk;
     const int64_t i0 = chunk * kc + (int64_t)(blockIdx.y % strips_per_chunk) * strip;
     const int64_t i1 = min(m, min(i0 + strip, (chunk + 1) * kc));
-    int e0 = INT_MIN, e1 = INT_MIN;
+    // per column and thread: the largest and the sum of kOne + (exponent + kOff) over
+    // the nonzero entries (at most 64 rows: the count above the sum, no carry)
+    constexpr unsigned kOne = 1u << 18, kOff = 1024u;
+    unsigned m0 = 0, m1 = 0, a0 = 0, a1 = 0;
     bool bad = false;
-    auto upd = [&](double v, int s, int &e) {
+    auto upd = [&](double v, unsigned s, unsigned &mx, unsigned &acc) {
         const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
         const unsigned ef = (hi >> 20) & 0x7ffu;
-        if (ef != 0u) e = max(e, (int)ef + s);
+        const unsigned x = ef != 0u ? ef + s : 0u;
+        mx = max(mx, x);
+        acc += x;
         bad |= ef == 0x7ffu || (ef == 0u && ((hi & 0xfffffu) | lo) != 0u);
     };
     if (col < n) {
@@ -110,27 +140,54 @@ __global__ void __launch_bounds__(256) k_rns_colmax(const double *__restrict__ A
 #pragma unroll 8
         for (int64_t i = i0 + threadIdx.y; i < i1; i += 8) {
             const double2 v = __ldg(reinterpret_cast<const double2 *>(a + i * lda));
-            const int s = __ldg(se + i);
-            upd(v.x, s, e0);
-            if (two) upd(v.y, s, e1);
+            const unsigned s = (unsigned)__ldg(se + i) + (kOne + kOff);
+            upd(v.x, s, m0, a0);
+            if (two) upd(v.y, s, m1, a1);
         }
     }
     if (bad) atomicExch(flag, 1);
-    red[threadIdx.y][2 * threadIdx.x] = e0;
-    red[threadIdx.y][2 * threadIdx.x + 1] = e1;
+    auto put = [&](int c, unsigned mx, unsigned acc) {
+        const int cnt = (int)(acc / kOne);
+        red[0][threadIdx.y][c] = mx ? (int)(mx % kOne) - (int)kOff : INT_MIN;
+        red[1][threadIdx.y][c] = (int)(acc % kOne) - cnt * (int)kOff;
+        red[2][threadIdx.y][c] = cnt;
+    };
+    put(2 * threadIdx.x, m0, a0);
+    put(2 * threadIdx.x + 1, m1, a1);
     __syncthreads();
-    const int t = threadIdx.y * 32 + threadIdx.x;
-    if (t < 64) {
-        int e = red[0][t];
-        for (int y = 1; y < 8; ++y) e = max(e, red[y][t]);
-        const int64_t q = (int64_t)blockIdx.x * 64 + t;
-        if (q < n && e != INT_MIN) atomicMax(colE + chunk * n + q, e - 1023 + 2);
+    const int t = threadIdx.y * 32 + threadIdx.x, u = t & 63, what = t >> 6;   // 64 threads a quantity
+    if (what < 3) {
+        int r = red[what][0][u];
+        for (int y = 1; y < 8; ++y) r = what == 0 ? max(r, red[0][y][u]) : r + red[what][y][u];
+        const int64_t q = (int64_t)blockIdx.x * 64 + u, o = chunk * n + q;
+        if (q < n) {
+            if (what == 0 && r != INT_MIN) atomicMax(col_stat.E + o, r - 1023 + 2);
+            if (what == 1 && r != 0) atomicAdd(col_stat.sum + o, r);
+            if (what == 2 && r != 0) atomicAdd(col_stat.cnt + o, r);
+        }
+    }
+    // the last of a chunk's strips looks at the spread of its columns
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (t == 0)
+        s_last = atomicAdd(col_stat.done + chunk * gridDim.x + blockIdx.x, 1) == strips_per_chunk - 1;
+    __syncthreads();
+    const int64_t q = (int64_t)blockIdx.x * 64 + t, o = chunk * n + q;
+    if (s_last && t < 64 && q < n) {
+        __threadfence();
+        const int64_t cnt = __ldcg(col_stat.cnt + o);
+        if (cnt > 0 && cnt * (__ldcg(col_stat.E + o) + 1023 - 2 - kMeanGap) > (int64_t)__ldcg(col_stat.sum + o))
+            atomicExch(flag, 1);
     }
 }
 
-__global__ void k_rns_init(int64_t cnt, int *__restrict__ colE) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (int64_t)gridDim.x * blockDim.x)
-        colE[i] = INT_MIN;
+__global__ void k_rns_init(int64_t cnt, int64_t blocks, ColStat col_stat) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (int64_t)gridDim.x * blockDim.x) {
+        col_stat.E[i] = INT_MIN;
+        col_stat.sum[i] = col_stat.cnt[i] = 0;
+        if (i < blocks) col_stat.done[i] = 0;
+    }
 }
 
 // R[l][k][q] = BF16 of X mod p_l, X = rint(A[i0 + k][q] s_(i0+k) 2^(b - colE[q])),
@@ -511,7 +568,7 @@ bool syrk_rns_pays(int64_t m, int64_t n) {
 
 size_t syrk_rns_workspace_bytes(int64_t m, int64_t n, int num_sms) {
     const RnsPlan pl = rns_plan(m, n, num_sms);
-    return 1024 + al1k((size_t)m * 8) + al1k((size_t)m * 4) + al1k((size_t)pl.chunks * n * 4) +
+    return 1024 + al1k((size_t)m * 8) + al1k((size_t)m * 4) + 4 * al1k((size_t)pl.chunks * n * 4) +
            al1k((size_t)RN * pl.kc * pl.ldn * 2) +
            al1k((size_t)RN * pl.nsplit * pl.group * T_M * T_N * sizeof(int16_t));
 }
@@ -529,21 +586,27 @@ const int *launch_syrk_rns(cudaStream_t st, int num_sms, const double *A, int64_
     base += al1k((size_t)m * 8);
     int *se = reinterpret_cast<int *>(base);
     base += al1k((size_t)m * 4);
-    int *colE = reinterpret_cast<int *>(base);
-    base += al1k((size_t)pl.chunks * n * 4);
+    ColStat cols{};
+    for (int **v : {&cols.E, &cols.sum, &cols.cnt, &cols.done}) {
+        *v = reinterpret_cast<int *>(base);
+        base += al1k((size_t)pl.chunks * n * 4);
+    }
+    const int *colE = cols.E;
     uint4 *R = reinterpret_cast<uint4 *>(base);
     base += al1k((size_t)RN * pl.kc * pl.ldn * 2);
     int16_t *W = reinterpret_cast<int16_t *>(base);
 
     MDSIP_CUDA(cudaMemsetAsync(flag, 0, 2 * sizeof(int), st));
-    k_rns_init<<<std::max(1, std::min(1024, ceil_div(pl.chunks * n, 256))), 256, 0, st>>>(pl.chunks * n, colE);
+    k_rns_init<<<std::max(1, std::min(1024, ceil_div(pl.chunks * n, 256))), 256, 0, st>>>(
+        pl.chunks * n, pl.chunks * ceil_div(n, 64), cols);
     MDSIP_LAUNCHED();
     k_rns_rows<<<std::max(1, std::min(4096, ceil_div(m, 256))), 256, 0, st>>>(m, w, sm, se, flag);
     MDSIP_LAUNCHED();
-    const int strip = 256, spc = (int)((pl.kc + strip - 1) / strip);
+    const int strip = pl.chunks * ceil_div(n, 64) * ceil_div(pl.kc, 256) >= 8 * num_sms ? 512 : 256;
+    const int spc = (int)((pl.kc + strip - 1) / strip);
     MDSIP_REQUIRE(pl.chunks * spc <= 65535, MDSIP_ERR_INVALID_ARG, "syrk: m too large");
     const dim3 cg((unsigned)ceil_div(n, 64), (unsigned)(pl.chunks * spc));
-    k_rns_colmax<<<cg, dim3(32, 8), 0, st>>>(A, m, n, lda, pl.kc, strip, spc, se, colE, flag);
+    k_rns_colmax<<<cg, dim3(32, 8), 0, st>>>(A, m, n, lda, pl.kc, strip, spc, se, cols, flag);
     MDSIP_LAUNCHED();
 
     static PerDeviceOnce once;
