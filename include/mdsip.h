@@ -334,9 +334,16 @@ mdsip_status mdsip_probe_fp64_fma(mdsip_ctx *ctx, int32_t blocks, int64_t iters,
  * geometric mean of a column's nonzero s_ip is more than 2^9 below the largest
  * in any such range of rows, or an operand is outside the form's range
  * (non-finite, subnormal, w not in 2^-1000 .. 2^1000), the FP64 pipe takes the
- * whole product, with errors relative to sum_i |A[i][p] A[i][q] / w[i]|. */
+ * whole product, with errors relative to sum_i |A[i][p] A[i][q] / w[i]|.
+ * Returns once the launches are enqueued.  Should a bounded device wait of the
+ * tensor-core form expire, C is set to NaN and the next call on the context
+ * after that returns DEVICE (once).  Errors: INVALID_ARG, OOM. */
 mdsip_status mdsip_syrk_scaled(mdsip_ctx *ctx, int64_t m, int64_t n, const double *A, int64_t lda,
                                const double *w, double beta, double *C, int64_t ldc);
+
+/* For tests of that report: the next mdsip_syrk_scaled on ctx that takes the
+ * tensor-core form behaves as if a device wait had expired. */
+mdsip_status mdsip_debug_expire_wait(mdsip_ctx *ctx);
 
 /* The same product on the tensor cores: precision MDSIP_PREC_TF32 or
  * MDSIP_PREC_BF16 operands A[i][p] * w_i^-1/2 (rounded to that type), FP32

@@ -121,6 +121,7 @@ _SIGS = {
     "mdsip_launch_count": (C.c_int64, []),
     "mdsip_syrk_scaled": (C.c_int, [C.c_void_p, C.c_int64, C.c_int64, C.c_void_p, C.c_int64,
                                     C.c_void_p, C.c_double, C.c_void_p, C.c_int64]),
+    "mdsip_debug_expire_wait": (C.c_int, [C.c_void_p]),
     "mdsip_syrk_scaled_tc": (C.c_int, [C.c_void_p, C.c_int64, C.c_int64, C.c_void_p, C.c_int64,
                                        C.c_void_p, C.c_double, C.c_void_p, C.c_int64, C.c_int]),
     "mdsip_gemv_pair_df": (C.c_int, [C.c_void_p, C.c_int64, C.c_int64, C.c_void_p, C.c_int64,
@@ -404,6 +405,10 @@ def mdsip_launch_count() -> int:
 
 def mdsip_syrk_scaled(ctx, m, n, A, lda, w, beta, Cmat, ldc):
     _check(lib().mdsip_syrk_scaled(ctx, m, n, _ptr(A), lda, _ptr(w), float(beta), _ptr(Cmat), ldc), ctx)
+
+
+def mdsip_debug_expire_wait(ctx):
+    _check(lib().mdsip_debug_expire_wait(ctx), ctx)
 
 
 def mdsip_syrk_scaled_tc(ctx, m, n, A, lda, w, beta, Cmat, ldc, precision):

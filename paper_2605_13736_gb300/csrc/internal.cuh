@@ -55,6 +55,10 @@ struct Ctx {
     int num_sms = 0;
     std::string last_error;
     int32_t ldlt_panels[2] = {0, 0};   // of the last mdsip_ldlt_factor* call
+    // pinned words the device can write: [0] nonzero once a wait expired in a call
+    // that had returned before (reported by the next call)
+    int *words = nullptr;
+    bool debug_expire = false;         // the next FP64 product ends as if a wait had expired
     // grow-only scratch arena for kernel-level calls
     void *scratch = nullptr;
     size_t scratch_bytes = 0;
@@ -79,6 +83,11 @@ struct DeviceGuard {
 // Runs fn, turning exceptions into a status and the context's last error.
 template <class F>
 inline mdsip_status guarded(Ctx *ctx, F &&fn) {
+    if (ctx && ctx->words && *(volatile int *)ctx->words) {
+        *(volatile int *)ctx->words = 0;
+        ctx->last_error = "a bounded device wait expired in an earlier mdsip_syrk_scaled (its C is NaN)";
+        return MDSIP_ERR_DEVICE;
+    }
     try {
         fn();
         return MDSIP_OK;
@@ -547,16 +556,19 @@ void launch_syrk_fp64(Ctx *ctx, const double *A, int64_t m, int64_t n, int64_t l
 size_t syrk_fp64_scratch_bytes(int64_t m, int64_t n, int num_sms);
 void launch_syrk_fp64_ws(cudaStream_t s, int num_sms, const double *A, int64_t m, int64_t n,
                          int64_t lda, const double *w, double beta, double *C, int64_t ldc,
-                         double *work, int bm = 0, void *rns_ws = nullptr);
+                         double *work, int bm = 0, void *rns_ws = nullptr, int *late_err = nullptr,
+                         bool expire = false);
 // The same product by residue numbers on the tensor cores (syrk_rns.cu), the
 // faster form from syrk_rns_pays on; ws as syrk_rns_workspace_bytes.  The
 // returned device flag is nonzero afterwards when the operands were outside
-// its range and C is untouched.
+// its range and C is untouched.  late_err: null, or a host word set to 1 when a
+// wait expired; expire: as if one had (a test of that path).
 bool syrk_rns_pays(int64_t m, int64_t n);
 size_t syrk_rns_workspace_bytes(int64_t m, int64_t n, int num_sms);
 inline const int *syrk_rns_err(const void *ws) { return static_cast<const int *>(ws) + 1; }   // nonzero: a wait expired
 const int *launch_syrk_rns(cudaStream_t s, int num_sms, const double *A, int64_t m, int64_t n, int64_t lda,
-                           const double *w, double beta, double *C, int64_t ldc, void *ws);
+                           const double *w, double beta, double *C, int64_t ldc, void *ws, int *late_err = nullptr,
+                           bool expire = false);
 
 // Tensor-core SYRK (syrk_tc.cu)
 struct TcPlan {

@@ -1580,6 +1580,10 @@ mdsip_status mdsip_ctx_create(int device, void *stream, const mdsip_alloc_hooks 
             c->has_hooks = true;
         }
         MDSIP_CUDA(cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device));
+        int *w = nullptr;
+        MDSIP_CUDA(cudaMallocHost(&w, 64));
+        std::fill(w, w + 16, 0);
+        c->words = w;
     });
     if (s != MDSIP_OK) {
         delete c;
@@ -1598,6 +1602,7 @@ void mdsip_ctx_destroy(mdsip_ctx *hctx) {
             cudaStreamSynchronize(ctx->stream);
             ctx->release(ctx->scratch, ctx->scratch_bytes);
         }
+        if (ctx->words) cudaFreeHost(ctx->words);
     } catch (...) {
     }
     delete ctx;
@@ -1904,6 +1909,12 @@ mdsip_status mdsip_syrk_scaled(mdsip_ctx *hctx, int64_t m, int64_t n, const doub
         MDSIP_REQUIRE(n == 0 || (A && w && C) || m == 0, MDSIP_ERR_INVALID_ARG, "syrk: null pointer");
         launch_syrk_fp64(ctx, A, m, n, lda, w, beta, C, ldc);
     });
+}
+
+mdsip_status mdsip_debug_expire_wait(mdsip_ctx *hctx) {
+    if (!hctx) return MDSIP_ERR_INVALID_ARG;
+    C_(hctx)->debug_expire = true;
+    return MDSIP_OK;
 }
 
 mdsip_status mdsip_syrk_scaled_tc(mdsip_ctx *hctx, int64_t m, int64_t n, const double *A, int64_t lda,

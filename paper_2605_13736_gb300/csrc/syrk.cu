@@ -247,9 +247,10 @@ size_t syrk_fp64_scratch_bytes(int64_t m, int64_t n, int num_sms) {
 // work: syrk_fp64_scratch_bytes(m, n, num_sms) bytes (split partials, then 1/w)
 void launch_syrk_fp64_ws(cudaStream_t st, int num_sms, const double *A, int64_t m, int64_t n,
                          int64_t lda, const double *w, double beta, double *C, int64_t ldc,
-                         double *work, int bm, void *rns_ws) {
+                         double *work, int bm, void *rns_ws, int *late_err, bool expire) {
     if (n <= 0) return;
-    const int *gate = rns_ws ? launch_syrk_rns(st, num_sms, A, m, n, lda, w, beta, C, ldc, rns_ws) : nullptr;
+    const int *gate =
+        rns_ws ? launch_syrk_rns(st, num_sms, A, m, n, lda, w, beta, C, ldc, rns_ws, late_err, expire) : nullptr;
     const Plan pl = plan_for(m, n, num_sms, bm == 32 || bm == 64 || bm == 80 ? bm : 0);
     SyrkArgs a{};
     a.A = A;
@@ -298,7 +299,8 @@ void launch_syrk_fp64(Ctx *ctx, const double *A, int64_t m, int64_t n, int64_t l
         }
         if (base) {
             launch_syrk_fp64_ws(ctx->stream, ctx->num_sms, A, m, n, lda, w, beta, C, ldc,
-                                reinterpret_cast<double *>(base), 0, base + ws);
+                                reinterpret_cast<double *>(base), 0, base + ws, ctx->words, ctx->debug_expire);
+            ctx->debug_expire = false;
             return;
         }
     }

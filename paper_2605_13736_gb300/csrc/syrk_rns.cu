@@ -431,16 +431,18 @@ __global__ void __launch_bounds__(MMA_THREADS, 1) k_rns_mma(const __grid_constan
 // residues of the splits added, y_l = r_l (M/p_l)^-1 mod p_l, the sum
 // X = sum_l y_l M/p_l - k M with k = rint(sum_l y_l / p_l) (|X| < M / 4, so FP32
 // finds k), rounded once to FP64.  A raised err word (a wait that expired in
-// k_rns_mma) poisons the result with NaN.  Bound by the latency of its loads: a
+// k_rns_mma) poisons the result with NaN and is passed on to late_err.  Bound by the latency of its loads: a
 // thread loads its next column's 14 residues under the arithmetic of this one,
 // whose 14 terms of five 30-bit limbs are seven pairs of four 32-bit ones (n =
 // 2000, 72 tiles: 98 us with a column a thread and three splits, 46 so).
 __global__ void __launch_bounds__(256) k_rns_combine(int64_t n, int tile0, int ntile, int nsplit, int b,
                                                      const int16_t *__restrict__ W, const int *__restrict__ colE,
                                                      double beta, double *__restrict__ C, int64_t ldc,
-                                                     const int *__restrict__ flag, const int *__restrict__ err) {
+                                                     const int *__restrict__ flag, const int *__restrict__ err,
+                                                     int *late_err) {
     if (*flag) return;
     const bool poison = *err != 0;
+    if (poison && late_err && threadIdx.x == 0 && blockIdx.x == 0 && blockIdx.y == 0) *(volatile int *)late_err = 1;
     int P, Q;
     rns_tile(tile0 + blockIdx.x, P, Q);
     const int row = threadIdx.x & 127;
@@ -577,7 +579,7 @@ size_t syrk_rns_workspace_bytes(int64_t m, int64_t n, int num_sms) {
 // allocator or here.  Returns the device flag that gates the DFMA kernel: it
 // is nonzero after these launches when C still has to be formed.
 const int *launch_syrk_rns(cudaStream_t st, int num_sms, const double *A, int64_t m, int64_t n, int64_t lda,
-                           const double *w, double beta, double *C, int64_t ldc, void *ws) {
+                           const double *w, double beta, double *C, int64_t ldc, void *ws, int *late_err, bool expire) {
     const RnsPlan pl = rns_plan(m, n, num_sms);
     char *base = static_cast<char *>(ws);
     int *flag = reinterpret_cast<int *>(base), *err = flag + 1;
@@ -597,6 +599,7 @@ const int *launch_syrk_rns(cudaStream_t st, int num_sms, const double *A, int64_
     int16_t *W = reinterpret_cast<int16_t *>(base);
 
     MDSIP_CUDA(cudaMemsetAsync(flag, 0, 2 * sizeof(int), st));
+    if (expire) MDSIP_CUDA(cudaMemsetAsync(err, 1, sizeof(int), st));
     k_rns_init<<<std::max(1, std::min(1024, ceil_div(pl.chunks * n, 256))), 256, 0, st>>>(
         pl.chunks * n, pl.chunks * ceil_div(n, 64), cols);
     MDSIP_LAUNCHED();
@@ -634,7 +637,7 @@ const int *launch_syrk_rns(cudaStream_t st, int num_sms, const double *A, int64_
             // four columns a thread where there are blocks enough, fewer for few tiles
             const int yb = nt >= 32 ? T_N / 8 : nt >= 8 ? T_N / 4 : T_N / 2;
             k_rns_combine<<<dim3((unsigned)nt, (unsigned)yb), 256, 0, st>>>(n, t0, nt, nsplit, b, W, colE + c * n,
-                                                                  c == 0 ? beta : 1.0, C, ldc, flag, err);
+                                                                  c == 0 ? beta : 1.0, C, ldc, flag, err, late_err);
             MDSIP_LAUNCHED();
         }
     }
