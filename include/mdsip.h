@@ -240,7 +240,9 @@ mdsip_status mdsip_set_start_predicted(mdsip_problem *p, const float *pred, doub
  * different streams run concurrently, one host worker thread per stream, at
  * most `max_concurrent` at a time (<= 0: no limit).  statuses[i] receives
  * problem i's mdsip_solve status.  Returns OK when every problem was attempted
- * (check the statuses), or INVALID_ARG. */
+ * (check the statuses), or INVALID_ARG.  A solve whose FP64 product is large
+ * holds a workspace of up to 0.75 GB while it runs (less, at a slower product,
+ * where that is not to be had), so max_concurrent also bounds that memory. */
 mdsip_status mdsip_batch_solve(mdsip_problem *const *problems, int32_t count, int32_t max_concurrent,
                                int32_t *statuses);
 

@@ -66,6 +66,9 @@ struct Ctx {
     void *alloc(size_t bytes);
     void release(void *p, size_t bytes);
     void *scratch_at_least(size_t bytes);
+    // memory for the length of one call: through the hooks, or stream-ordered
+    void *lease(size_t bytes);
+    void give_back(void *p, size_t bytes);
 };
 
 // Makes `dev` current for the scope of the object.
@@ -553,22 +556,50 @@ void launch_gemv_t(cudaStream_t s, const double *A, int64_t m, int64_t n, int64_
 // SYRK: C (column-major, ldc) = beta C + A^T diag(1/w) A (lower)
 void launch_syrk_fp64(Ctx *ctx, const double *A, int64_t m, int64_t n, int64_t lda, const double *w,
                       double beta, double *C, int64_t ldc);
-size_t syrk_fp64_scratch_bytes(int64_t m, int64_t n, int num_sms);
+// what the workspace has room for: residues of one chunk of rows (0: the DFMA
+// kernel alone) and the DFMA kernel's split partials, in bytes
+struct SyrkRoom {
+    size_t rns = 0, part = (size_t)1 << 30;
+};
+size_t syrk_workspace_bytes(int64_t m, int64_t n, int num_sms, const SyrkRoom &room);
 void launch_syrk_fp64_ws(cudaStream_t s, int num_sms, const double *A, int64_t m, int64_t n,
                          int64_t lda, const double *w, double beta, double *C, int64_t ldc,
-                         double *work, int bm = 0, void *rns_ws = nullptr, int *late_err = nullptr,
-                         bool expire = false);
+                         void *ws, const SyrkRoom &room, int bm = 0, int *late_err = nullptr, bool expire = false);
 // The same product by residue numbers on the tensor cores (syrk_rns.cu), the
 // faster form from syrk_rns_pays on; ws as syrk_rns_workspace_bytes.  The
 // returned device flag is nonzero afterwards when the operands were outside
 // its range and C is untouched.  late_err: null, or a host word set to 1 when a
 // wait expired; expire: as if one had (a test of that path).
 bool syrk_rns_pays(int64_t m, int64_t n);
-size_t syrk_rns_workspace_bytes(int64_t m, int64_t n, int num_sms);
+size_t syrk_rns_workspace_bytes(int64_t m, int64_t n, int num_sms, size_t cap);
 inline const int *syrk_rns_err(const void *ws) { return static_cast<const int *>(ws) + 1; }   // nonzero: a wait expired
 const int *launch_syrk_rns(cudaStream_t s, int num_sms, const double *A, int64_t m, int64_t n, int64_t lda,
-                           const double *w, double beta, double *C, int64_t ldc, void *ws, int *late_err = nullptr,
-                           bool expire = false);
+                           const double *w, double beta, double *C, int64_t ldc, void *ws, size_t cap,
+                           int *late_err = nullptr, bool expire = false);
+// Workspace of the product from `get(bytes)`, which throws OOM where that much is
+// not to be had: fewer rows of residues at a time then (m = 25600, n = 512: 377 MB
+// 266 us, 86 MB 599; m = 15053, n = 301: 140 MB 145 us, 38 MB 232), and only at last
+// the DFMA kernel (n = 301 1.6 ms with room for its split partials, 15.8 with none).
+template <class F>
+void *syrk_workspace(int64_t m, int64_t n, int num_sms, SyrkRoom &room, F &&get) {
+    constexpr size_t kMB = (size_t)1 << 20;
+    constexpr SyrkRoom rooms[] = {{512 * kMB, 1024 * kMB}, {128 * kMB, 128 * kMB}, {32 * kMB, 32 * kMB},
+                                  {0, 1024 * kMB}, {0, 32 * kMB}, {0, 0}};
+    size_t last = 0;
+    for (const SyrkRoom &r : rooms) {
+        if (r.rns && !syrk_rns_pays(m, n)) continue;
+        const size_t bytes = syrk_workspace_bytes(m, n, num_sms, r);
+        if (last && bytes >= last) continue;   // no less than what was refused
+        last = bytes;
+        room = r;
+        try {
+            return get(bytes);
+        } catch (const Error &e) {
+            if (e.status != MDSIP_ERR_OOM) throw;
+        }
+    }
+    throw Error{MDSIP_ERR_OOM, "no memory for the condensation product"};
+}
 
 // Tensor-core SYRK (syrk_tc.cu)
 struct TcPlan {

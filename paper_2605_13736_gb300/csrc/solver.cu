@@ -55,6 +55,27 @@ void Ctx::release(void *p, size_t bytes) {
         cudaFree(p);
 }
 
+void *Ctx::lease(size_t bytes) {
+    if (has_hooks) return alloc(bytes);
+    void *p = nullptr;
+    const cudaError_t e = cudaMallocAsync(&p, bytes, stream);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        throw Error{MDSIP_ERR_OOM, std::string("cudaMallocAsync: ") + cudaGetErrorString(e)};
+    }
+    return p;
+}
+
+void Ctx::give_back(void *p, size_t bytes) {
+    if (!p) return;
+    if (has_hooks) {
+        cudaStreamSynchronize(stream);   // the hook may hand the memory to anyone
+        release(p, bytes);
+    } else {
+        cudaFreeAsync(p, stream);
+    }
+}
+
 void *Ctx::scratch_at_least(size_t bytes) {
     if (bytes <= scratch_bytes) return scratch;
     if (scratch) {
@@ -110,8 +131,20 @@ struct Problem {
     DBuf bgrad, bgrad_t, bcg, bcg_t, bch, bch_t, bgl, bATy, bJdh, bHss, bHdd;
     DBuf bsig_x, bq, bsig_d, bw, bbt_g, bu, bATu, brhs, bAdx;
     // reduced matrix and factors
-    DBuf bS, bL, bDd, bDoff, bperm, bkind, binertia, bldlt_ws, berr, bsyrk_ws, brns_ws, btune;
-    bool rns_oom = false;   // the residue workspace did not fit once: the DFMA product from then on
+    DBuf bS, bL, bDd, bDoff, bperm, bkind, binertia, bldlt_ws, berr, bsyrk_ws, btune;
+    // workspace of the FP64 product where the residue form pays (hundreds of MB):
+    // held by a solve while it runs, otherwise the context's scratch
+    struct ProductWs {
+        void *ptr = nullptr;
+        size_t bytes = 0;
+        SyrkRoom room;
+        bool leased = false;
+    } pws;
+    bool in_solve = false;
+    void drop_product_ws() {
+        if (pws.leased) ctx->give_back(pws.ptr, pws.bytes);
+        pws = ProductWs{};
+    }
     // tensor-core condensation and refinement
     DBuf bAfT, bvf, btc_ws, btc_err, bref_b, bref_u, bref_r, bref_d, btmp_nd2, bsolve_ws, bsolve_err, bAu_run;
     DBuf bxq, bxnew, bqinv, bwinv, bwf, bsol_g;   // the refinement's one-pass sweeps
@@ -590,7 +623,8 @@ static void prepare_path(Problem *P) {
     P->bsolve_err.get<int>(ctx, 4);
     MDSIP_CUDA(cudaMemsetAsync(P->bsolve_err.ptr, 0, sizeof(int), ctx->stream));
     dvec(ctx, P->brhs, std::max<int64_t>(N, 1) * 2);
-    const size_t sw = path == MDSIP_PATH_P2 ? syrk_fp64_scratch_bytes(D.m_E, D.n_d, ctx->num_sms) : 0;
+    const size_t sw = path == MDSIP_PATH_P2 && !syrk_rns_pays(D.m_E, D.n_d)
+                          ? syrk_workspace_bytes(D.m_E, D.n_d, ctx->num_sms, SyrkRoom{}) : 0;
     if (sw) P->bsyrk_ws.get<char>(ctx, sw);
     else P->bsyrk_ws.reset();
     if (path == MDSIP_PATH_P2) {
@@ -701,7 +735,7 @@ static int tune_pick(Problem *P, const std::vector<int> &cands, F &&run) {
 // Tile edge of the FP64 condensation product for this problem's A (tuned when
 // the product is small enough for the extra runs not to matter: the many-
 // instance setting, where the analytic choice is least reliable).
-static int tuned_syrk_tile(Problem *P) {
+static int tuned_syrk_tile(Problem *P, const Problem::ProductWs &ws) {
     const Dims &D = P->D;
     if (!P->opt.autotune || (double)D.m_E * D.n_d * D.n_d > 4e10) return 0;
     // up to order 64 the analytic choice (32) stands: 11 us against 27 with 64, but
@@ -712,29 +746,30 @@ static int tuned_syrk_tile(Problem *P) {
     double *C = P->btune.get<double>(P->ctx, (size_t)std::max<int64_t>(D.n_d * D.n_d, 1));
     v = tune_pick(P, {64, 80}, [&](int bm) {
         launch_syrk_fp64_ws(P->ctx->stream, P->ctx->num_sms, P->Mv.A, D.m_E, D.n_d, D.lda, P->bw.as<double>(),
-                            0.0, C, D.n_d, P->bsyrk_ws.as<double>(), bm);
+                            0.0, C, D.n_d, ws.ptr, ws.room, bm);
     });
     P->btune.reset();
     tune_put(TUNE_SYRK_TILE, D.m_E, D.n_d, v);
     return v;
 }
 
-// Workspace of the residue form of the FP64 product, allocated at its first
-// use (a mixed-precision problem needs it only when a step falls back to the
-// FP64 product); null where that form does not pay or does not fit.
-static void *rns_workspace(Problem *P) {
+// Workspace of the FP64 product: the problem's own where only the DFMA kernel
+// pays; else, from the first FP64 product of a call on (a mixed-precision problem
+// needs it only when a step falls back), a lease for the rest of a solve -- many
+// instances may be resident, as many as there are workers solve at a time -- or
+// the context's scratch.
+static Problem::ProductWs product_workspace(Problem *P) {
     const Dims &D = P->D;
-    if (P->rns_oom || !syrk_rns_pays(D.m_E, D.n_d)) return nullptr;
-    if (!P->brns_ws.ptr) {
-        try {
-            P->brns_ws.get<char>(P->ctx, syrk_rns_workspace_bytes(D.m_E, D.n_d, P->ctx->num_sms));
-        } catch (const Error &e) {
-            if (e.status != MDSIP_ERR_OOM) throw;
-            P->rns_oom = true;
-            return nullptr;
-        }
-    }
-    return P->brns_ws.ptr;
+    if (P->bsyrk_ws.ptr) return Problem::ProductWs{P->bsyrk_ws.ptr, P->bsyrk_ws.bytes, SyrkRoom{}, false};
+    if (P->pws.ptr) return P->pws;
+    Problem::ProductWs w;
+    w.ptr = syrk_workspace(D.m_E, D.n_d, P->ctx->num_sms, w.room, [&](size_t bytes) {
+        w.bytes = bytes;
+        w.leased = P->in_solve;   // (a callback may use the context's scratch between two steps)
+        return w.leased ? P->ctx->lease(bytes) : P->ctx->scratch_at_least(bytes);
+    });
+    if (w.leased) P->pws = w;
+    return w;
 }
 
 // Run the factorization phase `enqueue` on the problem's stream: eagerly on
@@ -857,12 +892,12 @@ static Inertia factor_attempt(Problem *P, double dw, double dc, bool force_fp64 
             launch_syrk_tc(st, P->ctx->num_sms, (int)P->opt.precision, P->bAfT.as<float>(), D.m_E, D.n_d, w,
                            1.0, S, P->N, P->btc_ws.ptr, P->btc_err.as<int>());
         } else {
-            void *rns = rns_workspace(P);
-            const int bm = rns ? 0 : tuned_syrk_tile(P);
+            const Problem::ProductWs pw = product_workspace(P);
+            const int bm = pw.room.rns ? 0 : tuned_syrk_tile(P, pw);
             MDSIP_CUDA(cudaEventRecord(P->ev[8], st));   // the tile choice's trial runs are not the product
-            launch_syrk_fp64_ws(st, P->ctx->num_sms, P->Mv.A, D.m_E, D.n_d, D.lda, w, 1.0, S, P->N,
-                                P->bsyrk_ws.as<double>(), bm, rns);
-            rns_err = rns ? syrk_rns_err(rns) : nullptr;
+            launch_syrk_fp64_ws(st, P->ctx->num_sms, P->Mv.A, D.m_E, D.n_d, D.lda, w, 1.0, S, P->N, pw.ptr, pw.room,
+                                bm);
+            rns_err = pw.room.rns ? syrk_rns_err(pw.ptr) : nullptr;
         }
         MDSIP_CUDA(cudaEventRecord(P->ev[9], st));
     } else {
@@ -1802,6 +1837,14 @@ mdsip_status mdsip_solve(mdsip_problem *hp) {
     mdsip_status result = MDSIP_OK;
     mdsip_status s = guarded(p->ctx, [&] {
         DeviceGuard g(p->ctx->device);
+        struct InSolve {
+            Problem *p;
+            explicit InSolve(Problem *q) : p(q) { p->in_solve = true; }
+            ~InSolve() {
+                p->in_solve = false;
+                p->drop_product_ws();
+            }
+        } in_solve(p);
         result = run_ipm(p);
     });
     if (s != MDSIP_OK) {

@@ -200,8 +200,8 @@ struct Plan {
 
 // Tile edge with the least executed work (ragged edge + diagonal tiles), or
 // bm_force (32, 64 or 80) when given, then the split count whose (tile, split)
-// items fill whole waves of 2 CTAs per SM.
-Plan plan_for(int64_t m, int64_t n, int num_sms, int bm_force = 0) {
+// items fill whole waves of 2 CTAs per SM.  cap: bytes of split partials.
+Plan plan_for(int64_t m, int64_t n, int num_sms, size_t cap, int bm_force = 0) {
     Plan best{bm_force ? bm_force : 64, 0, 1};
     double best_work = 0;
     for (int bm : {32, 64, 80}) {
@@ -215,7 +215,6 @@ Plan plan_for(int64_t m, int64_t n, int num_sms, int bm_force = 0) {
         }
     }
     const int64_t slots = (int64_t)num_sms * 2;
-    const size_t cap = (size_t)1 << 30;  // split partials at most 1 GiB
     double best_eff = 0.0;
     // at least one slab per split: an order below one tile (n_d = 32, m = 1000)
     // has one tile; one CTA alone took 719 us, 62 splits of a 32 x 32 tile take 23
@@ -235,23 +234,32 @@ Plan plan_for(int64_t m, int64_t n, int num_sms, int bm_force = 0) {
 }  // namespace
 
 // enough for any tile edge
-size_t syrk_fp64_scratch_bytes(int64_t m, int64_t n, int num_sms) {
+static size_t syrk_fp64_scratch_bytes(int64_t m, int64_t n, int num_sms, size_t cap) {
     size_t part = 0;
     for (int bm : {32, 64, 80}) {
-        const Plan pl = plan_for(m, n, num_sms, bm);
+        const Plan pl = plan_for(m, n, num_sms, cap, bm);
         if (pl.nsplit > 1) part = std::max(part, (size_t)pl.nsplit * (size_t)n * (size_t)n * sizeof(double));
     }
     return part + ((size_t)std::max<int64_t>(m, 1) * sizeof(double) + 255) / 256 * 256;
 }
 
-// work: syrk_fp64_scratch_bytes(m, n, num_sms) bytes (split partials, then 1/w)
+// The DFMA kernel, which runs where the residue form left everything undone,
+// takes the same bytes behind that form's flags.
+size_t syrk_workspace_bytes(int64_t m, int64_t n, int num_sms, const SyrkRoom &room) {
+    const size_t dfma = (syrk_fp64_scratch_bytes(m, n, num_sms, room.part) + 1023) / 1024 * 1024;
+    return room.rns ? std::max(syrk_rns_workspace_bytes(m, n, num_sms, room.rns), 1024 + dfma) : dfma;
+}
+
+// ws: syrk_workspace_bytes(m, n, num_sms, room) bytes, 256-byte aligned
+// (split partials, then 1/w)
 void launch_syrk_fp64_ws(cudaStream_t st, int num_sms, const double *A, int64_t m, int64_t n,
                          int64_t lda, const double *w, double beta, double *C, int64_t ldc,
-                         double *work, int bm, void *rns_ws, int *late_err, bool expire) {
+                         void *ws, const SyrkRoom &room, int bm, int *late_err, bool expire) {
     if (n <= 0) return;
     const int *gate =
-        rns_ws ? launch_syrk_rns(st, num_sms, A, m, n, lda, w, beta, C, ldc, rns_ws, late_err, expire) : nullptr;
-    const Plan pl = plan_for(m, n, num_sms, bm == 32 || bm == 64 || bm == 80 ? bm : 0);
+        room.rns ? launch_syrk_rns(st, num_sms, A, m, n, lda, w, beta, C, ldc, ws, room.rns, late_err, expire) : nullptr;
+    double *work = reinterpret_cast<double *>(static_cast<char *>(ws) + (room.rns ? 1024 : 0));
+    const Plan pl = plan_for(m, n, num_sms, room.part, bm == 32 || bm == 64 || bm == 80 ? bm : 0);
     SyrkArgs a{};
     a.A = A;
     a.m = m;
@@ -289,23 +297,11 @@ void launch_syrk_fp64_ws(cudaStream_t st, int num_sms, const double *A, int64_t 
 
 void launch_syrk_fp64(Ctx *ctx, const double *A, int64_t m, int64_t n, int64_t lda, const double *w,
                       double beta, double *C, int64_t ldc) {
-    const size_t ws = (syrk_fp64_scratch_bytes(m, n, ctx->num_sms) + 1023) / 1024 * 1024;
-    if (syrk_rns_pays(m, n)) {
-        char *base = nullptr;
-        try {
-            base = static_cast<char *>(ctx->scratch_at_least(ws + syrk_rns_workspace_bytes(m, n, ctx->num_sms)));
-        } catch (const Error &e) {   // not enough memory for the residues: the DFMA kernel needs less
-            if (e.status != MDSIP_ERR_OOM) throw;
-        }
-        if (base) {
-            launch_syrk_fp64_ws(ctx->stream, ctx->num_sms, A, m, n, lda, w, beta, C, ldc,
-                                reinterpret_cast<double *>(base), 0, base + ws, ctx->words, ctx->debug_expire);
-            ctx->debug_expire = false;
-            return;
-        }
-    }
-    double *work = static_cast<double *>(ctx->scratch_at_least(ws));
-    launch_syrk_fp64_ws(ctx->stream, ctx->num_sms, A, m, n, lda, w, beta, C, ldc, work);
+    SyrkRoom room;
+    void *ws = syrk_workspace(m, n, ctx->num_sms, room, [&](size_t bytes) { return ctx->scratch_at_least(bytes); });
+    launch_syrk_fp64_ws(ctx->stream, ctx->num_sms, A, m, n, lda, w, beta, C, ldc, ws, room, 0, ctx->words,
+                        room.rns && ctx->debug_expire);
+    if (room.rns) ctx->debug_expire = false;
 }
 
 }  // namespace mdsip

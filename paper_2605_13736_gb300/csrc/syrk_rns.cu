@@ -508,16 +508,14 @@ struct RnsPlan {
     int tiles, group, nsplit, slabs_per_split;   // tiles, tiles per launch, K splits of a full chunk
 };
 
-constexpr size_t kRCap = (size_t)512 << 20;   // residues of one chunk
-constexpr size_t kWCap = (size_t)256 << 20;   // residues of the sums of one launch
-
 size_t al1k(size_t b) { return (b + 1023) / 1024 * 1024; }
 
-RnsPlan rns_plan(int64_t m, int64_t n, int num_sms) {
+// cap: bytes of one chunk's residues; half of it for the residues of one launch's sums
+RnsPlan rns_plan(int64_t m, int64_t n, int num_sms, size_t cap) {
     RnsPlan pl{};
     pl.ldn = (n + 7) / 8 * 8;
     const int64_t mp = (m + SLAB - 1) / SLAB * SLAB;
-    int64_t kc = (int64_t)(kRCap / (2 * RN * (size_t)pl.ldn)) / (SLAB * FOLD) * (SLAB * FOLD);
+    int64_t kc = (int64_t)(cap / (2 * RN * (size_t)pl.ldn)) / (SLAB * FOLD) * (SLAB * FOLD);
     kc = std::min<int64_t>(std::max<int64_t>(kc, SLAB * FOLD), 32768);
     pl.chunks = (mp + kc - 1) / kc;
     // equal chunks
@@ -545,7 +543,7 @@ RnsPlan rns_plan(int64_t m, int64_t n, int num_sms) {
     pl.slabs_per_split = ((nslab + pl.nsplit - 1) / pl.nsplit + FOLD - 1) / FOLD * FOLD;
     pl.nsplit = (nslab + pl.slabs_per_split - 1) / pl.slabs_per_split;
     const size_t per_tile = (size_t)RN * pl.nsplit * T_M * T_N * sizeof(int16_t);
-    pl.group = (int)std::min<int64_t>(pl.tiles, std::max<int64_t>(1, (int64_t)(kWCap / per_tile)));
+    pl.group = (int)std::min<int64_t>(pl.tiles, std::max<int64_t>(1, (int64_t)(cap / 2 / per_tile)));
     return pl;
 }
 
@@ -568,19 +566,19 @@ bool syrk_rns_pays(int64_t m, int64_t n) {
     return m >= 256 && work >= (n > 64 ? 1.5e7 : 3e7) && n <= (1 << 20) && m <= (1 << 23);
 }
 
-size_t syrk_rns_workspace_bytes(int64_t m, int64_t n, int num_sms) {
-    const RnsPlan pl = rns_plan(m, n, num_sms);
+size_t syrk_rns_workspace_bytes(int64_t m, int64_t n, int num_sms, size_t cap) {
+    const RnsPlan pl = rns_plan(m, n, num_sms, cap);
     return 1024 + al1k((size_t)m * 8) + al1k((size_t)m * 4) + 4 * al1k((size_t)pl.chunks * n * 4) +
            al1k((size_t)RN * pl.kc * pl.ldn * 2) +
            al1k((size_t)RN * pl.nsplit * pl.group * T_M * T_N * sizeof(int16_t));
 }
 
-// ws: syrk_rns_workspace_bytes(m, n, num_sms), 1024-byte aligned by the
-// allocator or here.  Returns the device flag that gates the DFMA kernel: it
+// ws: syrk_rns_workspace_bytes(m, n, num_sms, cap), 1024-byte aligned.  Returns the device flag that gates the DFMA kernel: it
 // is nonzero after these launches when C still has to be formed.
 const int *launch_syrk_rns(cudaStream_t st, int num_sms, const double *A, int64_t m, int64_t n, int64_t lda,
-                           const double *w, double beta, double *C, int64_t ldc, void *ws, int *late_err, bool expire) {
-    const RnsPlan pl = rns_plan(m, n, num_sms);
+                           const double *w, double beta, double *C, int64_t ldc, void *ws, size_t cap, int *late_err,
+                           bool expire) {
+    const RnsPlan pl = rns_plan(m, n, num_sms, cap);
     char *base = static_cast<char *>(ws);
     int *flag = reinterpret_cast<int *>(base), *err = flag + 1;
     base += 1024;
