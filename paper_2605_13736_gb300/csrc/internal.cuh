@@ -55,8 +55,9 @@ struct Ctx {
     int num_sms = 0;
     std::string last_error;
     int32_t ldlt_panels[2] = {0, 0};   // of the last mdsip_ldlt_factor* call
-    // pinned words the device can write: [0] nonzero once a wait expired in a call
-    // that had returned before (reported by the next call)
+    // 16 pinned words the device can write: [0] nonzero once a wait expired in a call
+    // that had returned before (reported by the next call); [2], [3] read back by the
+    // factorization
     int *words = nullptr;
     bool debug_expire = false;         // the next FP64 product ends as if a wait had expired
     // grow-only scratch arena for kernel-level calls
@@ -630,18 +631,18 @@ struct LdltOut {
 size_t ldlt_scratch_bytes(int64_t N);
 void launch_ldlt(cudaStream_t s, int num_sms, int64_t N, const double *S, int64_t ld,
                  const double *maxabs_dev, double zero_tol, LdltOut out, void *scratch,
-                 int *err_dev, bool fp32_update = false, int nb = 0, int spec = 1);
+                 int *err_dev, int *host2, bool fp32_update = false, int nb = 0, int spec = 1);
 size_t ldlt_blocked_scratch_bytes(int64_t N);
 bool ldlt_blocked_available(int64_t N);
 // Speculation mode of the blocked factorization: 0 every panel pivots; 1 and 2
 // the persistent no-interchange kernel first, then (FP32 updates) no-interchange
-// panels.  The persistent kernel reads back where it stopped (synchronises the
-// stream).
+// panels.  Where the persistent kernel stopped is read back into host2, two pinned
+// words (synchronises the stream).
 bool ldlt_persistent_path(int64_t N, int spec);
 std::vector<int> ldlt_blocked_widths(int64_t N, bool f32);
 void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, const double *maxabs_dev,
-                         double zero_tol, LdltOut out, void *scratch, bool fp32_update, int nb = 0,
-                         int spec = 1, int *err_dev = nullptr);
+                         double zero_tol, LdltOut out, void *scratch, bool fp32_update, int nb,
+                         int spec, int *err_dev, int *host2);
 void launch_ldlt_solve(cudaStream_t s, int64_t N, const double *L, const double *Dd,
                        const double *Doff, const int32_t *perm, int64_t nrhs, double *B,
                        int64_t ldb);

@@ -1841,10 +1841,9 @@ void launch_persist32(cudaStream_t s, int num_sms, int N, const PersistArgs &pa)
 }
 
 // Where the persistent kernel stopped (N: all panels kept); reads two words
-// back (synchronises the stream).
-int persist_stopped_at(cudaStream_t s, const PanelState *st, const PanelBar *bar) {
-    thread_local int *h = nullptr;
-    if (!h) MDSIP_CUDA(cudaMallocHost(&h, 4 * sizeof(int)));
+// back into the caller's pinned ones (synchronises the stream).  (Words of the
+// thread's own were never given back, and a batch starts its threads anew.)
+int persist_stopped_at(cudaStream_t s, const PanelState *st, const PanelBar *bar, int *h) {
     MDSIP_CUDA(cudaMemcpyAsync(h, &st->k, sizeof(int), cudaMemcpyDeviceToHost, s));
     MDSIP_CUDA(cudaMemcpyAsync(h + 1, &bar->err, sizeof(int), cudaMemcpyDeviceToHost, s));
     MDSIP_CUDA(cudaStreamSynchronize(s));
@@ -1886,7 +1885,7 @@ constexpr int64_t kRnsPanelMin = 96, kRnsTrailingMin = 32;
 // 256-byte aligned.  fp32_update: trailing products in FP32.  spec (with
 // fp32_update): each panel first tries the verified no-interchange path.
 void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, const double *maxabs_dev,
-                         double zero_tol, LdltOut out, void *scratch, bool fp32_update, int nb, int spec, int *err_dev) {
+                         double zero_tol, LdltOut out, void *scratch, bool fp32_update, int nb, int spec, int *err_dev, int *host2) {
     if (N <= 0) {
         MDSIP_CUDA(cudaMemsetAsync(out.inertia, 0, 3 * sizeof(int32_t), s));
         return;
@@ -1928,7 +1927,7 @@ void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, cons
         pa.wait_ns = 20LL * 1000 * 1000 * 1000;   // 20 s: far above the longest phase (FP64 update at N ~ 44000)
         if (fp32_update) launch_persist32(s, num_sms, (int)N, pa);
         else launch_persist64(s, num_sms, N, pa, w + lay.p64);
-        k0 = persist_stopped_at(s, st, bar);
+        k0 = persist_stopped_at(s, st, bar, host2);
         MDSIP_REQUIRE(k0 >= N || cfg.C > 0, MDSIP_ERR_INVALID_ARG,
                       "ldlt: a panel needs interchanges and N is too large for the pivoting panel");
     }
@@ -1968,10 +1967,10 @@ void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, cons
         MDSIP_CUDA(cudaMemsetAsync(w + lay.cmax, 0, 192 * sizeof(unsigned long long), s));
         launch_pdl(k_bk_panel<false>, (unsigned)cfg31.C, kPanelThreads, cfg31.smem, s, cfg31.C, panel_args(cfg31));
         launch_rns_trailing(s, num_sms, N, N - k0 - 31, npanel, S, out.L, out.Dd, out.Doff, Wg, maxabs_dev, st,
-                            err_dev ? err_dev : &bar->err, w + lay.p64);
+                            err_dev, w + lay.p64);
         MDSIP_CUDA(cudaMemsetAsync(&bar->count, 0, sizeof(unsigned), s));
         launch_persist64(s, num_sms, N, pa, w + lay.p64);
-        const int k1 = persist_stopped_at(s, st, bar);
+        const int k1 = persist_stopped_at(s, st, bar, host2);
         kept = k1 - (k0 + 32);
         k0 = k1;
     }
@@ -2040,7 +2039,7 @@ void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, cons
         const PanelState *cst = st;
         if (rns && rest > kRnsTrailingMin)
             launch_rns_trailing(s, num_sms, N, rest, npanel + p, S, out.L, out.Dd, out.Doff, Wg, maxabs_dev, st,
-                                err_dev ? err_dev : &bar->err, w + lay.p64);
+                                err_dev, w + lay.p64);
         else if (fp32_update)
             launch_pdl(k_bk_trailing<float>, tiles, kUpdThreads, usm, s, 1, (int)N, cfg.NB, S, cL, cWg, cLf, cWf, cst);
         else

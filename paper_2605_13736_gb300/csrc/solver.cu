@@ -858,7 +858,7 @@ static int tuned_ldlt_width(Problem *P, bool fp32) {
             LdltOut o{P->bL.as<double>(), P->bDd.as<double>(), P->bDoff.as<double>(), P->bperm.as<int32_t>(),
                       P->bkind.as<int32_t>(), P->binertia.as<int32_t>()};
             launch_ldlt(st, P->ctx->num_sms, N, S, N, sc + SC_MAXABS, P->opt.zero_tol, o, P->bldlt_ws.ptr,
-                        P->berr.as<int>(), fp32, nb, (int)P->opt.ldlt_spec);
+                        P->berr.as<int>(), P->ctx->words + 2, fp32, nb, (int)P->opt.ldlt_spec);
         });
         MDSIP_CUDA(cudaMemcpyAsync(S, Ssave, (size_t)N * N * sizeof(double), cudaMemcpyDeviceToDevice, st));
         MDSIP_CUDA(cudaStreamSynchronize(st));
@@ -917,7 +917,7 @@ static Inertia factor_attempt(Problem *P, double dw, double dc, bool force_fp64 
         LdltOut o{P->bL.as<double>(), P->bDd.as<double>(), P->bDoff.as<double>(), P->bperm.as<int32_t>(),
                   P->bkind.as<int32_t>(), P->binertia.as<int32_t>()};
         launch_ldlt(st, P->ctx->num_sms, P->N, S, P->N, sc + SC_MAXABS, P->opt.zero_tol, o, P->bldlt_ws.ptr,
-                    P->berr.as<int>(), tc_factor, nb, (int)P->opt.ldlt_spec);
+                    P->berr.as<int>(), P->ctx->words + 2, tc_factor, nb, (int)P->opt.ldlt_spec);
         launch_ldlt_solve_prepare(st, P->N, P->bL.as<double>(), P->bsolve_ws.ptr, P->solve_fp32);
     };
     run_factor_phase(P, tc_factor ? 1 : 0, factor_phase);
@@ -2092,7 +2092,8 @@ static mdsip_status ldlt_factor_impl(mdsip_ctx *hctx, int64_t N, double *S, int6
         MDSIP_CUDA(cudaMemsetAsync(err, 0, 3 * sizeof(int), ctx->stream));
         launch_maxabs_lower(ctx->stream, N, S, ld, maxabs);
         LdltOut o{L, Dd, Doff, perm, kind, inertia, err + 1};
-        launch_ldlt(ctx->stream, ctx->num_sms, N, S, ld, maxabs, zero_tol, o, w, err, fp32_update, 0, spec);
+        launch_ldlt(ctx->stream, ctx->num_sms, N, S, ld, maxabs, zero_tol, o, w, err, ctx->words + 2, fp32_update, 0,
+                    spec);
         int herr[3] = {0, 0, 0};
         MDSIP_CUDA(cudaMemcpyAsync(herr, err, 3 * sizeof(int), cudaMemcpyDeviceToHost, ctx->stream));
         MDSIP_CUDA(cudaStreamSynchronize(ctx->stream));
