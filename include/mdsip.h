@@ -418,11 +418,13 @@ mdsip_status mdsip_ldlt_factor(mdsip_ctx *ctx, int64_t N, double *S, int64_t ld,
  * every column of the panel (and no pivot is below zero_tol times the
  * largest |S_ij|); otherwise the pivoting panel factors it from the
  * unchanged matrix.  The flag makes every panel take the pivoting kernel.
- * The no-interchange panels of either precision first run in one persistent
- * cooperative kernel (with or without MDSIP_LDLT_PERSISTENT) that stops at the
+ * In FP64 at every order, and with FP32 updates from order 2048 on or, with
+ * MDSIP_LDLT_PERSISTENT, at any order, the no-interchange panels first run in one
+ * persistent cooperative kernel that stops at the
  * first panel the rule would not keep; the panels above take over from there
  * (where the pivoting panel does not fit shared memory, N above about 16 000,
- * such a panel is an INVALID_ARG error).  With FP32 updates that
+ * such a panel is an INVALID_ARG error).  With FP32 updates (whose products need
+ * entries and pivots within the range of FP32) that
  * kernel works on an FP32 copy of S (the FP32 updates are written back into
  * S before a hand-over; large trailing matrices are updated on the tensor
  * cores with a three-product TF32 split, about FP32 accuracy).  The call then

@@ -636,8 +636,9 @@ size_t ldlt_blocked_scratch_bytes(int64_t N);
 bool ldlt_blocked_available(int64_t N);
 // Speculation mode of the blocked factorization: 0 every panel pivots; 1 and 2
 // the persistent no-interchange kernel first, then (FP32 updates) no-interchange
-// panels.  Where the persistent kernel stopped is read back into host2, two pinned
+// panels; kSpecPanels (FP32 updates) no-interchange panels alone.  Where the persistent kernel stopped is read back into host2, two pinned
 // words (synchronises the stream).
+constexpr int kSpecPanels = 3;
 bool ldlt_persistent_path(int64_t N, int spec);
 std::vector<int> ldlt_blocked_widths(int64_t N, bool f32);
 void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, const double *maxabs_dev,

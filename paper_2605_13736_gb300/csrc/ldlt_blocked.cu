@@ -1871,7 +1871,7 @@ bool ldlt_blocked_available(int64_t N) { return blocked_config(N, true).C > 0 &&
 // updates (whose per-panel launches replayed as one graph): N = 562 0.23 / 0.49, 2050
 // 0.82 / 1.73 ms; 24 solves of 114 to 350 at once 79 / 84 ms in all.
 bool ldlt_persistent_path(int64_t N, int spec) {
-    return spec != 0 && N > 0 && N <= (int64_t)0x7fffffff / 2;
+    return spec != 0 && spec != kSpecPanels && N > 0 && N <= (int64_t)0x7fffffff / 2;
 }
 
 // Pivoting FP64 panels: columns left from which they are 31 wide with

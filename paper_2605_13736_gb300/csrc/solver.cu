@@ -2064,9 +2064,12 @@ mdsip_status mdsip_ldlt_factor_ex(mdsip_ctx *hctx, int64_t N, double *S, int64_t
         if (hctx) C_(hctx)->last_error = "ldlt: unknown or contradictory flags";
         return MDSIP_ERR_INVALID_ARG;
     }
-    const int spec = (flags & MDSIP_LDLT_NO_SPECULATION) ? 0 : ((flags & MDSIP_LDLT_PERSISTENT) ? 2 : 1);
-    return ldlt_factor_impl(hctx, N, S, ld, zero_tol, L, Dd, Doff, perm, kind, inertia,
-                            (flags & MDSIP_LDLT_FP32_UPDATES) != 0, spec);
+    const bool fp32 = (flags & MDSIP_LDLT_FP32_UPDATES) != 0;
+    int spec = (flags & MDSIP_LDLT_NO_SPECULATION) ? 0 : ((flags & MDSIP_LDLT_PERSISTENT) ? 2 : 1);
+    // the persistent kernel holds S itself in FP32 (reconstruction error 1e-7 against
+    // 1e-8 at N = 100 and 300): below this order only where it is asked for
+    if (fp32 && spec == 1 && N < 2048) spec = mdsip::kSpecPanels;
+    return ldlt_factor_impl(hctx, N, S, ld, zero_tol, L, Dd, Doff, perm, kind, inertia, fp32, spec);
 }
 
 static mdsip_status ldlt_factor_impl(mdsip_ctx *hctx, int64_t N, double *S, int64_t ld, double zero_tol,

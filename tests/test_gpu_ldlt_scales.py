@@ -87,3 +87,23 @@ def test_pivots_below_the_integer_form(ctx, i, j):
     want = np.ones(N)
     want[i], want[j] = 4 * t, 2 * t
     np.testing.assert_array_equal(np.sort(d.astype(float)), np.sort(want))
+
+
+@pytest.mark.parametrize("N", [40, 100, 300, 1000])
+def test_fp32_updates_keep_the_matrix_in_fp64(ctx, N):
+    """Below order 2048, without MDSIP_LDLT_PERSISTENT, FP32 enters through the
+    updates only: the first column of L, which takes none, is an FP64 quotient."""
+    torch = torch_cuda()
+    K = _convex(np.random.default_rng(N), N)
+    S = dev(np.tril(K).T.copy())
+    L = torch.zeros((N, N), dtype=torch.float64, device="cuda")
+    Dd, Doff = (torch.zeros(N, dtype=torch.float64, device="cuda") for _ in range(2))
+    perm, kind = (torch.zeros(N, dtype=torch.int32, device="cuda") for _ in range(2))
+    inr = torch.zeros(3, dtype=torch.int32, device="cuda")
+    m.mdsip_ldlt_factor_ex(ctx, N, S, N, 1e-14, m.MDSIP_LDLT_FP32_UPDATES, L, Dd, Doff, perm, kind, inr)
+    torch.cuda.synchronize()
+    assert tuple(inr.cpu().numpy()) == (N, 0, 0)
+    d0, col = float(Dd[0]), L[0].cpu().numpy()
+    assert d0 == K[0, 0]
+    # a reciprocal and a product: two roundings
+    np.testing.assert_allclose(col[1:], K[1:, 0] / K[0, 0], rtol=2.0 ** -51, atol=0)
