@@ -1702,8 +1702,9 @@ __global__ void k_bk_init(int N, int32_t *perm, PanelState *st, unsigned long lo
     }
 }
 
-__global__ void k_bk_finish(const PanelState *st, int32_t *inertia, int32_t *panels) {
+__global__ void k_bk_finish(const PanelState *st, const PanelBar *bar, int32_t *inertia, int32_t *panels, int *err) {
     pdl_wait();
+    if (bar->err) *err = 1;
     inertia[0] = st->npos;
     inertia[1] = st->nneg;
     inertia[2] = st->nzero;
@@ -1865,8 +1866,8 @@ bool ldlt_blocked_available(int64_t N) { return blocked_config(N, true).C > 0 &&
 
 // The persistent no-interchange factorization runs first (and the host reads
 // back where it stopped) at every order: it needs no pivoting panel unless a
-// panel fails the column test, and a first panel that fails costs one short
-// launch.  Convex Newton-step shape, persistent / per-panel launches, FP64: N =
+// panel fails the column test, and a first panel that fails costs some 10 us at
+// N <= 128 (where its first column fails) and 30 to 50 above.  Convex Newton-step shape, persistent / per-panel launches, FP64: N =
 // 33 0.085 / 0.14 ms, 351 0.35 / 1.47, 1036 0.98 / 4.46, 2050 2.42 / 11.1; FP32
 // updates (whose per-panel launches replayed as one graph): N = 562 0.23 / 0.49, 2050
 // 0.82 / 1.73 ms; 24 solves of 114 to 350 at once 79 / 84 ms in all.
@@ -1880,6 +1881,13 @@ bool ldlt_persistent_path(int64_t N, int spec) {
 // which such a panel's update takes them (a DFMA tile takes 38 us of the FP64
 // pipe however few there are, rows and update 7 + 12).
 constexpr int64_t kRnsPanelMin = 96, kRnsTrailingMin = 32;
+
+// Orders up to which the FP64 form does not read back where the persistent kernel
+// stopped: one or two empty pivoting panels cost less than that (convex, N = 16 62 ->
+// 61 us, 33 84 -> 76, 64 98 -> 90, 96 124 -> 119; with an interchange half way 24
+// 136 -> 116, 64 174 -> 165)
+constexpr int64_t kBlindMax = 96;
+static_assert(kBlindMax <= kRnsPanelMin, "the panels that follow are the wide ones");
 
 // S (lower, ld N) is overwritten.  scratch: ldlt_blocked_scratch_bytes(N),
 // 256-byte aligned.  fp32_update: trailing products in FP32.  spec (with
@@ -1927,7 +1935,10 @@ void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, cons
         pa.wait_ns = 20LL * 1000 * 1000 * 1000;   // 20 s: far above the longest phase (FP64 update at N ~ 44000)
         if (fp32_update) launch_persist32(s, num_sms, (int)N, pa);
         else launch_persist64(s, num_sms, N, pa, w + lay.p64);
-        k0 = persist_stopped_at(s, st, bar, host2);
+        // small FP64 matrices: the one or two pivoting panels follow unconditionally and,
+        // as a rule, find nothing left
+        if (!fp32_update && N <= kBlindMax && cfg.C > 0 && nb == 0) k0 = 0;
+        else k0 = persist_stopped_at(s, st, bar, host2);
         MDSIP_REQUIRE(k0 >= N || cfg.C > 0, MDSIP_ERR_INVALID_ARG,
                       "ldlt: a panel needs interchanges and N is too large for the pivoting panel");
     }
@@ -2046,7 +2057,8 @@ void launch_ldlt_blocked(cudaStream_t s, int num_sms, int64_t N, double *S, cons
             launch_pdl(k_bk_trailing<double>, tiles, kUpdThreads, usm, s, 1, (int)N, cfg.NB, S, cL, cWg, cLf, cWf, cst);
     }
     const PanelState *cst = st;
-    launch_pdl(k_bk_finish, 1, 1, 0, s, 1, cst, out.inertia, out.panels);
+    const PanelBar *cbar = bar;
+    launch_pdl(k_bk_finish, 1, 1, 0, s, 1, cst, cbar, out.inertia, out.panels, err_dev);
 }
 
 }  // namespace mdsip

@@ -51,6 +51,7 @@ constexpr int Q_THREADS = 544;          // warps 0-7 factor; 0-15 update, 0-12 i
 constexpr int Q_COMP = 256;             // threads of the factorization
 constexpr int Q_EPI = 16;               // warps of the trailing update
 constexpr int Q_OWN = 96;               // rows below the block staged at a time
+constexpr int kFirstTestMax = 128;      // orders whose first column is tested before its panel
 constexpr int VP = 33, LP = 33;         // shared-memory row pitches (doubles)
 constexpr int QA_BYTES = 128 * 64, QB_BYTES = 32 * 64;   // residues of 128 rows / 32 rows, 32 BF16 each
 constexpr int Q_STAGE = QA_BYTES + QB_BYTES;             // one modulus; a tile's 13 are loaded together
@@ -203,6 +204,21 @@ __device__ __forceinline__ void q_colmax(unsigned long long bm, unsigned long lo
     const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(bm >> 32));
     const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(bm >> 32) == hi ? (unsigned)bm : 0u);
     if (lane == 0 && (hi | lo)) atomicMax(dst, ((unsigned long long)hi << 32) | lo);
+}
+
+// whether the rule keeps a diagonal pivot d against the column's maximum.  (A pivot
+// below 2^-1000 has no scaling |d|^-1/2 in the integer form: its panel goes to the
+// pivoting kernel, as one that needs an interchange.)
+__device__ __forceinline__ bool q_keeps(double d, double colmax, double ztol) {
+    const double alpha = 0.6403882032022076;   // (1 + sqrt 17) / 8
+    return absbits64(d) >= absbits64(alpha * colmax) && fabs(d) > fmax(ztol, 0x1p-1000) && isfinite(d) &&
+           isfinite(colmax);
+}
+
+// the panel loop takes over at st->k
+__device__ __forceinline__ void q_hand_over(PanelState *st) {
+    st->kb = 0;
+    st->spec = 0;
 }
 
 // mbarriers of q_update, and -(bias + k M) modulo 2^128 in s_km (threads 0 .. 15)
@@ -395,6 +411,27 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
     // entries near the subnormal range would lose bits in the integer form: the
     // pivoting panels take such a matrix (st->k stays where it is)
     if (!(maxabs > 0x1p-900)) return;
+    // The rule's test on the first column, which takes no update: a small matrix that
+    // pivots at once leaves here, the same decision in every CTA (zero diagonal, with
+    // the read-back saved below order 96: N = 8 87 -> 67 us, 33 199 -> 160, 64 310 ->
+    // 262; at N = 350 the test would cost 9 us of 347 and save 30 of 1680)
+    if (N <= kFirstTestMax) {
+        if (tid == 0) s_cmax[0] = 0ULL;
+        __syncthreads();
+        const double *col = a.A + (int64_t)a.st->k * (N + 1);
+        unsigned long long bm = 0ULL;
+        for (int i = 1 + tid; i < N - a.st->k; i += Q_THREADS) {
+            const unsigned long long b = absbits64(__ldcg(col + i));
+            bm = b > bm ? b : bm;
+        }
+        q_colmax(bm, &s_cmax[0], lane);
+        __syncthreads();
+        const double d = __ldcg(col), colmax = __longlong_as_double((long long)s_cmax[0]);
+        if (!q_keeps(d, colmax, ztol)) {
+            if (g == 0 && tid == 0) q_hand_over(a.st);
+            return;
+        }
+    }
     if (tid == 0) {
         for (int j = 0; j < 16; ++j) tc::mbar_init(&colbar[j], 4);
     }
@@ -553,23 +590,11 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
         if (!panel_barrier(a.bar, epoch, a.wait_ns)) break;
         // ---------------- the rule's column test, the same in every CTA
         {
-            const double alpha = 0.6403882032022076;   // (1 + sqrt 17) / 8
             int keep = 1;
-            if (tid < nb) {
-                const double d = s_d[tid];
-                const double colmax = __longlong_as_double((long long)__ldcg(&a.cmax[buf * 64 + tid]));
-                // (a pivot below 2^-1000 has no scaling |d|^-1/2 in the integer form: its panel
-                // goes to the pivoting kernel, as one that needs an interchange)
-                if (absbits64(d) < absbits64(alpha * colmax) || fabs(d) <= fmax(ztol, 0x1p-1000) || !isfinite(d) ||
-                    !isfinite(colmax))
-                    keep = 0;
-            }
+            if (tid < nb)
+                keep = q_keeps(s_d[tid], __longlong_as_double((long long)__ldcg(&a.cmax[buf * 64 + tid])), ztol);
             if (!__syncthreads_and(keep)) {
-                if (g == 0 && tid == 0) {   // the panel loop takes over at column k
-                    a.st->k = k;
-                    a.st->kb = 0;
-                    a.st->spec = 0;
-                }
+                if (g == 0 && tid == 0) q_hand_over(a.st);   // st->k is this panel's first column
                 break;
             }
             if (g == 0) {
