@@ -438,8 +438,9 @@ mdsip_status mdsip_ldlt_factor_ex(mdsip_ctx *ctx, int64_t N, double *S, int64_t 
 
 /* Panel counts of the last mdsip_ldlt_factor / mdsip_ldlt_factor_ex call on
  * ctx (host array of 2): out2[0] = panels kept by the verified
- * no-interchange path, out2[1] = panels it handed to the pivoting kernel.
- * Both are 0 when that path did not run (MDSIP_LDLT_NO_SPECULATION or the
+ * no-interchange path, out2[1] = panels it handed to the pivoting kernel
+ * (FP64: times it did so; the last of them may have been followed by further
+ * pivoting panels).  Both are 0 when that path did not run (MDSIP_LDLT_NO_SPECULATION or the
  * unblocked kernel). */
 mdsip_status mdsip_ldlt_panel_counts(mdsip_ctx *ctx, int32_t *out2);
 

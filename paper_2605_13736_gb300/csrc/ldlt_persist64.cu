@@ -219,6 +219,7 @@ __device__ __forceinline__ bool q_keeps(double d, double colmax, double ztol) {
 __device__ __forceinline__ void q_hand_over(PanelState *st) {
     st->kb = 0;
     st->spec = 0;
+    st->nrej += 1;
 }
 
 // mbarriers of q_update, and -(bias + k M) modulo 2^128 in s_km (threads 0 .. 15)
@@ -410,7 +411,10 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
     const double maxabs = __ldg(a.maxabs), ztol = a.zero_tol * maxabs;
     // entries near the subnormal range would lose bits in the integer form: the
     // pivoting panels take such a matrix (st->k stays where it is)
-    if (!(maxabs > 0x1p-900)) return;
+    if (!(maxabs > 0x1p-900)) {
+        if (g == 0 && tid == 0) q_hand_over(a.st);
+        return;
+    }
     // The rule's test on the first column, which takes no update: a small matrix that
     // pivots at once leaves here, the same decision in every CTA (zero diagonal, with
     // the read-back saved below order 96: N = 8 87 -> 67 us, 33 199 -> 160, 64 310 ->

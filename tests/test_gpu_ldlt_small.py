@@ -54,3 +54,25 @@ def test_reconstruction(ctx, kind, N):
     R = np.abs(K[np.ix_(p, p)] - W @ Lh.T)
     b = np.abs(W) @ np.abs(Lh).T                # sum_j |w_ij| |l_kj|
     assert (R <= 4 * (N + 4) * 2.0 ** -53 * np.maximum(b, b.T).max()).all()
+
+
+@pytest.mark.parametrize("N,spots", [(20, ()), (20, (9,)), (80, (40,)), (300, (70,)), (1036, (100, 431, 800))])
+def test_panels_handed_over_are_counted(ctx, N, spots):
+    """mdsip_ldlt_panel_counts: one hand-over per interchange that stands alone, none without."""
+    torch = torch_cuda()
+    K = _matrix("convex", N)
+    for j in spots:                             # [[0, 3], [3, 0]], which only a 2x2 pivot gets past
+        K[j, j] = K[j + 1, j + 1] = 0.0
+        K[j, j + 1] = K[j + 1, j] = 3.0
+    S = dev(np.tril(K).T.copy())
+    L = torch.zeros((N, N), dtype=torch.float64, device="cuda")
+    Dd, Doff = (torch.zeros(N, dtype=torch.float64, device="cuda") for _ in range(2))
+    perm, kd = (torch.zeros(N, dtype=torch.int32, device="cuda") for _ in range(2))
+    inr = torch.zeros(3, dtype=torch.int32, device="cuda")
+    m.mdsip_ldlt_factor(ctx, N, S, N, 1e-14, L, Dd, Doff, perm, kd, inr)
+    torch.cuda.synchronize()
+    assert int((kd == 2).sum()) == len(spots)
+    assert m.mdsip_ldlt_panel_counts(ctx)[1] == len(spots)
+    m.mdsip_ldlt_factor(ctx, N, dev(np.tril(K * 2.0 ** -950).T.copy()), N, 1e-14, L, Dd, Doff, perm, kd, inr)
+    torch.cuda.synchronize()
+    assert m.mdsip_ldlt_panel_counts(ctx) == (0, 1)   # below the persistent kernel's range: handed over whole
