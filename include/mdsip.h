@@ -315,6 +315,19 @@ int64_t mdsip_launch_count(void);
  * blocks <= 0, iters <= 0 or sink == NULL: INVALID_ARG. */
 mdsip_status mdsip_probe_fp64_fma(mdsip_ctx *ctx, int32_t blocks, int64_t iters, double *sink);
 
+/* For tests: the scalar pieces that the kernels use in place of the division
+ * operator, log and square root, element by element (device pointers).
+ *   RCP:    out[i] = 1 / a[i] (0 for a zero)          within 0.51 units in the last place
+ *   DIV:    out[i] = a[i] / b[i]                      within 0.51
+ *   LOGSUM: out[i] = sum of log a[16 i .. 16 i + 15]
+ *   ADAM:   lr m / (sqrt(v) + eps) of the moments decayed from a[i], b[i] as FP32
+ *           (lr 1e-3, eps 1e-8, the second step's bias corrections): out[2 i] the
+ *           branch-free form (NaN outside its range), out[2 i + 1] the operators
+ *   RSQRT:  a[i]^-1/2 = (out[3 i] 2^32 + out[3 i + 1]) 2^(out[3 i + 2] - 63)
+ * Returns once the launch is enqueued. */
+enum { MDSIP_SCALAR_RCP = 0, MDSIP_SCALAR_DIV = 1, MDSIP_SCALAR_LOGSUM = 2, MDSIP_SCALAR_ADAM = 3, MDSIP_SCALAR_RSQRT = 4 };
+mdsip_status mdsip_debug_scalar(mdsip_ctx *ctx, int32_t op, int64_t n, const double *a, const double *b, double *out);
+
 /* ------------------------------------------------------------------------- */
 /* Kernel-level entry points (device pointers, context stream).              */
 /* ------------------------------------------------------------------------- */

@@ -121,6 +121,7 @@ _SIGS = {
     "mdsip_launch_count": (C.c_int64, []),
     "mdsip_syrk_scaled": (C.c_int, [C.c_void_p, C.c_int64, C.c_int64, C.c_void_p, C.c_int64,
                                     C.c_void_p, C.c_double, C.c_void_p, C.c_int64]),
+    "mdsip_debug_scalar": (C.c_int, [C.c_void_p, C.c_int32, C.c_int64, C.c_void_p, C.c_void_p, C.c_void_p]),
     "mdsip_debug_expire_wait": (C.c_int, [C.c_void_p]),
     "mdsip_syrk_scaled_tc": (C.c_int, [C.c_void_p, C.c_int64, C.c_int64, C.c_void_p, C.c_int64,
                                        C.c_void_p, C.c_double, C.c_void_p, C.c_int64, C.c_int]),
@@ -405,6 +406,10 @@ def mdsip_launch_count() -> int:
 
 def mdsip_syrk_scaled(ctx, m, n, A, lda, w, beta, Cmat, ldc):
     _check(lib().mdsip_syrk_scaled(ctx, m, n, _ptr(A), lda, _ptr(w), float(beta), _ptr(Cmat), ldc), ctx)
+
+
+def mdsip_debug_scalar(ctx, op, n, a, b, out):
+    _check(lib().mdsip_debug_scalar(ctx, int(op), int(n), _ptr(a), _ptr(b), _ptr(out)), ctx)
 
 
 def mdsip_debug_expire_wait(ctx):

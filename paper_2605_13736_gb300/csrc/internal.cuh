@@ -517,6 +517,8 @@ struct PerDeviceOnce {
 // probe.cu: blocks x 256 threads, each iters x 8 independent FP64 FMAs; sink
 // holds blocks x 256 doubles
 void launch_fp64_fma_probe(cudaStream_t s, int blocks, int64_t iters, double *sink);
+// as mdsip_debug_scalar
+void launch_scalar(cudaStream_t s, int op, int64_t n, const double *a, const double *b, double *out);
 
 // A passes (row-major A, m x n, leading dimension lda)
 void launch_gemv_rows(cudaStream_t s, const double *A, int64_t m, int64_t n, int64_t lda,

@@ -1938,6 +1938,19 @@ mdsip_status mdsip_probe_fp64_fma(mdsip_ctx *hctx, int32_t blocks, int64_t iters
     });
 }
 
+mdsip_status mdsip_debug_scalar(mdsip_ctx *hctx, int32_t op, int64_t n, const double *a, const double *b, double *out) {
+    if (!hctx) return MDSIP_ERR_INVALID_ARG;
+    Ctx *ctx = C_(hctx);
+    return guarded(ctx, [&] {
+        DeviceGuard g(ctx->device);
+        MDSIP_REQUIRE(op >= MDSIP_SCALAR_RCP && op <= MDSIP_SCALAR_RSQRT && n >= 0 && n < (1LL << 30),
+                      MDSIP_ERR_INVALID_ARG, "scalar: bad operation or count");
+        const bool two = op == MDSIP_SCALAR_DIV || op == MDSIP_SCALAR_ADAM;
+        MDSIP_REQUIRE(n == 0 || (a && out && (b || !two)), MDSIP_ERR_INVALID_ARG, "scalar: null pointer");
+        if (n > 0) launch_scalar(ctx->stream, op, n, a, b, out);
+    });
+}
+
 mdsip_status mdsip_syrk_scaled(mdsip_ctx *hctx, int64_t m, int64_t n, const double *A, int64_t lda,
                                const double *w, double beta, double *C, int64_t ldc) {
     if (!hctx) return MDSIP_ERR_INVALID_ARG;

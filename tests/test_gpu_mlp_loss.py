@@ -28,3 +28,23 @@ def test_loss_is_an_fp64_sum(batch, n_out, seed):
     finally:
         m.mdsip_mlp_destroy(mlp)
         m.mdsip_ctx_destroy(ctx)
+
+
+def test_a_step_on_overflowing_moments():
+    """Gradients so large that the second moment overflows move nothing: m / inf."""
+    torch = torch_cuda()
+    ctx = make_ctx()
+    mlp = m.mdsip_mlp_create(ctx, 8, 16, 200)
+    try:
+        n = m.mdsip_mlp_num_params(mlp)
+        P = torch.zeros(n, device="cuda")
+        m.mdsip_mlp_set_params(mlp, P, m.MDSIP_MEM_DEVICE, ctx)
+        X = torch.zeros(4, 8, dtype=torch.float64, device="cuda")
+        Y = torch.full((4, 200), 1e22, dtype=torch.float64, device="cuda")
+        for _ in range(3):                      # db3 = -1e20: v = 1e37, v / (1 - beta2^t) = inf
+            m.mdsip_mlp_train_step(mlp, X, 8, Y, 200, None, 4, 1e-3, ctx=ctx)
+        m.mdsip_mlp_get_params(mlp, P, m.MDSIP_MEM_DEVICE, ctx)
+        assert bool(torch.isfinite(P).all())
+    finally:
+        m.mdsip_mlp_destroy(mlp)
+        m.mdsip_ctx_destroy(ctx)
