@@ -75,7 +75,13 @@ __device__ __forceinline__ void rsqrt64(double v, unsigned long long &sm, int &s
     const unsigned long long mant =
         (((unsigned long long)__double_as_longlong(s) & 0xfffffffffffffULL) | 0x10000000000000ULL) << 11;
     const double cd = ldexp(0.5 * s * r, 63 - se);
-    sm = mant + (unsigned long long)__double2ll_rn(fmin(fmax(cd, -2047.0), 2047.0));
+    // (s is a rounded root's rounded reciprocal: up to 1.5 units, 3072 of cd, off)
+    const long long c = __double2ll_rn(cd);
+    sm = mant + (unsigned long long)c;
+    if (c > 0 && sm < mant) {              // past 2^64
+        sm = (sm >> 1) | (1ULL << 63);
+        ++se;
+    }
 }
 
 // |X| for X = rint(a s 2^(b - E)), s = sm 2^(se - 63), given that |a s| < 2^E; 0

@@ -134,3 +134,12 @@ def test_adam_quotient(ctx):
     assert np.isnan(far[:, 0]).all() and np.isfinite(far[:, 1]).all()
     assert far[2, 1] == 0.0                     # v / (1 - beta2^t) overflows: no step, as with the operators
 
+@needs_quad
+@pytest.mark.parametrize("lo,hi", [(30, 2010), (1022, 1024)])
+def test_reciprocal_root(ctx, lo, hi):
+    w = np.abs(_doubles(np.random.default_rng(hi), 200000, lo, hi))
+    out = _run(ctx, RSQRT, w, per=3).reshape(-1, 3)
+    got = np.ldexp(out[:, 0].astype(LD) * LD(2.0) ** 32 + out[:, 1].astype(LD), out[:, 2].astype(int) - 63)
+    want = 1 / np.sqrt(w.astype(LD))
+    # 64 bits, one Newton correction of a value good to 2^-52: 2^-62 from the integer, 2^-63 beside it
+    assert (np.abs(got / want - 1) <= LD(2.0) ** -61).all(), float(np.abs(got / want - 1).max() * LD(2.0) ** 61)
