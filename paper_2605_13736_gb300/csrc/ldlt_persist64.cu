@@ -209,10 +209,11 @@ __device__ __forceinline__ void q_colmax(unsigned long long bm, unsigned long lo
 // whether the rule keeps a diagonal pivot d against the column's maximum.  (A pivot
 // below 2^-1000 has no scaling |d|^-1/2 in the integer form: its panel goes to the
 // pivoting kernel, as one that needs an interchange.)
-__device__ __forceinline__ bool q_keeps(double d, double colmax, double ztol) {
+__device__ __forceinline__ bool q_keeps(double d, double colmax, unsigned long long zbits) {
     const double alpha = 0.6403882032022076;   // (1 + sqrt 17) / 8
-    return absbits64(d) >= absbits64(alpha * colmax) && fabs(d) > fmax(ztol, 0x1p-1000) && isfinite(d) &&
-           isfinite(colmax);
+    constexpr unsigned long long kInf = 0x7ff0000000000000ULL;
+    const unsigned long long bd = absbits64(d);
+    return bd >= absbits64(alpha * colmax) && bd > zbits && bd < kInf && absbits64(colmax) < kInf;
 }
 
 // the panel loop takes over at st->k
@@ -408,7 +409,8 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
     __shared__ uint32_t s_tmem;
     const int N = a.N, G = (int)gridDim.x, g = (int)blockIdx.x, tid = threadIdx.x;
     const int lane = tid & 31, wid = tid >> 5;
-    const double maxabs = __ldg(a.maxabs), ztol = a.zero_tol * maxabs;
+    const double maxabs = __ldg(a.maxabs);
+    const unsigned long long zbits = absbits64(fmax(a.zero_tol * maxabs, 0x1p-1000));
     // entries near the subnormal range would lose bits in the integer form: the
     // pivoting panels take such a matrix (st->k stays where it is)
     if (!(maxabs > 0x1p-900)) {
@@ -431,7 +433,7 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
         q_colmax(bm, &s_cmax[0], lane);
         __syncthreads();
         const double d = __ldcg(col), colmax = __longlong_as_double((long long)s_cmax[0]);
-        if (!q_keeps(d, colmax, ztol)) {
+        if (!q_keeps(d, colmax, zbits)) {
             if (g == 0 && tid == 0) q_hand_over(a.st);
             return;
         }
@@ -596,7 +598,7 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
         {
             int keep = 1;
             if (tid < nb)
-                keep = q_keeps(s_d[tid], __longlong_as_double((long long)__ldcg(&a.cmax[buf * 64 + tid])), ztol);
+                keep = q_keeps(s_d[tid], __longlong_as_double((long long)__ldcg(&a.cmax[buf * 64 + tid])), zbits);
             if (!__syncthreads_and(keep)) {
                 if (g == 0 && tid == 0) q_hand_over(a.st);   // st->k is this panel's first column
                 break;

@@ -37,9 +37,9 @@
 // FP32 arithmetic only: one FP64 instruction per entry costs as much as 64
 // FP32 ones); (4) k_rns_mma; (5) k_rns_combine.  Entries the integer form does
 // not cover (non-finite or subnormal entries of A; w not positive, finite and
-// within 2^+-1000; columns of too wide a spread) raise a device flag in (1) or
-// (2); the later passes then do nothing and the DFMA kernel, gated on the same
-// flag, forms the product.
+// within 2^+-1000; columns of too wide a spread) raise a device flag in (1), (2)
+// or, for the spread in any chunk, the first chunk's (3); the later passes then do
+// nothing and the DFMA kernel, gated on the same flag, forms the product.
 #include <cuda.h>
 
 #include <algorithm>
@@ -86,10 +86,9 @@ __host__ __device__ inline int rns_tiles(int64_t n) {
 
 constexpr int kMeanGap = 9;            // binary orders (see above)
 
-// of the columns of every chunk: exponent bound, sum and count of the exponents;
-// of every 64 of them: strips done
+// of the columns of every chunk: exponent bound, sum and count of the exponents
 struct ColStat {
-    int *E, *sum, *cnt, *done;
+    int *E, *sum, *cnt;
 };
 
 // w_i^-1/2 = sm[i] 2^(se[i] - 63)
@@ -108,10 +107,8 @@ __global__ void k_rns_rows(int64_t m, const double *__restrict__ w, unsigned lon
 // col[chunk][q]: E = 2 + max_i (exponent of A[i][q] + se[i]) over the chunk's
 // rows, |a s| < 2^E, and the sum and count of the exponents of its nonzero
 // entries.  32 x 8 threads, 64 columns and `strip` rows per block, strips of 512
-// rows where that leaves blocks enough (fewer atomics and tickets); HBM-bound
-// (one read of A).  The sums, counts and tickets cost 8 of 646 us at m = 30011, n =
-// 771 and 35 us of 6.9 ms at m = 100000, n = 2000; a look at the spread inside
-// k_rns_residues took that kernel from 64 to 104 registers and 370 us more there.
+// rows where that leaves blocks enough (fewer atomics); HBM-bound (one read of A; m =
+// 100000, n = 2000: 264 us, 255 with the maximum alone).
 __global__ void __launch_bounds__(256) k_rns_colmax(const double *__restrict__ A, int64_t m, int64_t n, int64_t lda,
                                                     int64_t kc, int strip, int strips_per_chunk,
                                                     const int *__restrict__ se, ColStat col_stat,
@@ -125,14 +122,15 @@ __global__ void __launch_bounds__(256) k_rns_colmax(const double *__restrict__ A
     // the nonzero entries (at most 64 rows: the count above the sum, no carry)
     constexpr unsigned kOne = 1u << 18, kOff = 1024u;
     unsigned m0 = 0, m1 = 0, a0 = 0, a1 = 0;
-    bool bad = false;
+    unsigned bad = 0;
     auto upd = [&](double v, unsigned s, unsigned &mx, unsigned &acc) {
-        const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
-        const unsigned ef = (hi >> 20) & 0x7ffu;
-        const unsigned x = ef != 0u ? ef + s : 0u;
-        mx = max(mx, x);
-        acc += x;
-        bad |= ef == 0x7ffu || (ef == 0u && ((hi & 0xfffffu) | lo) != 0u);
+        const unsigned h = (unsigned)__double2hiint(v) << 1, lo = (unsigned)__double2loint(v);
+        if (h - 0x200000u < 0xffc00000u) {   // a normal number
+            mx = __viaddmax_u32(h >> 21, s, mx);
+            acc += (h >> 21) + s;
+        } else {
+            bad |= h | lo;                   // zeros pass
+        }
     };
     if (col < n) {
         const bool two = col + 1 < n;
@@ -145,7 +143,7 @@ __global__ void __launch_bounds__(256) k_rns_colmax(const double *__restrict__ A
             if (two) upd(v.y, s, m1, a1);
         }
     }
-    if (bad) atomicExch(flag, 1);
+    if (bad != 0u) atomicExch(flag, 1);
     auto put = [&](int c, unsigned mx, unsigned acc) {
         const int cnt = (int)(acc / kOne);
         red[0][threadIdx.y][c] = mx ? (int)(mx % kOne) - (int)kOff : INT_MIN;
@@ -166,28 +164,21 @@ __global__ void __launch_bounds__(256) k_rns_colmax(const double *__restrict__ A
             if (what == 2 && r != 0) atomicAdd(col_stat.cnt + o, r);
         }
     }
-    // the last of a chunk's strips looks at the spread of its columns
-    __shared__ bool s_last;
-    __threadfence();
-    __syncthreads();
-    if (t == 0)
-        s_last = atomicAdd(col_stat.done + chunk * gridDim.x + blockIdx.x, 1) == strips_per_chunk - 1;
-    __syncthreads();
-    const int64_t q = (int64_t)blockIdx.x * 64 + t, o = chunk * n + q;
-    if (s_last && t < 64 && q < n) {
-        __threadfence();
-        const int64_t cnt = __ldcg(col_stat.cnt + o);
-        if (cnt > 0 && cnt * (__ldcg(col_stat.E + o) + 1023 - 2 - kMeanGap) > (int64_t)__ldcg(col_stat.sum + o))
-            atomicExch(flag, 1);
-    }
 }
 
-__global__ void k_rns_init(int64_t cnt, int64_t blocks, ColStat col_stat) {
+__global__ void k_rns_init(int64_t cnt, ColStat col_stat) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (int64_t)gridDim.x * blockDim.x) {
         col_stat.E[i] = INT_MIN;
         col_stat.sum[i] = col_stat.cnt[i] = 0;
-        if (i < blocks) col_stat.done[i] = 0;
     }
+}
+
+// Raises the flag where a column's spread is too wide.  Out of line: inside the
+// kernel below it took that from 64 to 104 registers.
+__device__ __noinline__ void rns_spread(ColStat cols, int64_t cnt, int *flag) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (int64_t)gridDim.x * blockDim.x)
+        if (cols.cnt[i] > 0 && (int64_t)cols.cnt[i] * (cols.E[i] + 1023 - 2 - kMeanGap) > (int64_t)cols.sum[i])
+            atomicExch(flag, 1);
 }
 
 // R[l][k][q] = BF16 of X mod p_l, X = rint(A[i0 + k][q] s_(i0+k) 2^(b - colE[q])),
@@ -201,8 +192,9 @@ __global__ void __launch_bounds__(256) k_rns_residues(const double *__restrict__
                                                       int rows, int kpad, int ldn, int b,
                                                       const unsigned long long *__restrict__ sm,
                                                       const int *__restrict__ se, const int *__restrict__ colE,
-                                                      uint4 *__restrict__ R, const int *__restrict__ flag) {
-    if (*flag) return;
+                                                      uint4 *__restrict__ R, int *flag, ColStat all, int64_t check) {
+    if (*(volatile int *)flag) return;
+    if (check) rns_spread(all, check, flag);
     const int groups = ldn / 8;
     const int64_t total = (int64_t)kpad * groups;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
@@ -568,7 +560,7 @@ bool syrk_rns_pays(int64_t m, int64_t n) {
 
 size_t syrk_rns_workspace_bytes(int64_t m, int64_t n, int num_sms, size_t cap) {
     const RnsPlan pl = rns_plan(m, n, num_sms, cap);
-    return 1024 + al1k((size_t)m * 8) + al1k((size_t)m * 4) + 4 * al1k((size_t)pl.chunks * n * 4) +
+    return 1024 + al1k((size_t)m * 8) + al1k((size_t)m * 4) + 3 * al1k((size_t)pl.chunks * n * 4) +
            al1k((size_t)RN * pl.kc * pl.ldn * 2) +
            al1k((size_t)RN * pl.nsplit * pl.group * T_M * T_N * sizeof(int16_t));
 }
@@ -587,7 +579,7 @@ const int *launch_syrk_rns(cudaStream_t st, int num_sms, const double *A, int64_
     int *se = reinterpret_cast<int *>(base);
     base += al1k((size_t)m * 4);
     ColStat cols{};
-    for (int **v : {&cols.E, &cols.sum, &cols.cnt, &cols.done}) {
+    for (int **v : {&cols.E, &cols.sum, &cols.cnt}) {
         *v = reinterpret_cast<int *>(base);
         base += al1k((size_t)pl.chunks * n * 4);
     }
@@ -598,8 +590,7 @@ const int *launch_syrk_rns(cudaStream_t st, int num_sms, const double *A, int64_
 
     MDSIP_CUDA(cudaMemsetAsync(flag, 0, 2 * sizeof(int), st));
     if (expire) MDSIP_CUDA(cudaMemsetAsync(err, 1, sizeof(int), st));
-    k_rns_init<<<std::max(1, std::min(1024, ceil_div(pl.chunks * n, 256))), 256, 0, st>>>(
-        pl.chunks * n, pl.chunks * ceil_div(n, 64), cols);
+    k_rns_init<<<std::max(1, std::min(1024, ceil_div(pl.chunks * n, 256))), 256, 0, st>>>(pl.chunks * n, cols);
     MDSIP_LAUNCHED();
     k_rns_rows<<<std::max(1, std::min(4096, ceil_div(m, 256))), 256, 0, st>>>(m, w, sm, se, flag);
     MDSIP_LAUNCHED();
@@ -621,7 +612,7 @@ const int *launch_syrk_rns(cudaStream_t st, int num_sms, const double *A, int64_
         const int b = std::min(56, (kModBits - 2 - ceil_log2(rows)) / 2);   // |sum| <= rows 2^(2b) < M / 4
         const int64_t total = (int64_t)kpad * (pl.ldn / 8);
         k_rns_residues<<<(int)std::min<int64_t>((int64_t)num_sms * 32, (total + 255) / 256), 256, 0, st>>>(
-            A, lda, n, i0, rows, kpad, (int)pl.ldn, b, sm, se, colE + c * n, R, flag);
+            A, lda, n, i0, rows, kpad, (int)pl.ldn, b, sm, se, colE + c * n, R, flag, cols, c == 0 ? pl.chunks * n : 0);
         MDSIP_LAUNCHED();
         CUtensorMap rmap;
         tc::encode_2d(&rmap, R, false, (uint64_t)pl.ldn, (uint64_t)RN * kpad, (uint64_t)pl.ldn, 64, SLAB);
