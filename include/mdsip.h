@@ -388,7 +388,7 @@ mdsip_status mdsip_syrk_scaled_tc(mdsip_ctx *ctx, int64_t m, int64_t n, const do
 mdsip_status mdsip_gemv_pair_df(mdsip_ctx *ctx, int64_t m, int64_t n, const double *A, int64_t lda,
                                 const double *x, const double *v, double *Ax, double *ATv);
 
-/* The same pass with the first half of the refinement's next approximate
+/* The same pass with the first half of a refinement's next approximate
  * solve folded in (the FP32 A^T product of the two-stage elimination of
  * Section 2.3, whose input needs the whole row sum of A x).  Besides Ax and
  * ATv as in mdsip_gemv_pair_df it writes

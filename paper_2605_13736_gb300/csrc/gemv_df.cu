@@ -167,8 +167,9 @@ __global__ void __launch_bounds__(NT) k_gemv_t_df(const float *__restrict__ Ahi,
 // needs the warps for its dependent chains); the per-thread row sums of a
 // batch are reduced over the block as double-float pairs (warp shuffles,
 // then one slot per warp).  Waits are bounded: on expiry the kernel sets
-// *err and stops.  The fused form (kFuse, one slice) also takes the first
-// half of the refinement's next approximate solve: each finished row sum
+// *err and stops.  The fused form (kFuse, one slice), which only the entry
+// mdsip_gemv_pair_df_next runs (the solver's refinement has whole sweeps in one
+// pass, refine_sweep.cu), also takes the first half of the next approximate solve: each finished row sum
 // gives v_i (BothNext), and A_hi^T v accumulates in FP32 one batch behind,
 // from the previous batch's A_hi chunk kept in registers (its stage is
 // already being refilled), so the batch keeps its single barrier.

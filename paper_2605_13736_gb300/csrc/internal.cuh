@@ -536,7 +536,8 @@ void launch_gemv_t_df(cudaStream_t s, const float *Ahi, const float *Alo, int64_
 // out_rows = A x and out_cols = A^T y from one read of A.  With nx, the same
 // read also gives out_v = A_hi^T v, v_i = fl32((cpre_i - (A x)_i) wf_i) with
 // the difference in double-float (FP32 products and sums): the first half of
-// the refinement's next approximate solve.  cw = cpre as FP32 halves
+// a refinement's next approximate solve (mdsip_gemv_pair_df_next; the solver's own
+// sweeps are in refine_sweep.cu).  cw = cpre as FP32 halves
 // (launch_split_vector), wf = fl32(1 / w) (launch_round_vector).  The fused
 // form needs the whole row in one slice: gemv_both_fusable(n).
 struct BothNextArgs {

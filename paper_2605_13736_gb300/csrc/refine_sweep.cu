@@ -34,6 +34,7 @@ constexpr int NT = kRedThreads;
 constexpr int kSwC = 512;                     // column threads: 16 warps
 constexpr int kSwThreads = 640;               // 20 warps, five a sub-partition: 96 registers a thread
 constexpr int kSwMaxSlots = 12;
+constexpr int KBR = 2;                        // rows of a group in a batch
 constexpr size_t kSwSmem = 224 * 1024;        // batches in flight or in use
 constexpr size_t kSwMin = 48 * 1024;          // the groups' column sums meet in the ring at the end
 
@@ -90,10 +91,10 @@ __device__ __forceinline__ float2 split64(double v) {
 // 358 us, with four columns and three batches of lag (whose row and column
 // parts interleave) 385, summing the rows in the finishing warps 377; m =
 // 200000, n = 4000 1360 us, with one row a batch 1770.
-template <int CH, int KBR, int kLag>
+template <int CH, int kLag>
 __global__ void __launch_bounds__(kSwThreads, 1) k_sweep(SweepArgs a) {
     extern __shared__ __align__(128) unsigned char sw_smem[];
-    constexpr int kVals = KBR * 16;            // (row, warp) sums of a batch
+    constexpr int kVals = KBR * 16;            // (row, warp) sums of a batch: one a lane of the finishing warp
     __shared__ float4 s_y[3][kVals];
     __shared__ float2 s_red[3][kVals];
     __shared__ float s_red2[3][kVals];
@@ -239,26 +240,24 @@ __global__ void __launch_bounds__(kSwThreads, 1) k_sweep(SweepArgs a) {
                 }
                 if (++rslot == S) rslot = 0, rph ^= 1;
                 float s = rs[0], c = rc[0], d = r2[0];
-                int row = g * KBR;
-                if constexpr (KBR == 2) {
-                    const bool up = (lane & 16) != 0;
-                    float es = up ? s : rs[1], ec = up ? c : rc[1], ed = up ? d : r2[1];
-                    s = up ? rs[1] : s;
-                    c = up ? rc[1] : c;
-                    d = up ? r2[1] : d;
-                    es = __shfl_xor_sync(0xffffffffu, es, 16);
-                    ec = __shfl_xor_sync(0xffffffffu, ec, 16);
-                    d += __shfl_xor_sync(0xffffffffu, ed, 16);
-                    df_add(s, c, es, ec);
-                    row += up ? 1 : 0;
-                }
+                const bool up = (lane & 16) != 0;
+                const int row = g * KBR + (up ? 1 : 0);
+                float es = up ? s : rs[1], ec = up ? c : rc[1], ed = up ? d : r2[1];
+                s = up ? rs[1] : s;
+                c = up ? rc[1] : c;
+                d = up ? r2[1] : d;
+                es = __shfl_xor_sync(0xffffffffu, es, 16);
+                ec = __shfl_xor_sync(0xffffffffu, ec, 16);
+                d += __shfl_xor_sync(0xffffffffu, ed, 16);
+                df_add(s, c, es, ec);
 #pragma unroll
-                for (int o = KBR == 2 ? 8 : 16; o > 0; o >>= 1) {
-                    const float es = __shfl_xor_sync(0xffffffffu, s, o), ec = __shfl_xor_sync(0xffffffffu, c, o);
+                for (int o = 8; o > 0; o >>= 1) {
+                    es = __shfl_xor_sync(0xffffffffu, s, o);
+                    ec = __shfl_xor_sync(0xffffffffu, c, o);
                     d += __shfl_xor_sync(0xffffffffu, d, o);
                     df_add(s, c, es, ec);
                 }
-                if ((lane & (KBR == 2 ? 15 : 31)) == 0) {
+                if ((lane & 15) == 0) {
                     s_red[rb][row * W + (t >> 5)] = make_float2(s, c);
                     s_red2[rb][row * W + (t >> 5)] = d;
                 }
@@ -365,18 +364,19 @@ __global__ void __launch_bounds__(kSwThreads, 1) k_sweep(SweepArgs a) {
     } else {
         // ---- finishing warps: lane = (row, warp sum)
         const int me = wid - 17, rho = lane / W, sub = lane - rho * W;
-        const bool mine = lane < kVals, lead = mine && sub == 0;
+        static_assert(kVals == 32, "a lane a sum");
+        const bool lead = sub == 0;
         uint32_t ph = 0;
         int e0 = 0, e1 = 0;
         auto rows_entries = [&](int b) {   // the row's entries, loaded a turn ahead
             const int x = b * RB + rho;
-            const bool live = mine && x < nrow && b < nbat;
+            const bool live = x < nrow && b < nbat;
             e0 = live ? __ldg(a.csr_ptr + r0 + x) : 0;
             e1 = live ? __ldg(a.csr_ptr + r0 + x + 1) : 0;
         };
         rows_entries(me);
         for (int b = me; b < nbat; b += 3) {
-            const bool live = mine && b * RB + rho < nrow;
+            const bool live = b * RB + rho < nrow;
             const int64_t i = r0 + b * RB + rho;
             double ug = 0.0, bt = 0.0, winv = 0.0, bg = 0.0;
             float wf = 0.0f;
@@ -404,7 +404,7 @@ __global__ void __launch_bounds__(kSwThreads, 1) k_sweep(SweepArgs a) {
             ok = __all_sync(0xffffffffu, tc::mbar_wait(&rowdone[me], ph));
             if (!ok) break;
             ph ^= 1;
-            float s = mine ? s_red[me][lane].x : 0.0f, c = mine ? s_red[me][lane].y : 0.0f, d = mine ? s_red2[me][lane] : 0.0f;
+            float s = s_red[me][lane].x, c = s_red[me][lane].y, d = s_red2[me][lane];
             for (int o = 1; o < W; o <<= 1) {
                 const float es = __shfl_xor_sync(0xffffffffu, s, o), ec = __shfl_xor_sync(0xffffffffu, c, o);
                 d += __shfl_xor_sync(0xffffffffu, d, o);
@@ -606,7 +606,7 @@ struct SweepParts {
     const float *pv;
 };
 
-template <int CH, int KBR, int kLag>
+template <int CH, int kLag>
 SweepParts launch_sweep_t(cudaStream_t st, int num_sms, SweepArgs a) {
     a.T = 32;
     while (a.T < kSwC && 4 * CH * a.T < a.n) a.T *= 2;
@@ -621,9 +621,9 @@ SweepParts launch_sweep_t(cudaStream_t st, int num_sms, SweepArgs a) {
     a.pv = reinterpret_cast<float *>(a.pu + grid * groups * a.n);
     static PerDeviceOnce once;
     MDSIP_CUDA(once.run([] {
-        return cudaFuncSetAttribute(k_sweep<CH, KBR, kLag>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSwSmem);
+        return cudaFuncSetAttribute(k_sweep<CH, kLag>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSwSmem);
     }));
-    k_sweep<CH, KBR, kLag><<<grid, kSwThreads, std::max(kSwMin, a.S * slot), st>>>(a);
+    k_sweep<CH, kLag><<<grid, kSwThreads, std::max(kSwMin, a.S * slot), st>>>(a);
     MDSIP_LAUNCHED();
     return SweepParts{grid, (int)groups, a.pv};
 }
@@ -680,7 +680,7 @@ void Refiner::sweep(const double *b, double *u, double *r, bool init, double dw,
     a.pu = colpart;
     a.err = solve_err;
     // up to 128 columns a warp of four columns a thread holds a row; wider rows go by eight
-    const SweepParts pt = D.n_d <= 128 ? launch_sweep_t<1, 2, 3>(st, num_sms, a) : launch_sweep_t<2, 2, 1>(st, num_sms, a);
+    const SweepParts pt = D.n_d <= 128 ? launch_sweep_t<1, 3>(st, num_sms, a) : launch_sweep_t<2, 1>(st, num_sms, a);
     k_sweep_residual<<<red_grid(std::max(std::max(D.n_s, D.m_E), 32 * D.n_d)), NT, 0, st>>>(
         D, M, b, u, r, q, qinv, sig_xd, sig_d, Jdh, tmp_m, sol_g, tmp_nd2, xnew, colpart,
         pt.pv, pt.n, pt.step, init ? 1 : 0, dw, dc, tmp_nd, rhsS,
