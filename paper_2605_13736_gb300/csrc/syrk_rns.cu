@@ -106,9 +106,8 @@ __global__ void k_rns_rows(int64_t m, const double *__restrict__ w, unsigned lon
 
 // col[chunk][q]: E = 2 + max_i (exponent of A[i][q] + se[i]) over the chunk's
 // rows, |a s| < 2^E, and the sum and count of the exponents of its nonzero
-// entries.  32 x 8 threads, 64 columns and `strip` rows per block, strips of 512
-// rows where that leaves blocks enough (fewer atomics); HBM-bound (one read of A; m =
-// 100000, n = 2000: 264 us, 255 with the maximum alone).
+// entries.  32 x 8 threads, 64 columns and `strip` rows per block; HBM-bound (one
+// read of A; m = 100000, n = 2000: 269 us, 255 with the maximum alone).
 __global__ void __launch_bounds__(256) k_rns_colmax(const double *__restrict__ A, int64_t m, int64_t n, int64_t lda,
                                                     int64_t kc, int strip, int strips_per_chunk,
                                                     const int *__restrict__ se, ColStat col_stat,
@@ -119,7 +118,7 @@ __global__ void __launch_bounds__(256) k_rns_colmax(const double *__restrict__ A
     const int64_t i0 = chunk * kc + (int64_t)(blockIdx.y % strips_per_chunk) * strip;
     const int64_t i1 = min(m, min(i0 + strip, (chunk + 1) * kc));
     // per column and thread: the largest and the sum of kOne + (exponent + kOff) over
-    // the nonzero entries (at most 64 rows: the count above the sum, no carry)
+    // the nonzero entries (at most 32 rows: the count above the sum, no carry)
     constexpr unsigned kOne = 1u << 18, kOff = 1024u;
     unsigned m0 = 0, m1 = 0, a0 = 0, a1 = 0;
     unsigned bad = 0;
@@ -193,7 +192,7 @@ __global__ void __launch_bounds__(256) k_rns_residues(const double *__restrict__
                                                       const unsigned long long *__restrict__ sm,
                                                       const int *__restrict__ se, const int *__restrict__ colE,
                                                       uint4 *__restrict__ R, int *flag, ColStat all, int64_t check) {
-    if (*(volatile int *)flag) return;
+    if (*flag) return;
     if (check) rns_spread(all, check, flag);
     const int groups = ldn / 8;
     const int64_t total = (int64_t)kpad * groups;
@@ -594,8 +593,7 @@ const int *launch_syrk_rns(cudaStream_t st, int num_sms, const double *A, int64_
     MDSIP_LAUNCHED();
     k_rns_rows<<<std::max(1, std::min(4096, ceil_div(m, 256))), 256, 0, st>>>(m, w, sm, se, flag);
     MDSIP_LAUNCHED();
-    const int strip = pl.chunks * ceil_div(n, 64) * ceil_div(pl.kc, 256) >= 8 * num_sms ? 512 : 256;
-    const int spc = (int)((pl.kc + strip - 1) / strip);
+    const int strip = 256, spc = (int)((pl.kc + strip - 1) / strip);
     MDSIP_REQUIRE(pl.chunks * spc <= 65535, MDSIP_ERR_INVALID_ARG, "syrk: m too large");
     const dim3 cg((unsigned)ceil_div(n, 64), (unsigned)(pl.chunks * spc));
     k_rns_colmax<<<cg, dim3(32, 8), 0, st>>>(A, m, n, lda, pl.kc, strip, spc, se, cols, flag);
