@@ -881,7 +881,8 @@ def run_gpu(args):
     syrk_ms = acc["t_syrk_ms"] / max(1, acc["n_syrk"])
     fp64_rate = flops / (syrk_ms / 1e3) / 1e12 if acc["n_syrk"] else None
     bf16_peak = measured_peak("bf16_tflops")
-    rns = D["m_E"] >= 256 and D["m_E"] * D["n_d"] ** 2 >= 3e7   # large enough for the tensor-core form
+    # large enough for the tensor-core form (syrk_rns_pays in syrk_rns.cu)
+    rns = D["m_E"] >= 256 and D["m_E"] * D["n_d"] ** 2 >= (1.5e7 if D["n_d"] > 64 else 3e7)
     achieved = SYRK_MODULI * fp64_rate if (fp64_rate and rns) else fp64_rate
     prod_peak = bf16_peak if rns else FP64_PEAK_TFLOPS
     roofline = {"kernel": ("k_rns_rows/colmax/residues/mma/combine (A^T W^-1 A in FP64 by exact BF16 tensor products "

@@ -22,7 +22,11 @@
 //      tensor-core contractions per 128 x 32 tile (bulk copies, tcgen05 into TMEM, the
 //      Chinese remainder in 128-bit integers on 16 warps, one rounding to FP64, one FP64
 //      subtraction per entry): sum_j sign(d_j) X_ij X_cj <= 32 2^108 in exact
-//      integers, an error below that of a 32-term FP64 dot product; grid barrier.
+//      integers.  An X is off by at most 2^-53 of its row's largest in the panel, an
+//      entry's update by 2^-53 (max|x_i| sum|x_c| + max|x_c| sum|x_i|), at most 2^-49
+//      sqrt(b_i b_c) with b_i = sum_j w_ij^2 / |d_j| (a 32-term FP64 dot product by
+//      2^-48 sum_j |x_ij x_cj|): the scale of the factorization's other roundings, not
+//      entry-wise; grid barrier.
 // Against the 64-column form with DFMA trailing tiles (its first panel's tiles
 // alone took 215 us): N = 2050 7.90 -> 2.42 ms, 4050 30.6 -> 8.1 ms.  A panel
 // takes 30 us at N = 351 to 1036, its pivot chain about 12 of them (32 columns

@@ -22,7 +22,7 @@ struct Tab {
     float inv[RN];                     // (M / p)^-1 mod p, symmetric
     // moduli taken in pairs (a last one alone): sum_l y_l M/p_l is the sum over
     // pairs of z M/(p q), z = y_p q + y_q p, |z| < 2^19
-    uint32_t mpair32[(RN + 1) / 2][4], mod32[4], bias32[4];   // M/(p q), M, 2^19 sum of M/(p q), 32-bit limbs
+    uint32_t mpair32[(RN + 1) / 2][4], mod32[4], bias32[4];   // M/(p q), M, 2^19 sum of M/(p q) modulo 2^128, 32-bit limbs
     float top, btop;                   // 2^96 / M; bias / M
 };
 
@@ -36,6 +36,7 @@ template <int RN>
 constexpr Tab<RN> make_tab() {
     Tab<RN> t{};
     unsigned __int128 M = 1, bias = 0;
+    double bias_M = 0.0;
     for (int l = 0; l < RN; ++l) M *= (unsigned)kModuli[l];
     for (int l = 0; l < RN; ++l) {
         const int p = kModuli[l];
@@ -52,6 +53,7 @@ constexpr Tab<RN> make_tab() {
     for (int l = 0; l < RN; l += 2) {
         const unsigned __int128 h = M / (unsigned)kModuli[l] / (unsigned)(l + 1 < RN ? kModuli[l + 1] : 1);
         bias += h << 19;
+        bias_M += (double)(1 << 19) / ((double)kModuli[l] * (l + 1 < RN ? kModuli[l + 1] : 1));
         for (int j = 0; j < 4; ++j) t.mpair32[l / 2][j] = (uint32_t)(h >> (32 * j));
     }
     for (int j = 0; j < 4; ++j) {
@@ -59,7 +61,7 @@ constexpr Tab<RN> make_tab() {
         t.bias32[j] = (uint32_t)(bias >> (32 * j));
     }
     t.top = (float)(79228162514264337593543950336.0 / (double)M);
-    t.btop = (float)((double)bias / (double)M);
+    t.btop = (float)bias_M;   // (the bias itself passes 2^128 with 14 moduli)
     return t;
 }
 

@@ -547,8 +547,8 @@ int ceil_log2(int64_t v) {
 }  // namespace
 
 // The rule of the dispatch, both sides measured (us per call, residues /
-// DFMA): 1003 x 130 57 / 70, 4000 x 80 63 / 82, 5000 x 100 62 / 181,
-// 15053 x 301 142 / 1588, 100000 x 2000 7494 / 336087; below, where the
+// DFMA): 1003 x 130 54 / 70, 4000 x 80 59 / 82, 5000 x 100 62 / 181,
+// 15053 x 301 141 / 1588, 100000 x 2000 6980 / 336087; below, where the
 // residue form's passes and launches cost about 55 us, 2000 x 64 56 / 35,
 // 3200 x 64 58 / 35, 1000 x 32 55 / 23 (orders up to 64 use the DFMA kernel's
 // 32 x 32 tiles, which spread better).
