@@ -198,6 +198,7 @@ struct Mlp {
         const int sms = ctx->num_sms;
         if (B > cap) {
             const int64_t c = std::max<int64_t>(B, 64);
+            cap = 0;   // until all of them are there: an allocation may fail
             Xb.get<bf16>(ctx, c * ldI);
             H1.get<bf16>(ctx, c * ldH);
             H2.get<bf16>(ctx, c * ldH);
@@ -207,6 +208,7 @@ struct Mlp {
         }
         if (train && B > tcap) {
             const int64_t c = std::max<int64_t>(B, 64);
+            tcap = 0;
             dY.get<bf16>(ctx, c * ldO);
             dZ2.get<bf16>(ctx, c * ldH);
             dZ1.get<bf16>(ctx, c * ldH);
