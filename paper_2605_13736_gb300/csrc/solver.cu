@@ -609,7 +609,7 @@ static void prepare_path(Problem *P) {
     if (path == P->path && N == P->N && P->bS.ptr) return;
     P->drop_graphs();   // the captured factorizations point at the old buffers
     P->path = path;
-    P->N = N;
+    P->N = -1;            // until every buffer below is there: an allocation may fail
     Ctx *ctx = P->ctx;
     dvec(ctx, P->bS, N * N);
     dvec(ctx, P->bL, N * N);
@@ -642,6 +642,7 @@ static void prepare_path(Problem *P) {
         dvec(ctx, P->bwf, D.m_E);       // m_E floats
         dvec(ctx, P->bsol_g, D.m_E);
     }
+    P->N = N;
 }
 
 // Tensor-core condensation: FP32 transposed copy of A (once; A is constant
@@ -669,6 +670,7 @@ static void prepare_tc(Problem *P) {
     if (!P->bAfT.ptr) P->bAfT.get<float>(ctx, (size_t)std::max<int64_t>(D.n_d, 1) * pl.ldt);
     if (!P->bvf.ptr) P->bvf.get<float>(ctx, (size_t)pl.ldt);
     if (P->tc_prec != prec) {
+        P->tc_prec = -1;
         P->btc_ws.get<char>(ctx, syrk_tc_workspace_bytes(pl, D.n_d, prec));
         P->btc_err.get<int>(ctx, 4);
         P->tc_prec = prec;
@@ -1190,7 +1192,7 @@ static void swap_trial(Problem *P) {
 static double fp64_direction_error(Problem *P, double mu, double dw, double dc) {
     const Dims &D = P->D;
     if (!P->Dchk.dx) {
-        DirView &C = P->Dchk;
+        DirView C;
         C.dx = dvec(P->ctx, P->bcx, D.n);
         C.dd = dvec(P->ctx, P->bcd, D.m_I);
         C.dyg = dvec(P->ctx, P->bcyg, D.m_E);
@@ -1199,6 +1201,7 @@ static double fp64_direction_error(Problem *P, double mu, double dw, double dc) 
         C.dzu = dvec(P->ctx, P->bczu, D.n);
         C.dvl = dvec(P->ctx, P->bcvl, D.m_I);
         C.dvu = dvec(P->ctx, P->bcvu, D.m_I);
+        P->Dchk = C;   // all of them or none
     }
     P->V.copy_dir(P->Dir, P->Dchk);
     Inertia in64 = factor_attempt(P, dw, dc, true);

@@ -90,3 +90,32 @@ def test_network_buffers():
     finally:
         m.mdsip_mlp_destroy(mlp)
         m.mdsip_ctx_destroy(ctx)
+
+
+@pytest.mark.parametrize("precision", [m.MDSIP_PREC_FP64, m.MDSIP_PREC_BF16])
+def test_problem_buffers(precision):
+    torch = torch_cuda()
+    inst = synth.make_instance(n_d=60, m_E=3000, m_I=4, sigma_a=0.01, seed=9)
+    want, at = None, -1
+    while True:
+        rec, ctx = _context()
+        prob = m.mdsip_problem_create_synthetic(ctx, **m.synth_arrays(inst))
+        try:
+            m.mdsip_set_option_int(prob, "precision", precision, ctx)
+            if precision != m.MDSIP_PREC_FP64:
+                m.mdsip_set_option_int(prob, "direction_check", 1, ctx)
+            out = torch.zeros(m.mdsip_packed_size(prob), dtype=torch.float64, device="cuda")
+            failed = at >= 0 and _oom(rec, at, lambda: m.mdsip_solve(prob, ctx))
+            assert m.STATUS[m.mdsip_solve(prob, ctx)] == "OK"
+            m.mdsip_get_iterate(prob, out, m.MDSIP_MEM_DEVICE, ctx)
+            got = out.cpu().numpy()
+            if want is None:
+                want = got
+            np.testing.assert_array_equal(got, want)
+            if at >= 0 and not failed:
+                break
+            at += 1
+        finally:
+            m.mdsip_problem_destroy(prob)
+            m.mdsip_ctx_destroy(ctx)
+    assert at >= 15
