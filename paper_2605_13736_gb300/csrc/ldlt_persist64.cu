@@ -79,70 +79,90 @@ __device__ __forceinline__ void bar_chain() { asm volatile("bar.sync 2, 128;" ::
 // The 16 x 16 diagonal sub-block at c0 and up to 32 rows below it, together.
 // Warps 0 .. 3 hold one element (ei, ej), ej >= 1, of the block's lower
 // triangle per lane, 30 lanes each; column j goes through `col` (two buffers of
-// 17, one barrier per column); v_it -= (w_i / d) w_t, in that order: w_i w_t
+// 18, one barrier per column); v_it -= (w_i / d) w_t, in that order: w_i w_t
 // leaves the range below 2^-511 and above 2^512, and w_i / d is the L that the
-// rows below use.  Lane 31 of each also
-// forms the next pivot from its value before the column (col[16]), so that its
-// reciprocal is under way while the column's elements are exchanged: a column
-// is one FMA, a reciprocal and two shuffles of latency.  Warps 4 .. 7 take the
-// rows on the FP64 pipes that the chain leaves idle, four threads each with
-// columns strided by four.  (Chain and rows one after the other, with the
-// second Newton step on the FP64 pipe, took 31 of a panel's 77 thousand cycles.)
+// rows below use.  An element gathers what the columns take off it apart until
+// its own four columns are due, so that it rounds at its own magnitude four
+// times at most, not once a column (reconstruction error at N = 100: 1.1e-16
+// rms entry-wise before, 0.67e-16 so; 0.56e-16 with one sum for all columns,
+// which costs an addition per column of the chain, 2 us a panel).  Lane 31 of
+// each warp also forms the next pivot from its value before the column (col[16],
+// col[17]), so that its reciprocal is under way while the column's elements are
+// exchanged: a column is a product, an FMA, a reciprocal and two shuffles of
+// latency.  Warps 4 .. 7 take the rows on the FP64 pipes that the chain leaves
+// idle, four threads each with columns strided by four.  (Chain and rows one
+// after the other, with the second Newton step on the FP64 pipe, took 31 of a
+// panel's 77 thousand cycles; all four columns unrolled, 0.7 us a panel less.)
 __device__ bool q_chain_rows(double *V, double *Ls, double *col, double *s_rc, uint64_t *colbar, uint32_t phase, int c0,
                              int cw, int ei, int ej, int nblk, int nr) {
     bool ok = true;
     const int tid = threadIdx.x, lane = tid & 31;
     if (tid < 128) {
         const bool elem = lane < 30;
-        double v = elem && ei < cw ? V[(c0 + ei) * VP + c0 + ej] : 0.0;
+        // y: the element from its own four columns on, what the columns before take off it until then
+        const double base = elem && ei < cw ? V[(c0 + ei) * VP + c0 + ej] : 0.0;
+        double y = ej < 4 ? base : 0.0;
         double r = rcp_newton(V[c0 * VP + c0]);
-        for (int j = 0; j < cw; ++j) {
-            double *cb = col + (j & 1) * 17;
-            if (j == 0) {
-                if (tid < 16) cb[tid] = V[(c0 + tid) * VP + c0];
-                if (tid == 16) cb[16] = V[(c0 + 1) * VP + c0 + 1];
-            } else if (elem && ej == j) {
-                cb[ei] = v;
-                V[(c0 + ei) * VP + c0 + j] = v;
-            }
-            if (j > 0 && elem && ei == j + 1 && ej == j + 1) cb[16] = v;
-            if (tid == 0) s_rc[c0 + j] = r;
-            __syncwarp();
-            if (lane == 0) tc::mbar_arrive(&colbar[j]);
-            bar_chain();
-            if (j + 1 < cw) {
-                const bool nd = lane == 31;
-                const double wi = cb[nd ? j + 1 : ei], wt = cb[nd ? j + 1 : ej];
-                const double nv = fma(-(wi * r), wt, nd ? cb[16] : v);
-                if (ej > j) v = nv;
-                r = rcp_newton(__shfl_sync(0xffffffffu, nv, 31));
+        for (int j0 = 0; j0 < cw; j0 += 4) {
+            const double add = lane == 31 ? 0.0 : ej >> 2 == (j0 >> 2) + 1 ? base : 0.0;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int j = j0 + u;
+                if (j >= cw) break;
+                double *cb = col + (u & 1) * 18;
+                if (j == 0) {
+                    if (tid < 16) cb[tid] = V[(c0 + tid) * VP + c0];
+                    if (tid == 16) cb[16] = V[(c0 + 1) * VP + c0 + 1];
+                } else if (elem && ej == j) {
+                    cb[ei] = y;
+                    V[(c0 + ei) * VP + c0 + j] = y;
+                }
+                if (j > 0 && elem && ei == j + 1 && ej == j + 1) {
+                    cb[16] = y;
+                    if (u == 3) cb[17] = base;
+                }
+                if (tid == 0) s_rc[c0 + j] = r;
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&colbar[j]);
+                bar_chain();
+                if (j + 1 < cw) {
+                    const bool nd = lane == 31;
+                    const double wi = cb[nd ? j + 1 : ei], wt = cb[nd ? j + 1 : ej];
+                    double x = fma(-(wi * r), wt, nd ? cb[16] : y);
+                    if (u == 3) x += nd ? cb[17] : add;
+                    if (ej > j) y = x;
+                    r = rcp_newton(__shfl_sync(0xffffffffu, x, 31));
+                }
             }
         }
     } else {
         const int q = lane & 3, x = (tid - 128) >> 2, total = min(32, nblk + nr);
         const bool live = x < total;
         const int row = live ? (x < nblk ? c0 + 16 + x : QN + x - nblk) : c0;
-        double v[4];
+        double v[4], y[4];
 #pragma unroll
-        for (int s = 0; s < 4; ++s) v[s] = live ? V[row * VP + c0 + q + 4 * s] : 0.0;
+        for (int s = 0; s < 4; ++s) {
+            v[s] = live ? V[row * VP + c0 + q + 4 * s] : 0.0;
+            y[s] = s == 0 ? v[s] : 0.0;
+        }
         const bool any = __any_sync(0xffffffffu, live);
-        for (int j = 0; j < cw; ++j) {
-            if (!any) break;
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+            if (!any || j >= cw) break;
             if (!tc::mbar_wait(&colbar[j], phase)) ok = false;   // column j and its reciprocal are there
-            const int sl = j >> 2;
-            const double own = sl == 0 ? v[0] : sl == 1 ? v[1] : sl == 2 ? v[2] : v[3];
-            const double l = __shfl_sync(0xffffffffu, own, (lane & ~3) | (j & 3)) * s_rc[c0 + j];
+            const double l = __shfl_sync(0xffffffffu, y[j >> 2], (lane & ~3) | (j & 3)) * s_rc[c0 + j];
             if (live && (j & 3) == q) Ls[row * LP + c0 + j] = l;
 #pragma unroll
             for (int s = 0; s < 4; ++s)
                 if (4 * s + 3 > j) {
                     const int t = q + 4 * s;
-                    v[s] = fma(-l, t > j ? V[(c0 + t) * VP + c0 + j] : 0.0, v[s]);
+                    y[s] = fma(-l, t > j ? V[(c0 + t) * VP + c0 + j] : 0.0, y[s]);
+                    if (4 * s == j + 1) y[s] += v[s];
                 }
         }
         if (live) {
 #pragma unroll
-            for (int s = 0; s < 4; ++s) V[row * VP + c0 + q + 4 * s] = v[s];
+            for (int s = 0; s < 4; ++s) V[row * VP + c0 + q + 4 * s] = y[s];
         }
     }
     return ok;
@@ -158,12 +178,15 @@ __device__ void q_rows(double *V, double *Ls, const double *s_rc, int c0, int fi
         const bool live = x < total;
         if (!__any_sync(0xffffffffu, live)) break;   // warp-uniform: no row in this warp
         const int row = live ? (x < nblk ? c0 + 16 + x : QN + x - nblk) : 0;
-        double v[4];
+        double v[4], y[4];   // as above
 #pragma unroll
-        for (int s = 0; s < 4; ++s) v[s] = live ? V[row * VP + c0 + q + 4 * s] : 0.0;
+        for (int s = 0; s < 4; ++s) {
+            v[s] = live ? V[row * VP + c0 + q + 4 * s] : 0.0;
+            y[s] = s == 0 ? v[s] : 0.0;
+        }
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
-            const double w = __shfl_sync(0xffffffffu, v[j >> 2], (lane & ~3) | (j & 3));
+            const double w = __shfl_sync(0xffffffffu, y[j >> 2], (lane & ~3) | (j & 3));
             const double l = w * s_rc[c0 + j];
             if (live && (j & 3) == q) Ls[row * LP + c0 + j] = l;
             if (j < 15) {
@@ -172,13 +195,14 @@ __device__ void q_rows(double *V, double *Ls, const double *s_rc, int c0, int fi
                     if ((j & 3) == 3 && s == (j >> 2)) continue;   // no column of this slot beyond j
                     const int t = q + 4 * s;
                     const double w2 = t > j ? V[(c0 + t) * VP + c0 + j] : 0.0;
-                    v[s] = fma(-l, w2, v[s]);
+                    y[s] = fma(-l, w2, y[s]);
+                    if (4 * s == j + 1) y[s] += v[s];
                 }
             }
         }
         if (live) {
 #pragma unroll
-            for (int s = 0; s < 4; ++s) V[row * VP + c0 + q + 4 * s] = v[s];
+            for (int s = 0; s < 4; ++s) V[row * VP + c0 + q + 4 * s] = y[s];
         }
     }
 }
@@ -191,15 +215,15 @@ __device__ void q_rank16(double *V, const double *Ls, int nb, bool blk, int nr) 
         const int x = e >> 3, c = 16 + 2 * (e & 7);
         const int row = x < nblk ? 16 + x : QN + x - nblk;
         if (x < nblk && c > row) continue;
-        double a0 = V[row * VP + c], a1 = V[row * VP + c + 1];
+        double a0 = 0.0, a1 = 0.0;
 #pragma unroll
         for (int j = 0; j < 16; ++j) {
             const double l = Ls[row * LP + j];
-            a0 = fma(-l, V[c * VP + j], a0);
-            a1 = fma(-l, V[(c + 1) * VP + j], a1);
+            a0 = fma(l, V[c * VP + j], a0);
+            a1 = fma(l, V[(c + 1) * VP + j], a1);
         }
-        V[row * VP + c] = a0;
-        V[row * VP + c + 1] = a1;
+        V[row * VP + c] -= a0;
+        V[row * VP + c + 1] -= a1;
     }
 }
 
@@ -404,7 +428,7 @@ __global__ void __launch_bounds__(Q_THREADS, 1) k_bk_persist64(P64Args q) {
     uint8_t *ring = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(psm_raw) + 1023) & ~uintptr_t(1023));
     double *V = reinterpret_cast<double *>(ring + RL * Q_STAGE);   // [32 + Q_OWN][VP]: block rows, own rows
     double *Ls = V + (QN + Q_OWN) * VP;                            // [32 + Q_OWN][LP]: L below the 16 x 16 sub-blocks
-    __shared__ double s_d[QN], s_rc[QN], s_col[34];
+    __shared__ double s_d[QN], s_rc[QN], s_col[36];
     __shared__ unsigned long long s_cmax[QN], s_sm[QN];
     __shared__ int s_se[QN];
     __shared__ uint4 s_km[16];   // -(bias + k M) modulo 2^128, k = -8 .. 7 at k + 8
