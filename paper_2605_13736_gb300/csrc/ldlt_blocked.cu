@@ -1868,7 +1868,7 @@ bool ldlt_blocked_available(int64_t N) { return blocked_config(N, true).C > 0 &&
 // back where it stopped) at every order: it needs no pivoting panel unless a
 // panel fails the column test, and a first panel that fails costs some 10 us at
 // N <= 128 (where its first column fails) and 30 to 50 above.  Convex Newton-step shape, persistent / per-panel launches, FP64: N =
-// 33 0.085 / 0.14 ms, 351 0.35 / 1.47, 1036 0.98 / 4.46, 2050 2.42 / 11.1; FP32
+// 33 0.077 / 0.14 ms, 351 0.35 / 1.47, 1036 0.95 / 4.46, 2050 2.37 / 11.1; FP32
 // updates (whose per-panel launches replayed as one graph): N = 562 0.23 / 0.49, 2050
 // 0.82 / 1.73 ms; 24 solves of 114 to 350 at once 79 / 84 ms in all.
 bool ldlt_persistent_path(int64_t N, int spec) {

@@ -28,7 +28,7 @@
 //      2^-48 sum_j |x_ij x_cj|): the scale of the factorization's other roundings, not
 //      entry-wise; grid barrier.
 // Against the 64-column form with DFMA trailing tiles (its first panel's tiles
-// alone took 215 us): N = 2050 7.90 -> 2.42 ms, 4050 30.6 -> 8.1 ms.  A panel
+// alone took 215 us): N = 2050 7.90 -> 2.37 ms, 4050 30.6 -> 8.1 ms.  A panel
 // takes 30 us at N = 351 to 1036, its pivot chain about 12 of them (32 columns
 // of an FP64 multiply and FMA, a reciprocal, an exchange); at N = 2050 37 us, 16
 // of them the tiles, whose read-back (13 residues to 128-bit integers per
