@@ -67,7 +67,8 @@ struct Ctx {
     void *alloc(size_t bytes);
     void release(void *p, size_t bytes);
     void *scratch_at_least(size_t bytes);
-    // memory for the length of one call: through the hooks, or stream-ordered
+    // memory for the length of one call: through the hooks, or stream-ordered from a pool
+    cudaMemPool_t pool = nullptr;
     void *lease(size_t bytes);
     void give_back(void *p, size_t bytes);
 };
