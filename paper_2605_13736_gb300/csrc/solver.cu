@@ -73,7 +73,10 @@ cudaMemPool_t join_lease_pool(int device) {
         props.allocType = cudaMemAllocationTypePinned;
         props.location.type = cudaMemLocationTypeDevice;
         props.location.id = device;
-        MDSIP_CUDA(cudaMemPoolCreate(&l.pool, &props));
+        if (cudaMemPoolCreate(&l.pool, &props) != cudaSuccess) {   // none here: plain allocations
+            cudaGetLastError();
+            return l.pool = nullptr;
+        }
         uint64_t keep = (uint64_t)4 << 30;
         cudaMemPoolSetAttribute(l.pool, cudaMemPoolAttrReleaseThreshold, &keep);
     }
@@ -92,10 +95,10 @@ void leave_lease_pool(int device) {
 }  // namespace
 
 void *Ctx::lease(size_t bytes) {
-    if (has_hooks) return alloc(bytes);
-    if (!pool && device < 64) pool = join_lease_pool(device);
+    if (!has_hooks && !pool && device < 64) pool = join_lease_pool(device);
+    if (!pool) return alloc(bytes);
     void *p = nullptr;
-    const cudaError_t e = pool ? cudaMallocFromPoolAsync(&p, bytes, pool, stream) : cudaMallocAsync(&p, bytes, stream);
+    const cudaError_t e = cudaMallocFromPoolAsync(&p, bytes, pool, stream);
     if (e != cudaSuccess) {
         cudaGetLastError();
         throw Error{MDSIP_ERR_OOM, std::string("device memory pool: ") + cudaGetErrorString(e)};
@@ -105,11 +108,11 @@ void *Ctx::lease(size_t bytes) {
 
 void Ctx::give_back(void *p, size_t bytes) {
     if (!p) return;
-    if (has_hooks) {
-        cudaStreamSynchronize(stream);   // the hook may hand the memory to anyone
-        release(p, bytes);
-    } else {
+    if (pool) {
         cudaFreeAsync(p, stream);
+    } else {
+        cudaStreamSynchronize(stream);   // a hook may hand the memory to anyone
+        release(p, bytes);
     }
 }
 
